@@ -98,7 +98,10 @@ typedef struct {
     void *cuda_stream;         /* cudaStream_t to run on; NULL = library-owned */
     int32_t myers_only;        /* 1: every pattern on the Myers/Hyyro bit-vector scan;
                                   0 (default): one-word patterns with K <= 2 use the
-                                  automaton scan where a class has >= 32 of them */
+                                  automaton scan where a class has >= 32 of them, and
+                                  large steps look candidate ends up in the gram index
+                                  (exact; same output) where that costs less than
+                                  scanning every pattern */
     int32_t graphs;            /* 1: launch each step as a captured CUDA graph,
                                   updated in place while its shape repeats */
     uint32_t groups_per_warp;  /* lane groups (32 patterns each) a scan warp runs
@@ -119,7 +122,8 @@ typedef struct {
                                   pattern's first 32 rows are computed while none
                                   of them comes within K of a match (the rows below
                                   then all exceed K), every word otherwise; same
-                                  output.  1: every word at every step */
+                                  output.  1: every word at every step, and no gram
+                                  index (as myers_only) */
     int32_t record_order;      /* filtered output only; same records either way.
                                   0 (default): automatic.  1: the filter writes
                                   each piece's records at a position fixed by the
@@ -149,8 +153,11 @@ typedef struct {
     uint64_t launches;       /* kernels launched by the library */
     uint64_t text_bytes;     /* new stream bytes processed */
     uint64_t cells;          /* Sellers cells: sum over patterns of l_p x bytes */
-    uint64_t word_steps;     /* bit-vector word updates of the forward scan */
-    uint64_t candidates;     /* ends with min distance <= K (forward scan) */
+    uint64_t word_steps;     /* bit-vector word updates of the forward scan (none for
+                                patterns that a step looks up in the gram index) */
+    uint64_t candidates;     /* ends with min distance <= K (forward scan, gram index;
+                                under edit costs the index adds ends whose edits
+                                alone would fit) */
     uint64_t hits;           /* hits of Eq. 2 handed to the filter */
     uint64_t kept;           /* records emitted */
     uint64_t reruns;         /* steps re-run after a buffer grew */

@@ -93,9 +93,16 @@ void free_ctx(oasm_ctx* c) {
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   auto f = [](void* p) { if (p) cudaFree(p); };
-  f(c->d_m); f(c->d_K); f(c->d_mem_off); f(c->d_peq_rev); f(c->d_wpat);
+  f(c->d_m); f(c->d_K); f(c->d_mem_off); f(c->d_peq_rev); f(c->d_bytes);
   f(c->d_pdir); f(c->d_pent); f(c->d_pbytes); f(c->d_poff); f(c->pset.p); f(c->d_pbloom);
-  for (auto& b : c->buckets) { f(b.d_groups); f(b.d_peq); f(b.d_peq_hi); f(b.d_wrow); }
+  for (auto* bs : {&c->buckets, &c->grams.rest})
+    for (auto& b : *bs) { f(b.d_groups); f(b.d_peq); f(b.d_peq_hi); f(b.d_wrow); }
+  {
+    Grams& gr = c->grams;
+    f(const_cast<uint32_t*>(gr.scan.bits)); f(const_cast<uint4*>(gr.scan.dir));
+    f(const_cast<GramEntry*>(gr.t.entries)); f(const_cast<uint8_t*>(gr.t.edits));
+    f(const_cast<uint32_t*>(gr.t.peq_fwd)); f(gr.susp.p); f(gr.ctr.p);
+  }
   f(c->d_tails); f(c->d_hdr); f(c->d_mem);
   f(c->arena.p); f(c->upload.p); f(c->stage[0].d.p); f(c->stage[1].d.p); f(c->cand.p); f(c->keys.p);
   f(c->keys_alt.p); f(c->out.p); f(c->pool_hdr.p); f(c->pool_mem.p); f(c->pair_pool.p);
@@ -269,7 +276,8 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
     if (prepare_scan_kernels(max_smem) != cudaSuccess ||
-        prepare_prefilter_kernel(64 << 10) != cudaSuccess) {
+        prepare_prefilter_kernel(64 << 10) != cudaSuccess ||
+        prepare_gram_kernels() != cudaSuccess) {
       cudaGetLastError();
       fail(ctx, OASM_ECUDA, "setting the scan kernels' shared-memory limit failed");
       return bail(OASM_ECUDA);
@@ -350,6 +358,12 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   // the records' copies to the host run on their own stream, beside the next step
   if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
     return bail(fail(ctx, OASM_ECUDA, "cudaStreamCreate failed"));
+  // the tables' copies and the cleared state are complete before the first
+  // step, which runs on a stream that does not wait for the default one
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+    cudaGetLastError();
+    return bail(fail(ctx, OASM_ECUDA, "preparing the context failed"));
+  }
   *out = ctx;
   return OASM_OK;
 }
@@ -881,6 +895,18 @@ int oasm_reset_stats(oasm_ctx* ctx) {
 
 void* oasm_cuda_stream(oasm_ctx* ctx) { return ctx ? static_cast<void*>(ctx->stream) : nullptr; }
 
+// The buckets beside the gram index take the settings of the class they are part of.
+static void share_tuning(oasm_ctx* ctx) {
+  for (Bucket& r : ctx->grams.rest)
+    for (const Bucket& b : ctx->buckets)
+      if (b.W == r.W && b.algo == r.algo && (b.max_nseg == 1) == (r.max_nseg == 1)) {
+        r.gpw = r.groups.size() > 1 ? b.gpw : 1;
+        r.warps = b.warps;
+        r.chunk = b.chunk;
+        r.region_scale = b.region_scale;
+      }
+}
+
 int oasm_get_tuning(oasm_ctx* ctx, oasm_tuning* out, uint32_t cap, uint32_t* n) {
   if (!ctx || !n) return OASM_EINVAL;
   *n = uint32_t(ctx->buckets.size());
@@ -922,6 +948,7 @@ int oasm_set_tuning(oasm_ctx* ctx, const oasm_tuning* t, uint32_t n) {
     b.chunk = t[i].chunk;
     b.region_scale = t[i].region_scale;
   }
+  share_tuning(ctx);
   return OASM_OK;
 }
 
@@ -1057,6 +1084,7 @@ int oasm_autotune(oasm_ctx* ctx, const uint8_t* dsample, size_t n, char* report,
     js += "]}";
   }
   js += "]}";
+  share_tuning(ctx);
   if (report && report_cap) {
     snprintf(report, report_cap, "%s", js.c_str());
   }

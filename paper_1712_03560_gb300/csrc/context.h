@@ -253,6 +253,20 @@ struct DevArray {
   size_t cap = 0;  // elements
 };
 
+// The gram index (grams.cu) of a context: its tables, and the buckets of the
+// patterns that stay on the forward scan while it runs.
+struct Grams {
+  uint32_t n_pat = 0;         // patterns it serves; 0: no index
+  GramTables t{};
+  GramScan scan{};            // tables; a step adds its text and buffers
+  double rate = 0;            // expected suspects per text symbol
+  double clk = 0;             // clocks of an SM per symbol it takes
+  double saved_clk = 0;       // and saves, against the forward scan of every pattern
+  std::vector<Bucket> rest;
+  DevArray<unsigned long long> susp;
+  DevArray<unsigned long long> ctr;  // suspects of each slice
+  int off_steps = 0;          // steps left without the index (suspects too dense)
+};
 
 struct StepPlan {
   std::vector<WorkItem> items;
@@ -265,6 +279,7 @@ struct StepPlan {
   int sb = 1, kb = 10;
   uint64_t new_bytes = 0;
   bool ordered = false;              // records written in canonical order (no record sort)
+  bool grams = false;                // the gram index and the rest buckets scan this step
 };
 
 // Pinned host staging for fed bytes, with its device copy.  Two of them
@@ -316,7 +331,7 @@ struct oasm_ctx {
   // replaces the bit-parallel scan and verification
   bool weighted = false;
   oasm_costs costs{1, 1, 1};
-  uint8_t* d_wpat = nullptr;  // [n_pat][OASM_MAX_PATTERN_LEN] pattern symbols
+  uint8_t* d_bytes = nullptr;  // [n_pat][OASM_MAX_PATTERN_LEN] pattern symbols
   std::vector<Bucket> buckets;
   // piece filter (cfg.prefilter_piece): tables of the patterns it serves
   uint32_t n_pref_pat = 0;
@@ -328,6 +343,7 @@ struct oasm_ctx {
   uint8_t* d_pbytes = nullptr;
   uint32_t* d_poff = nullptr;
   DevArray<unsigned long long> pset;  // (end, pattern) set, capacity a power of two
+  Grams grams;
 
   // streams
   std::vector<StreamRec> streams;
@@ -420,6 +436,10 @@ int wait_event(oasm_ctx* ctx, cudaEvent_t ev);
 void free_ctx(oasm_ctx* c);
 int build_prefilter(oasm_ctx* ctx, const std::vector<char>& pref);
 int build_tables(oasm_ctx* ctx);
+// Tables of the gram index; served[p] = 1 for the patterns it takes (all 0
+// when it would not pay).
+int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>& served);
+void finish_grams(oasm_ctx* ctx);
 void choose_piece_filter(const uint8_t* const* pat, const uint32_t* len, const uint32_t* k,
                          uint32_t n, uint32_t piece, uint8_t* on_filter);
 StepParams make_params(oasm_ctx* ctx, const WorkItem* d_items, uint32_t n_items, int sb, int kb,
@@ -430,6 +450,11 @@ int prepare_records(oasm_ctx* ctx, StepPlan& pl);
 int bucket_gpw(const oasm_ctx* ctx, const Bucket& b);
 int64_t region_len(oasm_ctx* ctx, const Bucket& b, int64_t total_ends);
 int plan_step(oasm_ctx* ctx, StepPlan& pl);
+void plan_regions(oasm_ctx* ctx, StepPlan& pl);
+// The buckets a step scans: all, or those of the patterns the gram index leaves.
+inline std::vector<Bucket>& step_buckets(oasm_ctx* ctx, const StepPlan& pl) {
+  return pl.grams ? ctx->grams.rest : ctx->buckets;
+}
 cudaError_t record_event(oasm_ctx* ctx, cudaEvent_t e, cudaStream_t s);
 int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Region* d_regions,
                  const CopyChunk* d_chunks);

@@ -1,0 +1,355 @@
+// gram_tables.cu -- which patterns the gram index (grams.cu) takes, their
+// grams, and the index's tables.
+#include <cmath>
+
+#include "context.h"
+
+namespace oasm {
+namespace {
+
+// Clocks of one SM per text symbol and forward-scan lane group, measured on a
+// GB300: 5.3 for a word of Myers/Hyyro (or the cut-off scan, one word) and for
+// the K = 2 automaton, 4.5 and 3.5 for the packed automata of K = 1 and K = 0;
+// 5.5 for a weighted wave-front group.
+double group_cost(int W, int algo) {
+  if (algo == kAlgoWeighted) return 5.5;
+  if (algo == 1) return 3.5;
+  if (algo == 2) return 4.5;
+  return algo == kAlgoCut || algo == 3 ? 5.3 : 5.3 * W;
+}
+double buckets_cost(const std::vector<Bucket>& bs) {
+  double c = 0;
+  for (const Bucket& b : bs)
+    for (const LaneGroup& g : b.groups) c += group_cost(b.W, b.algo) / g.nseg;
+  return c;
+}
+// Clocks of one SM per suspect (the ends run: about 25 for one word, 20 more
+// per further word), per false table bit (a directory look-up), and per text
+// symbol and gram length.
+constexpr double kEnds = 25.0, kEndsWord = 20.0, kLookup = 8.0, kLength = 0.12;
+
+constexpr int kMaxGram2 = 13;  // symbols of a gram, 2-bit text
+constexpr int kMaxPiece = 12;  // ... of a piece that may hold an edit
+const int kByteLens[] = {3, 4, 6, 8};
+
+// Grams of one length: key << 32 | pattern << 8 | pattern symbols after it.
+using GramList = std::vector<uint64_t>;
+
+// Orders the list by key (stable; three passes of 11 bits).
+void sort_by_key(GramList& g) {
+  GramList t(g.size());
+  for (int shift = 32; shift < 64; shift += 11) {
+    std::vector<uint32_t> at(2049, 0u);
+    for (uint64_t x : g) at[((x >> shift) & 2047u) + 1] += 1;
+    for (int i = 0; i < 2048; ++i) at[i + 1] += at[i];
+    for (uint64_t x : g) t[at[(x >> shift) & 2047u]++] = x;
+    g.swap(t);
+  }
+  g.erase(std::unique(g.begin(), g.end()), g.end());
+}
+
+// The j disjoint pieces of b symbols with the smallest sum of w (w[x] = chance
+// that a text position matches symbols x .. x + b - 1).  f: scratch.
+double place(const std::vector<double>& w, int m, int j, int b, std::vector<double>& f,
+             std::vector<int>* at) {
+  // f[t][e]: the best t pieces within the first e symbols (e >= b t)
+  const size_t row = size_t(m) + 1;
+  f.resize(size_t(j + 1) * row);
+  std::fill(f.begin(), f.begin() + row, 0.0);
+  for (int t = 1; t <= j; ++t) {
+    double* cur = &f[t * row];
+    const double* prev = &f[(t - 1) * row];
+    double best = 1e30;
+    for (int e = b * t; e <= m - b * (j - t); ++e)
+      cur[e] = best = std::min(best, prev[e - b] + w[e - b]);
+  }
+  at->assign(j, 0);
+  int e = m;
+  for (int t = j; t >= 1; --t) {
+    const double* cur = &f[t * row];
+    while (e > b * t && cur[e - 1] <= cur[e]) --e;
+    e -= b;
+    (*at)[t - 1] = e;
+  }
+  return f[j * row + m];
+}
+
+// Grams such that every string within one edit of s contains one of them,
+// each with the symbols of s up to its end: the strings with one symbol
+// missing (s without its last symbol is contained in s itself, in s with its
+// last symbol changed or missing and in s with an insertion before it; s
+// without its first symbol likewise), then changes and insertions further
+// inside.
+// s: b 2-bit symbols, the first in the low bits.
+template <class F>
+void one_edit(uint32_t s, int b, F put) {
+  auto sym = [&](int i) { return (s >> (2 * i)) & 3u; };
+  auto below = [&](int i) { return s & ((1u << (2 * i)) - 1u); };
+  for (int i = 0; i < b; ++i) {  // without symbol i (of a run of one symbol: its last)
+    if (i + 1 < b && sym(i) == sym(i + 1)) continue;
+    put(below(i) | ((s >> (2 * i + 2)) << (2 * i)), b - 1, i == b - 1 ? b - 1 : b);
+  }
+  for (int i = 1; i + 1 < b; ++i)
+    for (uint32_t c = 0; c < 4; ++c)
+      if (c != sym(i)) put((s & ~(3u << (2 * i))) | (c << (2 * i)), b, b);
+  for (int i = 2; i + 1 < b; ++i)  // before symbol i
+    for (uint32_t c = 0; c < 4; ++c)
+      if (c != sym(i))  // (equal: the same string as an insertion after it)
+        put(below(i) | (c << (2 * i)) | ((s >> (2 * i)) << (2 * i + 2)), b + 1, b);
+}
+
+}  // namespace
+
+int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>& served) {
+  const uint32_t n = ctx->n_pat;
+  served.assign(n, 0);
+  Grams& gr = ctx->grams;
+  // myers_only and full_words ask for the forward scan's own forms; the keys
+  // of the (end, pattern) set hold 24 pattern bits
+  if (ctx->cfg.myers_only || ctx->cfg.full_words || n >= (1u << 24)) return OASM_OK;
+  std::vector<double> cnt(256, 0.0);
+  double tot = 0;
+  int n_scan = 0;
+  for (uint32_t p = 0; p < n; ++p) {
+    if (pref[p]) continue;
+    ++n_scan;
+    for (uint8_t c : ctx->pats[p]) cnt[c] += 1, tot += 1;
+  }
+  if (n_scan < kLaneGroup) return OASM_OK;  // fewer run one group in the segment mapping
+  const double scan_all = buckets_cost(ctx->buckets);
+  const double share = scan_all / n_scan;  // the forward scan's clocks per pattern
+  // at most four symbols that two adjacent bits tell apart: 2-bit text (other
+  // symbols of the text read as one of the four; the ends run tells)
+  int shift2 = -1, distinct = 0;
+  for (int c = 0; c < 256; ++c) distinct += cnt[c] > 0;
+  for (int s = 0; s <= 6 && distinct <= 4 && shift2 < 0; ++s) {
+    int seen = 0;
+    bool ok = true;
+    for (int c = 0; c < 256; ++c)
+      if (cnt[c] > 0) {
+        const int bit = 1 << ((c >> s) & 3);
+        ok = ok && !(seen & bit);
+        seen |= bit;
+      }
+    if (ok) shift2 = s;
+  }
+  const bool two = shift2 >= 0;
+  std::vector<double> fr(256, 0.0);  // chance of a symbol (2-bit text: of its code)
+  for (int c = 0; c < 256; ++c) fr[two ? (c >> shift2) & 3 : c] += cnt[c] / tot;
+  if (two)
+    for (int c = 0; c < 4; ++c) fr[c] = std::max(fr[c], 1e-3);
+  std::vector<uint8_t> edits(n, 0);
+  const int cmin = ctx->weighted ? int(std::min({ctx->costs.sub, ctx->costs.ins, ctx->costs.del})) : 1;
+  GramList by_len[kMaxGram2 + 1];
+  double ends_clk = 0;
+  std::vector<double> ps, w, scratch;
+  std::vector<uint8_t> sym;
+  std::vector<int> at, best_at;
+  for (uint32_t p = 0; p < n; ++p) {
+    const int m = ctx->m[p], E = ctx->K[p] / cmin, W = (m + 31) / 32;
+    edits[p] = uint8_t(E);
+    if (pref[p]) continue;
+    sym.resize(m);
+    ps.resize(m);
+    for (int i = 0; i < m; ++i) {
+      const uint8_t c = ctx->pats[p][i];
+      sym[i] = two ? uint8_t((c >> shift2) & 3) : c;
+      ps[i] = fr[sym[i]];
+    }
+    auto windows = [&](int b) {
+      w.resize(m - b + 1);
+      for (int x = 0; x + b <= m; ++x) {
+        double r = 1;
+        for (int i = 0; i < b; ++i) r *= ps[x + i];
+        w[x] = r;
+      }
+    };
+    const double per_suspect = kEnds + kEndsWord * (W - 1);
+    // (a) E + 1 unedited pieces, as long as an equal split allows
+    double best = 1e30, best_q = 0;
+    int best_b = 0;
+    bool best_edit = false;
+    {
+      const int j = E + 1;
+      int b = std::min(m / j, kMaxGram2);
+      if (!two) {
+        int q = 0;
+        for (int L : kByteLens) q = L <= m / j ? L : q;
+        b = q;
+      }
+      if (b >= (two ? 5 : 3)) {
+        windows(b);
+        const double q = place(w, m, j, b, scratch, &at);
+        best = q * per_suspect + j * (kLookup / (32.0 * kGramMaxWords));
+        best_b = b;
+        best_at = at;
+        best_q = q;
+      }
+    }
+    // (b) E / 2 + 1 pieces with at most one edit each (2-bit text)
+    if (two && E >= 1) {
+      const int j = E / 2 + 1, b = std::min(m / j, kMaxPiece);
+      if (b >= 6) {
+        windows(b);
+        at.clear();
+        place(w, m, j, b, scratch, &at);
+        // deletions and changes of a uniform text symbol, about 7 b strings
+        const double q = j * (b / std::pow(4.0, b - 1) + 3.0 * (b - 2) / std::pow(4.0, b) +
+                              3.0 * (b - 3) / std::pow(4.0, b + 1));
+        const double cost = q * per_suspect + j * 7.0 * b * (kLookup / (32.0 * kGramMaxWords));
+        if (cost < best) {
+          best = cost;
+          best_b = b;
+          best_at = at;
+          best_edit = true;
+          best_q = q;
+        }
+      }
+    }
+    if (!best_b || best > 0.7 * share) continue;
+    served[p] = 1;
+    gr.n_pat += 1;
+    ends_clk += best_q * per_suspect;
+    gr.rate += best_q;
+    auto put = [&](uint32_t key, int len, int end) {  // end: pattern symbols up to the gram's end
+      by_len[len].push_back((uint64_t(key) << 32) | (uint64_t(p) << 8) | uint64_t(m - end));
+    };
+    for (int x : best_at) {
+      uint64_t k = 0;
+      for (int i = 0; i < best_b; ++i) k |= uint64_t(sym[x + i]) << ((two ? 2 : 8) * i);
+      if (best_edit)
+        one_edit(uint32_t(k), best_b, [&](uint32_t u, int len, int end) { put(u, len, x + end); });
+      else
+        put(two || best_b <= 4 ? uint32_t(k)
+                               : uint32_t(k) * kGramMixLo + uint32_t(k >> 32) * kGramMixHi,
+            best_b, x + best_b);
+    }
+  }
+  auto none = [&]() {
+    served.assign(n, 0);
+    gr.n_pat = 0;
+    return OASM_OK;
+  };
+  if (gr.n_pat < uint32_t(kLaneGroup)) return none();
+  // per length: a table of one bit per gram (direct, or hashed to the size
+  // that fits), and a directory
+  struct Len {
+    int len;
+    const GramList* g;
+    size_t distinct = 0;
+    int bits = 10;  // log2 of the table's bits
+  };
+  std::vector<Len> lens;
+  size_t n_grams = 0;
+  for (int len = 1; len <= kMaxGram2; ++len) {
+    GramList& g = by_len[len];
+    if (g.empty()) continue;
+    sort_by_key(g);
+    Len L{len, &g};
+    for (size_t i = 0; i < g.size(); ++i) L.distinct += i == 0 || (g[i] >> 32) != (g[i - 1] >> 32);
+    n_grams += g.size();
+    lens.push_back(L);
+  }
+  // a suspect holds 24 entry bits
+  if (n_grams >= (size_t(1) << 24) || lens.size() > size_t(kGramLens)) return none();
+  // doubles the table with the most grams per bit while the budget lasts
+  // (direct tables stop at one bit per key; 256 bits per gram is plenty)
+  auto most = [&](const Len& L) {
+    const int key_bits = two ? 2 * L.len : 32;
+    return key_bits <= L.bits || (size_t(1) << L.bits) >= 256 * L.distinct;
+  };
+  for (Len& L : lens)
+    if (two) L.bits = std::min(L.bits, 2 * L.len);
+  while (true) {
+    size_t words = 0;
+    Len* pick = nullptr;
+    for (Len& L : lens) {
+      words += std::max<size_t>(4, (size_t(1) << L.bits) / 32);
+      if (!most(L) && (!pick || double(L.distinct) / double(size_t(1) << L.bits) >
+                                    double(pick->distinct) / double(size_t(1) << pick->bits)))
+        pick = &L;
+    }
+    if (!pick || words + (size_t(1) << pick->bits) / 32 > kGramMaxWords) break;
+    pick->bits += 1;
+  }
+  std::vector<uint32_t> bits;
+  std::vector<uint4> dir;
+  std::vector<GramEntry> entries;
+  entries.reserve(n_grams);
+  double false_bits = 0;
+  GramScan& a = gr.scan;
+  a.n_len = int(lens.size());
+  a.two_bit = two ? 1 : 0;
+  a.shift2 = two ? uint32_t(shift2) : 0u;
+  for (size_t li = 0; li < lens.size(); ++li) {
+    const Len& L = lens[li];
+    const GramList& list = *L.g;
+    const int len = L.len, key_bits = two ? 2 * len : 32;
+    GramLen& g = a.len[li];
+    if (two) {
+      g.mask_lo = uint32_t((uint64_t(1) << (2 * len)) - 1);
+      g.mask_hi = 0;
+    } else {
+      g.mask_lo = len >= 4 ? 0xffffffffu : (1u << (8 * len)) - 1u;
+      g.mask_hi = len <= 4 ? 0u : len >= 8 ? 0xffffffffu : (1u << (8 * (len - 4))) - 1u;
+    }
+    const bool direct = key_bits <= L.bits;
+    g.mul = direct ? 1u : kGramBitMul;
+    g.shift = direct ? 0u : uint32_t(32 - L.bits);
+    g.word0 = uint32_t(bits.size());
+    bits.resize(bits.size() + std::max<size_t>(4, (size_t(1) << L.bits) / 32), 0u);
+    int db = 4;
+    while ((size_t(1) << db) < 2 * L.distinct) ++db;
+    g.dir0 = uint32_t(dir.size());
+    g.dir_shift = uint32_t(32 - db);
+    g.dir_mask = (1u << db) - 1u;
+    g.max_probe = 0;
+    dir.resize(dir.size() + (size_t(1) << db), make_uint4(0u, 0u, 0u, 0u));
+    for (size_t i = 0; i < list.size();) {
+      const uint32_t key = uint32_t(list[i] >> 32), h = (key * g.mul) >> g.shift;
+      const uint32_t first = uint32_t(entries.size());
+      for (; i < list.size() && uint32_t(list[i] >> 32) == key; ++i)
+        entries.push_back(GramEntry{uint32_t(list[i] >> 8) & 0xffffffu,
+                                    uint16_t(list[i] & 0xffu), uint16_t(len)});
+      bits[g.word0 + (h >> 5)] |= 1u << (h & 31);
+      uint32_t s = (key * kGramDirMul) >> g.dir_shift, pr = 0;
+      while (dir[g.dir0 + s].z != 0) {
+        s = (s + 1) & g.dir_mask;
+        ++pr;
+      }
+      dir[g.dir0 + s] = make_uint4(key, first, uint32_t(entries.size()) - first, 0u);
+      g.max_probe = std::max(g.max_probe, pr);
+    }
+    if (!direct) false_bits += double(L.distinct) / double(size_t(1) << L.bits);
+  }
+  a.n_words = uint32_t((bits.size() + 3) & ~size_t(3));
+  bits.resize(a.n_words, 0u);
+  gr.clk = ends_clk + kLength * double(lens.size()) + kLookup * false_bits;
+  if (gr.clk > 0.7 * scan_all) return none();  // not enough to gain
+  auto up = [&](auto** dst, const auto& v) -> cudaError_t {
+    using T = typename std::decay<decltype(v[0])>::type;
+    T* d = nullptr;
+    cudaError_t e = cudaMalloc(&d, v.size() * sizeof(T));
+    if (e != cudaSuccess) return e;
+    *dst = d;
+    return cudaMemcpy(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+  };
+  CK(up(&a.bits, bits));
+  CK(up(&a.dir, dir));
+  CK(up(&gr.t.entries, entries));
+  CK(up(&gr.t.edits, edits));
+  uint32_t* peq = nullptr;
+  CK(cudaMalloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t)));
+  gr.t.peq_fwd = peq;
+  CK(launch_peq(ctx->d_bytes, ctx->d_m, n, peq, false, ctx->stream));
+  return OASM_OK;
+}
+
+// Clocks per text symbol that the index saves, for the step rule.
+void finish_grams(oasm_ctx* ctx) {
+  Grams& gr = ctx->grams;
+  gr.saved_clk = buckets_cost(ctx->buckets) - buckets_cost(gr.rest) - gr.clk;
+  if (gr.saved_clk <= 0) gr.n_pat = 0;
+}
+
+}  // namespace oasm

@@ -107,6 +107,59 @@ constexpr int kPrefSegMax = 4096;  // start positions per segment
 cudaError_t launch_prefilter(const StepParams& p, const PrefArgs& f, cudaStream_t s);
 cudaError_t prepare_prefilter_kernel(int max_smem_bytes);
 
+// Gram index in front of the forward scan (grams.cu).
+constexpr int kGramThreads = 1024;            // threads of an index scan block (one per SM)
+constexpr uint32_t kGramMaxWords = 32768;     // 128 KiB of table bits in shared memory
+constexpr int kGramLens = 9;                  // gram lengths of an index
+constexpr unsigned kGramOverflow = 1u << 7;   // StepCounters::overflow: suspects over capacity
+// odd multipliers: byte grams of more than four symbols, table bits, directory
+constexpr uint32_t kGramMixLo = 0x9E3779B1u, kGramMixHi = 0x6C8E9CF5u;
+constexpr uint32_t kGramBitMul = 0x9E3779B1u, kGramDirMul = 0x2C1B3C6Du;
+struct GramLen {             // one gram length
+  uint32_t mask_lo, mask_hi; // the gram's symbols within 16 2-bit symbols, or 8 bytes
+  uint32_t mul, shift;       // table bit of a key: (key * mul) >> shift
+  uint32_t word0;            // first word of the length's table
+  uint32_t dir0;             // first directory slot
+  uint32_t dir_shift, dir_mask, max_probe;
+};
+struct GramEntry {           // one gram of a pattern
+  uint32_t pat;
+  uint16_t rest;             // pattern symbols after the gram
+  uint16_t len;              // symbols of the gram
+};
+struct EndSet {              // (arena offset of an end << 24 | pattern) keys; all ones = empty
+  unsigned long long* slots;
+  unsigned long long mask;   // capacity - 1 (a power of two)
+};
+struct GramTables {
+  const GramEntry* entries;
+  const uint8_t* edits;      // [n_pat] most edits of an occurrence (K under unit costs)
+  const uint32_t* peq_fwd;   // [n_pat][256][4] forward match masks
+};
+struct GramScan {
+  GramLen len[kGramLens];
+  int32_t n_len;
+  int32_t two_bit;           // 1: symbols as (byte >> shift2) & 3
+  uint32_t shift2;
+  uint32_t n_words;          // table words (a multiple of 4)
+  const uint32_t* bits;
+  const uint4* dir;          // {key, first entry, entries (0 = empty), -}
+  const uint8_t* arena;
+  unsigned long long t_begin, t_end;  // 512-symbol tiles of this slice
+  unsigned long long* susp;  // arena offset of a gram << 24 | entry
+  unsigned long long cap_susp;
+  unsigned long long* n_susp;
+  StepCounters* ctr;
+};
+cudaError_t prepare_gram_kernels();
+// Match masks [n_pat][256][4] from the patterns' bytes ([n_pat][128]): bit j
+// of a row is symbol j, or the j-th from the end.
+cudaError_t launch_peq(const uint8_t* bytes, const uint8_t* len, uint32_t n_pat, uint32_t* peq,
+                       bool reversed, cudaStream_t s);
+// scan and ends of one slice (two launches)
+cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramScan& a,
+                         const EndSet& set, cudaStream_t s);
+
 cudaError_t launch_verify(const StepParams& p, cudaStream_t s);
 
 constexpr int kSortMaxBins = 256;  // 8-bit digits

@@ -112,9 +112,11 @@ struct StepCounters {
   unsigned long long word_steps;
   unsigned int overflow;     // bit 0 candidates, 1 hits, 2 outputs, 3 pool,
                              // 5 the prefilter's candidate set (with bit 0),
-                             // 6 an ordered record outside its segment (a bug)
+                             // 6 an ordered record outside its segment (a bug),
+                             // 7 the gram index's suspects (with bit 0)
   unsigned int pad;
   unsigned long long n_pref;  // distinct (pattern, end) pairs the prefilter proposed
+  unsigned long long n_gram;  // distinct (pattern, end) pairs the gram index found
 };
 
 // Piece filter (exact pigeonhole prefilter).  A pattern with K errors split

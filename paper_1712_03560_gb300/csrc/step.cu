@@ -7,6 +7,21 @@
 namespace oasm {
 
 constexpr int64_t kPrefSeg = kPrefSegMax;  // start positions per piece-filter segment
+// Clocks per SM that the gram index has to save before a step runs it: its
+// launches and clearing its set cost about 15 us, and planning the regions of
+// a bucket beside it about 100 ns per stream.
+constexpr double kGramMinClk = 30e3, kGramPlanClk = 200.0;
+constexpr size_t kGramSlice = size_t(1) << 27;  // arena symbols per slice of suspects
+constexpr double kGramMaxRate = 2.0;            // suspects per symbol that a slice may hold
+
+// Slices of the arena that share the suspect buffer: their symbols (a
+// multiple of a tile's, at most 256 slices) and count.
+static size_t gram_slice(const StepPlan& pl) {
+  return std::max(kGramSlice, (pl.arena_bytes / 256 + 4095) & ~size_t(4095));
+}
+static size_t gram_slices(const StepPlan& pl) {
+  return (pl.arena_bytes + gram_slice(pl) - 1) / gram_slice(pl);
+}
 
 int plan_step(oasm_ctx* ctx, StepPlan& pl) {
   const int T = ctx->T;
@@ -64,8 +79,25 @@ int plan_step(oasm_ctx* ctx, StepPlan& pl) {
   pl.kb = pb + pl.sb + kLowBits;
   if (pl.kb > 64)
     return fail(ctx, OASM_EINVAL, "step too large for 64-bit hit keys (%d bits)", pl.kb);
-  // regions per bucket
-  for (const Bucket& b : ctx->buckets) {
+  Grams& gr = ctx->grams;
+  int64_t ends = 0;
+  for (const auto& w : pl.items) ends += w.e_new - w.base_pos;
+  pl.grams = gr.n_pat && gr.saved_clk * double(ends) >=
+                             (kGramMinClk + kGramPlanClk * double(pl.items.size()) *
+                                                double(gr.rest.size())) * ctx->num_sms;
+  if (pl.grams && gr.off_steps > 0) {
+    --gr.off_steps;
+    pl.grams = false;
+  }
+  plan_regions(ctx, pl);
+  return OASM_OK;
+}
+
+// Regions per bucket, then the piece filter's segments.
+void plan_regions(oasm_ctx* ctx, StepPlan& pl) {
+  pl.regions.clear();
+  pl.region_off.clear();
+  for (const Bucket& b : step_buckets(ctx, pl)) {
     pl.region_off.push_back(pl.regions.size());
     int64_t total = 0;
     for (const auto& w : pl.items) {
@@ -108,7 +140,6 @@ int plan_step(oasm_ctx* ctx, StepPlan& pl) {
     }
   }
   pl.region_off.push_back(pl.regions.size());
-  return OASM_OK;
 }
 
 cudaError_t record_event(oasm_ctx* ctx, cudaEvent_t e, cudaStream_t s) {
@@ -133,8 +164,34 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
   CK(launch_gather(d_chunks, int(pl.chunks.size()), ctx->arena.p, s));
   ctx->st.launches += pl.chunks.empty() ? 0 : 1;
   if (tm) CK(record_event(ctx, ctx->ev[1], s));
-  for (size_t bi = 0; bi < ctx->buckets.size(); ++bi) {
-    const Bucket& b = ctx->buckets[bi];
+  StepParams P = make_params(ctx, d_items, n_items, pl.sb, pl.kb, pl.ordered);
+  const std::vector<Bucket>& buckets = step_buckets(ctx, pl);
+  topo_add(pl.grams ? 0x61 : 0x60);
+  if (pl.grams || ctx->n_pref_pat)
+    CK(cudaMemsetAsync(ctx->pset.p, 0xff, ctx->pset.cap * sizeof(unsigned long long), s));
+  if (pl.grams) {
+    Grams& gr = ctx->grams;
+    const size_t slices = gram_slices(pl);
+    // whole tiles (the end padding is longer than a tile and holds no text)
+    const size_t n_tiles = (pl.arena_bytes - 16) / 512, slice = gram_slice(pl) / 512;
+    topo_add(slices);
+    CK(cudaMemsetAsync(gr.ctr.p, 0, slices * sizeof(unsigned long long), s));
+    for (size_t q = 0; q < slices; ++q) {
+      GramScan a = gr.scan;
+      a.arena = ctx->arena.p;
+      a.t_begin = std::min(n_tiles, q * slice);
+      a.t_end = std::min(n_tiles, (q + 1) * slice);
+      a.susp = gr.susp.p;
+      a.cap_susp = gr.susp.cap;
+      a.n_susp = gr.ctr.p + q;
+      a.ctr = ctx->d_ctr;
+      CK(launch_grams(P, gr.t, a, EndSet{ctx->pset.p, ctx->pset.cap - 1}, s));
+    }
+    ctx->st.launches += 2 * slices;
+    ctx->st.scan_launches += slices;
+  }
+  for (size_t bi = 0; bi < buckets.size(); ++bi) {
+    const Bucket& b = buckets[bi];
     ScanArgs a{};
     a.groups = b.d_groups;
     a.peq = b.d_peq;
@@ -164,9 +221,8 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
     ctx->st.launches += 1;
     ctx->st.scan_launches += 1;
   }
-  StepParams P = make_params(ctx, d_items, n_items, pl.sb, pl.kb, pl.ordered);
   if (ctx->n_pref_pat) {
-    const size_t nb = ctx->buckets.size();
+    const size_t nb = buckets.size();
     PrefArgs f{};
     f.dir = ctx->d_pdir;
     f.dir_bits = ctx->pdir_bits;
@@ -185,7 +241,6 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
     topo_add(f.n_segs > 0 ? 0x51 : 0x50);
     if (f.n_segs > 0) {
       if (tm) CK(record_event(ctx, ctx->ev[8], s));
-      CK(cudaMemsetAsync(ctx->pset.p, 0xff, ctx->pset.cap * sizeof(unsigned long long), s));
       CK(launch_prefilter(P, f, s));
       ctx->st.launches += 1;
     }
@@ -345,6 +400,37 @@ int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Regi
   return OASM_OK;
 }
 
+// Suspects a slice may hold: half as many again as expected, or, `most`, as
+// many as cost what the index saves (about 30 clocks each).
+static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) {
+  const Grams& gr = ctx->grams;
+  const double syms = double(std::min(pl.arena_bytes, gram_slice(pl)));
+  const double top = std::min(kGramMaxRate, gr.saved_clk / 30.0);
+  const double rate = most ? top : std::min(top, 1.5 * gr.rate + 0.03);
+  return size_t(syms * rate) + (size_t(1) << 14);
+}
+
+// One upload: items | regions | chunks.
+static int upload_plan(oasm_ctx* ctx, StepPlan& pl) {
+  int rc;
+  const size_t bi = pl.items.size() * sizeof(WorkItem);
+  const size_t br = pl.regions.size() * sizeof(Region);
+  const size_t bc = pl.chunks.size() * sizeof(CopyChunk);
+  const size_t o_r = (bi + 255) & ~size_t(255), o_c = (o_r + br + 255) & ~size_t(255);
+  const size_t total = o_c + bc + 256;
+  if ((rc = ensure_host(ctx, &ctx->h_upload, &ctx->h_upload_cap, total, 0))) return rc;
+  if ((rc = ensure(ctx, ctx->upload, total, "step upload"))) return rc;
+  memcpy(ctx->h_upload, pl.items.data(), bi);
+  memcpy(ctx->h_upload + o_r, pl.regions.data(), br);
+  memcpy(ctx->h_upload + o_c, pl.chunks.data(), bc);
+  CK(cudaMemcpyAsync(ctx->upload.p, ctx->h_upload, total, cudaMemcpyHostToDevice, ctx->stream));
+  Flight& f = ctx->flight;
+  f.d_items = reinterpret_cast<const WorkItem*>(ctx->upload.p);
+  f.d_regions = reinterpret_cast<const Region*>(ctx->upload.p + o_r);
+  f.d_chunks = reinterpret_cast<const CopyChunk*>(ctx->upload.p + o_c);
+  return OASM_OK;
+}
+
 // Waits for the launched step, then either grows the buffers that overflowed
 // (*overflow: the caller re-launches from unchanged state) or books the
 // step's timings and moves its records into the streams' queues.
@@ -386,8 +472,25 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     }
     if ((c.overflow & 4u) || c.n_out > P.cap_out)
       if ((rc = ensure_out(ctx, size_t(c.n_out * 5 / 4 + 1024), pl.ordered))) return rc;
-    if (c.overflow & 32u)  // the piece filter's set filled up: room for 4x its inserts
-      if ((rc = ensure_pow2(ctx, ctx->pset, size_t(c.n_pref) * 4, "piece filter set"))) return rc;
+    if (c.overflow & 32u)  // the (end, pattern) set filled up: room for 4x its inserts
+      if ((rc = ensure_pow2(ctx, ctx->pset,
+                            std::max(size_t(c.n_pref + c.n_gram) * 4, 2 * ctx->pset.cap),
+                            "piece filter set")))
+        return rc;
+    if (c.overflow & kGramOverflow) {
+      // suspects past the expected rate: more room up to the rate at which
+      // the index stops paying; past that the text is too repetitive for it,
+      // and this step and the next ones scan every pattern
+      const size_t cap = ctx->grams.susp.cap, most = gram_capacity(ctx, pl, true);
+      if (cap < most) {
+        if ((rc = ensure(ctx, ctx->grams.susp, std::min(most, 8 * cap), "gram suspects"))) return rc;
+      } else {
+        pl.grams = false;
+        ctx->grams.off_steps = 32;
+        plan_regions(ctx, pl);
+        if ((rc = upload_plan(ctx, pl))) return rc;
+      }
+    }
     if ((c.overflow & 8u) || c.n_pool > P.cap_pool) {
       const size_t want = size_t(c.n_pool * 5 / 4 + 1024);
       if ((rc = ensure(ctx, ctx->pool_hdr, want, "window pool"))) return rc;
@@ -399,7 +502,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
   if (tm) {
     float ms = 0;
     cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]); ctx->st.copy_ms += ms;
-    const size_t nb = ctx->buckets.size();
+    const size_t nb = step_buckets(ctx, pl).size();
     const bool pf = ctx->n_pref_pat && pl.region_off[nb + 1] > pl.region_off[nb];
     if (pf) {
       cudaEventElapsedTime(&ms, ctx->ev[1], ctx->ev[8]); ctx->st.scan_ms += ms;
@@ -572,28 +675,19 @@ int step_begin(oasm_ctx* ctx) {
     ctx->h_run_start = reinterpret_cast<unsigned long long*>(p);
     ctx->h_run_start_cap = cap_bytes / sizeof(unsigned long long);
   }
-  if (ctx->n_pref_pat && !ctx->pset.p &&
-      (rc = ensure_pow2(ctx, ctx->pset, size_t(1) << 20, "piece filter set")))
+  if ((ctx->n_pref_pat || pl.grams) && !ctx->pset.p &&
+      (rc = ensure_pow2(ctx, ctx->pset, pl.grams ? 4 * ctx->cand.cap : size_t(1) << 20,
+                        "piece filter set")))
+    return rc;
+  if (pl.grams && ((rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters")) ||
+                   (rc = ensure(ctx, ctx->grams.susp, gram_capacity(ctx, pl, false),
+                                "gram suspects"))))
     return rc;
   if (!ctx->pool_hdr.p) {
     if ((rc = ensure(ctx, ctx->pool_hdr, 1 << 14, "window pool"))) return rc;
     if ((rc = ensure(ctx, ctx->pool_mem, size_t(1 << 14) * (kMaxK + 1), "window pool"))) return rc;
   }
-  // one upload: items | regions | chunks
-  const size_t bi = pl.items.size() * sizeof(WorkItem);
-  const size_t br = pl.regions.size() * sizeof(Region);
-  const size_t bc = pl.chunks.size() * sizeof(CopyChunk);
-  const size_t o_r = (bi + 255) & ~size_t(255), o_c = (o_r + br + 255) & ~size_t(255);
-  const size_t total = o_c + bc + 256;
-  if ((rc = ensure_host(ctx, &ctx->h_upload, &ctx->h_upload_cap, total, 0))) return rc;
-  if ((rc = ensure(ctx, ctx->upload, total, "step upload"))) return rc;
-  memcpy(ctx->h_upload, pl.items.data(), bi);
-  memcpy(ctx->h_upload + o_r, pl.regions.data(), br);
-  memcpy(ctx->h_upload + o_c, pl.chunks.data(), bc);
-  CK(cudaMemcpyAsync(ctx->upload.p, ctx->h_upload, total, cudaMemcpyHostToDevice, ctx->stream));
-  f.d_items = reinterpret_cast<const WorkItem*>(ctx->upload.p);
-  f.d_regions = reinterpret_cast<const Region*>(ctx->upload.p + o_r);
-  f.d_chunks = reinterpret_cast<const CopyChunk*>(ctx->upload.p + o_c);
+  if ((rc = upload_plan(ctx, pl))) return rc;
   // the host staging copies must be done before bytes fed while this step
   // runs may move a staging buffer (a growing buffer is reallocated)
   if (copies) {
@@ -676,7 +770,7 @@ int step_end(oasm_ctx* ctx) {
   uint64_t msum = 0;
   for (uint32_t p = 0; p < ctx->n_pat; ++p) msum += ctx->m[p];
   ctx->st.cells += msum * pl.new_bytes;
-  for (const Bucket& b : ctx->buckets) {
+  for (const Bucket& b : step_buckets(ctx, pl)) {
     uint64_t lanes = 0;
     for (const auto& g : b.groups)
       for (int l = 0; l < kLaneGroup; l += g.nseg) lanes += g.pat[l] >= 0 ? 1 : 0;

@@ -135,15 +135,12 @@ void choose_piece_filter(const uint8_t* const* pat, const uint32_t* len, const u
 // the last row of its last lane; the rows above it in its first lane match
 // every symbol.  Patterns are packed into groups first-fit by decreasing
 // lane count, so short patterns share a warp.
-static int build_weighted(oasm_ctx* ctx) {
+static int build_weighted(oasm_ctx* ctx, std::vector<Bucket>& to, const std::vector<char>& skip) {
   const uint32_t n = ctx->n_pat;
-  std::vector<uint8_t> wp(size_t(n) * OASM_MAX_PATTERN_LEN, 0);
+  std::vector<uint32_t> ids;
   for (uint32_t p = 0; p < n; ++p)
-    std::copy(ctx->pats[p].begin(), ctx->pats[p].end(), wp.begin() + size_t(p) * OASM_MAX_PATTERN_LEN);
-  CK(cudaMalloc(&ctx->d_wpat, wp.size()));
-  CK(cudaMemcpy(ctx->d_wpat, wp.data(), wp.size(), cudaMemcpyHostToDevice));
-  std::vector<uint32_t> ids(n);
-  for (uint32_t p = 0; p < n; ++p) ids[p] = p;
+    if (!skip[p]) ids.push_back(p);
+  if (ids.empty()) return OASM_OK;
   std::stable_sort(ids.begin(), ids.end(),
                    [&](uint32_t a0, uint32_t b0) { return ctx->m[a0] > ctx->m[b0]; });
   std::vector<std::vector<uint32_t>> warps;  // patterns of each group, in lane order
@@ -205,28 +202,28 @@ static int build_weighted(oasm_ctx* ctx) {
                 cudaMemcpyHostToDevice));
   CK(cudaMalloc(&bk.d_wrow, rows.size() * sizeof(uint32_t)));
   CK(cudaMemcpy(bk.d_wrow, rows.data(), rows.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
-  ctx->buckets.push_back(bk);
+  to.push_back(bk);
   return OASM_OK;
 }
 
 int build_tables(oasm_ctx* ctx) {
   const uint32_t n = ctx->n_pat;
-  // reversed, bottom-aligned Peq (verification pass): [p][256][4]
-  std::vector<uint32_t> rev(size_t(n) * 256 * 4, 0u);
-  for (uint32_t p = 0; p < n; ++p) {
-    const auto& s = ctx->pats[p];
-    const int m = int(s.size());
-    for (int j = 0; j < m; ++j) {
-      const uint8_t c = s[m - 1 - j];
-      rev[(size_t(p) * 256 + c) * 4 + (j >> 5)] |= 1u << (j & 31);
-    }
-  }
-  CK(cudaMalloc(&ctx->d_peq_rev, rev.size() * 4));
-  CK(cudaMemcpy(ctx->d_peq_rev, rev.data(), rev.size() * 4, cudaMemcpyHostToDevice));
+  std::vector<uint8_t> bytes(size_t(n) * OASM_MAX_PATTERN_LEN, 0);
+  for (uint32_t p = 0; p < n; ++p)
+    std::copy(ctx->pats[p].begin(), ctx->pats[p].end(),
+              bytes.begin() + size_t(p) * OASM_MAX_PATTERN_LEN);
+  CK(cudaMalloc(&ctx->d_bytes, bytes.size()));
   CK(cudaMalloc(&ctx->d_m, n));
   CK(cudaMalloc(&ctx->d_K, n));
-  CK(cudaMemcpy(ctx->d_m, ctx->m.data(), n, cudaMemcpyHostToDevice));
+  // (on the context's stream, which the kernel that reads them runs on)
+  CK(cudaMemcpyAsync(ctx->d_bytes, bytes.data(), bytes.size(), cudaMemcpyHostToDevice,
+                     ctx->stream));
+  CK(cudaMemcpyAsync(ctx->d_m, ctx->m.data(), n, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpy(ctx->d_K, ctx->K.data(), n, cudaMemcpyHostToDevice));
+  // reversed, bottom-aligned Peq (verification pass): [p][256][4], made on the
+  // device (4 KiB per pattern would otherwise cross the link)
+  CK(cudaMalloc(&ctx->d_peq_rev, size_t(n) * 256 * 4 * sizeof(uint32_t)));
+  CK(launch_peq(ctx->d_bytes, ctx->d_m, n, ctx->d_peq_rev, true, ctx->stream));
   ctx->mem_off.resize(n);
   uint32_t off = 0;
   for (uint32_t p = 0; p < n; ++p) {
@@ -242,7 +239,8 @@ int build_tables(oasm_ctx* ctx) {
   // automaton classes (one per K) when there are at least 32 of them; their
   // lanes are packed with up to kMaxSlots patterns whose lengths sum to <= 32
   // (first-fit over lengths in decreasing order).
-  auto add_bucket = [&](int W, int algo, std::vector<uint32_t> ids) -> int {
+  auto add_bucket = [&](std::vector<Bucket>& to, int W, int algo,
+                        std::vector<uint32_t> ids) -> int {
     Bucket bk;
     bk.W = W;
     bk.algo = algo;
@@ -360,10 +358,18 @@ int build_tables(oasm_ctx* ctx) {
     }
     CK(cudaMalloc(&bk.d_peq, peq.size() * 4));
     CK(cudaMemcpy(bk.d_peq, peq.data(), peq.size() * 4, cudaMemcpyHostToDevice));
-    ctx->buckets.push_back(bk);
+    to.push_back(bk);
     return OASM_OK;
   };
-  if (ctx->weighted) return build_weighted(ctx);
+  if (ctx->weighted) {
+    std::vector<char> skip(n, 0), served;
+    int rc = build_weighted(ctx, ctx->buckets, skip);
+    if (rc) return rc;
+    if ((rc = build_grams(ctx, skip, served)) || !ctx->grams.n_pat) return rc;
+    if ((rc = build_weighted(ctx, ctx->grams.rest, served))) return rc;
+    finish_grams(ctx);
+    return OASM_OK;
+  }
   // patterns for the piece filter instead of the forward scan
   std::vector<char> pref(n, 0);
   if (ctx->cfg.prefilter_piece) {
@@ -381,29 +387,41 @@ int build_tables(oasm_ctx* ctx) {
     int rc = build_prefilter(ctx, pref);
     if (rc) return rc;
   }
-  for (int W = 1; W <= kMaxW; ++W) {
-    std::vector<uint32_t> ids;
-    for (uint32_t p = 0; p < n; ++p)
-      if ((ctx->m[p] + 31) / 32 == W && !pref[p]) ids.push_back(p);
-    if (W == 1 && !ctx->cfg.myers_only) {
-      for (int K = 0; K <= 2; ++K) {
-        std::vector<uint32_t> kid, rest;
-        for (uint32_t p : ids) (ctx->K[p] == K ? kid : rest).push_back(p);
-        if (kid.size() >= size_t(kLaneGroup)) {
-          int rc = add_bucket(1, 1 + K, kid);
-          if (rc) return rc;
-          ids.swap(rest);
+  // scan classes of the patterns that `skip` leaves
+  auto add_classes = [&](std::vector<Bucket>& to, const std::vector<char>& skip) -> int {
+    for (int W = 1; W <= kMaxW; ++W) {
+      std::vector<uint32_t> ids;
+      for (uint32_t p = 0; p < n; ++p)
+        if ((ctx->m[p] + 31) / 32 == W && !skip[p]) ids.push_back(p);
+      if (W == 1 && !ctx->cfg.myers_only) {
+        for (int K = 0; K <= 2; ++K) {
+          std::vector<uint32_t> kid, rest;
+          for (uint32_t p : ids) (ctx->K[p] == K ? kid : rest).push_back(p);
+          if (kid.size() >= size_t(kLaneGroup)) {
+            int rc = add_bucket(to, 1, 1 + K, kid);
+            if (rc) return rc;
+            ids.swap(rest);
+          }
         }
       }
+      if (ids.empty()) continue;
+      // multi-word classes of 32 or more patterns (dictionary mapping) run the
+      // cut-off form of the scan unless every word is asked for
+      const int algo = (W >= 2 && ids.size() >= size_t(kLaneGroup) && !ctx->cfg.full_words)
+                           ? kAlgoCut : 0;
+      int rc = add_bucket(to, W, algo, ids);
+      if (rc) return rc;
     }
-    if (ids.empty()) continue;
-    // multi-word classes of 32 or more patterns (dictionary mapping) run the
-    // cut-off form of the scan unless every word is asked for
-    const int algo = (W >= 2 && ids.size() >= size_t(kLaneGroup) && !ctx->cfg.full_words)
-                         ? kAlgoCut : 0;
-    int rc = add_bucket(W, algo, ids);
-    if (rc) return rc;
-  }
+    return OASM_OK;
+  };
+  int rc = add_classes(ctx->buckets, pref);
+  if (rc) return rc;
+  std::vector<char> served;
+  if ((rc = build_grams(ctx, pref, served))) return rc;
+  if (!ctx->grams.n_pat) return OASM_OK;
+  for (uint32_t p = 0; p < n; ++p) served[p] |= pref[p];
+  if ((rc = add_classes(ctx->grams.rest, served))) return rc;
+  finish_grams(ctx);
   return OASM_OK;
 }
 
@@ -414,7 +432,7 @@ StepParams make_params(oasm_ctx* ctx, const WorkItem* d_items, uint32_t n_items,
   P.K = ctx->d_K;
   P.mem_off = ctx->d_mem_off;
   P.peq_rev = ctx->d_peq_rev;
-  P.wpat = ctx->d_wpat;
+  P.wpat = ctx->d_bytes;
   P.weighted = ctx->weighted ? 1 : 0;
   P.c_sub = int(ctx->costs.sub);
   P.c_ins = int(ctx->costs.ins);

@@ -1,0 +1,148 @@
+"""GPU parity of the gram index (csrc/grams.cu): large steps look up grams of
+the text that a piece of a pattern may appear as, and examine only the ends
+they allow.  The records must equal the oracle's element by element, and those
+of the forward scan alone (cfg.full_words = 1 and myers_only = 1 keep every
+pattern on it), at sizes just above those from which the index runs."""
+import numpy as np
+import pytest
+
+from paper_1712_03560_gb300 import binding as B
+from paper_1712_03560_gb300 import workloads as W
+from parity_util import canon, oracle_rows, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+N_PAT = 1200  # with 100,000 symbols: a little more than the index's least work
+
+
+def dictionary(rng, sigma, n_pat, mlo, mhi, n, kfun, copies=2):
+    alphabet = np.frombuffer(b"ACGT", np.uint8) if sigma == 4 else \
+        rng.permutation(256).astype(np.uint8)[:sigma]
+    ms = rng.integers(mlo, mhi + 1, size=n_pat)
+    ks = [int(kfun(int(m))) for m in ms]
+    pats = [alphabet[rng.integers(0, sigma, size=int(m))] for m in ms]
+    text = alphabet[rng.integers(0, sigma, size=n)]
+    for p, k in zip(pats, ks):
+        for cp in W.edit_copies(rng, p, rng.integers(0, k + 1, size=copies), alphabet):
+            W.plant(rng, text, cp)
+    return pats, ks, text
+
+
+def runs_index(st, st_scan):
+    """The index runs no bit-vector words for the patterns it serves."""
+    return st["word_steps"] < 0.75 * st_scan["word_steps"]
+
+
+# (alphabet, pattern lengths, threshold, text symbols): one to four words, 2-bit
+# and byte text, whole pieces and pieces with an edit, the shortest to the
+# longest grams, odd sizes
+CASES = [(4, 8, 32, lambda m: m // 10, 130_003), (4, 24, 128, lambda m: m // 11, 110_007),
+         (4, 16, 40, lambda m: 0, 100_001), (256, 16, 128, lambda m: min(8, m // 4), 100_013),
+         (20, 33, 96, lambda m: 6, 105_019), (3, 30, 64, lambda m: 2, 100_151),
+         (4, 12, 30, lambda m: 1 + m // 10, 140_009), (256, 16, 32, lambda m: 4, 100_057)]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_index_equals_oracle_and_scan(case):
+    sigma, mlo, mhi, kfun, n = CASES[case]
+    rng = np.random.default_rng(800 + case)
+    pats, ks, text = dictionary(rng, sigma, N_PAT, mlo, mhi, n, kfun)
+    want = oracle_rows(pats, ks, text)
+    got, st = run_gpu(pats, ks, text)
+    scan, st_scan = run_gpu(pats, ks, text, cfg={"full_words": 1, "myers_only": 1})
+    assert len(want) > 0 and canon(got) == canon(scan) == want
+    assert runs_index(st, st_scan)
+    dev, _ = run_gpu(pats, ks, text, device_feed=True, cfg={"graphs": 1})
+    assert canon(dev) == want
+
+
+@pytest.mark.parametrize("mode,output", [("ends", "ends"), ("hits", "all_hits")])
+def test_index_raw_outputs(mode, output):
+    """Every end with D[e] <= K and every hit of Eq. 2: a missed end shows."""
+    rng = np.random.default_rng(820)
+    pats, ks, text = dictionary(rng, 4, N_PAT, 20, 60, 100_003, lambda m: m // 10)
+    got, _ = run_gpu(pats, ks, text, {"output": output})
+    assert canon(got) == oracle_rows(pats, ks, text, mode=mode)
+
+
+def test_index_over_steps_and_streams():
+    """Stream cuts inside occurrences (each step rescans its stored tail),
+    large steps with the index among small ones without it, and many streams
+    of odd lengths in one step."""
+    rng = np.random.default_rng(830)
+    pats, ks, text = dictionary(rng, 4, N_PAT, 18, 70, 260_011, lambda m: m // 10, copies=6)
+    want = oracle_rows(pats, ks, text)
+    cuts = [88_001, 88_002, 88_040, 176_500]
+    rows, _ = run_gpu(pats, ks, text, splits=cuts)
+    assert canon(rows) == want
+    lens = [1, 5, 63, 64, 65, 127, 1000, 4099, 20_001, 90_000]
+    ctx = B.oasm_create(pats, ks, None, {"max_streams": 16})
+    try:
+        parts = np.split(text[:sum(lens)], np.cumsum(lens)[:-1])
+        sids = [B.oasm_open_stream(ctx) for _ in parts]
+        for sid, t in zip(sids, parts):
+            B.oasm_feed(ctx, sid, t)
+            B.oasm_end_stream(ctx, sid)
+        B.oasm_step(ctx)
+        res = B.oasm_drain(ctx)
+        for sid, t in zip(sids, parts):
+            got = [(int(r["pattern_id"]), int(r["decided_at"]), int(r["k"]), int(r["start"]),
+                    int(r["len"])) for r in res[res["stream_id"] == sid]]
+            assert canon(got) == oracle_rows(pats, ks, t)
+    finally:
+        B.oasm_destroy(ctx)
+
+
+def test_index_gives_way_on_repetitive_text():
+    """Every piece matches nearly everywhere: the suspects outgrow their
+    buffer, the step is re-run on the forward scan, and so are the next
+    steps; symbols outside the patterns' alphabet match nothing."""
+    rng = np.random.default_rng(840)
+    unit = np.frombuffer(b"ACGGTCA", np.uint8)
+    pats = [np.roll(np.tile(unit, 5), i % 7)[:25 + i % 9].copy() for i in range(N_PAT)]
+    ks = [int(rng.integers(0, 3)) for _ in pats]
+    text = np.tile(unit, 24_000)[:90_000].copy()
+    text[rng.integers(0, text.size, size=400)] = ord("T")
+    text[40_000:40_100] = ord("N")
+    ctx = B.oasm_create(pats, ks)
+    try:
+        out = []
+        sid = B.oasm_open_stream(ctx)
+        for part in np.split(text, [85_000]):
+            B.oasm_feed(ctx, sid, part)
+            out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 1))
+        st = B.oasm_get_stats(ctx)
+    finally:
+        B.oasm_destroy(ctx)
+    got = [(int(r["pattern_id"]), int(r["decided_at"]), int(r["k"]), int(r["start"]),
+            int(r["len"])) for r in np.concatenate(out)]
+    assert canon(got) == oracle_rows(pats, ks, text)
+    assert st["reruns"] >= 1
+
+
+@pytest.mark.parametrize("costs", [(1, 2, 2), (2, 3, 2), (1, 1, 1), (9, 5, 7)])
+def test_index_under_edit_costs(costs):
+    """K bounds the cost, so the edits are at most K over the cheapest cost."""
+    rng = np.random.default_rng(850)
+    pats, ks, text = dictionary(rng, 4, N_PAT, 10, 40, 100_003, lambda m: m // 7)
+    got, st = run_gpu(pats, ks, text, costs=costs)
+    assert canon(got) == oracle_rows(pats, ks, text, costs=costs)
+    ends, _ = run_gpu(pats, ks, text, {"output": "ends"}, costs=costs)
+    assert canon(ends) == oracle_rows(pats, ks, text, mode="ends", costs=costs)
+
+
+def test_index_runs_of_one_symbol():
+    """Pieces with repeated symbols, where several edits give one string: DNA
+    patterns made of short runs, thresholds 1 to 3."""
+    rng = np.random.default_rng(860)
+    pats, ks = [], []
+    for i in range(N_PAT):
+        p = np.repeat(W.DNA[rng.integers(0, 4, size=20)], rng.integers(1, 4, size=20))
+        pats.append(p[:int(rng.integers(14, 32))].copy())
+        ks.append(1 + i % 3)
+    text = np.repeat(W.DNA[rng.integers(0, 4, size=60_000)], rng.integers(1, 4, size=60_000))
+    for p, k in zip(pats, ks):
+        for cp in W.edit_copies(rng, p, np.full(4, k), W.DNA):
+            W.plant(rng, text, cp)
+    got, _ = run_gpu(pats, ks, text)
+    assert canon(got) == oracle_rows(pats, ks, text)
