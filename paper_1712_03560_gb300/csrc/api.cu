@@ -271,7 +271,11 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   }
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
   if (ctx->num_sms < 1) ctx->num_sms = 1;
-  ctx->sort_blocks = 4 * ctx->num_sms;
+  if ((ctx->sort_blocks = sort_grid(ctx->num_sms)) < 1) {
+    cudaGetLastError();
+    fail(ctx, OASM_ECUDA, "the sort kernel does not fit the device");
+    return bail(OASM_ECUDA);
+  }
   {
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
@@ -343,7 +347,7 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   for (uint32_t i = 0; i < S; ++i) ctx->free_slots.push(i);
   if (cudaMalloc(&ctx->d_ctr, sizeof(StepCounters)) != cudaSuccess ||
       cudaHostAlloc(&ctx->h_ctr, sizeof(StepCounters), cudaHostAllocDefault) != cudaSuccess ||
-      cudaMalloc(&ctx->d_hist, size_t(kSortMaxBins) * ctx->sort_blocks * 4) != cudaSuccess) {
+      cudaMalloc(&ctx->d_hist, sort_hist_len(ctx->sort_blocks) * sizeof(unsigned int)) != cudaSuccess) {
     cudaGetLastError();
     fail(ctx, OASM_ENOMEM, "step counters");
     return bail(OASM_ENOMEM);

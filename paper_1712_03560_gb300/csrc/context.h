@@ -404,8 +404,8 @@ struct oasm_ctx {
   cudaEvent_t done = nullptr;
   cudaEvent_t staged = nullptr;  // host staging copies of the step in flight done
   // executable step graphs, one per step topology (which kernels a step
-  // launches: its scan classes, the piece filter, the sort passes the key
-  // width needs), each updated in place while its topology repeats; the least
+  // launches: its scan classes, the piece filter, the gram index, the record
+  // order), each updated in place while its topology repeats; the least
   // recently used one is dropped when a new topology needs a slot
   struct GraphSlot {
     uint64_t topo = 0;
@@ -416,7 +416,7 @@ struct oasm_ctx {
   std::vector<GraphSlot> graphs;
   uint64_t graph_clock = 0;
   uint64_t step_topo = 0;    // topology of the step being enqueued
-  int sort_blocks = 4 * 152; // radix-sort blocks: four per SM
+  int sort_blocks = 0;       // radix-sort blocks: as many as are resident together
   bool capturing = false;
 
   oasm_stats st{};

@@ -162,12 +162,11 @@ cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramSca
 
 cudaError_t launch_verify(const StepParams& p, cudaStream_t s);
 
-constexpr int kSortMaxBins = 256;  // 8-bit digits
-
 // Stable LSD radix sort (8-bit digits) of keys by bits [lo_bit, hi_bit),
-// with an optional 32-bit payload.  The element count is read on the device
-// from *count (clamped to cap).  On return *keys_out / *vals_out point at
-// whichever buffer of each pair holds the sorted data.
+// with an optional 32-bit payload, in one cooperative launch.  The element
+// count is read on the device from *count (clamped to cap).  On return
+// *keys_out / *vals_out point at whichever buffer of each pair holds the
+// sorted data.
 struct SortArgs {
   unsigned long long* keys;
   unsigned long long* keys_alt;
@@ -176,15 +175,19 @@ struct SortArgs {
   const unsigned long long* count;
   unsigned long long cap;
   int lo_bit, hi_bit;
-  unsigned int* hist;             // kSortMaxBins * nblocks
-  int nblocks;
+  unsigned int* hist;             // sort_hist_len(nblocks) entries
+  int nblocks;                    // sort_grid(): blocks that are resident together
+  unsigned int* bar;              // barrier arrivals, zero before the launch
+  StepCounters* ctr;
 };
+int sort_grid(int num_sms);       // 0: the device cannot say
+size_t sort_hist_len(int nblocks);
 cudaError_t launch_sort(const SortArgs& a, unsigned long long** keys_out, uint32_t** vals_out,
-                        int* launches, cudaStream_t s);
-// dst[i] = src[idx[i]] for i < min(*count, cap)
+                        cudaStream_t s);
+// dst[i] = src[idx[i]] for i < min(ctr->n_out, cap)
 cudaError_t launch_permute(const DevHit* src, const uint32_t* idx, DevHit* dst,
-                           const unsigned long long* count, unsigned long long cap,
-                           int num_sms, cudaStream_t s);
+                           const StepCounters* ctr, unsigned long long cap, int num_sms,
+                           cudaStream_t s);
 cudaError_t launch_filter(const StepParams& p, const unsigned long long* sorted, cudaStream_t s);
 // Carried windows: kFinFlush emits the decidable ones of pairs without hits,
 // kFinCommit writes the new window state; kFinAll does both.

@@ -114,6 +114,7 @@ struct StepCounters {
                              // 5 the prefilter's candidate set (with bit 0),
                              // 6 an ordered record outside its segment (a bug),
                              // 7 the gram index's suspects (with bit 0)
+  unsigned int bar[2];       // barrier arrivals of the hit sort, the record sort
   unsigned int pad;
   unsigned long long n_pref;  // distinct (pattern, end) pairs the prefilter proposed
   unsigned long long n_gram;  // distinct (pattern, end) pairs the gram index found

@@ -276,184 +276,278 @@ __global__ void __launch_bounds__(256) verify_kernel(const StepParams P) {
 }
 
 // ---------------------------------------------------------------- radix sort
+// Stable LSD radix sort, 8-bit digits, every pass in one cooperative launch
+// (the element count is on the device; a few launches per pass, most of them
+// over few keys, cost more than the passes themselves: 37 us a pass with a
+// histogram and a scatter kernel, whose blocks each walked every block's
+// histogram; 1 M keys of six digits 266 -> 122 us, up to 2,048 keys of two
+// digits 74 -> 8 us).
+//   up to kSortTile keys: one block, every pass in shared memory
+//   more: each active block owns a contiguous chunk.  Per pass: its digit
+//     counts; a scan of each digit's counts over the blocks (one digit per
+//     block and turn); the scatter, which ranks a tile of kSortTile keys in
+//     shared memory (warp matching per round of 32 keys with a running count
+//     per digit, scans over the warps and the digits) and writes the tile out
+//     digit run by digit run, consecutive threads on consecutive keys.
+// Blocks meet at bounded grid barriers; what other blocks wrote is read past
+// L1.
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-
-// Keys per block: an even split, but at least 1,024, so a small sort runs on
-// a few blocks and the rest leave at once (each active block reads the whole
-// histogram matrix to find its offsets).
-__device__ __forceinline__ unsigned long long sort_chunk(unsigned long long n) {
-  const unsigned long long even = (n + gridDim.x - 1) / gridDim.x;
-  return even > 1024ull ? even : 1024ull;
-}
-
-// 8-bit digits: one digit per thread in the per-digit scans.
 constexpr int kBins = 256;
-__global__ void __launch_bounds__(kSortThreads)
-    rs_hist(const unsigned long long* __restrict__ keys, const unsigned long long* count,
-            unsigned long long cap, int shift, unsigned int* hist) {
-  __shared__ unsigned int h[kBins];
-  for (int d = threadIdx.x; d < kBins; d += kSortThreads) h[d] = 0;
-  __syncthreads();
-  const unsigned long long n = min(*count, cap);
-  const unsigned long long chunk = sort_chunk(n);
-  const unsigned long long b0 = chunk * blockIdx.x, b1 = min(n, b0 + chunk);
-  const unsigned long long bd = blockDim.x;
-  unsigned long long i = b0 + threadIdx.x;
-  // four loads in flight per thread, then their four counts
-  for (; i + 3 * bd < b1; i += 4 * bd) {
-    const unsigned long long k0 = keys[i], k1 = keys[i + bd], k2 = keys[i + 2 * bd],
-                             k3 = keys[i + 3 * bd];
-    atomicAdd(&h[(k0 >> shift) & (kBins - 1u)], 1u);
-    atomicAdd(&h[(k1 >> shift) & (kBins - 1u)], 1u);
-    atomicAdd(&h[(k2 >> shift) & (kBins - 1u)], 1u);
-    atomicAdd(&h[(k3 >> shift) & (kBins - 1u)], 1u);
+constexpr int kSortPer = 8;                         // keys per thread and tile
+constexpr int kSortTile = kSortThreads * kSortPer;  // 2,048
+constexpr uint32_t kBarrierSpins = 1u << 22;
+
+struct SortSmem {
+  unsigned long long key[kSortTile];
+  uint32_t val[kSortTile];
+  unsigned int wcnt[kSortWarps][kBins];
+  unsigned int base[kBins];    // global position of the digit's next key
+  unsigned int tstart[kBins];  // the digit's first slot in the sorted tile
+  unsigned int wsum[kSortWarps];
+  int stop;
+};
+
+// Exclusive scan of one value per thread, in thread order.
+__device__ __forceinline__ unsigned int sort_scan(SortSmem& sm, unsigned int v) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int t = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += t;
   }
-  for (; i < b1; i += bd) atomicAdd(&h[(keys[i] >> shift) & (kBins - 1u)], 1u);
+  if (lane == 31) sm.wsum[warp] = incl;
   __syncthreads();
-  for (int d = threadIdx.x; d < kBins; d += kSortThreads)
-    hist[blockIdx.x * kBins + d] = h[d];  // block-major
+  unsigned int pre = 0;
+#pragma unroll
+  for (int w = 0; w < kSortWarps; ++w)
+    if (w < warp) pre += sm.wsum[w];
+  __syncthreads();  // wsum is reused by the next call
+  return pre + incl - v;
 }
 
-// Stable scatter.  Each block first finds where its keys of each digit go:
-// all keys of smaller digits, plus the keys of its digit in earlier blocks
-// (thread d walks column d of the block-major histogram).  It
-// then walks its contiguous chunk in tiles of kSortTile keys.  A warp ranks
-// its keys round by round (32 consecutive keys per round, warp matching for
-// the lanes of one digit, a running count per digit); per-digit scans over
-// the warps and over the digits give every key its place in the tile sorted
-// by digit, in shared memory; the tile then goes out with consecutive
-// threads writing consecutive keys of one digit's run.
-constexpr int kSortPer = 8;                             // keys per thread and tile
-constexpr int kSortTile = kSortThreads * kSortPer;      // 2,048
-__global__ void __launch_bounds__(kSortThreads)
-    rs_scatter(const unsigned long long* __restrict__ in, unsigned long long* __restrict__ out,
-               const uint32_t* __restrict__ vin, uint32_t* __restrict__ vout,
-               const unsigned long long* count, unsigned long long cap, int shift,
-               const unsigned int* __restrict__ hist) {
-  constexpr int kOwn = kBins / kSortThreads;  // digits per thread: 1
-  __shared__ unsigned long long skey[kSortTile];
-  __shared__ uint32_t sval[kSortTile];
-  __shared__ unsigned int wcnt[kSortWarps][kBins];
-  __shared__ unsigned int base[kBins];    // global position of the digit's next key
-  __shared__ unsigned int tstart[kBins];  // the digit's first slot in the sorted tile
-  __shared__ unsigned int wsum[kSortWarps];
+// Ranks the tile's keys (registers) by one digit: pos[r] = the key's slot in
+// the tile sorted by digit; returns this thread's digit's count (digit
+// threadIdx.x), its first slot in sm.tstart.
+__device__ __forceinline__ unsigned int rank_tile(SortSmem& sm,
+                                                  const unsigned long long (&key)[kSortPer],
+                                                  int tn, int shift,
+                                                  unsigned int (&pos)[kSortPer]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int d0 = threadIdx.x * kOwn;  // this thread's digits: d0 .. d0 + kOwn - 1
-  const unsigned long long n = min(*count, cap);
-  if (sort_chunk(n) * blockIdx.x >= n) return;  // no keys for this block
-  // exclusive scan of one value per thread, in thread order
-  auto block_excl = [&](unsigned int v) -> unsigned int {
-    unsigned int incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int t = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    unsigned int wpre = 0;
-    for (int w = 0; w < warp; ++w) wpre += wsum[w];
-    __syncthreads();  // wsum is reused by the next call
-    return wpre + incl - v;
-  };
-  {
-    unsigned int tot[kOwn], pre[kOwn], sum = 0;
-#pragma unroll
-    for (int q = 0; q < kOwn; ++q) tot[q] = pre[q] = 0;
-    for (int b = 0; b < int(gridDim.x); ++b) {
-#pragma unroll
-      for (int q = 0; q < kOwn; ++q) {
-        const unsigned int v = hist[b * kBins + d0 + q];
-        tot[q] += v;
-        if (b < int(blockIdx.x)) pre[q] += v;
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < kOwn; ++q) sum += tot[q];
-    unsigned int run = block_excl(sum);
-#pragma unroll
-    for (int q = 0; q < kOwn; ++q) {
-      base[d0 + q] = run + pre[q];
-      run += tot[q];
-    }
-  }
-  const unsigned long long chunk = sort_chunk(n);
-  const unsigned long long b0 = chunk * blockIdx.x, b1 = min(n, b0 + chunk);
   const unsigned lt = (1u << lane) - 1u;
-  for (unsigned long long t0 = b0; t0 < b1; t0 += kSortTile) {
-    const int tn = int(min((unsigned long long)kSortTile, b1 - t0));
 #pragma unroll
-    for (int w = 0; w < kSortWarps; ++w)
+  for (int w = 0; w < kSortWarps; ++w) sm.wcnt[w][threadIdx.x] = 0;
+  __syncthreads();
+  unsigned int dig[kSortPer];
 #pragma unroll
-      for (int q = 0; q < kOwn; ++q) wcnt[w][d0 + q] = 0;
-    __syncthreads();
+  for (int r = 0; r < kSortPer; ++r) {
+    const int e = warp * (kSortPer * 32) + r * 32 + lane;  // tile index: warp-major
+    const bool ok = e < tn;
+    const unsigned d = ok ? unsigned((key[r] >> shift) & (kBins - 1u)) : unsigned(kBins);
+    dig[r] = d;
+    const unsigned peers = __match_any_sync(kFull, d);
+    const unsigned below = __popc(peers & lt);
+    pos[r] = ok ? sm.wcnt[warp][d & (kBins - 1u)] + below : 0u;
+    __syncwarp();
+    if (ok && below == 0) sm.wcnt[warp][d] += __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  // per digit: offsets of the warps' keys, then the digit's start in the tile
+  unsigned int run = 0;
+#pragma unroll
+  for (int w = 0; w < kSortWarps; ++w) {
+    const unsigned int c = sm.wcnt[w][threadIdx.x];
+    sm.wcnt[w][threadIdx.x] = run;
+    run += c;
+  }
+  sm.tstart[threadIdx.x] = sort_scan(sm, run);
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kSortPer; ++r)
+    if (dig[r] < unsigned(kBins)) pos[r] += sm.tstart[dig[r]] + sm.wcnt[warp][dig[r]];
+  return run;
+}
+
+// All active blocks meet (*bar counts arrivals since the step began); false
+// when the bounded wait ran out.
+__device__ __forceinline__ bool sort_barrier(SortSmem& sm, unsigned int* bar, unsigned int target,
+                                             StepCounters* ctr) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    unsigned int seen = 0;
+    uint32_t it = 0;
+    for (; it < kBarrierSpins; ++it) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if (seen >= target) break;
+      __nanosleep(20);
+    }
+    sm.stop = it == kBarrierSpins;
+    // (bit 0 keeps the filter off the unsorted keys)
+    if (sm.stop) atomicOr(&ctr->overflow, (1u << 16) | 1u);
+    __threadfence();
+  }
+  __syncthreads();
+  return sm.stop == 0;
+}
+
+__global__ void __launch_bounds__(kSortThreads, 4)
+    sort_kernel(unsigned long long* keys, unsigned long long* keys_alt, uint32_t* vals,
+                uint32_t* vals_alt, const unsigned long long* count, unsigned long long cap,
+                int lo_bit, int hi_bit, unsigned int* hist, unsigned int* bar,
+                StepCounters* ctr) {
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  SortSmem& sm = *reinterpret_cast<SortSmem*>(sort_smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned long long n = min(*count, cap);
+  // keys per block: an even split, in whole tiles (two or more tiles to a block
+  // where one would do measured slower: 1 M keys of six digits 155 -> 179 us)
+  const unsigned long long tiles = (n + kSortTile - 1) / kSortTile;
+  const unsigned long long chunk = (tiles + gridDim.x - 1) / gridDim.x * kSortTile;
+  const unsigned int nb = n ? unsigned((n + chunk - 1) / chunk) : 0u;
+  if (blockIdx.x >= nb) return;
+  if (n <= kSortTile) {
+    const int passes = (hi_bit - lo_bit + 7) / 8;
     unsigned long long key[kSortPer];
     uint32_t val[kSortPer];
-    unsigned int dig[kSortPer], rank[kSortPer];
 #pragma unroll
     for (int r = 0; r < kSortPer; ++r) {
-      const int e = warp * (kSortPer * 32) + r * 32 + lane;  // tile index: warp-major
-      const bool ok = e < tn;
-      key[r] = ok ? in[t0 + e] : 0ull;
-      val[r] = (ok && vin) ? vin[t0 + e] : 0u;
-      const unsigned d = ok ? unsigned((key[r] >> shift) & (kBins - 1u)) : unsigned(kBins);
-      dig[r] = d;
-      const unsigned peers = __match_any_sync(kFull, d);
-      const unsigned below = __popc(peers & lt);
-      rank[r] = ok ? wcnt[warp][d & (kBins - 1u)] + below : 0u;
-      __syncwarp();
-      if (ok && below == 0) wcnt[warp][d] += __popc(peers);
-      __syncwarp();
+      const int e = warp * (kSortPer * 32) + r * 32 + lane;
+      key[r] = e < int(n) ? keys[e] : 0ull;
+      val[r] = vals && e < int(n) ? vals[e] : 0u;
     }
-    __syncthreads();
-    // per digit: offsets of the warps' keys, then the digit's start in the tile
-    unsigned int cnt[kOwn], sum = 0;
+    for (int shift = lo_bit; shift < hi_bit; shift += 8) {
+      unsigned int pos[kSortPer];
+      rank_tile(sm, key, int(n), shift, pos);
 #pragma unroll
-    for (int q = 0; q < kOwn; ++q) {
+      for (int r = 0; r < kSortPer; ++r)
+        if (warp * (kSortPer * 32) + r * 32 + lane < int(n)) {
+          sm.key[pos[r]] = key[r];
+          sm.val[pos[r]] = val[r];
+        }
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < kSortPer; ++r) {
+        const int e = warp * (kSortPer * 32) + r * 32 + lane;
+        if (e < int(n)) {
+          key[r] = sm.key[e];
+          val[r] = sm.val[e];
+        }
+      }
+      __syncthreads();
+    }
+    unsigned long long* ko = (passes & 1) ? keys_alt : keys;
+    uint32_t* vo = (passes & 1) ? vals_alt : vals;
+#pragma unroll
+    for (int r = 0; r < kSortPer; ++r) {
+      const int e = warp * (kSortPer * 32) + r * 32 + lane;
+      if (e < int(n)) {
+        ko[e] = key[r];
+        if (vals) vo[e] = val[r];
+      }
+    }
+    return;
+  }
+  const unsigned long long b0 = chunk * blockIdx.x, b1 = min(n, b0 + chunk);
+  unsigned int* total = hist + size_t(kBins) * gridDim.x;  // [kBins] keys of each digit
+  unsigned int target = 0;
+  for (int shift = lo_bit; shift < hi_bit; shift += 8) {
+    // digit counts of the block's chunk: hist[digit][block]
+    sm.base[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned long long i = b0 + threadIdx.x;
+    for (; i + 3 * kSortThreads < b1; i += 4 * kSortThreads) {
+      unsigned long long k4[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) k4[q] = __ldcg(keys + i + q * kSortThreads);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) atomicAdd(&sm.base[(k4[q] >> shift) & (kBins - 1u)], 1u);
+    }
+    for (; i < b1; i += kSortThreads)
+      atomicAdd(&sm.base[(__ldcg(keys + i) >> shift) & (kBins - 1u)], 1u);
+    __syncthreads();
+    hist[size_t(threadIdx.x) * gridDim.x + blockIdx.x] = sm.base[threadIdx.x];
+    if (!sort_barrier(sm, bar, target += nb, ctr)) return;
+    // each digit's counts scanned over the blocks: a digit per block and turn,
+    // or, where few blocks would take many turns, per warp (14,000 keys of four
+    // digits on 8 blocks: 114 -> 58 us; 3.7 M on 608: 196 us per block, 226 per
+    // warp)
+    const bool wide = nb >= kBins / 2;
+    for (unsigned int d = wide ? blockIdx.x : blockIdx.x * kSortWarps + warp; d < unsigned(kBins);
+         d += wide ? nb : nb * kSortWarps) {
+      unsigned int* row = hist + size_t(d) * gridDim.x;
       unsigned int run = 0;
+      for (unsigned int c = 0; c < nb; c += wide ? kSortThreads : 32) {
+        const unsigned int j = c + (wide ? threadIdx.x : lane);
+        const unsigned int v = j < nb ? __ldcg(row + j) : 0u;
+        if (wide) {
+          const unsigned int excl = sort_scan(sm, v);
+          if (j < nb) row[j] = run + excl;
+          for (int w = 0; w < kSortWarps; ++w) run += sm.wsum[w];
+          __syncthreads();
+        } else {
+          unsigned int incl = v;
 #pragma unroll
-      for (int w = 0; w < kSortWarps; ++w) {
-        const unsigned int c = wcnt[w][d0 + q];
-        wcnt[w][d0 + q] = run;
-        run += c;
+          for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+          }
+          if (j < nb) row[j] = run + incl - v;
+          run += __shfl_sync(kFull, incl, 31);
+        }
       }
-      cnt[q] = run;
-      sum += run;
+      if (lane == 0) total[d] = run;
     }
-    unsigned int ts = block_excl(sum);
+    if (!sort_barrier(sm, bar, target += nb, ctr)) return;
+    const unsigned int before = sort_scan(sm, __ldcg(total + threadIdx.x));
+    sm.base[threadIdx.x] = before + __ldcg(hist + size_t(threadIdx.x) * gridDim.x + blockIdx.x);
+    for (unsigned long long t0 = b0; t0 < b1; t0 += kSortTile) {
+      const int tn = int(min((unsigned long long)kSortTile, b1 - t0));
+      unsigned long long key[kSortPer];
+      uint32_t val[kSortPer];
+      unsigned int pos[kSortPer];
 #pragma unroll
-    for (int q = 0; q < kOwn; ++q) {
-      tstart[d0 + q] = ts;
-      ts += cnt[q];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kSortPer; ++r) {
-      if (dig[r] < unsigned(kBins)) {
-        const unsigned int pos = tstart[dig[r]] + wcnt[warp][dig[r]] + rank[r];
-        skey[pos] = key[r];
-        sval[pos] = val[r];
+      for (int r = 0; r < kSortPer; ++r) {
+        const int e = warp * (kSortPer * 32) + r * 32 + lane;
+        key[r] = e < tn ? __ldcg(keys + t0 + e) : 0ull;
+        val[r] = vals && e < tn ? __ldcg(vals + t0 + e) : 0u;
       }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < tn; e += kSortThreads) {
-      const unsigned long long k = skey[e];
-      const unsigned d = unsigned((k >> shift) & (kBins - 1u));
-      const unsigned int g = base[d] + unsigned(e) - tstart[d];
-      out[g] = k;
-      if (vout) vout[g] = sval[e];
-    }
-    __syncthreads();
+      const unsigned int cnt = rank_tile(sm, key, tn, shift, pos);
 #pragma unroll
-    for (int q = 0; q < kOwn; ++q) base[d0 + q] += cnt[q];
+      for (int r = 0; r < kSortPer; ++r)
+        if (warp * (kSortPer * 32) + r * 32 + lane < tn) {
+          sm.key[pos[r]] = key[r];
+          sm.val[pos[r]] = val[r];
+        }
+      __syncthreads();
+      for (int e = threadIdx.x; e < tn; e += kSortThreads) {
+        const unsigned long long k = sm.key[e];
+        const unsigned d = unsigned((k >> shift) & (kBins - 1u));
+        const unsigned int g = sm.base[d] + unsigned(e) - sm.tstart[d];
+        keys_alt[g] = k;
+        if (vals) vals_alt[g] = sm.val[e];
+      }
+      __syncthreads();
+      sm.base[threadIdx.x] += cnt;
+    }
+    if (shift + 8 < hi_bit && !sort_barrier(sm, bar, target += nb, ctr)) return;
+    unsigned long long* tk = keys;
+    keys = keys_alt;
+    keys_alt = tk;
+    uint32_t* tv = vals;
+    vals = vals_alt;
+    vals_alt = tv;
   }
 }
 
 __global__ void permute_kernel(const DevHit* __restrict__ src, const uint32_t* __restrict__ idx,
-                               DevHit* __restrict__ dst, const unsigned long long* count,
+                               DevHit* __restrict__ dst, const StepCounters* ctr,
                                unsigned long long cap) {
-  const unsigned long long n = min(*count, cap);
+  if (ctr->overflow & (1u << 16)) return;  // the record sort gave up: idx is incomplete
+  const unsigned long long n = min(ctr->n_out, cap);
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (unsigned long long)gridDim.x * blockDim.x)
     dst[i] = src[idx[i]];
@@ -958,30 +1052,43 @@ cudaError_t launch_verify(const StepParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+int sort_grid(int num_sms) {
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(sizeof(SortSmem))) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sort_kernel, kSortThreads,
+                                                    sizeof(SortSmem)) != cudaSuccess)
+    return 0;
+  return std::min(per_sm, 4) * num_sms;
+}
+
+size_t sort_hist_len(int nblocks) { return size_t(kBins) * (size_t(nblocks) + 1); }
+
 cudaError_t launch_sort(const SortArgs& a, unsigned long long** keys_out, uint32_t** vals_out,
-                        int* launches, cudaStream_t s) {
-  unsigned long long* ka = a.keys;
-  unsigned long long* kb = a.keys_alt;
-  uint32_t* va = a.vals;
-  uint32_t* vb = a.vals_alt;
-  int nl = 0;
-  for (int shift = a.lo_bit; shift < a.hi_bit; shift += 8) {
-    rs_hist<<<a.nblocks, kSortThreads, 0, s>>>(ka, a.count, a.cap, shift, a.hist);
-    rs_scatter<<<a.nblocks, kSortThreads, 0, s>>>(ka, kb, va, vb, a.count, a.cap, shift, a.hist);
-    nl += 2;
-    std::swap(ka, kb);
-    std::swap(va, vb);
-  }
-  *keys_out = ka;
-  if (vals_out) *vals_out = va;
-  *launches = nl;
-  return cudaGetLastError();
+                        cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(a.nblocks));
+  cfg.blockDim = dim3(kSortThreads);
+  cfg.dynamicSmemBytes = sizeof(SortSmem);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, sort_kernel, a.keys, a.keys_alt, a.vals, a.vals_alt, a.count, a.cap,
+                         a.lo_bit, a.hi_bit, a.hist, a.bar, a.ctr);
+  const bool odd = ((a.hi_bit - a.lo_bit + 7) / 8) & 1;
+  *keys_out = odd ? a.keys_alt : a.keys;
+  if (vals_out) *vals_out = odd ? a.vals_alt : a.vals;
+  return e;
 }
 
 cudaError_t launch_permute(const DevHit* src, const uint32_t* idx, DevHit* dst,
-                           const unsigned long long* count, unsigned long long cap,
-                           int num_sms, cudaStream_t s) {
-  permute_kernel<<<grid_for(cap, 256, num_sms * 8), 256, 0, s>>>(src, idx, dst, count, cap);
+                           const StepCounters* ctr, unsigned long long cap, int num_sms,
+                           cudaStream_t s) {
+  permute_kernel<<<grid_for(cap, 256, num_sms * 8), 256, 0, s>>>(src, idx, dst, ctr, cap);
   return cudaGetLastError();
 }
 

@@ -251,12 +251,11 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
   if (tm) CK(record_event(ctx, ctx->ev[3], s));
   unsigned long long* sorted = P.keys;
   if (ctx->rules.output == OASM_OUT_FILTERED) {
-    int nl = 0;
     SortArgs sa{P.keys, P.keys_alt, nullptr, nullptr, &ctx->d_ctr->n_hits, P.cap_hits,
-                kKBits, pl.kb, ctx->d_hist, ctx->sort_blocks};
-    CK(launch_sort(sa, &sorted, nullptr, &nl, s));
-    topo_add(0x100 + nl);
-    ctx->st.launches += uint64_t(nl);
+                kKBits, pl.kb, ctx->d_hist, ctx->sort_blocks, &ctx->d_ctr->bar[0], ctx->d_ctr};
+    CK(launch_sort(sa, &sorted, nullptr, s));
+    topo_add(0x100);
+    ctx->st.launches += 1;
     if (tm) CK(record_event(ctx, ctx->ev[4], s));
     if (pl.ordered) {
       // records by segment; the window state is written only after the scan
@@ -285,21 +284,21 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
                        s));
     ctx->st.launches += 2;
   } else {  // emitted records -> canonical order (work item, pattern, decided_at, k, length)
-    int nl = 0;
     unsigned long long* ks = nullptr;
     uint32_t* vs = nullptr;
     SortArgs sa{ctx->okeys.p, ctx->okeys_alt.p, ctx->ovals.p, ctx->ovals_alt.p,
-                &ctx->d_ctr->n_out, P.cap_out, 0, pl.kb, ctx->d_hist, ctx->sort_blocks};
-    CK(launch_sort(sa, &ks, &vs, &nl, s));
-    topo_add(0x200 + nl);
-    CK(launch_permute(ctx->out.p, vs, ctx->out_sorted[ctx->rec_buf].p, &ctx->d_ctr->n_out, P.cap_out,
+                &ctx->d_ctr->n_out, P.cap_out, 0, pl.kb, ctx->d_hist, ctx->sort_blocks,
+                &ctx->d_ctr->bar[1], ctx->d_ctr};
+    CK(launch_sort(sa, &ks, &vs, s));
+    topo_add(0x200);
+    CK(launch_permute(ctx->out.p, vs, ctx->out_sorted[ctx->rec_buf].p, ctx->d_ctr, P.cap_out,
                       ctx->num_sms, s));
     // where each work item's (stream's) run of records starts
     CK(launch_runs(ks, P, ctx->run_start.p, s));
     CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
                        (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                        s));
-    ctx->st.launches += uint64_t(nl) + 2;
+    ctx->st.launches += 3;
   }
   if (tm) CK(record_event(ctx, ctx->ev[5], s));
   CK(cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, sizeof(StepCounters), cudaMemcpyDeviceToHost, s));
