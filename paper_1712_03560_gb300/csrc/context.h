@@ -37,7 +37,8 @@ struct NvtxRange {
 
 constexpr size_t kFrontPad = 1024;   // arena bytes before the first work item
 constexpr size_t kEndPad = 2048;     // arena bytes after the last one
-constexpr size_t kChunk = 1 << 20;   // largest gather copy per block
+constexpr size_t kChunk = 1 << 16;   // largest gather copy per block
+constexpr size_t kShortChunk = 4096; // ... per warp, where no copy of a step is longer
 
 struct Piece {
   bool dev;
@@ -276,6 +277,7 @@ struct StepPlan {
   std::vector<size_t> region_off;    // per bucket
   std::vector<CopyChunk> chunks;
   size_t arena_bytes = 0;
+  size_t longest_chunk = 0;
   int sb = 1, kb = 10;
   uint64_t new_bytes = 0;
   bool ordered = false;              // records written in canonical order (no record sort)

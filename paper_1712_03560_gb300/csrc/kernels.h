@@ -79,7 +79,9 @@ struct CopyChunk {
   uint32_t len;
   uint32_t pad;
 };
-cudaError_t launch_gather(const CopyChunk* chunks, int n, uint8_t* arena, cudaStream_t s);
+// short_chunks: a warp per chunk instead of a block
+cudaError_t launch_gather(const CopyChunk* chunks, int n, bool short_chunks, uint8_t* arena,
+                          cudaStream_t s);
 
 // Piece filter over segments of the step's text: exact matches of pattern
 // pieces propose candidate ends, deduplicated through an open-addressing set.

@@ -26,20 +26,82 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr uint32_t kInvalid = 0xffffffffu;
 
 // ---------------------------------------------------------------- gather
-__global__ void gather_kernel(const CopyChunk* __restrict__ chunks, int n, uint8_t* arena) {
-  for (int c = blockIdx.x; c < n; c += gridDim.x) {
+// 16 bytes at byte offset `mis` of the 32 bytes a | b.
+__device__ __forceinline__ uint4 shift_bytes(const uint4& a, const uint4& b, unsigned mis) {
+  const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  const unsigned r = 8 * (mis & 3);
+  uint4 o;
+  switch (mis >> 2) {  // uniform over a chunk
+    case 0:
+      o = make_uint4(__funnelshift_r(w[0], w[1], r), __funnelshift_r(w[1], w[2], r),
+                     __funnelshift_r(w[2], w[3], r), __funnelshift_r(w[3], w[4], r));
+      break;
+    case 1:
+      o = make_uint4(__funnelshift_r(w[1], w[2], r), __funnelshift_r(w[2], w[3], r),
+                     __funnelshift_r(w[3], w[4], r), __funnelshift_r(w[4], w[5], r));
+      break;
+    case 2:
+      o = make_uint4(__funnelshift_r(w[2], w[3], r), __funnelshift_r(w[3], w[4], r),
+                     __funnelshift_r(w[4], w[5], r), __funnelshift_r(w[5], w[6], r));
+      break;
+    default:
+      o = make_uint4(__funnelshift_r(w[3], w[4], r), __funnelshift_r(w[4], w[5], r),
+                     __funnelshift_r(w[5], w[6], r), __funnelshift_r(w[6], w[7], r));
+  }
+  return o;
+}
+
+// Copies of any alignment, one per block (long chunks) or per warp (short
+// ones: packets and tails).  Whole 16-byte vectors at the destination's
+// alignment; a source of another alignment is read in its own aligned vectors
+// (only those that lie inside the chunk), each once, the other half coming
+// from the next lane.  The bytes before and after go one by one.  Bound by
+// memory: 64 MiB 122 -> 33 us (byte copies of unaligned texts ran at 70 GB/s).
+template <bool kWarp>
+__global__ void __launch_bounds__(256)
+    gather_kernel(const CopyChunk* __restrict__ chunks, int n, uint8_t* arena) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int me = kWarp ? lane : int(threadIdx.x), team = kWarp ? 32 : 256;
+  const int first = kWarp ? int(blockIdx.x) * 8 + warp : int(blockIdx.x);
+  const int step = kWarp ? int(gridDim.x) * 8 : int(gridDim.x);
+  for (int c = first; c < n; c += step) {
     const CopyChunk ch = chunks[c];
     uint8_t* dst = arena + ch.dst_off;
     const uint8_t* src = ch.src;
-    const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) |
-                       ch.len) & 15u) == 0;
-    if (vec) {
-      const uint4* s4 = reinterpret_cast<const uint4*>(src);
-      uint4* d4 = reinterpret_cast<uint4*>(dst);
-      for (uint32_t i = threadIdx.x; i < ch.len / 16; i += blockDim.x) d4[i] = s4[i];
-    } else {
-      for (uint32_t i = threadIdx.x; i < ch.len; i += blockDim.x) dst[i] = src[i];
+    uint32_t head = min(ch.len, uint32_t(-reinterpret_cast<uintptr_t>(dst)) & 15u);
+    const unsigned mis = unsigned(reinterpret_cast<uintptr_t>(src + head)) & 15u;
+    if (mis > head) head = min(ch.len, head + 16u);  // the first aligned vector starts in the chunk
+    const uint32_t body = ch.len - head;
+    // vectors whose source (two aligned vectors where it is unaligned) lies
+    // inside the chunk
+    const uint32_t nv = mis == 0 ? body / 16 : body + mis < 32 ? 0u : (body + mis - 16) / 16;
+    const uint4* s4 = reinterpret_cast<const uint4*>(src + head - mis);
+    uint4* d4 = reinterpret_cast<uint4*>(dst + head);
+    if (mis == 0) {
+      uint32_t i = me;
+      for (; i + 3 * team < nv; i += 4 * team) {
+        const uint4 v0 = s4[i], v1 = s4[i + team], v2 = s4[i + 2 * team], v3 = s4[i + 3 * team];
+        d4[i] = v0;
+        d4[i + team] = v1;
+        d4[i + 2 * team] = v2;
+        d4[i + 3 * team] = v3;
+      }
+      for (; i < nv; i += team) d4[i] = s4[i];
+    } else if (nv) {
+      // (vector nv is the last one's second half: inside the chunk)
+      for (uint32_t i = me; i - lane < nv; i += team) {
+        const uint4 a = s4[min(i, nv)];
+        uint4 b;
+        b.x = __shfl_down_sync(kFull, a.x, 1);
+        b.y = __shfl_down_sync(kFull, a.y, 1);
+        b.z = __shfl_down_sync(kFull, a.z, 1);
+        b.w = __shfl_down_sync(kFull, a.w, 1);
+        if (lane == 31) b = s4[min(i + 1, nv)];
+        if (i < nv) d4[i] = shift_bytes(a, b, mis);
+      }
     }
+    for (uint32_t i = me; i < head; i += team) dst[i] = src[i];
+    for (uint32_t i = head + 16 * nv + me; i < ch.len; i += team) dst[i] = src[i];
   }
 }
 
@@ -1039,9 +1101,13 @@ int grid_for(unsigned long long n, int threads, int cap_blocks) {
 
 }  // namespace
 
-cudaError_t launch_gather(const CopyChunk* chunks, int n, uint8_t* arena, cudaStream_t s) {
+cudaError_t launch_gather(const CopyChunk* chunks, int n, bool short_chunks, uint8_t* arena,
+                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  gather_kernel<<<min(n, 65535), 256, 0, s>>>(chunks, n, arena);
+  if (short_chunks)
+    gather_kernel<true><<<min((n + 7) / 8, 65535), 256, 0, s>>>(chunks, n, arena);
+  else
+    gather_kernel<false><<<min(n, 65535), 256, 0, s>>>(chunks, n, arena);
   return cudaGetLastError();
 }
 

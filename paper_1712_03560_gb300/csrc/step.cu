@@ -54,6 +54,7 @@ int plan_step(oasm_ctx* ctx, StepPlan& pl) {
       if (left <= 0) break;
       const size_t n = size_t(std::min<int64_t>(left, int64_t(pc.n)));
       const uint8_t* src = pc.dev ? pc.dptr : ctx->stage[pc.sb].d.p + pc.host_off;
+      pl.longest_chunk = std::max(pl.longest_chunk, std::min(kChunk, n));
       for (size_t o = 0; o < n; o += kChunk) {
         CopyChunk ch{src + o, dst + o, uint32_t(std::min(kChunk, n - o)), 0};
         pl.chunks.push_back(ch);
@@ -161,7 +162,9 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
   if (tm) CK(record_event(ctx, ctx->ev[0], s));
   CK(cudaMemsetAsync(ctx->d_ctr, 0, sizeof(StepCounters), s));
   CK(cudaMemsetAsync(ctx->pair_pool.p, 0xff, size_t(n_items) * ctx->n_pat * sizeof(int32_t), s));
-  CK(launch_gather(d_chunks, int(pl.chunks.size()), ctx->arena.p, s));
+  const bool short_chunks = pl.longest_chunk <= kShortChunk;
+  topo_add(short_chunks ? 1 : 0);
+  CK(launch_gather(d_chunks, int(pl.chunks.size()), short_chunks, ctx->arena.p, s));
   ctx->st.launches += pl.chunks.empty() ? 0 : 1;
   if (tm) CK(record_event(ctx, ctx->ev[1], s));
   StepParams P = make_params(ctx, d_items, n_items, pl.sb, pl.kb, pl.ordered);
