@@ -616,40 +616,63 @@ __global__ void permute_kernel(const DevHit* __restrict__ src, const uint32_t* _
 }
 
 // ---------------------------------------------------------------- filter
-struct Hit {
-  uint32_t pair;
-  int64_t start;
-  int32_t len;
-  int32_t k;
+// A pair's keys decoded: the hit's start, length and level.
+struct PairKeys {
+  int64_t base;          // base_pos
+  int32_t len0;          // m - K
+  uint64_t mask;         // start bits
+  __device__ __forceinline__ int64_t start(uint64_t key) const {
+    return base + int64_t((key >> kLowBits) & mask);
+  }
+  __device__ __forceinline__ int len(uint64_t key) const {
+    return int(uint32_t(key) >> kKBits & 31u) + len0;
+  }
 };
 
-__device__ __forceinline__ Hit decode(uint64_t key, const StepParams& P) {
-  Hit h;
-  h.pair = uint32_t(key >> (P.start_bits + kLowBits));
-  const int p = int(h.pair % P.n_pat);
-  const WorkItem& w = P.items[h.pair / P.n_pat];
-  h.start = w.base_pos + int64_t((key >> kLowBits) & ((1ull << P.start_bits) - 1));
-  h.len = int32_t((key >> kKBits) & 31u) + P.m[p] - P.K[p];
-  h.k = int32_t(key & 15u);
-  return h;
-}
-
+// Filter window of one pair.  The level that is pending (idx) is also kept in
+// registers, so a hit's rules touch the level rows only to store.
 struct Window {
   int pend;
   int idx;
-  MemRow rows[kMaxK + 1];
+  uint32_t valid;           // levels that hold a row
+  int64_t top_start;        // row idx
+  int32_t top_len;
+  int64_t start[kMaxK + 1];
+  int32_t len[kMaxK + 1];
   unsigned long long rpos;  // ordered records: the segment's first position
   uint32_t nrec;            // records the segment wrote so far
 };
 
-__device__ void emit(const StepParams& P, Window& W, uint32_t pair, int p, int lv,
-                     const MemRow& r, int64_t f, const WorkItem& w) {
+__device__ __forceinline__ void open_window(Window& W, int K) {
+  W.pend = 0;
+  W.idx = K;
+  W.valid = 0;
+  W.nrec = 0;
+  W.rpos = 0;
+}
+
+__device__ __forceinline__ void load_window(Window& W, const WinHdr& hd, const MemRow* rows,
+                                            int K) {
+  W.pend = 1;
+  W.idx = hd.idx;
+  for (int lv = 0; lv <= K; ++lv) {
+    const MemRow r = rows[lv];
+    W.start[lv] = r.start;
+    W.len[lv] = r.len;
+    W.valid |= r.valid ? 1u << lv : 0u;
+  }
+  W.top_start = W.start[W.idx];
+  W.top_len = W.len[W.idx];
+}
+
+__device__ void emit(const StepParams& P, Window& W, uint32_t pair, int p, int lv, int64_t start,
+                     int len, int64_t f, const WorkItem& w) {
   DevHit h;
-  h.start = uint64_t(r.start);
+  h.start = uint64_t(start);
   h.decided_at = uint64_t(f);
   h.pattern = uint32_t(p);
   h.slot = w.slot;
-  h.len = uint32_t(r.len);
+  h.len = uint32_t(len);
   h.k = uint32_t(lv);
   if (P.ordered) {
     const unsigned long long o = W.rpos + W.nrec++;
@@ -662,7 +685,7 @@ __device__ void emit(const StepParams& P, Window& W, uint32_t pair, int p, int l
     atomicOr(&P.ctr->overflow, 4u);
     return;
   }
-  put_record(P, o, h, out_key(P, pair, w, f, lv, r.len, P.m[p], P.K[p]));
+  put_record(P, o, h, out_key(P, pair, w, f, lv, len, P.m[p], P.K[p]));
 }
 
 // A segment's record count, read by the scan (ordered records).
@@ -676,49 +699,44 @@ __device__ __forceinline__ void close_segment(const StepParams& P, const Window&
 // at 1 on insertion and grows by one per processed symbol.
 __device__ void flush(const StepParams& P, Window& W, uint32_t pair, int p, int K,
                       const WorkItem& w) {
-  const MemRow& top = W.rows[W.idx];
-  const int64_t f = top.start + top.len - 1;
+  const int64_t f = W.top_start + W.top_len - 1;
   int64_t acc = 0;
-  for (int lv = W.idx; lv <= K; ++lv) {
-    const MemRow& r = W.rows[lv];
-    if (!r.valid) continue;
-    const int64_t lhs = (f - r.start + 1) - acc;
-    const bool keep = (lv == W.idx) || (P.rules.cmp == OASM_CMP_GT ? lhs > r.len : lhs >= r.len);
+  for (uint32_t left = W.valid & (~0u << W.idx); left; left &= left - 1) {
+    const int lv = __ffs(left) - 1;
+    const int64_t start = W.start[lv];
+    const int len = W.len[lv];
+    const int64_t lhs = (f - start + 1) - acc;
+    const bool keep = (lv == W.idx) || (P.rules.cmp == OASM_CMP_GT ? lhs > len : lhs >= len);
     if (keep) {
-      emit(P, W, pair, p, lv, r, f, w);
-      acc = (P.rules.acc == OASM_ACC_SUM) ? acc + r.len : r.len;
+      emit(P, W, pair, p, lv, start, len, f, w);
+      acc = (P.rules.acc == OASM_ACC_SUM) ? acc + len : len;
     }
   }
   W.pend = 0;
   W.idx = K;
-  for (int lv = 0; lv <= K; ++lv) W.rows[lv].valid = 0;
+  W.valid = 0;
 }
 
 // R1-R3 applied to one hit met in (i, l) order (event form of Algorithm 1).
-__device__ void apply(const StepParams& P, Window& W, uint32_t pair, int p, int K,
-                      const WorkItem& w, const Hit& h) {
-  if (W.pend) {
-    const MemRow& top = W.rows[W.idx];
-    if (h.start > top.start + top.len - 1) flush(P, W, pair, p, K, w);
-  }
-  MemRow nr;
-  nr.start = h.start;
-  nr.len = h.len;
-  nr.valid = 1;
+__device__ __forceinline__ void apply(const StepParams& P, Window& W, uint32_t pair, int p, int K,
+                                      const WorkItem& w, int64_t start, int len, int k) {
+  if (W.pend && start > W.top_start + W.top_len - 1) flush(P, W, pair, p, K, w);
+  bool put = false;
   if (!W.pend) {  // an empty window opens at the hit's level
     W.pend = 1;
-    W.idx = h.k;
-    W.rows[h.k] = nr;
-  } else if (h.k < W.idx) {  // R1
-    W.idx = h.k;
-    W.rows[h.k] = nr;
-  } else if (h.k == W.idx) {  // R2 / R3
-    const MemRow& cur = W.rows[W.idx];
-    const int64_t ce = cur.start + cur.len - 1, ne = h.start + h.len - 1;
-    bool rep = false;
-    if (P.rules.replace == OASM_REPLACE_CONTAINED) rep = h.start >= cur.start && ne <= ce;
-    else if (P.rules.replace == OASM_REPLACE_SAME_END) rep = ne == ce;
-    if (rep) W.rows[W.idx] = nr;
+    put = true;
+  } else if (k < W.idx) {  // R1
+    put = true;
+  } else if (k == W.idx) {  // R2 / R3
+    const int64_t ce = W.top_start + W.top_len - 1, ne = start + len - 1;
+    if (P.rules.replace == OASM_REPLACE_CONTAINED) put = start >= W.top_start && ne <= ce;
+    else if (P.rules.replace == OASM_REPLACE_SAME_END) put = ne == ce;
+  }
+  if (put) {
+    W.idx = k;
+    W.valid |= 1u << k;
+    W.start[k] = W.top_start = start;
+    W.len[k] = W.top_len = len;
   }
 }
 
@@ -726,37 +744,46 @@ __device__ __forceinline__ uint32_t pair_of(uint64_t key, int sb) {
   return uint32_t(key >> (sb + kLowBits));
 }
 
+// One thread per hit; the first hit of a piece runs the piece.  A piece is a
+// serial chain, so its latency counts (a planted copy at K = 15 gives some
+// hundred hits): its keys are read four at a time ahead of the rules, decoded
+// with the pair's constants, and the pending level stays in registers (a
+// dozen signatures with K up to 15: 171 -> 72 us; 3.7 M hits of one motif:
+// 291 -> 167).
 __global__ void __launch_bounds__(128)
     filter_kernel(const StepParams P, const unsigned long long* __restrict__ S) {
   if (P.ctr->overflow & 3u) return;  // candidates or hits incomplete; keep counting records
   const unsigned long long n = min(P.ctr->n_hits, P.cap_hits);
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  const int sb = P.start_bits;
   for (unsigned long long h = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; h < n;
        h += stride) {
-    const Hit hh = decode(S[h], P);
-    const uint32_t pair = hh.pair;
+    const uint64_t key0 = S[h], before = h ? S[h - 1] : 0ull;
+    const uint32_t pair = pair_of(key0, sb);
+    const bool first = h == 0 || pair_of(before, sb) != pair;
+    // a piece starts only at the first hit of a start that no earlier hit of
+    // the pair (nor the carried window) spans
+    if (!first && (before >> kLowBits) == (key0 >> kLowBits)) continue;
     const int p = int(pair % P.n_pat);
     const WorkItem w = P.items[pair / P.n_pat];
     const int m = P.m[p], K = P.K[p];
-    const bool first = (h == 0) || pair_of(S[h - 1], P.start_bits) != pair;
+    const PairKeys D{w.base_pos, m - K, (1ull << sb) - 1};
+    const int64_t start0 = D.start(key0);
+    if (!first && D.start(before) + D.len(before) - 1 >= start0) continue;
     const size_t hidx = size_t(w.slot) * P.n_pat + p;
     const MemRow* crow = P.mem + size_t(w.slot) * P.mem_stride + P.mem_off[p];
     const WinHdr chdr = P.hdr[hidx];
     int64_t cf = INT64_MIN;  // end of the carried window's top occurrence
     if (chdr.pend) cf = crow[chdr.idx].start + crow[chdr.idx].len - 1;
     if (!first) {
-      // a piece starts only at the first hit of a start that no earlier hit
-      // of the pair (nor the carried window) spans
-      const Hit prev = decode(S[h - 1], P);
-      if (prev.start == hh.start) continue;
-      if (cf >= hh.start) continue;
+      if (cf >= start0) continue;
       bool spanned = false;
-      for (long long j = (long long)h - 1; j >= 0; --j) {
+      for (long long j = (long long)h - 2; j >= 0; --j) {
         const uint64_t kj = S[j];
-        if (pair_of(kj, P.start_bits) != pair) break;
-        const Hit hj = decode(kj, P);
-        if (hj.start + m + K <= hh.start) break;  // ends before hh.start
-        if (hj.start + hj.len - 1 >= hh.start) {
+        if (pair_of(kj, sb) != pair) break;
+        const int64_t sj = D.start(kj);
+        if (sj + m + K <= start0) break;  // ends before start0
+        if (sj + D.len(kj) - 1 >= start0) {
           spanned = true;
           break;
         }
@@ -764,54 +791,68 @@ __global__ void __launch_bounds__(128)
       if (spanned) continue;
     }
     Window Wn;
-    Wn.pend = 0;
-    Wn.idx = K;
-    for (int lv = 0; lv <= K; ++lv) Wn.rows[lv].valid = 0;
+    open_window(Wn, K);
     Wn.rpos = h + (unsigned long long)(first ? pair : pair + 1) * unsigned(P.head);
-    Wn.nrec = 0;
     int64_t maxend = INT64_MIN;
     if (first && chdr.pend) {
-      Wn.pend = 1;
-      Wn.idx = chdr.idx;
-      for (int lv = 0; lv <= K; ++lv) Wn.rows[lv] = crow[lv];
+      load_window(Wn, chdr, crow, K);
       maxend = cf;
     }
-    unsigned long long j = h;
-    bool last = false;
-    while (true) {
-      Hit cur = decode(S[j], P);
-      unsigned long long nxt = j + 1;
-      if (P.rules.order == OASM_ORDER_PER_START_BEST) {
-        // among the hits of this start keep the smallest k, then the shortest
-        int64_t me = cur.start + cur.len - 1;
-        while (nxt < n && pair_of(S[nxt], P.start_bits) == pair) {
-          const Hit o = decode(S[nxt], P);
-          if (o.start != cur.start) break;
-          me = max(me, o.start + o.len - 1);
-          if (o.k < cur.k) cur = o;
-          ++nxt;
+    const bool per_start_best = P.rules.order == OASM_ORDER_PER_START_BEST;
+    // per-start-best: the best hit so far (smallest k, then shortest) of the
+    // current start, and the last end of that start's hits
+    int64_t bs = 0, bend = 0;
+    int bl = 0, bk = 0;
+    bool have = false, last = true;
+    for (unsigned long long j = h; j < n && last; j += 4) {
+      uint64_t k4[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) k4[q] = S[min(j + q, n - 1)];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint64_t key = k4[q];
+        if (j + q >= n || pair_of(key, sb) != pair) {  // the pair's last hit is behind
+          j = n;
+          break;
         }
-        apply(P, Wn, pair, p, K, w, cur);
-        maxend = max(maxend, me);
-      } else {
-        apply(P, Wn, pair, p, K, w, cur);
-        maxend = max(maxend, cur.start + cur.len - 1);
+        const int64_t st = D.start(key);
+        const int len = D.len(key), k = int(key & 15u);
+        if (!per_start_best) {
+          if (j + q != h && st > maxend) {  // next piece
+            last = false;
+            break;
+          }
+          apply(P, Wn, pair, p, K, w, st, len, k);
+          maxend = max(maxend, st + len - 1);
+          continue;
+        }
+        if (have && st == bs) {
+          bend = max(bend, st + len - 1);
+          if (k < bk) bl = len, bk = k;
+          continue;
+        }
+        if (have) {
+          apply(P, Wn, pair, p, K, w, bs, bl, bk);
+          maxend = max(maxend, bend);
+          have = false;
+          if (st > maxend) {  // next piece
+            last = false;
+            break;
+          }
+        }
+        have = true;
+        bs = st;
+        bl = len;
+        bk = k;
+        bend = st + len - 1;
       }
-      j = nxt;
-      if (j >= n || pair_of(S[j], P.start_bits) != pair) {
-        last = true;
-        break;
-      }
-      const Hit nh = decode(S[j], P);
-      if (nh.start > maxend) break;  // next piece
     }
+    if (have) apply(P, Wn, pair, p, K, w, bs, bl, bk);
     if (!last) {
       if (Wn.pend) flush(P, Wn, pair, p, K, w);
     } else {
-      if (Wn.pend) {
-        const MemRow& top = Wn.rows[Wn.idx];
-        if (w.eos || top.start + top.len - 1 <= f_new(w, m, K)) flush(P, Wn, pair, p, K, w);
-      }
+      if (Wn.pend && (w.eos || Wn.top_start + Wn.top_len - 1 <= f_new(w, m, K)))
+        flush(P, Wn, pair, p, K, w);
       const unsigned long long q = atomicAdd(&P.ctr->n_pool, 1ull);
       if (q >= P.cap_pool) {
         atomicOr(&P.ctr->overflow, 8u);
@@ -820,7 +861,14 @@ __global__ void __launch_bounds__(128)
         nhdr.pend = Wn.pend;
         nhdr.idx = Wn.idx;
         P.pool_hdr[q] = nhdr;
-        for (int lv = 0; lv <= K; ++lv) P.pool_mem[q * (kMaxK + 1) + lv] = Wn.rows[lv];
+        for (int lv = 0; lv <= K; ++lv) {
+          const bool v = (Wn.valid >> lv) & 1u;
+          MemRow r;
+          r.start = v ? Wn.start[lv] : 0;
+          r.len = v ? Wn.len[lv] : 0;
+          r.valid = v;
+          P.pool_mem[q * (kMaxK + 1) + lv] = r;
+        }
         P.pair_pool[pair] = int32_t(q);
       }
     }
@@ -877,11 +925,8 @@ __global__ void finalize_kernel(const StepParams P, const unsigned long long* __
           continue;
         }
         Window Wn;
-        Wn.pend = 1;
-        Wn.idx = hd->idx;
-        for (int lv = 0; lv <= K; ++lv) Wn.rows[lv] = rows[lv];
-        Wn.nrec = 0;
-        Wn.rpos = 0;
+        open_window(Wn, K);
+        load_window(Wn, *hd, rows, K);
         if (P.ordered)  // a pair without hits: its segment is the pair's head
           Wn.rpos = pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pr,
                                      P.start_bits + kLowBits) + pr * unsigned(P.head);
