@@ -265,7 +265,8 @@ struct Grams {
   double saved_clk = 0;       // and saves, against the forward scan of every pattern
   std::vector<Bucket> rest;
   DevArray<unsigned long long> susp;
-  DevArray<unsigned long long> ctr;  // suspects of each slice
+  DevArray<unsigned long long> longs;
+  DevArray<GramCounters> ctr;
   int off_steps = 0;          // steps left without the index (suspects too dense)
 };
 

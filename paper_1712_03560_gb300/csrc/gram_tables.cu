@@ -23,29 +23,28 @@ double buckets_cost(const std::vector<Bucket>& bs) {
     for (const LaneGroup& g : b.groups) c += group_cost(b.W, b.algo) / g.nseg;
   return c;
 }
-// Clocks of one SM per suspect (the ends run: about 25 for one word, 20 more
-// per further word), per false table bit (a directory look-up), and per text
-// symbol and gram length.
-constexpr double kEnds = 25.0, kEndsWord = 20.0, kLookup = 8.0, kLength = 0.12;
+// Clocks of one SM per suspect (the ends kernel's first round, and both), per
+// table hit (a directory look-up), and per text symbol and key length.
+constexpr double kPair = 6.0, kEnds = 25.0, kLookup = 4.0, kLength = 0.12;
 
-constexpr int kMaxGram2 = 13;  // symbols of a gram, 2-bit text
-constexpr int kMaxPiece = 12;  // ... of a piece that may hold an edit
-const int kByteLens[] = {3, 4, 6, 8};
+constexpr int kMaxGram2 = 16, kMaxGram = 8;  // symbols of a gram: 2-bit text, bytes
+constexpr int kMaxPiece = 12;                // ... of a piece that may hold an edit
+constexpr int kMaxKey2 = 10, kMaxKey = 4;    // symbols that are looked up
+constexpr int kPairRows = 8;                 // symbols of a pair looked at beside a gram
 
-// Grams of one length: key << 32 | pattern << 8 | pattern symbols after it.
-using GramList = std::vector<uint64_t>;
+// Grams of one key length, ordered by key (stable; three passes of 11 bits).
+using GramList = std::vector<GramEntry>;
 
-// Orders the list by key (stable; three passes of 11 bits).
-void sort_by_key(GramList& g) {
+void sort_by_key(GramList& g, uint32_t mask) {
   GramList t(g.size());
-  for (int shift = 32; shift < 64; shift += 11) {
+  for (int shift = 0; shift < 32; shift += 11) {
+    if (shift && (mask >> shift) == 0) break;
     std::vector<uint32_t> at(2049, 0u);
-    for (uint64_t x : g) at[((x >> shift) & 2047u) + 1] += 1;
+    for (const GramEntry& x : g) at[(((x.lo & mask) >> shift) & 2047u) + 1] += 1;
     for (int i = 0; i < 2048; ++i) at[i + 1] += at[i];
-    for (uint64_t x : g) t[at[(x >> shift) & 2047u]++] = x;
+    for (const GramEntry& x : g) t[at[((x.lo & mask) >> shift) & 2047u]++] = x;
     g.swap(t);
   }
-  g.erase(std::unique(g.begin(), g.end()), g.end());
 }
 
 // The j disjoint pieces of b symbols with the smallest sum of w (w[x] = chance
@@ -74,29 +73,35 @@ double place(const std::vector<double>& w, int m, int j, int b, std::vector<doub
   return f[j * row + m];
 }
 
-// Grams such that every string within one edit of s contains one of them,
-// each with the symbols of s up to its end: the strings with one symbol
-// missing (s without its last symbol is contained in s itself, in s with its
-// last symbol changed or missing and in s with an insertion before it; s
-// without its first symbol likewise), then changes and insertions further
-// inside.
+// Grams such that every string within one edit of s contains one of them, as
+// (gram, its symbols, the part of s it stands for, edits between the two).  s
+// without its last symbol, standing for itself, is contained in s, in s with
+// its last symbol changed or missing and in s with an insertion before it; s
+// without its first symbol likewise.  The rest, an edit further inside, stands
+// for all of s.  (A missing symbol of a run is the run's last one, or its
+// first at the start of s: the same string.)
 // s: b 2-bit symbols, the first in the low bits.
 template <class F>
 void one_edit(uint32_t s, int b, F put) {
   auto sym = [&](int i) { return (s >> (2 * i)) & 3u; };
   auto below = [&](int i) { return s & ((1u << (2 * i)) - 1u); };
-  for (int i = 0; i < b; ++i) {  // without symbol i (of a run of one symbol: its last)
-    if (i + 1 < b && sym(i) == sym(i + 1)) continue;
-    put(below(i) | ((s >> (2 * i + 2)) << (2 * i)), b - 1, i == b - 1 ? b - 1 : b);
-  }
+  put(below(b - 1), b - 1, 0, b - 1, 0);
+  put(s >> 2, b - 1, 1, b, 0);
+  int head = 0;  // last symbol of the run that s starts with
+  while (head + 1 < b && sym(head + 1) == sym(0)) ++head;
+  for (int i = head + 1; i + 1 < b; ++i)  // without symbol i
+    if (sym(i) != sym(i + 1)) put(below(i) | ((s >> (2 * i + 2)) << (2 * i)), b - 1, 0, b, 1);
   for (int i = 1; i + 1 < b; ++i)
     for (uint32_t c = 0; c < 4; ++c)
-      if (c != sym(i)) put((s & ~(3u << (2 * i))) | (c << (2 * i)), b, b);
+      if (c != sym(i)) put((s & ~(3u << (2 * i))) | (c << (2 * i)), b, 0, b, 1);
   for (int i = 2; i + 1 < b; ++i)  // before symbol i
     for (uint32_t c = 0; c < 4; ++c)
       if (c != sym(i))  // (equal: the same string as an insertion after it)
-        put(below(i) | (c << (2 * i)) | ((s >> (2 * i)) << (2 * i + 2)), b + 1, b);
+        put(below(i) | (c << (2 * i)) | ((s >> (2 * i)) << (2 * i + 2)), b + 1, 0, b, 1);
 }
+
+// Whether piece t of E + 1 is half of a pair.
+bool paired(int t, int E) { return t < E || (E & 1); }
 
 }  // namespace
 
@@ -140,13 +145,13 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     for (int c = 0; c < 4; ++c) fr[c] = std::max(fr[c], 1e-3);
   std::vector<uint8_t> edits(n, 0);
   const int cmin = ctx->weighted ? int(std::min({ctx->costs.sub, ctx->costs.ins, ctx->costs.del})) : 1;
-  GramList by_len[kMaxGram2 + 1];
+  GramList by_len[kMaxKey2 + 1];
   double ends_clk = 0;
   std::vector<double> ps, w, scratch;
   std::vector<uint8_t> sym;
   std::vector<int> at, best_at;
   for (uint32_t p = 0; p < n; ++p) {
-    const int m = ctx->m[p], E = ctx->K[p] / cmin, W = (m + 31) / 32;
+    const int m = ctx->m[p], E = ctx->K[p] / cmin;
     edits[p] = uint8_t(E);
     if (pref[p]) continue;
     sym.resize(m);
@@ -164,26 +169,42 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
         w[x] = r;
       }
     };
-    const double per_suspect = kEnds + kEndsWord * (W - 1);
-    // (a) E + 1 unedited pieces, as long as an equal split allows
-    double best = 1e30, best_q = 0;
-    int best_b = 0;
-    bool best_edit = false;
-    {
-      const int j = E + 1;
-      int b = std::min(m / j, kMaxGram2);
-      if (!two) {
-        int q = 0;
-        for (int L : kByteLens) q = L <= m / j ? L : q;
-        b = q;
+    // a byte piece is looked up by its rarest four symbols (and compared from
+    // there on); 2-bit pieces from their start
+    auto key_at = [&](int x, int b) {
+      if (two || b <= kMaxKey) return x;
+      int at = x;
+      double least = 1e30;
+      for (int y = x; y + kMaxKey <= x + b; ++y) {
+        double key = 1, all = 1;
+        for (int i = 0; i < kMaxKey; ++i) key *= ps[y + i];
+        for (int i = y; i < x + b; ++i) all *= ps[i];
+        const double cost = key * kLookup + all * kPair;
+        if (cost < least) least = cost, at = y;
       }
-      if (b >= (two ? 5 : 3)) {
-        windows(b);
-        const double q = place(w, m, j, b, scratch, &at);
-        best = q * per_suspect + j * (kLookup / (32.0 * kGramMaxWords));
-        best_b = b;
-        best_at = at;
-        best_q = q;
+      return at;
+    };
+    double best = 1e30, best_q = 0, best_clk = 0;
+    int best_b = 0, best_h = 0;
+    bool best_edit = false;
+    // (a) E + 1 pieces of h symbols, two by two: a pair of them holds at most
+    // one edit, so one of its halves none, or, for even E, the last piece holds
+    // none (E / 2 pairs with two edits or more leave no edit for it)
+    {
+      const int h = std::min(m / (E + 1), two ? kMaxGram2 : kMaxGram);
+      if (h >= (two ? 5 : 3)) {
+        windows(h);
+        best_q = place(w, m, E + 1, h, scratch, &best_at);
+        const int kb = std::min(h, two ? kMaxKey2 : kMaxKey);
+        double cost = 0;
+        for (int t = 0; t <= E; ++t) {
+          const int x = best_at[t], y = key_at(x, h);
+          double key = 1;
+          for (int i = 0; i < kb; ++i) key *= ps[y + i];
+          cost += key * kLookup + w[x] * (paired(t, E) ? kPair : kEnds);
+        }
+        best = best_clk = cost;
+        best_h = h;
       }
     }
     // (b) E / 2 + 1 pieces with at most one edit each (2-bit text)
@@ -196,9 +217,10 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
         // deletions and changes of a uniform text symbol, about 7 b strings
         const double q = j * (b / std::pow(4.0, b - 1) + 3.0 * (b - 2) / std::pow(4.0, b) +
                               3.0 * (b - 3) / std::pow(4.0, b + 1));
-        const double cost = q * per_suspect + j * 7.0 * b * (kLookup / (32.0 * kGramMaxWords));
+        const double look = j * 7.0 * b / std::pow(4.0, std::min(b, kMaxKey2));
+        const double cost = q * kEnds + look * kLookup;
         if (cost < best) {
-          best = cost;
+          best = best_clk = cost;
           best_b = b;
           best_at = at;
           best_edit = true;
@@ -206,23 +228,40 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
         }
       }
     }
-    if (!best_b || best > 0.7 * share) continue;
+    if (best > 0.7 * share) continue;
     served[p] = 1;
     gr.n_pat += 1;
-    ends_clk += best_q * per_suspect;
+    ends_clk += best_clk;
     gr.rate += best_q;
-    auto put = [&](uint32_t key, int len, int end) {  // end: pattern symbols up to the gram's end
-      by_len[len].push_back((uint64_t(key) << 32) | (uint64_t(p) << 8) | uint64_t(m - end));
+    // a gram for pattern symbols [from, to)
+    auto put = [&](uint64_t sym8, int len, int from, int to, int pair) {
+      if (from > 32 || m - to > 32) gr.t.any_long = 1;
+      by_len[std::min(len, two ? kMaxKey2 : kMaxKey)].push_back(
+          GramEntry{p, uint8_t(from), uint8_t(m - to), uint8_t(pair), uint8_t(len), uint32_t(sym8),
+                    uint32_t(sym8 >> 32)});
     };
-    for (int x : best_at) {
+    auto packed = [&](int x, int len) {
       uint64_t k = 0;
-      for (int i = 0; i < best_b; ++i) k |= uint64_t(sym[x + i]) << ((two ? 2 : 8) * i);
-      if (best_edit)
-        one_edit(uint32_t(k), best_b, [&](uint32_t u, int len, int end) { put(u, len, x + end); });
-      else
-        put(two || best_b <= 4 ? uint32_t(k)
-                               : uint32_t(k) * kGramMixLo + uint32_t(k >> 32) * kGramMixHi,
-            best_b, x + best_b);
+      for (int i = 0; i < len; ++i) k |= uint64_t(sym[x + i]) << ((two ? 2 : 8) * i);
+      return k;
+    };
+    if (best_edit) {
+      for (int x : best_at)
+        one_edit(uint32_t(packed(x, best_b)), best_b,
+                 [&](uint32_t u, int l, int from, int to, int edit) {
+                   put(u, l, x + from, x + to, edit ? kGramEdit : 0);
+                 });
+    }
+    // each piece, and how far its pair reaches on the other side (of which
+    // kPairRows symbols tell enough: more would only make a warp's lanes wait
+    // for the longest)
+    for (int t = 0; !best_edit && t <= E; ++t) {
+      const int y = key_at(best_at[t], best_h), to = best_at[t] + best_h;
+      int pair = 0;
+      if (paired(t, E))
+        pair = t & 1 ? std::min(kPairRows, y - best_at[t - 1]) | kGramLeft
+                     : std::min(kPairRows, best_at[t + 1] + best_h - to);
+      put(packed(y, to - y), to - y, y, to, pair);
     }
   }
   auto none = [&]() {
@@ -231,36 +270,37 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     return OASM_OK;
   };
   if (gr.n_pat < uint32_t(kLaneGroup)) return none();
-  // per length: a table of one bit per gram (direct, or hashed to the size
+  // per key length: a table of one bit per key (direct, or hashed to the size
   // that fits), and a directory
   struct Len {
     int len;
+    uint32_t mask;
     const GramList* g;
     size_t distinct = 0;
     int bits = 10;  // log2 of the table's bits
   };
   std::vector<Len> lens;
   size_t n_grams = 0;
-  for (int len = 1; len <= kMaxGram2; ++len) {
+  for (int len = 1; len <= kMaxKey2; ++len) {
     GramList& g = by_len[len];
     if (g.empty()) continue;
-    sort_by_key(g);
-    Len L{len, &g};
-    for (size_t i = 0; i < g.size(); ++i) L.distinct += i == 0 || (g[i] >> 32) != (g[i - 1] >> 32);
+    const int kb = (two ? 2 : 8) * len;
+    Len L{len, kb >= 32 ? ~0u : (1u << kb) - 1u, &g};
+    sort_by_key(g, L.mask);
+    for (size_t i = 0; i < g.size(); ++i)
+      L.distinct += i == 0 || ((g[i].lo ^ g[i - 1].lo) & L.mask) != 0;
     n_grams += g.size();
     lens.push_back(L);
   }
   // a suspect holds 24 entry bits
   if (n_grams >= (size_t(1) << 24) || lens.size() > size_t(kGramLens)) return none();
-  // doubles the table with the most grams per bit while the budget lasts
-  // (direct tables stop at one bit per key; 256 bits per gram is plenty)
-  auto most = [&](const Len& L) {
-    const int key_bits = two ? 2 * L.len : 32;
-    return key_bits <= L.bits || (size_t(1) << L.bits) >= 256 * L.distinct;
-  };
+  // 2-bit keys index their table directly (all lengths together fit); a byte
+  // length's table is doubled, the fullest first, while the budget lasts (256
+  // bits per gram are plenty)
+  auto most = [&](const Len& L) { return (size_t(1) << L.bits) >= 256 * L.distinct; };
   for (Len& L : lens)
-    if (two) L.bits = std::min(L.bits, 2 * L.len);
-  while (true) {
+    if (two) L.bits = 2 * L.len;
+  while (!two) {
     size_t words = 0;
     Len* pick = nullptr;
     for (Len& L : lens) {
@@ -284,18 +324,10 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   for (size_t li = 0; li < lens.size(); ++li) {
     const Len& L = lens[li];
     const GramList& list = *L.g;
-    const int len = L.len, key_bits = two ? 2 * len : 32;
     GramLen& g = a.len[li];
-    if (two) {
-      g.mask_lo = uint32_t((uint64_t(1) << (2 * len)) - 1);
-      g.mask_hi = 0;
-    } else {
-      g.mask_lo = len >= 4 ? 0xffffffffu : (1u << (8 * len)) - 1u;
-      g.mask_hi = len <= 4 ? 0u : len >= 8 ? 0xffffffffu : (1u << (8 * (len - 4))) - 1u;
-    }
-    const bool direct = key_bits <= L.bits;
-    g.mul = direct ? 1u : kGramBitMul;
-    g.shift = direct ? 0u : uint32_t(32 - L.bits);
+    g.mask = L.mask;
+    g.mul = two ? 1u : kGramBitMul;
+    g.shift = two ? 0u : uint32_t(32 - L.bits);
     g.word0 = uint32_t(bits.size());
     bits.resize(bits.size() + std::max<size_t>(4, (size_t(1) << L.bits) / 32), 0u);
     int db = 4;
@@ -306,11 +338,9 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     g.max_probe = 0;
     dir.resize(dir.size() + (size_t(1) << db), make_uint4(0u, 0u, 0u, 0u));
     for (size_t i = 0; i < list.size();) {
-      const uint32_t key = uint32_t(list[i] >> 32), h = (key * g.mul) >> g.shift;
+      const uint32_t key = list[i].lo & L.mask, h = (key * g.mul) >> g.shift;
       const uint32_t first = uint32_t(entries.size());
-      for (; i < list.size() && uint32_t(list[i] >> 32) == key; ++i)
-        entries.push_back(GramEntry{uint32_t(list[i] >> 8) & 0xffffffu,
-                                    uint16_t(list[i] & 0xffu), uint16_t(len)});
+      for (; i < list.size() && (list[i].lo & L.mask) == key; ++i) entries.push_back(list[i]);
       bits[g.word0 + (h >> 5)] |= 1u << (h & 31);
       uint32_t s = (key * kGramDirMul) >> g.dir_shift, pr = 0;
       while (dir[g.dir0 + s].z != 0) {
@@ -320,7 +350,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
       dir[g.dir0 + s] = make_uint4(key, first, uint32_t(entries.size()) - first, 0u);
       g.max_probe = std::max(g.max_probe, pr);
     }
-    if (!direct) false_bits += double(L.distinct) / double(size_t(1) << L.bits);
+    if (!two) false_bits += double(L.distinct) / double(size_t(1) << L.bits);
   }
   a.n_words = uint32_t((bits.size() + 3) & ~size_t(3));
   bits.resize(a.n_words, 0u);
@@ -341,6 +371,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   uint32_t* peq = nullptr;
   CK(cudaMalloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t)));
   gr.t.peq_fwd = peq;
+  a.entries = gr.t.entries;
   CK(launch_peq(ctx->d_bytes, ctx->d_m, n, peq, false, ctx->stream));
   return OASM_OK;
 }

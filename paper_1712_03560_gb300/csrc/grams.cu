@@ -1,34 +1,38 @@
 // grams.cu -- gram index in front of the exact forward scan (sm_103a).
 //
 // Pigeonhole principle for edit distance: an alignment of a pattern with at
-// most E edits (Eq. 1, Eq. 2; E = K under unit costs) leaves one of E + 1
-// disjoint pieces of the pattern unedited, and one of E / 2 + 1 pieces with
-// at most one edit.  The index holds every string such a piece may appear as
-// (the piece itself, or every string one edit away from it) as a gram of the
-// text, with the pattern symbols that remain after it; a gram found at a text
-// position allows the ends within E of that many symbols further on.  Only
-// those ends are examined, with the whole pattern's column recurrence, and
-// the ones with D[e] <= E become candidates: the forward scan's own
-// candidates under unit costs, a superset of them under edit costs (a
-// distance is at least the cheapest cost times the number of edits), which
-// verification then measures.
+// most E edits (Eq. 1, Eq. 2; E = K under unit costs) leaves
+//   one of E + 1 disjoint pieces of the pattern unedited; with the pieces taken
+//   two by two, one of a pair that has at most one edit in all (or the odd
+//   last one);
+//   one of E / 2 + 1 disjoint pieces with at most one edit.
+// The index holds grams: the pieces themselves, or (2-bit text) the strings
+// one edit away from longer pieces.  A gram found at a text position allows
+// the ends within E edits of its diagonal; the pattern symbols beside it are
+// matched with the text beside it, and an end that all of them reach within E
+// edits becomes a candidate: the forward scan's own candidates under unit
+// costs, a superset of them under edit costs (a distance is at least the
+// cheapest cost times the number of edits) or where 2-bit text holds other
+// symbols; verification measures them.
 //
-//   scan   one text position per step of a lane: for each gram length, a bit
-//          of a table in shared memory, and where it is set the length's
-//          directory (open addressing, in L2): suspects (position, entry)
-//   ends   one thread per suspect: the recurrence over the ends the entry
-//          allows; each (pattern, end) becomes a candidate once (an
+//   scan   one text position per step of a lane: for each key length, a bit of
+//          a table in shared memory; where it is set, the length's directory
+//          (open addressing, in L2) and the grams with that key: suspects
+//          (position, gram)
+//   ends   one thread per suspect: the pattern beside the gram against the
+//          text beside it; each (pattern, end) becomes a candidate once (an
 //          open-addressing set: an occurrence holds several grams)
+//   long   what passed of patterns longer than 32 symbols beside their gram
 //
-// The cost per text position depends on the number of gram lengths and on
-// how often grams appear, not on the number of patterns.
+// The cost per text position depends on the number of key lengths and on how
+// often grams appear, not on the number of patterns.
 #include "kernels.h"
 
 namespace oasm {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kQueue = 96;  // suspects buffered per warp
+constexpr int kQueue = 64;  // table hits, and suspects, buffered per warp
 
 // ------------------------------------------------------------------- scan
 // 2-bit symbols: (byte >> shift) & 3, 16 of them to a word.
@@ -38,49 +42,130 @@ __device__ __forceinline__ uint32_t pack2(uint32_t w, uint32_t shift) {
   return (((w >> shift) & 0x03030303u) * 0x01041040u) >> 24;
 }
 
-// Key of the gram of length g.len at symbol j of the lane's 16 (2-bit text:
-// the packed symbols; bytes: up to four bytes as they are, more hashed).
+// The text at symbol j of the lane's 16: 16 2-bit symbols, or eight bytes.
 template <bool kTwoBit>
-__device__ __forceinline__ uint32_t gram_key(const GramLen& g, const uint32_t (&t)[6], int j) {
-  if (kTwoBit) return __funnelshift_r(t[0], t[1], 2 * j) & g.mask_lo;
-  const int q = j >> 2, r = 8 * (j & 3);
-  const uint32_t lo = r ? __funnelshift_r(t[q], t[q + 1], r) : t[q];
-  if (g.mask_hi == 0u) return lo & g.mask_lo;
-  const uint32_t hi = r ? __funnelshift_r(t[q + 1], t[q + 2], r) : t[q + 1];
-  return lo * kGramMixLo + (hi & g.mask_hi) * kGramMixHi;
+__device__ __forceinline__ void window(const uint32_t (&t)[6], int j, uint32_t& lo, uint32_t& hi) {
+  if (kTwoBit) {
+    lo = __funnelshift_r(t[0], t[1], 2 * j);
+    hi = 0u;
+    return;
+  }
+  const int q = j >> 2, r = 8 * (j & 3);  // (selects where j is known only here)
+  const uint32_t a = q == 0 ? t[0] : q == 1 ? t[1] : q == 2 ? t[2] : t[3];
+  const uint32_t b = q == 0 ? t[1] : q == 1 ? t[2] : q == 2 ? t[3] : t[4];
+  const uint32_t c = q == 0 ? t[2] : q == 1 ? t[3] : q == 2 ? t[4] : t[5];
+  lo = __funnelshift_r(a, b, r);
+  hi = __funnelshift_r(b, c, r);
 }
 
 // One block per SM; its warps walk 512-symbol tiles of the text arena, 16
-// symbols per lane.  Bound by instruction issue (about nine instructions per
-// position and gram length) and by the shared-memory conflicts of the random
-// table reads; the directory reads of one warp hide behind the others.
+// symbols per lane.  A gram is indexed by its first symbols (up to ten 2-bit
+// symbols, whose tables are direct: 4^10 bits; three or four bytes, hashed)
+// and compared with the text in full where its table bit and directory slot
+// are found.  Table hits go through a per-warp queue, so that the directory
+// (L2) is read 32 look-ups at a time, and the entries of those look-ups are
+// dealt out one per lane.  Bound by instruction issue and the shared-memory
+// conflicts of the random table reads.
+// (First forms: hashed tables for every gram length, up to 13 symbols, let
+// four positions in ten through to the directory, one look-up per lane and
+// length at a time: 535 us per 64 MiB of DNA against 1,024 patterns; with the
+// queue 430; this form 186.  4,096 byte patterns over 32 MiB: 200, now 126.)
+struct GramWarp {
+  unsigned long long hit_pos[kQueue];  // arena offset << 4 | key length's number
+  unsigned long long susp[kQueue];
+  uint32_t hit_lo[kQueue], hit_hi[kQueue];
+};
+
 template <bool kTwoBit>
 __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramScan A) {
   extern __shared__ __align__(16) uint32_t bits_s[];
   constexpr int kWarps = kGramThreads / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned long long* queue =
-      reinterpret_cast<unsigned long long*>(bits_s + A.n_words) + size_t(warp) * kQueue;
+  const unsigned below = (1u << lane) - 1u;
+  GramWarp& Q = reinterpret_cast<GramWarp*>(bits_s + A.n_words)[warp];
   {
     const uint4* src = reinterpret_cast<const uint4*>(A.bits);
     uint4* dst = reinterpret_cast<uint4*>(bits_s);
     for (uint32_t i = threadIdx.x; i < A.n_words / 4; i += kGramThreads) dst[i] = src[i];
   }
   __syncthreads();
-  int qn = 0;         // queued suspects of this warp
-  bool dead = false;  // the suspect buffer is full
+  int hn = 0, qn = 0;  // queued table hits and suspects of this warp
+  bool dead = false;   // the suspect buffer is full
   auto flush = [&]() {
     __syncwarp();
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(A.n_susp, (unsigned long long)qn);
+    if (lane == 0) base = atomicAdd(&A.ctr_slice->n_susp, (unsigned long long)qn);
     base = __shfl_sync(kFull, base, 0);
     for (int i = lane; i < qn; i += 32)
-      if (base + i < A.cap_susp) A.susp[base + i] = queue[i];
+      if (base + i < A.cap_susp) A.susp[base + i] = Q.susp[i];
     if (base + qn > A.cap_susp) {
       dead = true;
       if (lane == 0) atomicOr(&A.ctr->overflow, kGramOverflow | 1u);
     }
     qn = 0;
+    __syncwarp();
+  };
+  // The last 32 (or all) queued table hits: a directory look-up each, then
+  // all their entries, one per lane and round, against the text.
+  auto look_up = [&]() {
+    __syncwarp();
+    const int i = max(hn - 32, 0) + lane;
+    uint32_t first = 0, left = 0, lo = 0, hi = 0;
+    unsigned long long pos = 0;
+    if (i < hn) {
+      lo = Q.hit_lo[i];
+      hi = Q.hit_hi[i];
+      pos = Q.hit_pos[i];
+      const GramLen& g = A.len[pos & 15u];
+      const uint32_t key = lo & g.mask;
+      uint32_t s = (key * kGramDirMul) >> g.dir_shift;
+      for (uint32_t pr = 0; pr <= g.max_probe; ++pr) {
+        const uint4 sl = __ldg(A.dir + g.dir0 + s);
+        if (sl.z == 0) break;
+        if (sl.x == key) {
+          first = sl.y;
+          left = sl.z;
+          break;
+        }
+        s = (s + 1) & g.dir_mask;
+      }
+      pos >>= 4;
+    }
+    hn = max(hn - 32, 0);
+    uint32_t incl = left;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(kFull, incl, d);
+      if (lane >= d) incl += x;
+    }
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+    for (uint32_t base = 0; base < total && !dead; base += 32) {
+      const uint32_t item = base + unsigned(lane);
+      int own = 0;  // the lane whose look-up found the item: lanes with incl <= item
+#pragma unroll
+      for (int d = 16; d; d >>= 1) {
+        const uint32_t x = __shfl_sync(kFull, incl, own + d - 1);
+        if (x <= item) own += d;
+      }
+      own = min(own, 31);
+      const uint32_t e = __shfl_sync(kFull, first - (incl - left), own) + item;
+      const uint32_t olo = __shfl_sync(kFull, lo, own), ohi = __shfl_sync(kFull, hi, own);
+      const unsigned long long opos = __shfl_sync(kFull, pos, own);
+      bool ok = false;
+      if (item < total) {
+        const uint4 en = __ldg(reinterpret_cast<const uint4*>(A.entries + e));
+        const uint32_t len = en.y >> 24;
+        const uint32_t nb = kTwoBit ? 2 * len : 8 * len;  // bits of the gram
+        const uint32_t mlo = nb >= 32 ? ~0u : (1u << nb) - 1u;
+        const uint32_t mhi = nb <= 32 ? 0u : nb >= 64 ? ~0u : (1u << (nb - 32)) - 1u;
+        ok = (((olo ^ en.z) & mlo) | ((ohi ^ en.w) & mhi)) == 0;
+      }
+      const unsigned m = __ballot_sync(kFull, ok);
+      if (!m) continue;
+      if (qn > kQueue - 32) flush();
+      if (ok) Q.susp[qn + __popc(m & below)] = (opos << 24) | e;
+      qn += __popc(m);
+    }
     __syncwarp();
   };
   const uint4* text = reinterpret_cast<const uint4*>(A.arena);
@@ -112,67 +197,43 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
     }
 #pragma unroll 1
     for (int l = 0; l < A.n_len; ++l) {
-      const GramLen g = A.len[l];
+      const GramLen& g = A.len[l];
       // table bit of every position, shifted in from the top: position j of
       // the lane ends at bit 16 + j
       uint32_t acc = 0;
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const uint32_t h = (gram_key<kTwoBit>(g, t, j) * g.mul) >> g.shift;
+        uint32_t h;
+        if (kTwoBit) {
+          h = __funnelshift_r(t[0], t[1], 2 * j) & g.mask;
+        } else {
+          const uint32_t lo = (j & 3) ? __funnelshift_r(t[j >> 2], t[(j >> 2) + 1], 8 * (j & 3))
+                                      : t[j >> 2];
+          h = ((lo & g.mask) * g.mul) >> g.shift;
+        }
         const uint32_t w = bits_s[g.word0 + (h >> 5)];
         acc = __funnelshift_r(acc, __funnelshift_r(w, w, h), 1);
       }
       uint32_t hits = acc >> 16;
-      // directory look-ups, one per lane and round; then one entry per lane
-      // and round into the queue
-      uint32_t e = 0, left = 0;
-      unsigned long long pos = 0;
-      while (__any_sync(kFull, (hits | left) != 0)) {
-        if (left == 0 && hits) {
+      unsigned m;
+      while ((m = __ballot_sync(kFull, hits != 0)) != 0) {
+        if (hn > kQueue - 32) look_up();
+        if (hits) {
           const int j = __ffs(hits) - 1;
           hits &= hits - 1;
-          pos = tile * 512 + unsigned(lane) * 16 + unsigned(j);
-          // the key again, at a position known only here
-          uint32_t key;
-          if (kTwoBit) {
-            key = __funnelshift_r(t[0], t[1], 2 * j) & g.mask_lo;
-          } else {
-            const int q = j >> 2;
-            const uint32_t a = q == 0 ? t[0] : q == 1 ? t[1] : q == 2 ? t[2] : t[3];
-            const uint32_t b = q == 0 ? t[1] : q == 1 ? t[2] : q == 2 ? t[3] : t[4];
-            const uint32_t c = q == 0 ? t[2] : q == 1 ? t[3] : q == 2 ? t[4] : t[5];
-            const uint32_t lo = __funnelshift_r(a, b, 8 * (j & 3));
-            const uint32_t hi = __funnelshift_r(b, c, 8 * (j & 3));
-            key = g.mask_hi == 0u ? (lo & g.mask_lo)
-                                  : lo * kGramMixLo + (hi & g.mask_hi) * kGramMixHi;
-          }
-          uint32_t s = (key * kGramDirMul) >> g.dir_shift;
-          for (uint32_t pr = 0; pr <= g.max_probe; ++pr) {
-            const uint4 sl = __ldg(A.dir + g.dir0 + s);
-            if (sl.z == 0) break;
-            if (sl.x == key) {
-              e = sl.y;
-              left = sl.z;
-              break;
-            }
-            s = (s + 1) & g.dir_mask;
-          }
+          uint32_t lo, hi;
+          window<kTwoBit>(t, j, lo, hi);
+          const int at = hn + __popc(m & below);
+          Q.hit_lo[at] = lo;
+          Q.hit_hi[at] = hi;
+          Q.hit_pos[at] = ((tile * 512 + unsigned(lane) * 16 + unsigned(j)) << 4) | unsigned(l);
         }
-        const unsigned m = __ballot_sync(kFull, left != 0);
-        if (!m) continue;
-        if (qn > kQueue - 32) flush();
-        if (left) {
-          queue[qn + __popc(m & ((1u << lane) - 1u))] = (pos << 24) | e;
-          ++e;
-          --left;
-        }
-        qn += __popc(m);
-        if (dead) break;
+        hn += __popc(m);
       }
-      if (dead) break;
     }
   }
-  if (qn) flush();
+  while (hn && !dead) look_up();
+  if (qn && !dead) flush();
 }
 
 // ------------------------------------------------------------------- ends
@@ -216,6 +277,7 @@ __device__ uint32_t ends_run(const uint32_t* __restrict__ peq, const uint8_t* __
   const int64_t start = max(lo - (m + E - 1), int64_t(0));
   const int warm = int(lo - start), n = warm + span + 1;
   const uint8_t* t = text + start;
+#pragma unroll 4
   for (int i = 0; i < n; ++i) {
     const uint32_t* row = peq + size_t(t[i]) * 4;
     uint32_t eq[W];
@@ -251,115 +313,297 @@ __device__ uint32_t ends_run(const uint32_t* __restrict__ peq, const uint8_t* __
   return hit;
 }
 
-constexpr int kEndThreads = 256;
+// A suspect decoded: the pattern, the ends [lo, lo + span] (relative to the
+// item's first symbol) that its gram allows (none: span < 0), and where the
+// gram lies.
+struct Suspect {
+  uint32_t wi, pat;
+  int m, E, span;
+  int before, after, pair, len;   // as in the entry
+  int64_t lo, x, n_text;          // x: the gram's first symbol; n_text: symbols of the text
+  uint64_t arena0;
+};
 
+__device__ __forceinline__ Suspect decode_suspect(const StepParams& P, const GramTables& G,
+                                                  unsigned long long key) {
+  Suspect s;
+  s.span = -1;
+  const uint2 en = __ldg(reinterpret_cast<const uint2*>(G.entries + (key & 0xffffffu)));
+  const uint64_t x = key >> 24;  // arena offset of the gram
+  s.pat = en.x;
+  s.before = int(en.y & 255u);
+  s.after = int((en.y >> 8) & 255u);
+  s.pair = int((en.y >> 16) & 255u);
+  s.len = int(en.y >> 24);
+  s.m = P.m[s.pat];
+  s.E = G.edits[s.pat];
+  const int K = P.K[s.pat];
+  // the last item that starts at or before the gram
+  uint32_t a = 0, b = P.n_items;
+  while (a < b) {
+    const uint32_t mid = (a + b) >> 1;
+    if (P.items[mid].arena_base <= x)
+      a = mid + 1;
+    else
+      b = mid;
+  }
+  if (a == 0) return s;
+  s.wi = a - 1;
+  const WorkItem w = P.items[s.wi];
+  s.arena0 = w.arena_base;
+  s.x = int64_t(x - s.arena0);
+  s.n_text = w.e_new - w.base_pos;
+  const int64_t last = s.x + s.len - 1;
+  if (last >= s.n_text) return s;
+  s.lo = max(last + s.after - s.E, max(int64_t(0), w.e_prev - 2 * int64_t(K)) - w.base_pos);
+  const int64_t hi = min(last + int64_t(s.after) + s.E, s.n_text - 1);
+  if (s.lo <= hi) s.span = int(hi - s.lo);
+  return s;
+}
+
+// Least edits between r (at most 32) pattern symbols beside a found gram and
+// the text beside it, if at most lim (a larger value otherwise): the anchored
+// column recurrence (dummy row 0, 1, 2, ...) over text symbols t[0], t[d],
+// t[2 d], ..., at most avail, against bits o, o + 1, ... of the mask rows.
+// ends: bit j - r + lim is set where the r symbols match the first j of the
+// text within lim.  A cell within lim of a column lies at most lim off the
+// diagonal, so a diagonal value over 2 lim ends it.
+__device__ __forceinline__ int side(const uint32_t* __restrict__ peq, int o,
+                                    const uint8_t* __restrict__ t, int d, int r, int avail,
+                                    int lim, uint32_t& ends) {
+  if (r == 0) {  // nothing left to match: every text symbol is an insertion
+    ends = (0xffffffffu >> (31 - min(lim, avail))) << lim;
+    return 0;
+  }
+  ends = r <= lim ? 1u << (lim - r) : 0u;  // no text symbol: r deletions
+  int best = r;
+  uint32_t Pv = 0xffffffffu, Mv = 0u;
+  int score = r, diag = 0;
+  const int n = min(r + lim, avail), q = o >> 5, sh = o & 31;
+  if (n <= 0) return best;
+  // the masks of the next column and the symbol after it are on their way
+  // while a column is computed
+  auto mask = [&](uint32_t c) {
+    const uint32_t* row = peq + size_t(c) * 4;
+    return __funnelshift_r(__ldg(row + q), q < 3 ? __ldg(row + q + 1) : 0u, sh);
+  };
+  uint32_t eq_next = mask(t[0]), c_next = t[min(1, n - 1) * d];
+  for (int j = 0; j < n; ++j) {
+    const uint32_t eq = eq_next;
+    eq_next = mask(c_next);
+    c_next = t[min(j + 2, n - 1) * d];
+    const uint32_t sum = (eq & Pv) + Pv;
+    const uint32_t xv = eq | Mv;
+    const uint32_t xh = (sum ^ Pv) | eq;
+    const uint32_t ph = Mv | ~(xh | Pv), mh = Pv & xh;
+    score += int((ph >> (r - 1)) & 1u) - int((mh >> (r - 1)) & 1u);
+    best = min(best, score);
+    if (score <= lim) ends |= 1u << (j + 1 - r + lim);
+    if (j < r) {
+      diag += 1 - int(((xh | Mv) >> j) & 1u);
+      if (diag > 2 * lim) return lim + 1;
+    }
+    const uint32_t phs = (ph << 1) | 1u, mhs = mh << 1;
+    Pv = mhs | ~(xv | phs);
+    Mv = phs & xv;
+  }
+  return best;
+}
+
+// The found ends (bit j of hit: lo + j) as candidates, each (pattern, end)
+// pair once, one reservation per warp.  Called by whole warps.
+__device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, const Suspect& s,
+                                         uint32_t hit) {
+  if (!__any_sync(kFull, hit != 0)) return;
+  const unsigned lane = threadIdx.x & 31;
+  bool full = false;
+  for (uint32_t h = hit; h; h &= h - 1)
+    if (!insert_key(S, ((s.arena0 + uint64_t(s.lo + __ffs(h) - 1)) << 24) | s.pat, &full))
+      hit &= ~(h & (0u - h));
+  if (full) atomicOr(&P.ctr->overflow, 1u | 32u);
+  __syncwarp();
+  const int nf = __popc(hit);
+  int incl = nf;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(kFull, incl, d);
+    if (int(lane) >= d) incl += t;
+  }
+  const int tot = __shfl_sync(kFull, incl, 31);
+  if (!tot) return;
+  unsigned long long o = 0;
+  if (lane == 0) {
+    o = atomicAdd(&P.ctr->n_cand, (unsigned long long)tot);
+    const unsigned long long filled =
+        atomicAdd(&P.ctr->n_gram, (unsigned long long)tot) + (unsigned long long)tot;
+    if (filled > (S.mask + 1) / 4) atomicOr(&P.ctr->overflow, 1u | 32u);
+  }
+  o = __shfl_sync(kFull, o, 0) + unsigned(incl - nf);
+  bool over = false;
+  for (uint32_t h = hit; h; h &= h - 1, ++o) {
+    if (o < P.cap_cand) {
+      Candidate c;
+      c.wi = s.wi;
+      c.pat = s.pat;
+      c.e_rel = uint64_t(s.lo + __ffs(h) - 1);
+      P.cand[o] = c;
+    } else {
+      over = true;
+    }
+  }
+  if (over) atomicOr(&P.ctr->overflow, 1u);
+}
+
+constexpr int kEndThreads = 256;
+constexpr int kEndList = 64;
+
+// One thread per suspect, in two rounds so that warps stay full: the rest of
+// the gram's double piece against the text beside it, within one edit, drops
+// nearly every chance find after a few columns; what stays waits in a list per
+// warp.  The second round matches the pattern symbols on the gram's left, then
+// those on its right with the edits that are left: the right side's columns
+// are the ends.  (An occurrence keeps one double piece within one edit and one
+// half of it unedited, or one gram with its edit; that one's suspect finds its
+// end.)  With more than 32 symbols on a side, the 32 next to the gram are
+// matched, and the few suspects that pass are left to gram_long_kernel.
+// (4,096 byte patterns over 32 MiB, 3 M suspects: the whole pattern for every
+// suspect 892 us; its first 32 rows first 576; both sides at once, 9 lanes of a
+// warp busy, 965; in two rounds, but with the long patterns' runs among the
+// others', 660; this form 375, and 85 in gram_long_kernel.)
 __global__ void __launch_bounds__(kEndThreads)
     gram_ends_kernel(const StepParams P, const GramTables G,
-                     const unsigned long long* __restrict__ susp, const unsigned long long* n_susp,
-                     unsigned long long cap, const EndSet S) {
-  if (P.ctr->overflow & 1u) return;
-  __shared__ int cnt[4];
-  __shared__ unsigned long long order[kEndThreads];
-  const unsigned long long n = min(*n_susp, cap);
-  const unsigned lane = threadIdx.x & 31;
-  const unsigned long long stride = (unsigned long long)gridDim.x * kEndThreads;
-  for (unsigned long long base = (unsigned long long)blockIdx.x * kEndThreads; base < n;
-       base += stride) {
-    // the block's suspects by word count, so that a warp's patterns agree
-    if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
-    __syncthreads();
-    const unsigned long long i = base + threadIdx.x;
-    const unsigned long long key = i < n ? susp[i] : 0ull;
-    GramEntry en{};
-    int W = 3;
-    if (i < n) {
-      en = G.entries[key & 0xffffffu];
-      W = (P.m[en.pat] - 1) >> 5;
-    }
-    const int rank = atomicAdd(&cnt[W], 1);
-    __syncthreads();
-    int at = rank;
-    for (int w = 0; w < W; ++w) at += cnt[w];
-    order[at] = i < n ? key : ~0ull;
-    __syncthreads();
-    const unsigned long long mine = order[threadIdx.x];
+                     const unsigned long long* __restrict__ susp, GramCounters* C,
+                     unsigned long long cap, unsigned long long* __restrict__ longs,
+                     unsigned long long cap_long, const EndSet S) {
+  __shared__ unsigned long long list[kEndThreads / 32][kEndList];
+  const unsigned long long n = min(C->n_susp, cap);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (__any_sync(kFull, P.ctr->overflow & 1u)) return;
+  unsigned long long* mine = list[warp];
+  int ln = 0;  // listed suspects of this warp
+  // the second round for the last 32 (or all) listed suspects
+  auto resolve = [&]() {
+    __syncwarp();
+    const int i = max(ln - 32, 0) + lane;
+    Suspect s;
     uint32_t hit = 0;
-    uint32_t wi = 0, pat = 0;
-    int64_t lo = 0;
-    uint64_t arena0 = 0;
-    if (mine != ~0ull) {
-      en = G.entries[mine & 0xffffffu];
-      pat = en.pat;
-      const uint64_t x = mine >> 24;  // arena offset of the gram
-      const int m = P.m[pat], K = P.K[pat], E = G.edits[pat];
-      // the last item that starts at or before the gram
-      uint32_t a = 0, b = P.n_items;
-      while (a < b) {
-        const uint32_t mid = (a + b) >> 1;
-        if (P.items[mid].arena_base <= x)
-          a = mid + 1;
-        else
-          b = mid;
-      }
-      if (a > 0) {
-        wi = a - 1;
-        const WorkItem w = P.items[wi];
-        arena0 = w.arena_base;
-        const int64_t last = int64_t(x - arena0) + en.len - 1;  // the gram's last symbol
-        const int64_t n_text = w.e_new - w.base_pos;
-        lo = max(last + en.rest - E,
-                 max(int64_t(0), w.e_prev - 2 * int64_t(K)) - w.base_pos);
-        const int64_t hi = min(last + int64_t(en.rest) + E, n_text - 1);
-        if (last < n_text && lo <= hi) {
-          const uint32_t* peq = G.peq_fwd + size_t(pat) * 256 * 4;
-          const uint8_t* text = P.arena + arena0;
-          const int span = int(hi - lo);
-          if (m <= 32) hit = ends_run<1>(peq, text, lo, span, m, E);
-          else if (m <= 64) hit = ends_run<2>(peq, text, lo, span, m, E);
-          else if (m <= 96) hit = ends_run<3>(peq, text, lo, span, m, E);
-          else hit = ends_run<4>(peq, text, lo, span, m, E);
+    s.span = -1;
+    const unsigned long long key = i < ln ? mine[i] : 0ull;
+    int w = -1;
+    if (i < ln) s = decode_suspect(P, G, key);
+    ln = max(ln - 32, 0);
+    if (s.span >= 0) {
+      const uint32_t* fwd = G.peq_fwd + size_t(s.pat) * 256 * 4;
+      const uint8_t* text = P.arena + s.arena0;
+      const int lim = s.E - ((s.pair & kGramEdit) ? 1 : 0);
+      if (s.before <= 32 && s.after <= 32) {
+        uint32_t ends;
+        const int kl = side(P.peq_rev + size_t(s.pat) * 256 * 4, s.m - s.before, text + s.x - 1,
+                            -1, s.before, int(min(s.x, int64_t(64))), lim, ends);
+        const int left = lim - kl;  // edits left for the right side
+        if (left >= 0) {
+          const int64_t next = s.x + s.len;
+          side(fwd, s.m - s.after, text + next, 1, s.after,
+               int(min(s.n_text - next, int64_t(64))), left, ends);
+          // bit b: the end after + b - left symbols past the gram; hit: from lo on
+          const int64_t sh = s.lo - (next - 1 + s.after - left);
+          hit = sh >= 0 ? (sh < 32 ? ends >> sh : 0u) : ends << -sh;
+          hit &= 0xffffffffu >> (31 - s.span);
         }
+      } else {
+        // up to 32 symbols next to the gram on each side; what is left runs
+        // whole (gram_long_kernel)
+        uint32_t ends;
+        const int kl = side(P.peq_rev + size_t(s.pat) * 256 * 4, s.m - s.before, text + s.x - 1,
+                            -1, min(s.before, 32), int(min(s.x, int64_t(64))), lim, ends);
+        const int64_t next = s.x + s.len;
+        if (kl <= lim && side(fwd, s.m - s.after, text + next, 1, min(s.after, 32),
+                              int(min(s.n_text - next, int64_t(64))), lim - kl, ends) <= lim - kl)
+          w = ((s.m - 1) >> 5) - 1;
+      }
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const unsigned b = __ballot_sync(kFull, w == l);
+      if (!b) continue;
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd(&C->n_long[l], (unsigned long long)__popc(b));
+      at = __shfl_sync(kFull, at, 0) + __popc(b & ((1u << lane) - 1u));
+      if (w == l) {
+        if (at < cap_long) longs[l * cap_long + at] = key;
+        else atomicOr(&P.ctr->overflow, kGramOverflow | 1u);
       }
     }
     __syncwarp();
-    // distinct (pattern, end) pairs, one reservation per warp
-    bool full = false;
-    for (uint32_t h = hit; h; h &= h - 1)
-      if (!insert_key(S, ((arena0 + uint64_t(lo + __ffs(h) - 1)) << 24) | pat, &full))
-        hit &= ~(h & (0u - h));
-    if (full) atomicOr(&P.ctr->overflow, 1u | 32u);
-    const int nf = __popc(hit);
-    int incl = nf;
+    put_ends(P, S, s, hit);
+    __syncwarp();
+  };
+  const unsigned long long stride = (unsigned long long)gridDim.x * kEndThreads;
+  for (unsigned long long base = (unsigned long long)blockIdx.x * kEndThreads + warp * 32; base < n;
+       base += stride) {
+    const unsigned long long i = base + lane;
+    unsigned long long key = 0;
+    bool keep = false;
+    if (i < n) {
+      key = susp[i];
+      const Suspect s = decode_suspect(P, G, key);
+      keep = s.span >= 0;
+      const int r = s.pair & 63;
+      if (keep && r) {
+        const int lim = min(s.E, 1);
+        const uint8_t* text = P.arena + s.arena0 + s.x;
+        const size_t p0 = size_t(s.pat) * 256 * 4;
+        const bool lf = (s.pair & kGramLeft) != 0;
+        uint32_t ends;
+        keep = side(lf ? P.peq_rev + p0 : G.peq_fwd + p0, s.m - (lf ? s.before : s.after),
+                    lf ? text - 1 : text + s.len, lf ? -1 : 1, r,
+                    int(min(lf ? s.x : s.n_text - s.x - s.len, int64_t(64))), lim, ends) <= lim;
+      }
+    }
+    const unsigned m = __ballot_sync(kFull, keep);
+    if (!m) continue;
+    if (keep) mine[ln + __popc(m & ((1u << lane) - 1u))] = key;
+    ln += __popc(m);
+    if (ln >= 32) resolve();
+  }
+  if (ln) resolve();
+}
+
+// The whole pattern over the ends of the listed suspects, whole warps of one
+// word count.
+__global__ void __launch_bounds__(kEndThreads)
+    gram_long_kernel(const StepParams P, const GramTables G, const GramCounters* C,
+                     const unsigned long long* __restrict__ longs, unsigned long long cap_long,
+                     const EndSet S) {
+  if (__any_sync(kFull, P.ctr->overflow & 1u)) return;
+  unsigned long long n[3], warps = 0;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(kFull, incl, d);
-      if (int(lane) >= d) incl += t;
+  for (int l = 0; l < 3; ++l) {
+    n[l] = min(C->n_long[l], cap_long);
+    warps += (n[l] + 31) / 32;
+  }
+  const int lane = threadIdx.x & 31;
+  const unsigned long long stride = (unsigned long long)gridDim.x * (kEndThreads / 32);
+  for (unsigned long long wj = (unsigned long long)blockIdx.x * (kEndThreads / 32) +
+                               (threadIdx.x >> 5);
+       wj < warps; wj += stride) {
+    unsigned long long t = wj;
+    int l = 0;
+    while (l < 2 && t >= (n[l] + 31) / 32) t -= (n[l++] + 31) / 32;
+    const unsigned long long i = t * 32 + lane;
+    Suspect s;
+    uint32_t hit = 0;
+    if (i < n[l]) {
+      s = decode_suspect(P, G, longs[l * cap_long + i]);
+      const uint32_t* peq = G.peq_fwd + size_t(s.pat) * 256 * 4;
+      const uint8_t* text = P.arena + s.arena0;
+      if (l == 0) hit = ends_run<2>(peq, text, s.lo, s.span, s.m, s.E);
+      else if (l == 1) hit = ends_run<3>(peq, text, s.lo, s.span, s.m, s.E);
+      else hit = ends_run<4>(peq, text, s.lo, s.span, s.m, s.E);
     }
-    const int tot = __shfl_sync(kFull, incl, 31);
-    if (tot) {
-      unsigned long long o = 0;
-      if (lane == 0) {
-        o = atomicAdd(&P.ctr->n_cand, (unsigned long long)tot);
-        const unsigned long long filled =
-            atomicAdd(&P.ctr->n_gram, (unsigned long long)tot) + (unsigned long long)tot;
-        if (filled > (S.mask + 1) / 4) atomicOr(&P.ctr->overflow, 1u | 32u);
-      }
-      o = __shfl_sync(kFull, o, 0) + unsigned(incl - nf);
-      bool over = false;
-      for (uint32_t h = hit; h; h &= h - 1, ++o) {
-        if (o < P.cap_cand) {
-          Candidate c;
-          c.wi = wi;
-          c.pat = pat;
-          c.e_rel = uint64_t(lo + __ffs(h) - 1);
-          P.cand[o] = c;
-        } else {
-          over = true;
-        }
-      }
-      if (over) atomicOr(&P.ctr->overflow, 1u);
-    }
-    __syncthreads();  // cnt and order are reused
+    __syncwarp();
+    put_ends(P, S, s, hit);
+    __syncwarp();
   }
 }
 
@@ -381,7 +625,7 @@ __global__ void __launch_bounds__(256)
 }
 
 size_t gram_smem(uint32_t n_words) {
-  return size_t(n_words) * 4 + size_t(kGramThreads / 32) * kQueue * 8;
+  return size_t(n_words) * 4 + size_t(kGramThreads / 32) * sizeof(GramWarp);
 }
 
 }  // namespace
@@ -413,7 +657,11 @@ cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramSca
     gram_scan_kernel<true><<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
   else
     gram_scan_kernel<false><<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
-  gram_ends_kernel<<<p.num_sms * 6, kEndThreads, 0, s>>>(p, g, a.susp, a.n_susp, a.cap_susp, set);
+  gram_ends_kernel<<<p.num_sms * 6, kEndThreads, 0, s>>>(p, g, a.susp, a.ctr_slice, a.cap_susp,
+                                                         a.longs, a.cap_long, set);
+  if (g.any_long)
+    gram_long_kernel<<<p.num_sms * 6, kEndThreads, 0, s>>>(p, g, a.ctr_slice, a.longs, a.cap_long,
+                                                           set);
   return cudaGetLastError();
 }
 

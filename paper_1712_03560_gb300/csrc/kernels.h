@@ -111,32 +111,40 @@ cudaError_t prepare_prefilter_kernel(int max_smem_bytes);
 
 // Gram index in front of the forward scan (grams.cu).
 constexpr int kGramThreads = 1024;            // threads of an index scan block (one per SM)
-constexpr uint32_t kGramMaxWords = 32768;     // 128 KiB of table bits in shared memory
-constexpr int kGramLens = 9;                  // gram lengths of an index
+constexpr uint32_t kGramMaxWords = 45056;     // 176 KiB of table bits in shared memory
+constexpr int kGramLens = 6;                  // key lengths of an index
 constexpr unsigned kGramOverflow = 1u << 7;   // StepCounters::overflow: suspects over capacity
-// odd multipliers: byte grams of more than four symbols, table bits, directory
-constexpr uint32_t kGramMixLo = 0x9E3779B1u, kGramMixHi = 0x6C8E9CF5u;
+// odd multipliers: table bits of hashed keys, directory
 constexpr uint32_t kGramBitMul = 0x9E3779B1u, kGramDirMul = 0x2C1B3C6Du;
-struct GramLen {             // one gram length
-  uint32_t mask_lo, mask_hi; // the gram's symbols within 16 2-bit symbols, or 8 bytes
+struct GramLen {             // one key length: the first symbols of a gram
+  uint32_t mask;             // the key within 16 2-bit symbols, or four bytes
   uint32_t mul, shift;       // table bit of a key: (key * mul) >> shift
   uint32_t word0;            // first word of the length's table
   uint32_t dir0;             // first directory slot
   uint32_t dir_shift, dir_mask, max_probe;
 };
+constexpr int kGramLeft = 128, kGramEdit = 64;
 struct GramEntry {           // one gram of a pattern
   uint32_t pat;
-  uint16_t rest;             // pattern symbols after the gram
-  uint16_t len;              // symbols of the gram
+  uint8_t before, after;     // pattern symbols beside the part that the gram stands for
+  uint8_t pair;              // symbols of its double piece beyond the gram (at most 32),
+                             // kGramLeft: before it; kGramEdit: the gram holds an edit
+  uint8_t len;               // symbols of the gram
+  uint32_t lo, hi;           // 16 2-bit symbols (lo), or eight bytes
 };
 struct EndSet {              // (arena offset of an end << 24 | pattern) keys; all ones = empty
   unsigned long long* slots;
   unsigned long long mask;   // capacity - 1 (a power of two)
 };
+struct GramCounters {        // one per slice of the arena
+  unsigned long long n_susp;
+  unsigned long long n_long[3];  // suspects left of patterns of two, three, four words
+};
 struct GramTables {
   const GramEntry* entries;
   const uint8_t* edits;      // [n_pat] most edits of an occurrence (K under unit costs)
   const uint32_t* peq_fwd;   // [n_pat][256][4] forward match masks
+  int32_t any_long;          // 1: a gram has more than 32 pattern symbols on a side
 };
 struct GramScan {
   GramLen len[kGramLens];
@@ -146,11 +154,14 @@ struct GramScan {
   uint32_t n_words;          // table words (a multiple of 4)
   const uint32_t* bits;
   const uint4* dir;          // {key, first entry, entries (0 = empty), -}
+  const GramEntry* entries;
   const uint8_t* arena;
   unsigned long long t_begin, t_end;  // 512-symbol tiles of this slice
   unsigned long long* susp;  // arena offset of a gram << 24 | entry
   unsigned long long cap_susp;
-  unsigned long long* n_susp;
+  unsigned long long* longs; // [3][cap_long] suspects left, by word count
+  unsigned long long cap_long;
+  GramCounters* ctr_slice;
   StepCounters* ctr;
 };
 cudaError_t prepare_gram_kernels();
@@ -158,7 +169,7 @@ cudaError_t prepare_gram_kernels();
 // of a row is symbol j, or the j-th from the end.
 cudaError_t launch_peq(const uint8_t* bytes, const uint8_t* len, uint32_t n_pat, uint32_t* peq,
                        bool reversed, cudaStream_t s);
-// scan and ends of one slice (two launches)
+// scan, ends and long of one slice (two or three launches)
 cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramScan& a,
                          const EndSet& set, cudaStream_t s);
 

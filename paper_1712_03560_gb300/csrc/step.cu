@@ -178,7 +178,7 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
     // whole tiles (the end padding is longer than a tile and holds no text)
     const size_t n_tiles = (pl.arena_bytes - 16) / 512, slice = gram_slice(pl) / 512;
     topo_add(slices);
-    CK(cudaMemsetAsync(gr.ctr.p, 0, slices * sizeof(unsigned long long), s));
+    CK(cudaMemsetAsync(gr.ctr.p, 0, slices * sizeof(GramCounters), s));
     for (size_t q = 0; q < slices; ++q) {
       GramScan a = gr.scan;
       a.arena = ctx->arena.p;
@@ -186,11 +186,13 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
       a.t_end = std::min(n_tiles, (q + 1) * slice);
       a.susp = gr.susp.p;
       a.cap_susp = gr.susp.cap;
-      a.n_susp = gr.ctr.p + q;
+      a.longs = gr.longs.p;
+      a.cap_long = gr.longs.cap / 3;
+      a.ctr_slice = gr.ctr.p + q;
       a.ctr = ctx->d_ctr;
       CK(launch_grams(P, gr.t, a, EndSet{ctx->pset.p, ctx->pset.cap - 1}, s));
     }
-    ctx->st.launches += 2 * slices;
+    ctx->st.launches += (gr.t.any_long ? 3 : 2) * slices;
     ctx->st.scan_launches += slices;
   }
   for (size_t bi = 0; bi < buckets.size(); ++bi) {
@@ -412,6 +414,14 @@ static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) 
   return size_t(syms * rate) + (size_t(1) << 14);
 }
 
+// Room for n suspects of a slice; those of long patterns that a second look
+// keeps are a small part.
+static int ensure_grams(oasm_ctx* ctx, size_t n) {
+  const int rc = ensure(ctx, ctx->grams.susp, n, "gram suspects");
+  if (rc || !ctx->grams.t.any_long) return rc;
+  return ensure(ctx, ctx->grams.longs, 3 * (n / 4 + (size_t(1) << 14)), "gram suspects");
+}
+
 // One upload: items | regions | chunks.
 static int upload_plan(oasm_ctx* ctx, StepPlan& pl) {
   int rc;
@@ -485,7 +495,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
       // and this step and the next ones scan every pattern
       const size_t cap = ctx->grams.susp.cap, most = gram_capacity(ctx, pl, true);
       if (cap < most) {
-        if ((rc = ensure(ctx, ctx->grams.susp, std::min(most, 8 * cap), "gram suspects"))) return rc;
+        if ((rc = ensure_grams(ctx, std::min(most, 8 * cap)))) return rc;
       } else {
         pl.grams = false;
         ctx->grams.off_steps = 32;
@@ -682,8 +692,7 @@ int step_begin(oasm_ctx* ctx) {
                         "piece filter set")))
     return rc;
   if (pl.grams && ((rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters")) ||
-                   (rc = ensure(ctx, ctx->grams.susp, gram_capacity(ctx, pl, false),
-                                "gram suspects"))))
+                   (rc = ensure_grams(ctx, gram_capacity(ctx, pl, false)))))
     return rc;
   if (!ctx->pool_hdr.p) {
     if ((rc = ensure(ctx, ctx->pool_hdr, 1 << 14, "window pool"))) return rc;
