@@ -255,7 +255,9 @@ struct DevArray {
 };
 
 // The gram index (grams.cu) of a context: its tables, and the buckets of the
-// patterns that stay on the forward scan while it runs.
+// patterns that stay on the forward scan while it runs.  It also takes the
+// piece filter's patterns; if it cannot take all of them the piece filter runs
+// beside it (both put their ends through one set).
 struct Grams {
   uint32_t n_pat = 0;         // patterns it serves; 0: no index
   GramTables t{};
@@ -263,6 +265,7 @@ struct Grams {
   double rate = 0;            // expected suspects per text symbol
   double clk = 0;             // clocks of an SM per symbol it takes
   double saved_clk = 0;       // and saves, against the forward scan of every pattern
+  bool all_pref = false;      // serves every pattern of the piece filter
   std::vector<Bucket> rest;
   DevArray<unsigned long long> susp;
   DevArray<unsigned long long> longs;

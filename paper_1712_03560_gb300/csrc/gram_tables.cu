@@ -25,6 +25,8 @@ double buckets_cost(const std::vector<Bucket>& bs) {
 }
 // Clocks of one SM per suspect (the ends kernel's first round, and both), per
 // table hit (a directory look-up), and per text symbol and key length.
+// (kFilter: the piece filter and the verification of its proposals, per symbol.)
+constexpr double kFilter = 15.0;
 constexpr double kPair = 6.0, kEnds = 25.0, kLookup = 4.0, kLength = 0.12;
 
 constexpr int kMaxGram2 = 16, kMaxGram = 8;  // symbols of a gram: 2-bit text, bytes
@@ -114,15 +116,15 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   if (ctx->cfg.myers_only || ctx->cfg.full_words || n >= (1u << 24)) return OASM_OK;
   std::vector<double> cnt(256, 0.0);
   double tot = 0;
-  int n_scan = 0;
+  int n_pref = 0;
   for (uint32_t p = 0; p < n; ++p) {
-    if (pref[p]) continue;
-    ++n_scan;
+    n_pref += pref[p] != 0;
     for (uint8_t c : ctx->pats[p]) cnt[c] += 1, tot += 1;
   }
-  if (n_scan < kLaneGroup) return OASM_OK;  // fewer run one group in the segment mapping
-  const double scan_all = buckets_cost(ctx->buckets);
-  const double share = scan_all / n_scan;  // the forward scan's clocks per pattern
+  // clocks per pattern of the forward scan and of the piece filter
+  const double scan_all = buckets_cost(ctx->buckets) + (n_pref ? kFilter : 0.0);
+  const double scan_share = buckets_cost(ctx->buckets) / std::max(1, int(n) - n_pref);
+  const double filter_share = kFilter / std::max(1, n_pref);
   // at most four symbols that two adjacent bits tell apart: 2-bit text (other
   // symbols of the text read as one of the four; the ends run tells)
   int shift2 = -1, distinct = 0;
@@ -153,7 +155,6 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   for (uint32_t p = 0; p < n; ++p) {
     const int m = ctx->m[p], E = ctx->K[p] / cmin;
     edits[p] = uint8_t(E);
-    if (pref[p]) continue;
     sym.resize(m);
     ps.resize(m);
     for (int i = 0; i < m; ++i) {
@@ -228,7 +229,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
         }
       }
     }
-    if (best > 0.7 * share) continue;
+    if (best > 0.7 * (pref[p] ? filter_share : scan_share)) continue;
     served[p] = 1;
     gr.n_pat += 1;
     ends_clk += best_clk;
@@ -269,7 +270,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     gr.n_pat = 0;
     return OASM_OK;
   };
-  if (gr.n_pat < uint32_t(kLaneGroup)) return none();
+  if (!gr.n_pat) return OASM_OK;
   // per key length: a table of one bit per key (direct, or hashed to the size
   // that fits), and a directory
   struct Len {
@@ -356,6 +357,8 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   bits.resize(a.n_words, 0u);
   gr.clk = ends_clk + kLength * double(lens.size()) + kLookup * false_bits;
   if (gr.clk > 0.7 * scan_all) return none();  // not enough to gain
+  gr.all_pref = true;
+  for (uint32_t p = 0; p < n; ++p) gr.all_pref = gr.all_pref && (!pref[p] || served[p]);
   auto up = [&](auto** dst, const auto& v) -> cudaError_t {
     using T = typename std::decay<decltype(v[0])>::type;
     T* d = nullptr;
@@ -379,7 +382,8 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
 // Clocks per text symbol that the index saves, for the step rule.
 void finish_grams(oasm_ctx* ctx) {
   Grams& gr = ctx->grams;
-  gr.saved_clk = buckets_cost(ctx->buckets) - buckets_cost(gr.rest) - gr.clk;
+  gr.saved_clk = buckets_cost(ctx->buckets) - buckets_cost(gr.rest) - gr.clk +
+                 (ctx->n_pref_pat && gr.all_pref ? kFilter : 0.0);
   if (gr.saved_clk <= 0) gr.n_pat = 0;
 }
 

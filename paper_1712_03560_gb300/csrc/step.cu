@@ -127,7 +127,7 @@ void plan_regions(oasm_ctx* ctx, StepPlan& pl) {
   // piece filter: start positions x with t[x .. x + 3] in the text, in
   // segments of kPrefSeg (every piece of an occurrence whose end is reported
   // this step starts at or after base_pos, inside the stored tail)
-  if (ctx->n_pref_pat) {
+  if (ctx->n_pref_pat && !(pl.grams && ctx->grams.all_pref)) {
     for (uint32_t i = 0; i < pl.items.size(); ++i) {
       const WorkItem& w = pl.items[i];
       const int64_t x_end = w.e_new - 3;  // exclusive

@@ -146,3 +146,30 @@ def test_index_runs_of_one_symbol():
             W.plant(rng, text, cp)
     got, _ = run_gpu(pats, ks, text)
     assert canon(got) == oracle_rows(pats, ks, text)
+
+
+@pytest.mark.parametrize("piece", [1, 4])
+def test_index_takes_the_piece_filters_patterns(piece):
+    """A large step looks the piece filter's patterns up in the index too, or,
+    with a pattern that the index leaves (one repeated symbol), runs the piece
+    filter beside it; small steps of the same stream run the filter."""
+    rng = np.random.default_rng(870 + piece)
+    pats, ks, text = dictionary(rng, 256, N_PAT, 12, 100, 400_003, lambda m: min(8, m // 6))
+    cuts = [390_000, 390_500, 399_990]
+    for extra in (False, True):
+        if extra:
+            pats = pats + [np.full(40, text[0], np.uint8)]
+            ks = ks + [1]
+            text[200_000:200_300] = text[0]
+        got, _ = run_gpu(pats, ks, text, splits=cuts, cfg={"prefilter_piece": piece})
+        assert canon(got) == oracle_rows(pats, ks, text)
+
+
+def test_index_of_a_few_long_patterns():
+    """Fewer patterns than a warp has lanes, thresholds up to 15."""
+    rng = np.random.default_rng(880)
+    pats, ks, text = dictionary(rng, 256, 9, 60, 128, 1_000_003, lambda m: 3 + m // 11, copies=40)
+    got, st = run_gpu(pats, ks, text)
+    scan, st_scan = run_gpu(pats, ks, text, cfg={"full_words": 1})
+    assert runs_index(st, st_scan)
+    assert canon(got) == canon(scan) == oracle_rows(pats, ks, text)
