@@ -394,11 +394,7 @@ int oasm_open_stream(oasm_ctx* ctx, uint32_t* sid) {
                        size_t(ctx->mem_stride) * sizeof(MemRow), ctx->stream));
   }
   ctx->free_slots.pop();
-  HitVec keep;  // the slot's queue storage, kept from its last stream
-  keep.swap(s.ready);
-  keep.clear();
-  s = StreamRec();
-  s.ready.swap(keep);
+  s.reset();
   s.open = true;
   ++ctx->n_open;
   *sid = i;
@@ -419,13 +415,7 @@ int oasm_close_stream(oasm_ctx* ctx, uint32_t sid) {
     if (!pc.dev) ctx->stage[pc.sb].pending -= pc.n;
   // a stream that never fed anything since its last end has empty windows
   const bool clean = s.clean && s.pos == 0;
-  // the slot keeps its queue's storage for the next stream it serves (no new
-  // pages to touch when large outputs repeat)
-  HitVec keep;
-  keep.swap(s.ready);
-  keep.clear();
-  s = StreamRec();
-  s.ready.swap(keep);
+  s.reset();
   s.clean = clean;
   --ctx->n_open;
   ctx->free_slots.push(sid);
@@ -631,7 +621,7 @@ int oasm_feed_many(oasm_ctx* ctx, uint32_t n, const uint32_t* sid, const uint8_t
     dst[j] = base[sid[j]];
     base[sid[j]] += len[j];
   }
-  parallel_parts(n, total > (size_t(4) << 20) ? std::max<size_t>(1, n / 16) : n + 1,
+  parallel_parts(n, total > (size_t(1) << 18) ? std::max<size_t>(1, n / 16) : n + 1,
                  [&](size_t lo, size_t hi) {
                    for (size_t j = lo; j < hi; ++j)
                      if (len[j]) memcpy(sg->h + dst[j], buf + off[j], len[j]);

@@ -204,6 +204,16 @@ struct StreamRec {
   const oasm_hit* lent = nullptr;
   size_t lent_n = 0;
   int lent_buf = 0;
+  // A fresh record that keeps the storage of its queue and its pieces (no new
+  // pages to touch, no allocation per stream).
+  void reset() {
+    StreamRec fresh;
+    ready.clear();
+    pieces.clear();
+    fresh.ready.swap(ready);
+    fresh.pieces.swap(pieces);
+    *this = std::move(fresh);
+  }
 };
 
 // A finished step whose records are still on their way to the host: the
@@ -286,6 +296,21 @@ struct StepPlan {
   uint64_t new_bytes = 0;
   bool ordered = false;              // records written in canonical order (no record sort)
   bool grams = false;                // the gram index and the rest buckets scan this step
+  // An empty plan that keeps its vectors' storage.
+  void clear() {
+    StepPlan fresh;
+    const auto keep = [](auto& to, auto& from) {
+      from.clear();
+      to.swap(from);
+    };
+    keep(fresh.items, items);
+    keep(fresh.sids, sids);
+    keep(fresh.take, take);
+    keep(fresh.regions, regions);
+    keep(fresh.region_off, region_off);
+    keep(fresh.chunks, chunks);
+    *this = std::move(fresh);
+  }
 };
 
 // Pinned host staging for fed bytes, with its device copy.  Two of them

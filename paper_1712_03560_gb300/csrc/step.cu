@@ -106,22 +106,33 @@ void plan_regions(oasm_ctx* ctx, StepPlan& pl) {
       total += std::max<int64_t>(0, w.e_new - lo);
     }
     const int64_t R = region_len(ctx, b, total);
+    // longest first: a block's warps get regions of similar length (a block
+    // holds its SM until its slowest warp ends) and long work starts early.
+    // Whole regions come first, each item's last one by its length in 64ths of
+    // a whole one (placed by counting: a sort took 0.3 ms of a step of 29,000
+    // regions, or of 4,096 streams)
+    const auto item_lo = [&](const WorkItem& w) {
+      return std::max<int64_t>(0, w.e_prev - 2 * b.kmax);
+    };
+    const auto bin = [&](int64_t len) { return size_t(63 - std::min<int64_t>(63, len * 64 / R)); };
+    size_t whole = 0, at[65] = {};
+    for (const WorkItem& w : pl.items) {
+      const int64_t len = w.e_new - item_lo(w);
+      if (len <= 0) continue;
+      whole += size_t(len / R);
+      if (len % R) at[bin(len % R) + 1] += 1;
+    }
     const size_t first = pl.regions.size();
+    at[0] = first + whole;
+    for (int q = 0; q < 64; ++q) at[q + 1] += at[q];
+    pl.regions.resize(at[64]);
+    size_t next = first;
     for (uint32_t i = 0; i < pl.items.size(); ++i) {
       const WorkItem& w = pl.items[i];
-      const int64_t lo = std::max<int64_t>(0, w.e_prev - 2 * b.kmax);
-      for (int64_t a = lo; a < w.e_new; a += R) {
-        Region r{};
-        r.wi = i;
-        r.a = a;
-        r.b = std::min(w.e_new, a + R);
-        pl.regions.push_back(r);
-      }
+      int64_t a = item_lo(w);
+      for (; a + R <= w.e_new; a += R) pl.regions[next++] = Region{i, 0, a, a + R};
+      if (a < w.e_new) pl.regions[at[bin(w.e_new - a)]++] = Region{i, 0, a, w.e_new};
     }
-    // longest first: a block's warps get regions of similar length (a block
-    // holds its SM until its slowest warp ends) and long work starts early
-    std::stable_sort(pl.regions.begin() + first, pl.regions.end(),
-                     [](const Region& x, const Region& y) { return (x.b - x.a) > (y.b - y.a); });
   }
   pl.region_off.push_back(pl.regions.size());
   // piece filter: start positions x with t[x .. x + 3] in the text, in
@@ -649,7 +660,7 @@ int step_begin(oasm_ctx* ctx) {
   int rc;
   const auto t_plan = std::chrono::steady_clock::now();
   Flight& f = ctx->flight;
-  f.pl = StepPlan();
+  f.pl.clear();
   StepPlan& pl = f.pl;
   // device copies of the staging buffers first: plan_step takes their addresses
   for (Stage& sg : ctx->stage)
