@@ -223,6 +223,7 @@ struct StreamRec {
 // streams (settle_records).
 struct PendingRecords {
   bool on = false;
+  bool direct = false;  // already in the pinned buffer (a small step wrote them)
   int buf = 0;
   size_t n = 0;
   std::vector<uint32_t> sids;                 // stream of each work item
@@ -295,6 +296,7 @@ struct StepPlan {
   int sb = 1, kb = 10;
   uint64_t new_bytes = 0;
   bool ordered = false;              // records written in canonical order (no record sort)
+  bool small = false;                // everything after the candidates in one launch
   bool grams = false;                // the gram index and the rest buckets scan this step
   // An empty plan that keeps its vectors' storage.
   void clear() {
@@ -447,6 +449,7 @@ struct oasm_ctx {
   std::vector<GraphSlot> graphs;
   uint64_t graph_clock = 0;
   uint64_t step_topo = 0;    // topology of the step being enqueued
+  int small_blocks = 0;      // blocks of the small steps' launch (0: never used)
   int sort_blocks = 0;       // radix-sort blocks: as many as are resident together
   bool capturing = false;
 

@@ -218,6 +218,25 @@ cudaError_t launch_ordered_scan(const StepParams& p, unsigned long long* part, c
 cudaError_t launch_ordered_emit(const StepParams& p, const unsigned long long* sorted,
                                 DevHit* dst, unsigned long long* run_start, cudaStream_t s);
 cudaError_t launch_tails(const StepParams& p, cudaStream_t s);
+// Everything after the candidates of a small step with ordered records, in one
+// cooperative launch (p.pair_pool and p.seg need no filling before it).
+struct SmallStep {
+  DevHit* dst;                    // records in canonical order
+  DevHit* direct;                 // pinned host memory for up to direct_cap of them
+  unsigned long long direct_cap;  // (more go to dst)
+  unsigned long long* run_start;  // pinned host memory, [n_items + 1]
+  StepCounters* counters;         // pinned host memory
+  unsigned long long* part;       // [nblocks]
+  unsigned int* hist;             // sort_hist_len(nblocks)
+  unsigned int* bar;              // barrier arrivals, zero before the launch
+  unsigned int* sort_bar;
+  // set by the launcher
+  const unsigned long long* sorted;
+  size_t seg_len;
+  int lo_bit, hi_bit;
+};
+int small_step_grid(int num_sms);  // most blocks of the launch; 0: it does not fit
+cudaError_t launch_small_step(const StepParams& p, SmallStep a, int nblocks, cudaStream_t s);
 // start[w] = first canonically sorted record of work item w, w = 0..n_items
 // (start[n_items] = the record count), from the sorted record keys
 cudaError_t launch_runs(const unsigned long long* sorted_keys, const StepParams& p,

@@ -225,7 +225,7 @@ __device__ __forceinline__ void put_record(const StepParams& P, unsigned long lo
   P.ovals[o] = uint32_t(o);
 }
 
-__global__ void __launch_bounds__(256) verify_kernel(const StepParams P) {
+__device__ void verify_body(const StepParams& P) {
   const unsigned long long n = min(P.ctr->n_cand, P.cap_cand);
   // stop only on an upstream overflow: the hit count must stay exact when this
   // kernel's own output overflows, so the re-run can size the buffer at once
@@ -336,6 +336,8 @@ __global__ void __launch_bounds__(256) verify_kernel(const StepParams P) {
     }
   }
 }
+
+__global__ void __launch_bounds__(256) verify_kernel(const StepParams P) { verify_body(P); }
 
 // ---------------------------------------------------------------- radix sort
 // Stable LSD radix sort, 8-bit digits, every pass in one cooperative launch
@@ -456,13 +458,10 @@ __device__ __forceinline__ bool sort_barrier(SortSmem& sm, unsigned int* bar, un
   return sm.stop == 0;
 }
 
-__global__ void __launch_bounds__(kSortThreads, 4)
-    sort_kernel(unsigned long long* keys, unsigned long long* keys_alt, uint32_t* vals,
-                uint32_t* vals_alt, const unsigned long long* count, unsigned long long cap,
-                int lo_bit, int hi_bit, unsigned int* hist, unsigned int* bar,
-                StepCounters* ctr) {
-  extern __shared__ __align__(16) unsigned char sort_smem[];
-  SortSmem& sm = *reinterpret_cast<SortSmem*>(sort_smem);
+__device__ void sort_body(SortSmem& sm, unsigned long long* keys, unsigned long long* keys_alt,
+                          uint32_t* vals, uint32_t* vals_alt, const unsigned long long* count,
+                          unsigned long long cap, int lo_bit, int hi_bit, unsigned int* hist,
+                          unsigned int* bar, StepCounters* ctr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned long long n = min(*count, cap);
   // keys per block: an even split, in whole tiles (two or more tiles to a block
@@ -603,6 +602,16 @@ __global__ void __launch_bounds__(kSortThreads, 4)
     vals = vals_alt;
     vals_alt = tv;
   }
+}
+
+__global__ void __launch_bounds__(kSortThreads, 4)
+    sort_kernel(unsigned long long* keys, unsigned long long* keys_alt, uint32_t* vals,
+                uint32_t* vals_alt, const unsigned long long* count, unsigned long long cap,
+                int lo_bit, int hi_bit, unsigned int* hist, unsigned int* bar,
+                StepCounters* ctr) {
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  sort_body(*reinterpret_cast<SortSmem*>(sort_smem), keys, keys_alt, vals, vals_alt, count, cap,
+            lo_bit, hi_bit, hist, bar, ctr);
 }
 
 __global__ void permute_kernel(const DevHit* __restrict__ src, const uint32_t* __restrict__ idx,
@@ -750,8 +759,7 @@ __device__ __forceinline__ uint32_t pair_of(uint64_t key, int sb) {
 // with the pair's constants, and the pending level stays in registers (a
 // dozen signatures with K up to 15: 171 -> 72 us; 3.7 M hits of one motif:
 // 291 -> 167).
-__global__ void __launch_bounds__(128)
-    filter_kernel(const StepParams P, const unsigned long long* __restrict__ S) {
+__device__ void filter_body(const StepParams& P, const unsigned long long* S) {
   if (P.ctr->overflow & 3u) return;  // candidates or hits incomplete; keep counting records
   const unsigned long long n = min(P.ctr->n_hits, P.cap_hits);
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -876,6 +884,11 @@ __global__ void __launch_bounds__(128)
   }
 }
 
+__global__ void __launch_bounds__(128)
+    filter_kernel(const StepParams P, const unsigned long long* __restrict__ S) {
+  filter_body(P, S);
+}
+
 // First index of the sorted hit keys S[0, n) whose pair is >= pr.
 __device__ __forceinline__ unsigned long long pair_lower_bound(const unsigned long long* S,
                                                                unsigned long long n,
@@ -896,8 +909,7 @@ __device__ __forceinline__ unsigned long long pair_lower_bound(const unsigned lo
 // clears the decided ones) in the stream state.  The ordered record path
 // runs the two apart, so the state changes only once the record count is
 // known to fit (a step that overflows is re-run from unchanged state).
-__global__ void finalize_kernel(const StepParams P, const unsigned long long* __restrict__ S,
-                                int phase) {
+__device__ void finalize_body(const StepParams& P, const unsigned long long* S, int phase) {
   if (P.ctr->overflow) return;
   const unsigned long long npairs = (unsigned long long)P.n_items * P.n_pat;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -943,7 +955,12 @@ __global__ void finalize_kernel(const StepParams P, const unsigned long long* __
   }
 }
 
-__global__ void tails_kernel(const StepParams P) {
+__global__ void finalize_kernel(const StepParams P, const unsigned long long* __restrict__ S,
+                                int phase) {
+  finalize_body(P, S, phase);
+}
+
+__device__ void tails_body(const StepParams& P) {
   if (P.ctr->overflow) return;
   for (uint32_t i = blockIdx.x; i < P.n_items; i += gridDim.x) {
     const WorkItem w = P.items[i];
@@ -954,6 +971,8 @@ __global__ void tails_kernel(const StepParams P) {
     for (int64_t b = threadIdx.x; b < nt; b += blockDim.x) dst[b] = src[b];
   }
 }
+
+__global__ void tails_kernel(const StepParams P) { tails_body(P); }
 
 // Run boundaries of the canonically sorted records: the records of work item
 // w are [start[w], start[w + 1]), the first index whose key belongs to a pair
@@ -1002,8 +1021,7 @@ __device__ __forceinline__ unsigned long long scan_chunk(unsigned long long n) {
   return (tiles + gridDim.x - 1) / gridDim.x * kScanTile;
 }
 
-__global__ void __launch_bounds__(kScanThreads)
-    seg_reduce_kernel(const StepParams P, unsigned long long* __restrict__ part) {
+__device__ void seg_reduce_body(const StepParams& P, unsigned long long* part) {
   __shared__ unsigned long long ws[kScanThreads / 32];
   const unsigned long long n = seg_count(P);
   const unsigned long long chunk = scan_chunk(n);
@@ -1022,6 +1040,11 @@ __global__ void __launch_bounds__(kScanThreads)
     for (int w = 0; w < kScanThreads / 32; ++w) t += ws[w];
     part[blockIdx.x] = t;
   }
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+    seg_reduce_kernel(const StepParams P, unsigned long long* __restrict__ part) {
+  seg_reduce_body(P, part);
 }
 
 // One block: exclusive offsets of the block sums; the total is the record
@@ -1056,15 +1079,13 @@ __global__ void __launch_bounds__(kScanMaxBlocks)
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads)
-    seg_down_kernel(const StepParams P, const unsigned long long* __restrict__ part) {
+__device__ void seg_down_body(const StepParams& P, uint32_t run) {
   __shared__ uint32_t ws[kScanThreads / 32];
   __shared__ uint32_t tile_total;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const unsigned long long n = seg_count(P);
   const unsigned long long chunk = scan_chunk(n);
   const unsigned long long b0 = chunk * blockIdx.x, b1 = min(n, b0 + chunk);
-  uint32_t run = uint32_t(part[blockIdx.x]);  // offsets fit 32 bits (cap_out does)
   for (unsigned long long base = b0; base < b1; base += kScanTile) {
     const unsigned long long i = base + unsigned(t) * kScanPer;
     uint4 v = *reinterpret_cast<const uint4*>(P.seg + i);
@@ -1105,9 +1126,14 @@ __global__ void __launch_bounds__(kScanThreads)
   }
 }
 
+__global__ void __launch_bounds__(kScanThreads)
+    seg_down_kernel(const StepParams P, const unsigned long long* __restrict__ part) {
+  seg_down_body(P, uint32_t(part[blockIdx.x]));  // offsets fit 32 bits (cap_out does)
+}
+
 // Segment c holds seg[c + 1] - seg[c] records at rtmp[c ...): they go to
 // the output at seg[c].
-__global__ void compact_kernel(const StepParams P, DevHit* __restrict__ dst) {
+__device__ void compact_body(const StepParams& P, DevHit* dst) {
   const unsigned long long n = seg_count(P) - 1;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long c = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; c < n;
@@ -1120,21 +1146,96 @@ __global__ void compact_kernel(const StepParams P, DevHit* __restrict__ dst) {
   }
 }
 
+__global__ void compact_kernel(const StepParams P, DevHit* __restrict__ dst) {
+  compact_body(P, dst);
+}
+
 // start[w] = the first output record of work item w: the offset of the head
 // segment of its first pair (w x n_pat); start[n_items] = the record count.
+__device__ void runs_ordered_body(const StepParams& P, const unsigned long long* S,
+                                  unsigned long long* start) {
+  const unsigned long long n = seg_count(P) - 1;
+  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w <= P.n_items;
+       w += gridDim.x * blockDim.x) {
+    if (w == P.n_items) {
+      start[w] = P.seg[n];
+      continue;
+    }
+    const unsigned long long pr = (unsigned long long)w * P.n_pat;
+    const unsigned long long h =
+        pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pr, P.start_bits + kLowBits);
+    start[w] = P.seg[h + pr * unsigned(P.head)];
+  }
+}
+
 __global__ void runs_ordered_kernel(const StepParams P, const unsigned long long* __restrict__ S,
                                     unsigned long long* __restrict__ start) {
-  const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w > P.n_items) return;
-  const unsigned long long n = seg_count(P) - 1;
-  if (w == P.n_items) {
-    start[w] = P.seg[n];
-    return;
+  runs_ordered_body(P, S, start);
+}
+
+// ------------------------------------------------- small steps
+// Everything after the candidates of a small step (filtered output, ordered
+// records) in one cooperative launch: verification, the hit sort, the filter,
+// the carried windows, the records' offsets, and the new state, with bounded
+// grid barriers between them.  As launches of their own these are a dozen
+// kernels of 3 to 14 us and two fills, with a gap after each and 2 us of the
+// host before it; small steps are made of that.  The counters, each stream's
+// first record and, if there are at most direct_cap, the records go straight
+// to pinned host memory.
+// A step of one motif over 1,500 bytes: 125 -> 73 us a call.
+__global__ void __launch_bounds__(kSortThreads, 2) small_step_kernel(const StepParams P,
+                                                                     const SmallStep A) {
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  SortSmem& sm = *reinterpret_cast<SortSmem*>(sort_smem);
+  __shared__ unsigned long long before_s, total_s;
+  unsigned int target = 0;
+  const unsigned long long me = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x,
+                           all = (unsigned long long)gridDim.x * blockDim.x;
+  // (the timeout bit is set by the barrier; the host gives up on the step)
+  auto meet = [&]() { return sort_barrier(sm, A.bar, target += gridDim.x, P.ctr); };
+  for (unsigned long long i = me; i < (unsigned long long)P.n_items * P.n_pat; i += all)
+    P.pair_pool[i] = -1;
+  for (unsigned long long i = me; i < A.seg_len / 4; i += all)
+    reinterpret_cast<uint4*>(P.seg)[i] = make_uint4(0u, 0u, 0u, 0u);
+  verify_body(P);
+  if (!meet()) return;
+  sort_body(sm, P.keys, P.keys_alt, nullptr, nullptr, &P.ctr->n_hits, P.cap_hits, A.lo_bit,
+            A.hi_bit, A.hist, A.sort_bar, P.ctr);
+  if (!meet()) return;
+  filter_body(P, A.sorted);
+  if (!meet()) return;
+  finalize_body(P, A.sorted, kFinFlush);
+  if (!meet()) return;
+  seg_reduce_body(P, A.part);
+  if (!meet()) return;
+  if (threadIdx.x < 32) {  // the sums of the blocks before this one, and of all
+    unsigned long long b = 0, t = 0;
+    for (unsigned int q = threadIdx.x; q < gridDim.x; q += 32) {
+      const unsigned long long v = __ldcg(A.part + q);
+      t += v;
+      if (q < blockIdx.x) b += v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      b += __shfl_down_sync(kFull, b, o);
+      t += __shfl_down_sync(kFull, t, o);
+    }
+    if (threadIdx.x == 0) {
+      before_s = b;
+      total_s = t;
+    }
   }
-  const unsigned long long pr = (unsigned long long)w * P.n_pat;
-  const unsigned long long h =
-      pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pr, P.start_bits + kLowBits);
-  start[w] = P.seg[h + pr * unsigned(P.head)];
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    P.ctr->n_out = total_s;
+    if (total_s > P.cap_out) atomicOr(&P.ctr->overflow, 4u);
+  }
+  seg_down_body(P, uint32_t(before_s));
+  if (!meet()) return;
+  finalize_body(P, A.sorted, kFinCommit);
+  tails_body(P);
+  compact_body(P, total_s <= A.direct_cap ? A.direct : A.dst);
+  runs_ordered_body(P, A.sorted, A.run_start);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *A.counters = *P.ctr;
 }
 
 int grid_for(unsigned long long n, int threads, int cap_blocks) {
@@ -1171,6 +1272,34 @@ int sort_grid(int num_sms) {
                                                     sizeof(SortSmem)) != cudaSuccess)
     return 0;
   return std::min(per_sm, 4) * num_sms;
+}
+
+int small_step_grid(int num_sms) {
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(sizeof(SortSmem))) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_step_kernel, kSortThreads,
+                                                    sizeof(SortSmem)) != cudaSuccess)
+    return 0;
+  return per_sm < 1 ? 0 : num_sms;
+}
+
+cudaError_t launch_small_step(const StepParams& p, SmallStep a, int nblocks, cudaStream_t s) {
+  a.seg_len = ordered_seg_len(p.cap_rtmp);
+  a.lo_bit = kKBits;
+  a.hi_bit = p.key_bits;
+  a.sorted = (((a.hi_bit - a.lo_bit + 7) / 8) & 1) ? p.keys_alt : p.keys;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(nblocks));
+  cfg.blockDim = dim3(kSortThreads);
+  cfg.dynamicSmemBytes = sizeof(SortSmem);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, small_step_kernel, p, a);
 }
 
 size_t sort_hist_len(int nblocks) { return size_t(kBins) * (size_t(nblocks) + 1); }

@@ -7,6 +7,12 @@
 namespace oasm {
 
 constexpr int64_t kPrefSeg = kPrefSegMax;  // start positions per piece-filter segment
+// Steps that run everything after the scan in one launch: at most this much new
+// text and this many head slots (pairs x (K_max + 1)).
+constexpr uint64_t kSmallBytes = 1 << 20;
+constexpr size_t kSmallSlots = 1 << 15;
+constexpr size_t kDirectRecords = 4096;  // records such a step writes to the host itself
+
 // Clocks per SM that the gram index has to save before a step runs it: its
 // launches and clearing its set cost about 15 us, and planning the regions of
 // a bucket beside it about 100 ns per stream.
@@ -172,7 +178,8 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
   topo_add(pl.chunks.empty() ? 0 : 1);
   if (tm) CK(record_event(ctx, ctx->ev[0], s));
   CK(cudaMemsetAsync(ctx->d_ctr, 0, sizeof(StepCounters), s));
-  CK(cudaMemsetAsync(ctx->pair_pool.p, 0xff, size_t(n_items) * ctx->n_pat * sizeof(int32_t), s));
+  if (!pl.small)
+    CK(cudaMemsetAsync(ctx->pair_pool.p, 0xff, size_t(n_items) * ctx->n_pat * sizeof(int32_t), s));
   const bool short_chunks = pl.longest_chunk <= kShortChunk;
   topo_add(short_chunks ? 1 : 0);
   CK(launch_gather(d_chunks, int(pl.chunks.size()), short_chunks, ctx->arena.p, s));
@@ -261,6 +268,23 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
       ctx->st.launches += 1;
     }
   }
+  if (pl.small) {
+    SmallStep a{};
+    a.dst = ctx->out_sorted[ctx->rec_buf].p;
+    a.direct = ctx->h_out[ctx->rec_buf];
+    a.direct_cap = kDirectRecords;
+    a.run_start = ctx->h_run_start;
+    a.counters = ctx->h_ctr;
+    a.part = ctx->seg_part.p;
+    a.hist = ctx->d_hist;
+    a.bar = &ctx->d_ctr->bar[1];
+    a.sort_bar = &ctx->d_ctr->bar[0];
+    CK(launch_small_step(P, a, ctx->small_blocks, s));
+    ctx->st.launches += 1;
+    topo_add(0x400);
+    ctx->step_topo = topo;
+    return OASM_OK;
+  }
   if (tm) CK(record_event(ctx, ctx->ev[2], s));
   CK(launch_verify(P, s));
   ctx->st.launches += 1;
@@ -339,11 +363,46 @@ int prepare_records(oasm_ctx* ctx, StepPlan& pl) {
   const int ro = ctx->cfg.record_order;
   pl.ordered = ctx->rules.output == OASM_OUT_FILTERED &&
                (ro == 1 || (ro == 0 && npairs * head <= cap_hits));
+  // (with cfg.timing each kernel class is timed, so they are launched one by one)
+  pl.small = pl.ordered && !ctx->cfg.timing && pl.new_bytes <= kSmallBytes &&
+             npairs * head <= kSmallSlots;
   if (!pl.ordered) return OASM_OK;
   int rc;
   if ((rc = ensure(ctx, ctx->rtmp, cap_hits + npairs * head, "ordered records"))) return rc;
   if ((rc = ensure(ctx, ctx->seg, ordered_seg_len(ctx->rtmp.cap), "record segments"))) return rc;
   return ensure(ctx, ctx->seg_part, size_t(ordered_scan_blocks(ctx->num_sms)), "record scan");
+}
+
+// Records lent from pinned buffer b (by a step two steps ago) move to their
+// queues: the buffer is about to be written.
+static void reclaim_lent(oasm_ctx* ctx, int b) {
+  std::vector<CopyTask> keep;
+  for (StreamRec& sr : ctx->streams)
+    if (sr.lent_n && sr.lent_buf == b) {
+      sr.ready.clear();
+      sr.head = 0;
+      sr.runs.assign(1, 0);
+      sr.ready.resize(sr.lent_n);
+      keep.push_back(CopyTask{sr.ready.data(), sr.lent, sr.lent_n});
+      sr.lent = nullptr;
+      sr.lent_n = 0;
+    }
+  if (!keep.empty()) parallel_copy(keep);
+}
+
+// Pinned record buffer b of at least n records.
+static int ensure_h_out(oasm_ctx* ctx, int b, size_t n) {
+  if (n <= ctx->h_out_cap[b]) return OASM_OK;
+  if (ctx->h_out[b]) cudaFreeHost(ctx->h_out[b]);
+  ctx->h_out[b] = nullptr;
+  ctx->h_out_cap[b] = 0;
+  ctx->st.buffer_grows += 1;
+  if (cudaHostAlloc(&ctx->h_out[b], n * sizeof(DevHit), cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(ctx, OASM_ENOMEM, "pinned allocation for %zu records failed", n);
+  }
+  ctx->h_out_cap[b] = n;
+  return OASM_OK;
 }
 
 // Launches one step's device work (as a graph or directly) and records the
@@ -354,6 +413,12 @@ int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Regi
   cudaStream_t s = ctx->stream;
   int rc;
   if ((rc = prepare_records(ctx, pl))) return rc;
+  if (pl.small) {  // the step may write its records straight into the pinned buffer
+    reclaim_lent(ctx, ctx->rec_buf);
+    if ((rc = ensure_h_out(ctx, ctx->rec_buf, kDirectRecords))) return rc;
+    // the kernel writes the counters at its end: one that gave up leaves this
+    ctx->h_ctr->overflow = 1u << 16;
+  }
   if (ctx->cfg.graphs) {
     // capture the step, then update the cached executable graph in place when
     // the step has the same shape (kernel arguments and grids may differ)
@@ -480,7 +545,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
             pl.items.size(), c.overflow, c.n_cand, ctx->cand.cap, c.n_hits,
             (size_t)P.cap_hits, c.n_out, P.cap_out, c.n_pool, P.cap_pool);
   if (c.overflow & (1u << 16))
-    return fail(ctx, OASM_ETIMEOUT, "a bounded wait for a TMA copy ran out in the scan");
+    return fail(ctx, OASM_ETIMEOUT, "a bounded wait on the device (a TMA copy, a grid barrier) ran out");
   if (c.overflow & 64u)
     return fail(ctx, OASM_ECUDA, "internal error: an ordered record fell outside its segment");
   *overflow = c.overflow != 0;
@@ -550,41 +615,20 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
   // the caller (and the next step on the device) go on.
   if ((rc = settle_records(ctx))) return rc;
   const int b = ctx->rec_buf;
-  {  // records lent from buffer b (two steps old) move to their queues first
-    std::vector<CopyTask> keep;
-    for (StreamRec& sr : ctx->streams)
-      if (sr.lent_n && sr.lent_buf == b) {
-        sr.ready.clear();
-        sr.head = 0;
-        sr.runs.assign(1, 0);
-        sr.ready.resize(sr.lent_n);
-        keep.push_back(CopyTask{sr.ready.data(), sr.lent, sr.lent_n});
-        sr.lent = nullptr;
-        sr.lent_n = 0;
-      }
-    if (!keep.empty()) parallel_copy(keep);
-  }
+  reclaim_lent(ctx, b);
   if (c.n_out) {
     const size_t n = size_t(c.n_out);
-    if (n > ctx->h_out_cap[b]) {
-      if (ctx->h_out[b]) cudaFreeHost(ctx->h_out[b]);
-      ctx->h_out[b] = nullptr;
-      ctx->h_out_cap[b] = 0;
-      ctx->st.buffer_grows += 1;
-      if (cudaHostAlloc(&ctx->h_out[b], n * sizeof(DevHit), cudaHostAllocDefault) !=
-          cudaSuccess) {
-        cudaGetLastError();
-        return fail(ctx, OASM_ENOMEM, "pinned allocation for %zu records failed", n);
-      }
-      ctx->h_out_cap[b] = n;
-    }
+    if ((rc = ensure_h_out(ctx, b, n))) return rc;
     // the step's work is complete (its event was waited for above), so the
     // copy stream needs no dependency on the step's stream
-    CK(cudaMemcpyAsync(ctx->h_out[b], ctx->out_sorted[b].p, n * sizeof(DevHit),
-                       cudaMemcpyDeviceToHost, ctx->copy_stream));
-    CK(cudaEventRecord(ctx->copy_done[b], ctx->copy_stream));
-    ctx->st.record_bytes += n * sizeof(DevHit);
     PendingRecords& pr = ctx->pend;
+    pr.direct = pl.small && n <= kDirectRecords;  // the step wrote them there itself
+    if (!pr.direct) {
+      CK(cudaMemcpyAsync(ctx->h_out[b], ctx->out_sorted[b].p, n * sizeof(DevHit),
+                         cudaMemcpyDeviceToHost, ctx->copy_stream));
+      CK(cudaEventRecord(ctx->copy_done[b], ctx->copy_stream));
+    }
+    ctx->st.record_bytes += n * sizeof(DevHit);
     pr.on = true;
     pr.buf = b;
     pr.n = n;
@@ -600,7 +644,7 @@ int settle_records(oasm_ctx* ctx) {
   if (!pr.on) return OASM_OK;
   pr.on = false;
   const auto t_copy = std::chrono::steady_clock::now();
-  const int rc = wait_event(ctx, ctx->copy_done[pr.buf]);
+  const int rc = pr.direct ? OASM_OK : wait_event(ctx, ctx->copy_done[pr.buf]);
   ctx->st.host_copy_ms += ms_since(t_copy);
   if (rc) return rc;
   const oasm_hit* recs = reinterpret_cast<const oasm_hit*>(ctx->h_out[pr.buf]);
