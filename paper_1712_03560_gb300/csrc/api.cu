@@ -272,7 +272,7 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
   if (ctx->num_sms < 1) ctx->num_sms = 1;
   if ((ctx->sort_blocks = sort_grid(ctx->num_sms)) < 1 ||
-      (ctx->small_blocks = std::min(64, small_step_grid(ctx->num_sms))) < 1) {
+      (ctx->small_blocks = small_step_grid(ctx->num_sms)) < 1) {
     cudaGetLastError();
     fail(ctx, OASM_ECUDA, "the sort kernel does not fit the device");
     return bail(OASM_ECUDA);

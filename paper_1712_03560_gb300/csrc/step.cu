@@ -9,14 +9,17 @@ namespace oasm {
 constexpr int64_t kPrefSeg = kPrefSegMax;  // start positions per piece-filter segment
 // Steps that run everything after the scan in one launch: at most this much new
 // text and this many head slots (pairs x (K_max + 1)).
-constexpr uint64_t kSmallBytes = 1 << 20;
-constexpr size_t kSmallSlots = 1 << 15;
+constexpr uint64_t kSmallBytes = 8 << 20;
+constexpr size_t kSmallSlots = 1 << 18;
 constexpr size_t kDirectRecords = 4096;  // records such a step writes to the host itself
 
-// Clocks per SM that the gram index has to save before a step runs it: its
-// launches and clearing its set cost about 15 us, and planning the regions of
-// a bucket beside it about 100 ns per stream.
-constexpr double kGramMinClk = 30e3, kGramPlanClk = 200.0;
+// When the gram index runs: its launches, clearing its set and its table loads
+// cost about 20 us (in clocks of an SM), a scan launch that it saves 3 us at
+// least, and planning the regions of a bucket beside it about 15 ns per stream.
+// Measured: 300 byte patterns over 50,000 symbols 148 -> 73 us a call, 4,096
+// over 4,096 symbols 168 -> 76, 300 DNA patterns over 100,000 125 -> 98, over
+// 30,000 105 -> 92 (left to the scan).
+constexpr double kGramClk = 40e3, kScanLaunchClk = 6e3, kGramPlanClk = 30.0;
 constexpr size_t kGramSlice = size_t(1) << 27;  // arena symbols per slice of suspects
 constexpr double kGramMaxRate = 2.0;            // suspects per symbol that a slice may hold
 
@@ -89,9 +92,10 @@ int plan_step(oasm_ctx* ctx, StepPlan& pl) {
   Grams& gr = ctx->grams;
   int64_t ends = 0;
   for (const auto& w : pl.items) ends += w.e_new - w.base_pos;
-  pl.grams = gr.n_pat && gr.saved_clk * double(ends) >=
-                             (kGramMinClk + kGramPlanClk * double(pl.items.size()) *
-                                                double(gr.rest.size())) * ctx->num_sms;
+  pl.grams = gr.n_pat &&
+             gr.saved_clk * double(ends) / ctx->num_sms +
+                     kScanLaunchClk * (double(ctx->buckets.size()) - double(gr.rest.size())) >=
+                 kGramClk + kGramPlanClk * double(pl.items.size()) * double(gr.rest.size());
   if (pl.grams && gr.off_steps > 0) {
     --gr.off_steps;
     pl.grams = false;

@@ -12,7 +12,7 @@ from parity_util import canon, gpu_rows, oracle_rows, random_case, run_gpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [1, 2, 40, 5000, (1 << 20) - 1, 1 << 20, (1 << 20) + 1])
+@pytest.mark.parametrize("n", [1, 2, 40, 5000, (8 << 20) - 1, 8 << 20, (8 << 20) + 1])
 def test_text_sizes(n):
     rng = np.random.default_rng(1000 + n)
     pats = [W.DNA[rng.integers(0, 4, size=m)] for m in (8, 11, 20)]
@@ -25,7 +25,7 @@ def test_text_sizes(n):
     timed, st_t = run_gpu(pats, ks, text, cfg={"timing": 1})  # one launch per kernel class
     assert canon(timed) == want
     assert (st["launches"] / (st["steps"] + st["reruns"]) <
-            st_t["launches"] / (st_t["steps"] + st_t["reruns"])) == (n <= 1 << 20)
+            st_t["launches"] / (st_t["steps"] + st_t["reruns"])) == (n <= 8 << 20)
 
 
 @pytest.mark.parametrize("records", [4095, 4096, 4097, 9000])
