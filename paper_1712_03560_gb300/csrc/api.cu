@@ -100,7 +100,7 @@ void free_ctx(oasm_ctx* c) {
   {
     Grams& gr = c->grams;
     f(const_cast<uint32_t*>(gr.scan.bits)); f(const_cast<uint4*>(gr.scan.dir));
-    f(const_cast<GramEntry*>(gr.t.entries)); f(const_cast<uint8_t*>(gr.t.edits));
+    f(const_cast<GramEntry*>(gr.t.entries));
     f(const_cast<uint32_t*>(gr.t.peq_fwd)); f(gr.susp.p); f(gr.longs.p); f(gr.ctr.p);
   }
   f(c->d_tails); f(c->d_hdr); f(c->d_mem);

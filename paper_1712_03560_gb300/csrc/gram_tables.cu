@@ -32,7 +32,6 @@ constexpr double kPair = 6.0, kEnds = 25.0, kLookup = 4.0, kLength = 0.12;
 constexpr int kMaxGram2 = 16, kMaxGram = 8;  // symbols of a gram: 2-bit text, bytes
 constexpr int kMaxPiece = 12;                // ... of a piece that may hold an edit
 constexpr int kMaxKey2 = 10, kMaxKey = 4;    // symbols that are looked up
-constexpr int kPairRows = 8;                 // symbols of a pair looked at beside a gram
 
 // Grams of one key length, ordered by key (stable; three passes of 11 bits).
 using GramList = std::vector<GramEntry>;
@@ -145,7 +144,6 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   for (int c = 0; c < 256; ++c) fr[two ? (c >> shift2) & 3 : c] += cnt[c] / tot;
   if (two)
     for (int c = 0; c < 4; ++c) fr[c] = std::max(fr[c], 1e-3);
-  std::vector<uint8_t> edits(n, 0);
   const int cmin = ctx->weighted ? int(std::min({ctx->costs.sub, ctx->costs.ins, ctx->costs.del})) : 1;
   GramList by_len[kMaxKey2 + 1];
   double ends_clk = 0;
@@ -154,7 +152,6 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   std::vector<int> at, best_at;
   for (uint32_t p = 0; p < n; ++p) {
     const int m = ctx->m[p], E = ctx->K[p] / cmin;
-    edits[p] = uint8_t(E);
     sym.resize(m);
     ps.resize(m);
     for (int i = 0; i < m; ++i) {
@@ -238,8 +235,9 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     auto put = [&](uint64_t sym8, int len, int from, int to, int pair) {
       if (from > 32 || m - to > 32) gr.t.any_long = 1;
       by_len[std::min(len, two ? kMaxKey2 : kMaxKey)].push_back(
-          GramEntry{p, uint8_t(from), uint8_t(m - to), uint8_t(pair), uint8_t(len), uint32_t(sym8),
-                    uint32_t(sym8 >> 32)});
+          GramEntry{p | uint32_t(ctx->K[p]) << 24 | uint32_t(E) << 28, uint8_t(from),
+                    uint8_t(m - to), uint8_t(pair | (to - from - len + 1) << 4), uint8_t(len),
+                    uint32_t(sym8), uint32_t(sym8 >> 32)});
     };
     auto packed = [&](int x, int len) {
       uint64_t k = 0;
@@ -254,14 +252,14 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
                  });
     }
     // each piece, and how far its pair reaches on the other side (of which
-    // kPairRows symbols tell enough: more would only make a warp's lanes wait
+    // kGramPair symbols tell enough: more would only make a warp's lanes wait
     // for the longest)
     for (int t = 0; !best_edit && t <= E; ++t) {
       const int y = key_at(best_at[t], best_h), to = best_at[t] + best_h;
       int pair = 0;
       if (paired(t, E))
-        pair = t & 1 ? std::min(kPairRows, y - best_at[t - 1]) | kGramLeft
-                     : std::min(kPairRows, best_at[t + 1] + best_h - to);
+        pair = t & 1 ? std::min(kGramPair, y - best_at[t - 1]) | kGramLeft
+                     : std::min(kGramPair, best_at[t + 1] + best_h - to);
       put(packed(y, to - y), to - y, y, to, pair);
     }
   }
@@ -370,7 +368,6 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   CK(up(&a.bits, bits));
   CK(up(&a.dir, dir));
   CK(up(&gr.t.entries, entries));
-  CK(up(&gr.t.edits, edits));
   uint32_t* peq = nullptr;
   CK(cudaMalloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t)));
   gr.t.peq_fwd = peq;

@@ -330,14 +330,14 @@ __device__ __forceinline__ Suspect decode_suspect(const StepParams& P, const Gra
   s.span = -1;
   const uint2 en = __ldg(reinterpret_cast<const uint2*>(G.entries + (key & 0xffffffu)));
   const uint64_t x = key >> 24;  // arena offset of the gram
-  s.pat = en.x;
+  s.pat = en.x & 0xffffffu;
+  s.E = int(en.x >> 28);
+  const int K = int((en.x >> 24) & 15u);
   s.before = int(en.y & 255u);
   s.after = int((en.y >> 8) & 255u);
   s.pair = int((en.y >> 16) & 255u);
   s.len = int(en.y >> 24);
-  s.m = P.m[s.pat];
-  s.E = G.edits[s.pat];
-  const int K = P.K[s.pat];
+  s.m = s.before + s.after + s.len + ((s.pair >> 4) & 3) - 1;
   // the last item that starts at or before the gram
   uint32_t a = 0, b = P.n_items;
   while (a < b) {
@@ -361,31 +361,39 @@ __device__ __forceinline__ Suspect decode_suspect(const StepParams& P, const Gra
   return s;
 }
 
-// Least edits between r (at most 32) pattern symbols beside a found gram and
-// the text beside it, if at most lim (a larger value otherwise): the anchored
-// column recurrence (dummy row 0, 1, 2, ...) over text symbols t[0], t[d],
-// t[2 d], ..., at most avail, against bits o, o + 1, ... of the mask rows.
-// ends: bit j - r + lim is set where the r symbols match the first j of the
-// text within lim.  A cell within lim of a column lies at most lim off the
-// diagonal, so a diagonal value over 2 lim ends it.
+// Edits between r (at most 32) pattern symbols beside a found gram and the
+// text beside it: the anchored column recurrence (dummy row 0, 1, 2, ...) over
+// text symbols t[0], t[d], t[2 d], ..., at most avail, against bits o, o + 1,
+// ... of the mask rows.  Returns a value over lim if there are more than lim;
+// otherwise
+//   kTest  a value of at most lim
+//   kLeast the least, over all ends in the text
+//   kEnds  the least, and bit j - r + lim of ends for each end j (text
+//          symbols matched) within lim
+// A cell within lim of a column lies at most lim off the diagonal, so a
+// diagonal value over 2 lim ends it.
+enum Side { kTest, kLeast, kEnds };
+template <Side kMode>
 __device__ __forceinline__ int side(const uint32_t* __restrict__ peq, int o,
                                     const uint8_t* __restrict__ t, int d, int r, int avail,
                                     int lim, uint32_t& ends) {
-  if (r == 0) {  // nothing left to match: every text symbol is an insertion
-    ends = (0xffffffffu >> (31 - min(lim, avail))) << lim;
+  if (r == 0) {  // nothing to match: every text symbol is an insertion
+    if (kMode == kEnds) ends = (0xffffffffu >> (31 - min(lim, avail))) << lim;
     return 0;
   }
-  ends = r <= lim ? 1u << (lim - r) : 0u;  // no text symbol: r deletions
-  int best = r;
-  uint32_t Pv = 0xffffffffu, Mv = 0u;
-  int score = r, diag = 0;
+  if (kMode == kEnds) ends = r <= lim ? 1u << (lim - r) : 0u;  // no text symbol: r deletions
+  if (kMode == kTest && r <= lim) return r;
+  int best = r, score = r, diag = 0;
   const int n = min(r + lim, avail), q = o >> 5, sh = o & 31;
   if (n <= 0) return best;
+  uint32_t Pv = 0xffffffffu, Mv = 0u;
   // the masks of the next column and the symbol after it are on their way
-  // while a column is computed
+  // while a column is computed (four columns at a time, symbols from aligned
+  // words, read less but measured slower: 300 -> 421 us on DNA)
+  const bool two_words = sh + r > 32;
   auto mask = [&](uint32_t c) {
-    const uint32_t* row = peq + size_t(c) * 4;
-    return __funnelshift_r(__ldg(row + q), q < 3 ? __ldg(row + q + 1) : 0u, sh);
+    const uint32_t* row = peq + c * 4 + q;
+    return __funnelshift_r(__ldg(row), two_words ? __ldg(row + 1) : 0u, sh);
   };
   uint32_t eq_next = mask(t[0]), c_next = t[min(1, n - 1) * d];
   for (int j = 0; j < n; ++j) {
@@ -397,8 +405,9 @@ __device__ __forceinline__ int side(const uint32_t* __restrict__ peq, int o,
     const uint32_t xh = (sum ^ Pv) | eq;
     const uint32_t ph = Mv | ~(xh | Pv), mh = Pv & xh;
     score += int((ph >> (r - 1)) & 1u) - int((mh >> (r - 1)) & 1u);
+    if (kMode == kTest && score <= lim) return score;
     best = min(best, score);
-    if (score <= lim) ends |= 1u << (j + 1 - r + lim);
+    if (kMode == kEnds && score <= lim) ends |= 1u << (j + 1 - r + lim);
     if (j < r) {
       diag += 1 - int(((xh | Mv) >> j) & 1u);
       if (diag > 2 * lim) return lim + 1;
@@ -408,6 +417,18 @@ __device__ __forceinline__ int side(const uint32_t* __restrict__ peq, int o,
     Mv = phs & xv;
   }
   return best;
+}
+
+// side() on one side of a suspect's gram, r of the symbols there.
+template <Side kMode>
+__device__ __forceinline__ int suspect_side(const StepParams& P, const GramTables& G,
+                                            const Suspect& s, bool left, int r, int lim,
+                                            uint32_t& ends) {
+  const size_t p0 = size_t(s.pat) * 256 * 4;
+  const uint8_t* text = P.arena + s.arena0 + s.x;
+  return side<kMode>(left ? P.peq_rev + p0 : G.peq_fwd + p0, s.m - (left ? s.before : s.after),
+                     left ? text - 1 : text + s.len, left ? -1 : 1, r,
+                     int(min(left ? s.x : s.n_text - s.x - s.len, int64_t(64))), lim, ends);
 }
 
 // The found ends (bit j of hit: lo + j) as candidates, each (pattern, end)
@@ -457,116 +478,121 @@ __device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, c
 constexpr int kEndThreads = 256;
 constexpr int kEndList = 64;
 
-// One thread per suspect, in two rounds so that warps stay full: the rest of
-// the gram's double piece against the text beside it, within one edit, drops
-// nearly every chance find after a few columns; what stays waits in a list per
-// warp.  The second round matches the pattern symbols on the gram's left, then
-// those on its right with the edits that are left: the right side's columns
-// are the ends.  (An occurrence keeps one double piece within one edit and one
-// half of it unedited, or one gram with its edit; that one's suspect finds its
-// end.)  With more than 32 symbols on a side, the 32 next to the gram are
-// matched, and the few suspects that pass are left to gram_long_kernel.
+// One thread per suspect, in three rounds so that warps stay full (what stays
+// after a round waits in a list per warp):
+//   the rest of the gram's pair against the text beside it, within one edit,
+//     drops nearly every chance find after a few columns;
+//   the pattern symbols on the gram's longer side, then those on the other
+//     with the edits that are left;
+//   the left side again, and the right side's columns, which are the ends.
+// (An occurrence keeps one pair within one edit and one half of it unedited,
+// or one gram with its edit; that one's suspect finds its end.)  With more than
+// 32 symbols on a side, the 32 next to the gram are matched, and the few
+// suspects that pass are left to gram_long_kernel.
 // (4,096 byte patterns over 32 MiB, 3 M suspects: the whole pattern for every
 // suspect 892 us; its first 32 rows first 576; both sides at once, 9 lanes of a
-// warp busy, 965; in two rounds, but with the long patterns' runs among the
-// others', 660; this form 375, and 85 in gram_long_kernel.)
+// warp busy, 965; two rounds, long patterns apart, 375; this form 331; and 85
+// in gram_long_kernel.)
 __global__ void __launch_bounds__(kEndThreads)
     gram_ends_kernel(const StepParams P, const GramTables G,
                      const unsigned long long* __restrict__ susp, GramCounters* C,
                      unsigned long long cap, unsigned long long* __restrict__ longs,
                      unsigned long long cap_long, const EndSet S) {
-  __shared__ unsigned long long list[kEndThreads / 32][kEndList];
+  __shared__ unsigned long long list[2][kEndThreads / 32][kEndList];
   const unsigned long long n = min(C->n_susp, cap);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
   if (__any_sync(kFull, P.ctr->overflow & 1u)) return;
-  unsigned long long* mine = list[warp];
-  int ln = 0;  // listed suspects of this warp
-  // the second round for the last 32 (or all) listed suspects
-  auto resolve = [&]() {
+  unsigned long long *pairs = list[0][warp], *passed = list[1][warp];
+  int np = 0, nq = 0;  // listed suspects of this warp: whose pair, whose sides matched
+  // the ends of the last 32 (or all) suspects that passed
+  auto finish = [&]() {
     __syncwarp();
-    const int i = max(ln - 32, 0) + lane;
+    const int i = max(nq - 32, 0) + lane;
     Suspect s;
     uint32_t hit = 0;
     s.span = -1;
-    const unsigned long long key = i < ln ? mine[i] : 0ull;
-    int w = -1;
-    if (i < ln) s = decode_suspect(P, G, key);
-    ln = max(ln - 32, 0);
+    if (i < nq) s = decode_suspect(P, G, passed[i]);
+    nq = max(nq - 32, 0);
     if (s.span >= 0) {
-      const uint32_t* fwd = G.peq_fwd + size_t(s.pat) * 256 * 4;
-      const uint8_t* text = P.arena + s.arena0;
       const int lim = s.E - ((s.pair & kGramEdit) ? 1 : 0);
-      if (s.before <= 32 && s.after <= 32) {
-        uint32_t ends;
-        const int kl = side(P.peq_rev + size_t(s.pat) * 256 * 4, s.m - s.before, text + s.x - 1,
-                            -1, s.before, int(min(s.x, int64_t(64))), lim, ends);
-        const int left = lim - kl;  // edits left for the right side
-        if (left >= 0) {
-          const int64_t next = s.x + s.len;
-          side(fwd, s.m - s.after, text + next, 1, s.after,
-               int(min(s.n_text - next, int64_t(64))), left, ends);
-          // bit b: the end after + b - left symbols past the gram; hit: from lo on
-          const int64_t sh = s.lo - (next - 1 + s.after - left);
-          hit = sh >= 0 ? (sh < 32 ? ends >> sh : 0u) : ends << -sh;
-          hit &= 0xffffffffu >> (31 - s.span);
-        }
-      } else {
-        // up to 32 symbols next to the gram on each side; what is left runs
-        // whole (gram_long_kernel)
-        uint32_t ends;
-        const int kl = side(P.peq_rev + size_t(s.pat) * 256 * 4, s.m - s.before, text + s.x - 1,
-                            -1, min(s.before, 32), int(min(s.x, int64_t(64))), lim, ends);
-        const int64_t next = s.x + s.len;
-        if (kl <= lim && side(fwd, s.m - s.after, text + next, 1, min(s.after, 32),
-                              int(min(s.n_text - next, int64_t(64))), lim - kl, ends) <= lim - kl)
-          w = ((s.m - 1) >> 5) - 1;
-      }
-    }
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      const unsigned b = __ballot_sync(kFull, w == l);
-      if (!b) continue;
-      unsigned long long at = 0;
-      if (lane == 0) at = atomicAdd(&C->n_long[l], (unsigned long long)__popc(b));
-      at = __shfl_sync(kFull, at, 0) + __popc(b & ((1u << lane) - 1u));
-      if (w == l) {
-        if (at < cap_long) longs[l * cap_long + at] = key;
-        else atomicOr(&P.ctr->overflow, kGramOverflow | 1u);
+      uint32_t ends;
+      const int left = lim - suspect_side<kLeast>(P, G, s, true, s.before, lim, ends);
+      if (left >= 0) {  // edits left for the right side
+        suspect_side<kEnds>(P, G, s, false, s.after, left, ends);
+        // bit i: the end i + after - left symbols past the gram; hit: from lo on
+        const int64_t sh = s.lo - (s.x + s.len - 1 + s.after - left);
+        hit = sh >= 0 ? (sh < 32 ? ends >> sh : 0u) : ends << -sh;
+        hit &= 0xffffffffu >> (31 - s.span);
       }
     }
     __syncwarp();
     put_ends(P, S, s, hit);
     __syncwarp();
   };
+  // both sides of the last 32 (or all) suspects whose pair matched, up to 32
+  // symbols each, the longer side first: it ends most of them
+  auto sides = [&]() {
+    __syncwarp();
+    const int i = max(np - 32, 0) + lane;
+    const unsigned long long key = i < np ? pairs[i] : 0ull;
+    int w = -1;  // 0 .. 2: runs whole (gram_long_kernel); 3: finish
+    if (i < np) {
+      const Suspect s = decode_suspect(P, G, key);
+      const int lim = s.E - ((s.pair & kGramEdit) ? 1 : 0);
+      const bool left1 = s.before > s.after;
+      uint32_t ends;
+      const int k1 = suspect_side<kLeast>(P, G, s, left1, min(left1 ? s.before : s.after, 32), lim,
+                                          ends);
+      if (k1 <= lim &&
+          suspect_side<kTest>(P, G, s, !left1, min(left1 ? s.after : s.before, 32), lim - k1,
+                              ends) <= lim - k1)
+        w = s.before > 32 || s.after > 32 ? ((s.m - 1) >> 5) - 1 : 3;
+    }
+    np = max(np - 32, 0);
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const unsigned b = __ballot_sync(kFull, w == l);
+      if (!b) continue;
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd(&C->n_long[l], (unsigned long long)__popc(b));
+      at = __shfl_sync(kFull, at, 0) + __popc(b & below);
+      if (w == l) {
+        if (at < cap_long) longs[l * cap_long + at] = key;
+        else atomicOr(&P.ctr->overflow, kGramOverflow | 1u);
+      }
+    }
+    const unsigned b = __ballot_sync(kFull, w == 3);
+    if (w == 3) passed[nq + __popc(b & below)] = key;
+    nq += __popc(b);
+    if (nq >= 32) finish();
+    __syncwarp();
+  };
   const unsigned long long stride = (unsigned long long)gridDim.x * kEndThreads;
-  for (unsigned long long base = (unsigned long long)blockIdx.x * kEndThreads + warp * 32; base < n;
-       base += stride) {
-    const unsigned long long i = base + lane;
-    unsigned long long key = 0;
+  const unsigned long long first = (unsigned long long)blockIdx.x * kEndThreads + warp * 32;
+  unsigned long long next = first + lane < n ? susp[first + lane] : 0ull;
+  for (unsigned long long base = first; base < n; base += stride) {
+    const unsigned long long i = base + lane, key = next;
     bool keep = false;
+    next = i + stride < n ? susp[i + stride] : 0ull;
     if (i < n) {
-      key = susp[i];
       const Suspect s = decode_suspect(P, G, key);
       keep = s.span >= 0;
-      const int r = s.pair & 63;
+      const int r = s.pair & 15;
       if (keep && r) {
-        const int lim = min(s.E, 1);
-        const uint8_t* text = P.arena + s.arena0 + s.x;
-        const size_t p0 = size_t(s.pat) * 256 * 4;
-        const bool lf = (s.pair & kGramLeft) != 0;
         uint32_t ends;
-        keep = side(lf ? P.peq_rev + p0 : G.peq_fwd + p0, s.m - (lf ? s.before : s.after),
-                    lf ? text - 1 : text + s.len, lf ? -1 : 1, r,
-                    int(min(lf ? s.x : s.n_text - s.x - s.len, int64_t(64))), lim, ends) <= lim;
+        const int lim = min(s.E, 1);
+        keep = suspect_side<kTest>(P, G, s, (s.pair & kGramLeft) != 0, r, lim, ends) <= lim;
       }
     }
     const unsigned m = __ballot_sync(kFull, keep);
     if (!m) continue;
-    if (keep) mine[ln + __popc(m & ((1u << lane) - 1u))] = key;
-    ln += __popc(m);
-    if (ln >= 32) resolve();
+    if (keep) pairs[np + __popc(m & below)] = key;
+    np += __popc(m);
+    if (np >= 32) sides();
   }
-  if (ln) resolve();
+  if (np) sides();
+  if (nq) finish();
 }
 
 // The whole pattern over the ends of the listed suspects, whole warps of one
@@ -657,7 +683,7 @@ cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramSca
     gram_scan_kernel<true><<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
   else
     gram_scan_kernel<false><<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
-  gram_ends_kernel<<<p.num_sms * 6, kEndThreads, 0, s>>>(p, g, a.susp, a.ctr_slice, a.cap_susp,
+  gram_ends_kernel<<<p.num_sms * 4, kEndThreads, 0, s>>>(p, g, a.susp, a.ctr_slice, a.cap_susp,
                                                          a.longs, a.cap_long, set);
   if (g.any_long)
     gram_long_kernel<<<p.num_sms * 6, kEndThreads, 0, s>>>(p, g, a.ctr_slice, a.longs, a.cap_long,

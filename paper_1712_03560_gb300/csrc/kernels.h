@@ -123,12 +123,15 @@ struct GramLen {             // one key length: the first symbols of a gram
   uint32_t dir0;             // first directory slot
   uint32_t dir_shift, dir_mask, max_probe;
 };
+constexpr int kGramPair = 8;  // symbols of a pair looked at beside a gram
 constexpr int kGramLeft = 128, kGramEdit = 64;
 struct GramEntry {           // one gram of a pattern
-  uint32_t pat;
+  uint32_t pat;              // pattern | K << 24 | most edits of an occurrence << 28
+                             // (K under unit costs)
   uint8_t before, after;     // pattern symbols beside the part that the gram stands for
-  uint8_t pair;              // symbols of its double piece beyond the gram (at most 32),
-                             // kGramLeft: before it; kGramEdit: the gram holds an edit
+  uint8_t pair;              // symbols of its pair beyond the gram (at most kGramPair),
+                             // kGramLeft: before it; kGramEdit: the gram holds an edit;
+                             // bits 4-5: symbols of that part - len + 1
   uint8_t len;               // symbols of the gram
   uint32_t lo, hi;           // 16 2-bit symbols (lo), or eight bytes
 };
@@ -142,7 +145,6 @@ struct GramCounters {        // one per slice of the arena
 };
 struct GramTables {
   const GramEntry* entries;
-  const uint8_t* edits;      // [n_pat] most edits of an occurrence (K under unit costs)
   const uint32_t* peq_fwd;   // [n_pat][256][4] forward match masks
   int32_t any_long;          // 1: a gram has more than 32 pattern symbols on a side
 };
