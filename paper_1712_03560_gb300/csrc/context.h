@@ -239,7 +239,7 @@ inline bool canon_less(const oasm_hit& a, const oasm_hit& b) {
 
 struct Bucket {
   int W = 0;
-  int algo = 0;           // 0: Myers/Hyyro bit-vectors; 1 + K: automaton for K <= 2;
+  int algo = 0;           // 0: Myers/Hyyro bit-vectors; 1 + K: automaton for K <= 3;
                           // kAlgoCut: multi-word Myers/Hyyro with the cut-off
   int max_nseg = 1;
   int warps = 8;          // warps per scan block
@@ -474,6 +474,7 @@ int build_tables(oasm_ctx* ctx);
 // when it would not pay).
 int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>& served);
 void finish_grams(oasm_ctx* ctx);
+double group_cost(int W, int algo);
 void choose_piece_filter(const uint8_t* const* pat, const uint32_t* len, const uint32_t* k,
                          uint32_t n, uint32_t piece, uint8_t* on_filter);
 StepParams make_params(oasm_ctx* ctx, const WorkItem* d_items, uint32_t n_items, int sb, int kb,

@@ -5,18 +5,22 @@
 #include "context.h"
 
 namespace oasm {
-namespace {
 
 // Clocks of one SM per text symbol and forward-scan lane group, measured on a
 // GB300: 5.3 for a word of Myers/Hyyro (or the cut-off scan, one word) and for
-// the K = 2 automaton, 4.5 and 3.5 for the packed automata of K = 1 and K = 0;
+// the K = 2 automaton, 4.5 and 3.5 for the packed automata of K = 1 and K = 0,
+// 6.5 for two K = 3 patterns a lane;
 // 5.5 for a weighted wave-front group.
 double group_cost(int W, int algo) {
   if (algo == kAlgoWeighted) return 5.5;
   if (algo == 1) return 3.5;
   if (algo == 2) return 4.5;
+  if (algo == 4) return 6.5;
   return algo == kAlgoCut || algo == 3 ? 5.3 : 5.3 * W;
 }
+
+namespace {
+
 double buckets_cost(const std::vector<Bucket>& bs) {
   double c = 0;
   for (const Bucket& b : bs)

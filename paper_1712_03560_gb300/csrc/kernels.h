@@ -19,7 +19,7 @@ struct ScanArgs {
   int32_t resv;              // candidate slots a warp reserves at a time
   int32_t dict;              // 1: dictionary mapping (one pattern per lane, nseg = 1)
   int32_t chunk;             // text bytes per TMA buffer (dictionary mapping)
-  int32_t algo;              // 0: Myers/Hyyro bit-vectors; 1 + K: automaton for K <= 2 (W = 1);
+  int32_t algo;              // 0: Myers/Hyyro bit-vectors; 1 + K: automaton for K <= 3 (W = 1);
                              // kAlgoCut: Myers/Hyyro with the cut-off (W >= 2)
   int32_t gpw;               // lane groups per warp: 1, or 2 (dictionary mapping, W = 1)
   int32_t c_sub, c_ins, c_del;  // edit costs (algo == kAlgoWeighted)
@@ -33,6 +33,7 @@ struct ScanArgs {
   StepCounters* ctr;
   uint32_t two;              // 2, and the bytes of one symbol's Peq row, as kernel
   uint32_t row_bytes;        // arguments (set by the launchers; see fma_dbl in scan.cu)
+  uint32_t half;             // 2^31 (see half_plus in scan.cu)
 };
 
 // Weighted dynamic program over patterns' rows (oasm_create_weighted).  A
@@ -53,10 +54,10 @@ constexpr uint32_t kWFirstLane = 1u << 24;
 
 // Words per symbol row of a class's staged table: W for the Myers/Hyyro
 // classes, word 0 only for the cut-off classes, the match mask B for the
-// automaton classes of K = 0 and 1, and B and B >> 1 for those of K = 2 (see
-// nfa_step in scan.cu).
+// automaton classes of K = 0 and 1, and B and B >> 1 for those of K = 2 and 3
+// (see nfa_step in scan.cu).
 inline int staged_words(int W, int algo) {
-  return algo == kAlgoCut ? 1 : algo == 3 ? 2 : (algo >= 1 && algo <= 2) ? 1 : W;
+  return algo == kAlgoCut ? 1 : algo == 3 || algo == 4 ? 2 : (algo >= 1 && algo <= 2) ? 1 : W;
 }
 
 // Shared memory of one scan block: the Peq tables of its gpw lane groups (256

@@ -122,6 +122,13 @@ __device__ __forceinline__ uint32_t fma_dbl(uint32_t x, uint32_t two, uint32_t c
   return r;
 }
 
+// (x >> 1) + c with `half` a kernel argument (2^31).
+__device__ __forceinline__ uint32_t half_plus(uint32_t x, uint32_t half, uint32_t c) {
+  uint32_t r;
+  asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(half), "r"(c));
+  return r;
+}
+
 template <int W>
 __device__ __forceinline__ void add_words(const uint32_t (&a)[W], const uint32_t (&b)[W],
                                           uint32_t (&s)[W]);
@@ -204,9 +211,8 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
 struct Emitter {
   unsigned long long rbase = 0;
   int rleft = 0;
-  __device__ __forceinline__ void put(const ScanArgs& A, int lane, uint32_t cm, int64_t pos0,
-                                      uint32_t wi, int pid, int64_t base_pos, int top = 15) {
-    const int nc = __popc(cm);
+  // Where this lane's nc candidates go (in the warp's reservation).
+  __device__ __forceinline__ unsigned long long slots(const ScanArgs& A, int lane, int nc) {
     int incl = nc;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -228,7 +234,11 @@ struct Emitter {
       rleft -= tot;
     }
     mybase = __shfl_sync(kFull, mybase, 0);
-    unsigned long long o = mybase + unsigned(incl - nc);
+    return mybase + unsigned(incl - nc);
+  }
+  __device__ __forceinline__ void write(const ScanArgs& A, unsigned long long& o, uint32_t cm,
+                                        int64_t pos0, uint32_t wi, int pid, int64_t base_pos,
+                                        int top) {
     bool over = false;
     while (cm) {
       const int bit = 31 - __clz(cm);
@@ -246,6 +256,11 @@ struct Emitter {
       ++o;
     }
     if (over) atomicOr(&A.ctr->overflow, 1u);
+  }
+  __device__ __forceinline__ void put(const ScanArgs& A, int lane, uint32_t cm, int64_t pos0,
+                                      uint32_t wi, int pid, int64_t base_pos, int top = 15) {
+    unsigned long long o = slots(A, lane, __popc(cm));
+    write(A, o, cm, pos0, wi, pid, base_pos, top);
   }
   __device__ __forceinline__ void finish(const ScanArgs& A, int lane) {
     if (lane == 0)
@@ -728,6 +743,66 @@ __device__ void scan_dict_nfa(const ScanArgs& A, const char* peq, uint8_t* tbuf,
   if (ok) em.finish(A, lane);
 }
 
+// ---------------------- dictionary mapping, NFA for K = 3, two patterns a lane
+// Patterns of up to 16 symbols with K = 3, one in each half of the lane word
+// and ended at bits 15 and 31.  Candidates are frequent (a short pattern with
+// three errors ends within K every few hundred symbols of DNA, so that most
+// 32-symbol blocks of a group of 64 hold one): every step records both halves'
+// last bits with one shift and one three-input operation, and no block is
+// replayed.  Bound by the logic pipe (ncu: 71% busy, 73% of the issue slots),
+// so the shifts go to the other one.  64 MiB of DNA, 55 patterns: two
+// Myers/Hyyro groups 2.85 ms; this form with shifts on the logic pipe 2.0, as
+// it stands 1.69 (the packed automaton above, with its replays, 4.5).  The bits between two patterns may hold anything: the first bit of
+// a pattern is set by E at every level above 0, and by E & B at level 0.
+__device__ void scan_dict_pairs(const ScanArgs& A, const char* peq, uint8_t* tbuf, uint32_t bar0,
+                                const GroupSet<1>& GS, const Region& R, const WorkItem& wi,
+                                int lane) {
+  constexpr int KL = 3;
+  const LaneGroup& G = *GS.g[0];
+  const LaneSetup L = lane_setup(A, G, R, wi, lane, GS.ov);
+  const int pid1 = L.pid < 0 ? -1 : G.xpat[0][lane];
+  const uint32_t E = L.pid < 0 ? 0u : G.first[lane];
+  uint32_t Rs[KL + 1];
+#pragma unroll
+  for (int j = 0; j <= KL; ++j) Rs[j] = E * ((1u << j) - 1u);
+  const char* tab = peq + uint32_t(lane) * 4u;
+  Emitter em;
+  const int nbytes = (L.nvec * 16 + kBlk - 1) / kBlk * kBlk;
+  const bool ok = stream_blocks(A, tbuf, bar0, A.arena + L.ad_al, nbytes, lane,
+                                [&](const uint8_t* tv, int v) {
+    uint32_t acc[2] = {0u, 0u};  // bits j and 16 + j: step j of each half block
+#pragma unroll
+    for (int j = 0; j < kBlk; ++j) {
+      const char* row = tab + uint32_t(tv[j]) * 256u;
+      const uint32_t B = *reinterpret_cast<const uint32_t*>(row);
+      const uint32_t Bs = *reinterpret_cast<const uint32_t*>(row + 128);
+      // (nfa_step, shifts as multiply-adds: R_j-1 is part of R_j, so that
+      // W_j = R_j | E | shifted term)
+      uint32_t old = Rs[0];
+      Rs[0] = (fma_dbl(old, A.two) | E) & B;
+      uint32_t w = old | Rs[0];
+#pragma unroll
+      for (int l = 1; l <= KL; ++l) {
+        const uint32_t x = fma_dbl((Rs[l] & Bs) | w, A.two);
+        if (l < KL) w = Rs[l] | x | E;
+        const uint32_t r = x | E | old;
+        old = Rs[l];
+        Rs[l] = r;
+      }
+      acc[j >> 4] = half_plus(acc[j >> 4], A.half, Rs[KL] & 0x80008000u);
+    }
+    const uint32_t vm = block_mask32(L.t_lo, L.t_hi, v);
+    const uint32_t c0 = L.pid < 0 ? 0u : __brev(__byte_perm(acc[0], acc[1], 0x5410u)) & vm;
+    const uint32_t c1 = pid1 < 0 ? 0u : __brev(__byte_perm(acc[0], acc[1], 0x7632u)) & vm;
+    if (__any_sync(kFull, (c0 | c1) != 0)) {
+      unsigned long long o = em.slots(A, lane, __popc(c0) + __popc(c1));
+      em.write(A, o, c0, L.spos + kBlk * v, R.wi, L.pid, wi.base_pos, kBlk - 1);
+      em.write(A, o, c1, L.spos + kBlk * v, R.wi, pid1, wi.base_pos, kBlk - 1);
+    }
+  });
+  if (ok) em.finish(A, lane);
+}
+
 // ---------------------------------------------------- segment mapping
 template <int W>
 __device__ void scan_segments(const ScanArgs& A, const char* peq, const LaneGroup& G,
@@ -967,7 +1042,7 @@ __global__ void __launch_bounds__(512) scan_cut_kernel(const ScanArgs A) {
 template <int W, bool kDict, int ALG, int GPW>
 __global__ void __launch_bounds__(512) scan_kernel(const ScanArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
-  constexpr uint32_t kPeqBytes = 256u * 128u * (ALG == 3 ? 2 : ALG > 0 ? 1 : W);
+  constexpr uint32_t kPeqBytes = 256u * 128u * (ALG >= 3 ? 2 : ALG > 0 ? 1 : W);
   const int ngb = (A.n_groups + GPW - 1) / GPW;
   const int g0 = (blockIdx.x % ngb) * GPW;
   const int rb = blockIdx.x / ngb;
@@ -1021,7 +1096,9 @@ __global__ void __launch_bounds__(512) scan_kernel(const ScanArgs A) {
     }
     uint8_t* tb = tbase + size_t(warp) * 2 * A.chunk;
     const uint32_t bar0 = smem_u32(bars + 1 + 2 * warp);
-    if constexpr (ALG > 0) {
+    if constexpr (ALG == 4) {
+      scan_dict_pairs(A, peq, tb, bar0, GS, R, wi, lane);
+    } else if constexpr (ALG > 0) {
       if (single)
         scan_dict_nfa<ALG - 1, true, GPW>(A, peq, tb, bar0, GS, R, wi, lane);
       else
@@ -1218,6 +1295,7 @@ template <int W, bool kDict, int ALG = 0, int GPW = 1>
 cudaError_t launch_w(const ScanArgs& a0, cudaStream_t st) {
   ScanArgs a = a0;
   a.two = 2u;
+  a.half = 1u << 31;
   a.row_bytes = 128u * W;  // one symbol's row of the group's table
   const size_t smem = scan_smem_bytes(W, a.warps, kDict ? a.chunk : 0, GPW, ALG);
   const long long blocks_r = (a.n_regions + a.warps - 1) / a.warps;
@@ -1263,6 +1341,7 @@ cudaError_t prepare_scan_kernels(int max_smem_bytes) {
   set(allow_smem<1, true, 1>(max_smem_bytes));
   set(allow_smem<1, true, 2>(max_smem_bytes));
   set(allow_smem<1, true, 3>(max_smem_bytes));
+  set(allow_smem<1, true, 4>(max_smem_bytes));
   set(allow_smem<1, true, 0, 2>(max_smem_bytes));
   set(allow_smem<1, true, 1, 2>(max_smem_bytes));
   set(allow_smem<1, true, 2, 2>(max_smem_bytes));
@@ -1305,6 +1384,7 @@ cudaError_t launch_scan(const ScanArgs& a, cudaStream_t s) {
       case 1: return launch_w<1, true, 1>(a, s);
       case 2: return launch_w<1, true, 2>(a, s);
       case 3: return launch_w<1, true, 3>(a, s);
+      case 4: return launch_w<1, true, 4>(a, s);
       default: return cudaErrorInvalidValue;
     }
   }

@@ -261,6 +261,9 @@ int build_tables(oasm_ctx* ctx) {
         lanes[l].push_back(p);
         used[l] += ctx->m[p];
       }
+    } else if (algo == 4) {  // two a lane, ended at bits 15 and 31
+      for (size_t i = 0; i < ids.size(); i += 2)
+        lanes.emplace_back(ids.begin() + i, ids.begin() + std::min(i + 2, ids.size()));
     } else {
       std::stable_sort(ids.begin(), ids.end(),
                        [&](uint32_t a0, uint32_t b0) { return ctx->m[a0] < ctx->m[b0]; });
@@ -304,6 +307,7 @@ int build_tables(oasm_ctx* ctx) {
           const uint32_t p = lp[q];
           const auto& s = ctx->pats[p];
           const int m = int(s.size());
+          if (algo == 4) off = 16 * int(q) + 16 - m;
           if (q > 0) G.xpat[q - 1][l] = int32_t(p);
           G.m[l] = std::max<uint8_t>(G.m[l], uint8_t(m));
           G.ov = std::max(G.ov, m + ctx->K[p] - 1);
@@ -312,7 +316,7 @@ int build_tables(oasm_ctx* ctx) {
             const int bit = off + j;
             peq[base + size_t(s[j]) * RW + size_t(bit >> 5) * 32 + l] |= 1u << (bit & 31);
           }
-          if (algo > 0 && algo <= 3) {
+          if (algo > 0 && algo <= 4) {
             G.first[l] |= 1u << off;
             G.last[l] |= 1u << (off + m - 1);
             G.lastbit[q][l] = uint8_t(off + m - 1);
@@ -330,6 +334,9 @@ int build_tables(oasm_ctx* ctx) {
     const size_t ng = bk.groups.size();
     bk.gpw = (algo == 0 && W == 1 && bk.max_nseg == 1 && ng >= 2 && (ng % 2 == 0 || ng >= 7))
                  ? 2 : 1;
+    // (two K = 3 patterns a lane, 55 patterns over 64 MiB of DNA: 8 warps and
+    // 1,024-byte buffers 1.79 ms, 16 and 512 with regions twice as long 1.69)
+    if (algo == 4) bk.warps = 16, bk.chunk = 512, bk.region_scale = 2.0;
     CK(cudaMalloc(&bk.d_groups, bk.groups.size() * sizeof(LaneGroup)));
     CK(cudaMemcpy(bk.d_groups, bk.groups.data(), bk.groups.size() * sizeof(LaneGroup),
                   cudaMemcpyHostToDevice));
@@ -345,8 +352,8 @@ int build_tables(oasm_ctx* ctx) {
       CK(cudaMemcpy(bk.d_peq_hi, peq.data(), peq.size() * 4, cudaMemcpyHostToDevice));
       peq.swap(w0);
     }
-    if (algo == 3) {
-      // automaton classes of K = 2: each symbol row holds the match masks B
+    if (algo >= 3 && algo <= 4) {
+      // automaton classes of K = 2 and 3: each symbol row holds the match masks B
       // and B >> 1
       std::vector<uint32_t> two(bk.groups.size() * size_t(256) * 64);
       for (size_t r = 0; r < bk.groups.size() * size_t(256); ++r)
@@ -388,7 +395,13 @@ int build_tables(oasm_ctx* ctx) {
     if (rc) return rc;
   }
   // scan classes of the patterns that `skip` leaves
-  auto add_classes = [&](std::vector<Bucket>& to, const std::vector<char>& skip) -> int {
+  // cost of a one-word Myers/Hyyro class of x patterns
+  auto words_cost = [&](size_t x) {
+    const size_t L = size_t(kLaneGroup);
+    return group_cost(1, 0) * (x >= L ? double((x + L - 1) / L) : x ? 1.0 / double(L / x) : 0.0);
+  };
+  auto add_classes = [&](std::vector<Bucket>& to, const std::vector<char>& skip,
+                         bool rest) -> int {
     for (int W = 1; W <= kMaxW; ++W) {
       std::vector<uint32_t> ids;
       for (uint32_t p = 0; p < n; ++p)
@@ -404,6 +417,20 @@ int build_tables(oasm_ctx* ctx) {
           }
         }
       }
+      // beside the gram index: patterns of up to 16 symbols with K = 3, two a
+      // lane, where that is cheaper than one a lane (55 of them over 64 MiB of
+      // DNA: 2.85 ms as two Myers/Hyyro groups, 1.69 as one of these)
+      if (rest && W == 1) {
+        std::vector<uint32_t> kid, others;
+        for (uint32_t p : ids) (ctx->K[p] == 3 && ctx->m[p] <= 16 ? kid : others).push_back(p);
+        if (kid.size() > size_t(kLaneGroup) &&
+            double((kid.size() + 63) / 64) * group_cost(1, 4) + words_cost(others.size()) <
+                words_cost(ids.size())) {
+          int rc = add_bucket(to, 1, 4, kid);
+          if (rc) return rc;
+          ids.swap(others);
+        }
+      }
       if (ids.empty()) continue;
       // multi-word classes of 32 or more patterns (dictionary mapping) run the
       // cut-off form of the scan unless every word is asked for
@@ -414,13 +441,13 @@ int build_tables(oasm_ctx* ctx) {
     }
     return OASM_OK;
   };
-  int rc = add_classes(ctx->buckets, pref);
+  int rc = add_classes(ctx->buckets, pref, false);
   if (rc) return rc;
   std::vector<char> served;
   if ((rc = build_grams(ctx, pref, served))) return rc;
   if (!ctx->grams.n_pat) return OASM_OK;
   for (uint32_t p = 0; p < n; ++p) served[p] |= pref[p];
-  if ((rc = add_classes(ctx->grams.rest, served))) return rc;
+  if ((rc = add_classes(ctx->grams.rest, served, true))) return rc;
   finish_grams(ctx);
   return OASM_OK;
 }
@@ -482,7 +509,7 @@ StepParams make_params(oasm_ctx* ctx, const WorkItem* d_items, uint32_t n_items,
 // Lane groups per warp for a bucket: the configured value where the kernel
 // has that form (one-word class, dictionary mapping), else the tuned one.
 int bucket_gpw(const oasm_ctx* ctx, const Bucket& b) {
-  if (b.W != 1 || b.max_nseg != 1 || b.algo == kAlgoWeighted) return 1;
+  if (b.W != 1 || b.max_nseg != 1 || b.algo == kAlgoWeighted || b.algo == 4) return 1;
   const uint32_t c = ctx->cfg.groups_per_warp;
   return c == 1 || c == 2 ? int(c) : b.gpw;
 }

@@ -173,3 +173,21 @@ def test_index_of_a_few_long_patterns():
     scan, st_scan = run_gpu(pats, ks, text, cfg={"full_words": 1})
     assert runs_index(st, st_scan)
     assert canon(got) == canon(scan) == oracle_rows(pats, ks, text)
+
+
+@pytest.mark.parametrize("short", [33, 55, 64, 65, 97])
+def test_short_patterns_of_three_errors_beside_the_index(short):
+    """Patterns too short for the index, two a lane: one to two groups, a last
+    lane with one pattern, lengths from K + 1 on."""
+    rng = np.random.default_rng(860 + short)
+    n = 130_003
+    pats, ks, text = dictionary(rng, 4, 500, 40, 64, n, lambda m: 3)
+    few = [np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, size=m)]
+           for m in [4, 5] + [9 + j % 5 for j in range(short - 2)]]
+    high = np.uint8(0x80 * (short & 1))  # symbols in either half of the table
+    pats, ks = [p | high for p in few[:3] + pats + few[3:]], [3] * (short + 500)
+    text = text | high
+    want = oracle_rows(pats, ks, text)
+    got, st = run_gpu(pats, ks, text)
+    assert canon(got) == want
+    assert st["word_steps"] == (short + 1) // 2 * n
