@@ -171,33 +171,89 @@ __device__ void anchored_pass(const uint32_t* __restrict__ peq, const uint8_t* _
 // Weighted verification (integer edit costs): the column dynamic program of
 // Eq. 1 with costs c_sub, c_ins, c_del, the reversed pattern against t[e],
 // t[e-1], ... (an alignment read backwards keeps its operations, so the
-// distance is unchanged), one column of l_p + 1 cells per length.  Writes
-// dist[l] = weighted distance of t[e-l+1..e] for l = 1..lmax.
-__device__ void weighted_anchored(const StepParams& P, int p, const uint8_t* __restrict__ tend,
-                                  int m, int lmax, int8_t* dist) {
-  const uint8_t* pat = P.wpat + size_t(p) * OASM_MAX_PATTERN_LEN;
-  const int cs = P.c_sub, ci = P.c_ins, cd = P.c_del;
-  int col[OASM_MAX_PATTERN_LEN + 1];
-  for (int r = 0; r <= m; ++r) col[r] = r * cd;
+// distance is unchanged).  An alignment of cost <= K holds at most
+// K / min(c_ins, c_del) insertions and deletions, so it stays within that many
+// diagonals of the main one: only those cells are filled, with a bound above
+// every distance outside, and every value <= K is exact.  Writes dist[l] for
+// l = 1..lmax (127 where the length is too far from l_p to be within K).
+// B: half width of the band, whose cells stay in registers (cell d of column l
+// is row l + d - B).
+// (1,024 DNA patterns of up to 32 symbols over 16 MiB, 178,000 ends: all rows
+// in local memory 199 us, this form 31.)
+template <int B>
+__device__ __noinline__ void weighted_band(const uint8_t* __restrict__ pat,
+                                           const uint8_t* __restrict__ tend, int m, int lmax,
+                                           int cs, int ci, int cd, int8_t* dist) {
+  constexpr int kFar = 1 << 24;
+  int x[2 * B + 1];
+  uint32_t sym[2 * B + 1];  // symbol of the cell's row (row r: p[m - r])
+#pragma unroll
+  for (int d = 0; d <= 2 * B; ++d) {
+    x[d] = d < B ? kFar : (d - B) * cd;
+    const int r = 1 + d - B;
+    sym[d] = r >= 1 && r <= m ? pat[m - r] : 256u;
+  }
   for (int l = 1; l <= lmax; ++l) {
-    const uint8_t c = tend[-(l - 1)];
-    int diag = col[0];
-    col[0] = l * ci;
-    for (int r = 1; r <= m; ++r) {
-      const int left = col[r];
-      const int v = min(min(left + ci, col[r - 1] + cd), diag + (pat[m - r] == c ? 0 : cs));
-      diag = left;
-      col[r] = v;
+    const uint32_t c = tend[-(l - 1)];
+#pragma unroll
+    for (int d = 0; d <= 2 * B; ++d) {
+      int v = x[d] + (sym[d] == c ? 0 : cs);
+      if (d < 2 * B) v = min(v, x[d + 1] + ci);
+      if (d > 0) v = min(v, x[d - 1] + cd);
+      if (d < B && d <= B - l) v = d == B - l ? l * ci : kFar;  // row 0 and above
+      x[d] = v;
     }
-    dist[l] = int8_t(min(col[m], 127));
+    int at = 127;  // row m
+#pragma unroll
+    for (int d = 0; d <= 2 * B; ++d)
+      if (d == m - l + B) at = x[d];
+    dist[l] = int8_t(min(at, 127));
+#pragma unroll
+    for (int d = 0; d < 2 * B; ++d) sym[d] = sym[d + 1];
+    const int r = l + 1 + B;
+    sym[2 * B] = r <= m ? pat[m - r] : 256u;
   }
 }
 
+// Bands too wide for registers: one column in local memory.
+__device__ __noinline__ void weighted_column(const uint8_t* __restrict__ pat,
+                                             const uint8_t* __restrict__ tend, int m, int lmax,
+                                             int cs, int ci, int cd, int b, int8_t* dist) {
+  constexpr int kFar = 1 << 24;
+  int col[OASM_MAX_PATTERN_LEN + 1];
+  for (int r = 0; r <= m; ++r) col[r] = r <= b ? r * cd : kFar;
+  for (int l = 1; l <= lmax; ++l) {
+    const uint8_t c = tend[-(l - 1)];
+    const int r0 = max(1, l - b), r1 = min(m, l + b);
+    int diag = r0 <= r1 ? col[r0 - 1] : 0;
+    int up = r0 == 1 ? l * ci : kFar;
+    col[r0 - 1 <= m ? r0 - 1 : 0] = up;
+    for (int r = r0; r <= r1; ++r) {
+      const int left = col[r];
+      up = min(min(left + ci, up + cd), diag + (pat[m - r] == c ? 0 : cs));
+      diag = left;
+      col[r] = up;
+    }
+    dist[l] = int8_t(r1 == m && r0 <= m ? min(up, 127) : 127);
+  }
+}
+
+__device__ __forceinline__ void weighted_anchored(const StepParams& P, int p,
+                                                  const uint8_t* __restrict__ tend, int m,
+                                                  int lmax, int8_t* dist) {
+  const uint8_t* pat = P.wpat + size_t(p) * OASM_MAX_PATTERN_LEN;
+  const int b = int(P.K[p]) / min(P.c_ins, P.c_del);
+  if (b <= 1) weighted_band<1>(pat, tend, m, lmax, P.c_sub, P.c_ins, P.c_del, dist);
+  else if (b <= 3) weighted_band<3>(pat, tend, m, lmax, P.c_sub, P.c_ins, P.c_del, dist);
+  else weighted_column(pat, tend, m, lmax, P.c_sub, P.c_ins, P.c_del, b, dist);
+}
+
 // Distances of every length ending at tend (bit-parallel, or the weighted
-// dynamic program).
+// dynamic program: a kernel of its own each, for its registers and stack).
+template <bool kWeighted>
 __device__ __forceinline__ void lengths_at(const StepParams& P, int p, const uint8_t* tend,
                                            int m, int lmax, int8_t* dist) {
-  if (P.weighted) {
+  if (kWeighted) {
     weighted_anchored(P, p, tend, m, lmax, dist);
     return;
   }
@@ -225,6 +281,7 @@ __device__ __forceinline__ void put_record(const StepParams& P, unsigned long lo
   P.ovals[o] = uint32_t(o);
 }
 
+template <bool kWeighted>
 __device__ void verify_body(const StepParams& P) {
   const unsigned long long n = min(P.ctr->n_cand, P.cap_cand);
   // stop only on an upstream overflow: the hit count must stay exact when this
@@ -252,7 +309,7 @@ __device__ void verify_body(const StepParams& P) {
         if (P.rules.output == OASM_OUT_ENDS) {
           if (e >= w.e_prev && e < w.e_new) {
             const int lmax = int(min(int64_t(m + K), e - lo_start + 1));
-            lengths_at(P, p, tend, m, lmax, dist);
+            lengths_at<kWeighted>(P, p, tend, m, lmax, dist);
             int best = 127, bl = 0;
             for (int l = 1; l <= lmax; ++l)
               if (dist[l] < best) { best = dist[l]; bl = l; }
@@ -273,7 +330,7 @@ __device__ void verify_body(const StepParams& P) {
           const int lmax = int(min(int64_t(m + K), e - smin + 1));
           const int lmin = int(max(int64_t(max(1, m - K)), e - fn + 1));
           if (lmin <= lmax) {
-            lengths_at(P, p, tend, m, lmax, dist);
+            lengths_at<kWeighted>(P, p, tend, m, lmax, dist);
             const uint64_t pair = uint64_t(c.wi) * P.n_pat + uint64_t(p);
             for (int l = lmin; l <= lmax; ++l) {
               const int k = dist[l];
@@ -337,7 +394,10 @@ __device__ void verify_body(const StepParams& P) {
   }
 }
 
-__global__ void __launch_bounds__(256) verify_kernel(const StepParams P) { verify_body(P); }
+template <bool kWeighted>
+__global__ void __launch_bounds__(256) verify_kernel(const StepParams P) {
+  verify_body<kWeighted>(P);
+}
 
 // ---------------------------------------------------------------- radix sort
 // Stable LSD radix sort, 8-bit digits, every pass in one cooperative launch
@@ -1202,8 +1262,9 @@ __global__ void runs_ordered_kernel(const StepParams P, const unsigned long long
 // first record and, if there are at most direct_cap, the records go straight
 // to pinned host memory.
 // A step of one motif over 1,500 bytes: 125 -> 73 us a call.
-__global__ void __launch_bounds__(kSortThreads, 2) small_step_kernel(const StepParams P,
-                                                                     const SmallStep A) {
+template <bool kWeighted>
+__global__ void __launch_bounds__(kSortThreads, 2)
+    small_step_kernel(const StepParams P, const SmallStep A) {
   extern __shared__ __align__(16) unsigned char sort_smem[];
   SortSmem& sm = *reinterpret_cast<SortSmem*>(sort_smem);
   __shared__ unsigned long long before_s, total_s;
@@ -1216,7 +1277,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) small_step_kernel(const StepP
     P.pair_pool[i] = -1;
   for (unsigned long long i = me; i < A.seg_len / 4; i += all)
     reinterpret_cast<uint4*>(P.seg)[i] = make_uint4(0u, 0u, 0u, 0u);
-  verify_body(P);
+  verify_body<kWeighted>(P);
   if (!meet()) return;
   sort_body(sm, P.keys, P.keys_alt, nullptr, nullptr, &P.ctr->n_hits, P.cap_hits, A.lo_bit,
             A.hi_bit, A.hist, A.sort_bar, P.ctr);
@@ -1279,7 +1340,8 @@ cudaError_t launch_gather(const CopyChunk* chunks, int n, bool short_chunks, uin
 cudaError_t launch_verify(const StepParams& p, cudaStream_t s) {
   // the candidate count lives on the device: size for the capacity, loop inside
   const int grid = grid_for(p.cap_cand, 256, p.num_sms * 16);
-  verify_kernel<<<grid, 256, 0, s>>>(p);
+  if (p.weighted) verify_kernel<true><<<grid, 256, 0, s>>>(p);
+  else verify_kernel<false><<<grid, 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -1294,13 +1356,16 @@ int sort_grid(int num_sms) {
 }
 
 int small_step_grid(int num_sms) {
-  int per_sm = 0;
-  if (cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(sizeof(SortSmem))) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_step_kernel, kSortThreads,
-                                                    sizeof(SortSmem)) != cudaSuccess)
-    return 0;
-  return per_sm < 1 ? 0 : num_sms;
+  for (auto* kernel : {small_step_kernel<false>, small_step_kernel<true>}) {
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(sizeof(SortSmem))) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kSortThreads,
+                                                      sizeof(SortSmem)) != cudaSuccess ||
+        per_sm < 1)
+      return 0;
+  }
+  return num_sms;
 }
 
 cudaError_t launch_small_step(const StepParams& p, SmallStep a, int nblocks, cudaStream_t s) {
@@ -1318,7 +1383,8 @@ cudaError_t launch_small_step(const StepParams& p, SmallStep a, int nblocks, cud
   at.val.cooperative = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, small_step_kernel, p, a);
+  return cudaLaunchKernelEx(&cfg, p.weighted ? small_step_kernel<true> : small_step_kernel<false>,
+                            p, a);
 }
 
 size_t sort_hist_len(int nblocks) {

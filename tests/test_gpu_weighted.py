@@ -214,3 +214,23 @@ def test_weighted_large_costs_long_patterns(costs):
     assert canon(got2) == want
     if costs[0] == 2:
         assert len(want) >= 10
+
+
+@pytest.mark.parametrize("costs", [(16, 20, 30), (3, 9, 8), (7, 14, 6), (2, 4, 5), (1, 3, 4),
+                                   (2, 15, 1), (1, 1, 2)])
+def test_weighted_verification_bands(costs):
+    """K / min(c_ins, c_del) = 0, 1, 2, 3, 5 and 15 diagonals beside the main
+    one; patterns from K + 1 symbols on, ends near the start of the text."""
+    rng = np.random.default_rng(47 + sum(costs))
+    alphabet = np.arange(40, 48, dtype=np.uint8)
+    pats = [alphabet[rng.integers(0, 8, size=m)] for m in (16, 17, 31, 33, 64, 70, 128)]
+    ks = [15, 14, 15, 13, 15, 12, 15]
+    text = alphabet[rng.integers(0, 8, size=9001)]
+    for p, k in zip(pats, ks):
+        for cp in W.edit_copies(rng, p, rng.integers(0, k // min(costs) + 1, size=6), alphabet):
+            W.plant(rng, text, cp)
+    text[:30] = pats[2][1:]
+    text[-17:] = pats[1]
+    for mode, output in (("ends", "ends"), ("hits", "all_hits")):
+        got, _ = run_gpu(pats, ks, text, {"output": output}, costs=costs)
+        assert canon(got) == oracle_rows(pats, ks, text, mode=mode, costs=costs)
