@@ -5,9 +5,10 @@
 // input of every stream, lays it out in a device text arena behind each
 // stream's stored tail, and runs the device path on the context's CUDA
 // stream:
-//   gather -> scan (one launch per word-count class) [-> piece filter]
+//   gather -> [gram index ->] scan (one launch per class, of the patterns that
+//   the index leaves where it runs) [-> piece filter]
 //   -> verify -> radix sort -> filter -> finalize -> tails
-// then copies the per-step counters and the emitted records back.  If a
+// (from verify on in one launch for small steps), then copies the per-step counters and the emitted records back.  If a
 // device buffer was too small, the kernels that change stream state skip
 // their work, the host grows the buffer and re-runs the step from the same
 // (unchanged) state.  This file holds context creation, streams and input,
@@ -29,10 +30,6 @@ int fail(oasm_ctx* c, int code, const char* fmt, ...) {
 }
 
 thread_local std::string g_create_err;
-
-
-
-
 
 int ensure_host(oasm_ctx* ctx, uint8_t** p, size_t* cap, size_t n, size_t keep) {
   if (*cap >= n && *p) return OASM_OK;
