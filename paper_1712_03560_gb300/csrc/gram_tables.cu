@@ -392,11 +392,16 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     *dst = d;
     return cudaMemcpy(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
   };
-  CK(up(&a.bits, bits));
-  CK(up(&a.dir, dir));
-  CK(up(&gr.t.entries, entries));
   uint32_t* peq = nullptr;
-  CK(cudaMalloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t)));
+  cudaError_t e = up(&a.bits, bits);
+  if (e == cudaSuccess) e = up(&a.dir, dir);
+  if (e == cudaSuccess) e = up(&gr.t.entries, entries);
+  if (e == cudaSuccess) e = cudaMalloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t));
+  if (e == cudaErrorMemoryAllocation) {  // no room for the index: the scan needs none
+    cudaGetLastError();
+    return none();  // (what was allocated goes with the context)
+  }
+  CK(e);
   gr.t.peq_fwd = peq;
   a.entries = gr.t.entries;
   CK(launch_peq(ctx->d_bytes, ctx->d_m, n, peq, false, ctx->stream));

@@ -523,6 +523,18 @@ static int upload_plan(oasm_ctx* ctx, StepPlan& pl) {
   return OASM_OK;
 }
 
+// The step, and the next ones, without the index: every pattern is scanned
+// (or filtered) with the buffers that this needs.  Used where the text is too
+// repetitive for the index, and where its buffers find no memory.
+static int leave_grams(oasm_ctx* ctx, StepPlan& pl) {
+  pl.grams = false;
+  ctx->grams.off_steps = 32;
+  ctx->err.clear();
+  plan_regions(ctx, pl);
+  return ctx->n_pref_pat && !ctx->pset.p
+             ? ensure_pow2(ctx, ctx->pset, size_t(1) << 20, "piece filter set") : OASM_OK;
+}
+
 // Waits for the launched step, then either grows the buffers that overflowed
 // (*overflow: the caller re-launches from unchanged state) or books the
 // step's timings and moves its records into the streams' queues.
@@ -564,25 +576,24 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     }
     if ((c.overflow & 4u) || c.n_out > P.cap_out)
       if ((rc = ensure_out(ctx, size_t(c.n_out * 5 / 4 + 1024), pl.ordered))) return rc;
-    if (c.overflow & 32u)  // the (end, pattern) set filled up: room for 4x its inserts
-      if ((rc = ensure_pow2(ctx, ctx->pset,
-                            std::max(size_t(c.n_pref + c.n_gram) * 4, 2 * ctx->pset.cap),
-                            "piece filter set")))
-        return rc;
+    bool leave = false;
+    if (c.overflow & 32u) {  // the (end, pattern) set filled up: room for 4x its inserts
+      rc = ensure_pow2(ctx, ctx->pset,
+                       std::max(size_t(c.n_pref + c.n_gram) * 4, 2 * ctx->pset.cap),
+                       "piece filter set");
+      leave = rc == OASM_ENOMEM && pl.grams;
+      if (rc && !leave) return rc;
+    }
     if (c.overflow & kGramOverflow) {
       // suspects past the expected rate: more room up to the rate at which
       // the index stops paying; past that the text is too repetitive for it,
       // and this step and the next ones scan every pattern
       const size_t cap = ctx->grams.susp.cap, most = gram_capacity(ctx, pl, true);
-      if (cap < most) {
-        if ((rc = ensure_grams(ctx, std::min(most, 8 * cap)))) return rc;
-      } else {
-        pl.grams = false;
-        ctx->grams.off_steps = 32;
-        plan_regions(ctx, pl);
-        if ((rc = upload_plan(ctx, pl))) return rc;
-      }
+      rc = cap < most ? ensure_grams(ctx, std::min(most, 8 * cap)) : OASM_ENOMEM;
+      if (rc && rc != OASM_ENOMEM) return rc;
+      leave = leave || rc;
     }
+    if (leave && ((rc = leave_grams(ctx, pl)) || (rc = upload_plan(ctx, pl)))) return rc;
     if ((c.overflow & 8u) || c.n_pool > P.cap_pool) {
       const size_t want = size_t(c.n_pool * 5 / 4 + 1024);
       if ((rc = ensure(ctx, ctx->pool_hdr, want, "window pool"))) return rc;
@@ -746,13 +757,15 @@ int step_begin(oasm_ctx* ctx) {
     ctx->h_run_start = reinterpret_cast<unsigned long long*>(p);
     ctx->h_run_start_cap = cap_bytes / sizeof(unsigned long long);
   }
-  if ((ctx->n_pref_pat || pl.grams) && !ctx->pset.p &&
-      (rc = ensure_pow2(ctx, ctx->pset, pl.grams ? 4 * ctx->cand.cap : size_t(1) << 20,
-                        "piece filter set")))
+  if (ctx->n_pref_pat && !pl.grams && !ctx->pset.p &&
+      (rc = ensure_pow2(ctx, ctx->pset, size_t(1) << 20, "piece filter set")))
     return rc;
-  if (pl.grams && ((rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters")) ||
-                   (rc = ensure_grams(ctx, gram_capacity(ctx, pl, false)))))
-    return rc;
+  if (pl.grams) {
+    rc = ctx->pset.p ? OASM_OK : ensure_pow2(ctx, ctx->pset, 4 * ctx->cand.cap, "piece filter set");
+    if (!rc) rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters");
+    if (!rc) rc = ensure_grams(ctx, gram_capacity(ctx, pl, false));
+    if (rc && (rc != OASM_ENOMEM || (rc = leave_grams(ctx, pl)))) return rc;
+  }
   if (!ctx->pool_hdr.p) {
     if ((rc = ensure(ctx, ctx->pool_hdr, 1 << 14, "window pool"))) return rc;
     if ((rc = ensure(ctx, ctx->pool_mem, size_t(1 << 14) * (kMaxK + 1), "window pool"))) return rc;
