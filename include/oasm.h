@@ -160,7 +160,8 @@ typedef struct {
                                 alone would fit) */
     uint64_t hits;           /* hits of Eq. 2 handed to the filter */
     uint64_t kept;           /* records emitted */
-    uint64_t reruns;         /* steps re-run after a buffer grew */
+    uint64_t reruns;         /* steps re-run after a buffer grew, or after the wait of
+                                a small step's blocks for one another ran out */
     double scan_ms;          /* with timing=1: forward scan kernels */
     double verify_ms;        /* anchored verification */
     double order_ms;         /* radix sort of hits */
@@ -457,6 +458,16 @@ int oasm_restore_stream(oasm_ctx *ctx, uint32_t sid, const void *buf, size_t n);
 int oasm_get_stats(oasm_ctx *ctx, oasm_stats *st);
 int oasm_reset_stats(oasm_ctx *ctx);
 
+/* Which way the context's steps went (cumulative; the records are the same
+ * either way). */
+typedef struct {
+    uint64_t small_steps; /* steps whose work after the scan ran in one launch */
+    uint64_t small_left;  /* steps that left that launch for separate ones: too many
+                             hits for it, or a wait of its blocks for one another
+                             ran out */
+} oasm_routes;
+int oasm_get_routes(oasm_ctx *ctx, oasm_routes *out);
+
 /* The cudaStream_t the context runs on (for timing with CUDA events). */
 void *oasm_cuda_stream(oasm_ctx *ctx);
 
@@ -531,6 +542,18 @@ int oasm_set_tuning(oasm_ctx *ctx, const oasm_tuning *t, uint32_t n);
  * trap or hang is involved; the device stays usable.  Errors: OASM_EINVAL
  * (spin_limit == 0), OASM_ENOMEM, OASM_ECUDA. */
 int oasm_selftest_wait(int device, uint32_t spin_limit, int arrive);
+
+/* Lower bounds inside the library, so that a test reaches what lies behind
+ * them with little work (no paper passage).  A field of 0 keeps the library's
+ * own bound; l == NULL restores them all.  Finishes a step in flight first.
+ * Results never depend on these bounds. */
+typedef struct {
+    uint64_t small_hits;     /* hits over which a small step leaves its launch */
+    uint32_t barrier_polls;  /* polls at a grid barrier, which then also waits for an
+                                arrival that never comes: the wait runs out */
+    uint32_t reserved;
+} oasm_limits;
+int oasm_selftest_limits(oasm_ctx *ctx, const oasm_limits *l);
 
 /* ---- search without device allocation (no counterpart in the paper) ----
  * For callers that cannot call cudaMalloc: code running inside a framework

@@ -83,6 +83,15 @@ class oasm_stats(ctypes.Structure):
                 ("record_bytes", ctypes.c_uint64)]
 
 
+class oasm_routes(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_uint64) for n in ("small_steps", "small_left")]
+
+
+class oasm_limits(ctypes.Structure):
+    _fields_ = [("small_hits", ctypes.c_uint64), ("barrier_polls", ctypes.c_uint32),
+                ("reserved", ctypes.c_uint32)]
+
+
 class oasm_costs(ctypes.Structure):
     _fields_ = [("sub", ctypes.c_uint32), ("ins", ctypes.c_uint32), ("del_", ctypes.c_uint32)]
 
@@ -142,7 +151,7 @@ EXPORTS = ["oasm_config_default", "oasm_rules_default", "oasm_create", "oasm_cre
            "oasm_save_stream", "oasm_restore_stream", "oasm_replay", "oasm_register_host",
            "oasm_unregister_host", "oasm_step_begin", "oasm_step_end", "oasm_replay_ops",
            "oasm_piece_filter_choice", "oasm_selftest_wait", "oasm_get_tuning",
-           "oasm_set_tuning"]
+           "oasm_set_tuning", "oasm_get_routes", "oasm_selftest_limits"]
 
 _lib = None
 _lock = threading.Lock()
@@ -192,6 +201,8 @@ def load(path: str | None = None):
             "oasm_strerror": ([i32], ctypes.c_char_p),
             "oasm_autotune": ([vp, vp, ctypes.c_size_t, ctypes.c_char_p, ctypes.c_size_t], i32),
             "oasm_selftest_wait": ([i32, u32, i32], i32),
+            "oasm_get_routes": ([vp, ctypes.POINTER(oasm_routes)], i32),
+            "oasm_selftest_limits": ([vp, ctypes.POINTER(oasm_limits)], i32),
             "oasm_get_tuning": ([vp, ctypes.POINTER(oasm_tuning), u32, ctypes.POINTER(u32)], i32),
             "oasm_set_tuning": ([vp, ctypes.POINTER(oasm_tuning), u32], i32),
             "oasm_measure_int_peak": ([i32, ctypes.POINTER(ctypes.c_double),
@@ -408,6 +419,12 @@ def oasm_get_stats(ctx) -> dict:
     return {n: getattr(st, n) for n, _ in oasm_stats._fields_}
 
 
+def oasm_get_routes(ctx) -> dict:
+    r = oasm_routes()
+    _check(load().oasm_get_routes(ctx, ctypes.byref(r)), ctx)
+    return {n: getattr(r, n) for n, _ in oasm_routes._fields_}
+
+
 def oasm_reset_stats(ctx):
     return _check(load().oasm_reset_stats(ctx), ctx)
 
@@ -471,6 +488,13 @@ def oasm_selftest_wait(device: int = 0, spin_limit: int = 1 << 16, arrive: bool 
     """Bounded-wait self-test: the library's status code (OASM_ETIMEOUT when
     nothing completes the barrier, OASM_OK when it completes)."""
     return int(load().oasm_selftest_wait(device, spin_limit, 1 if arrive else 0))
+
+
+def oasm_selftest_limits(ctx, **kw):
+    """Lower bounds inside the library for a test; without arguments the
+    library's own ones again."""
+    lim = oasm_limits(**kw)
+    return _check(load().oasm_selftest_limits(ctx, ctypes.byref(lim) if kw else None), ctx)
 
 
 def _check_device_buffer(d, need_bytes: int, what: str):

@@ -885,6 +885,24 @@ int oasm_reset_stats(oasm_ctx* ctx) {
   return OASM_OK;
 }
 
+int oasm_get_routes(oasm_ctx* ctx, oasm_routes* out) {
+  if (!ctx || !out) return OASM_EINVAL;
+  *out = ctx->routes;
+  return OASM_OK;
+}
+
+int oasm_selftest_limits(oasm_ctx* ctx, const oasm_limits* l) {
+  if (!ctx) return OASM_EINVAL;
+  int rc = step_end(ctx);
+  if (rc) return rc;
+  ctx->limits = Limits();
+  ctx->many_hits = false;
+  if (!l) return OASM_OK;
+  if (l->small_hits) ctx->limits.small_hits = l->small_hits;
+  if (l->barrier_polls) ctx->limits.barrier = BarrierBound{l->barrier_polls, 1};
+  return OASM_OK;
+}
+
 void* oasm_cuda_stream(oasm_ctx* ctx) { return ctx ? static_cast<void*>(ctx->stream) : nullptr; }
 
 // The buckets beside the gram index take the settings of the class they are part of.

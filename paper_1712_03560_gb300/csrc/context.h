@@ -284,6 +284,23 @@ struct Grams {
   int off_steps = 0;          // steps left without the index (suspects too dense)
 };
 
+// Where a step's launches begin: at its text, or, after a small step that left
+// its launch, at the verification or at the sort.
+enum { kFromText = 0, kFromCandidates, kFromHits };
+
+// Bounds that tests lower to reach what lies behind them (oasm_selftest_limits).
+struct Limits {
+  // A small step of more candidates or hits goes on as separate launches.  In a
+  // text of one repeated symbol all hits of a pattern are one chain that a
+  // thread walks at 175 ns a hit (46 ms for so many), while the others wait at a
+  // barrier, for a second or more: 33 M hits in 1 MiB ran out of that wait.  The
+  // separate launches are as fast by then (a motif of 8 symbols, K = 3: 212,000
+  // hits 171 us a step here and 208 there, 424,000 238 and 233, 844,000 369 and
+  // 288).
+  unsigned long long small_cand = 1ull << 22, small_hits = 1ull << 18;
+  BarrierBound barrier;
+};
+
 struct StepPlan {
   std::vector<WorkItem> items;
   std::vector<uint32_t> sids;
@@ -297,6 +314,8 @@ struct StepPlan {
   uint64_t new_bytes = 0;
   bool ordered = false;              // records written in canonical order (no record sort)
   bool small = false;                // everything after the candidates in one launch
+  bool no_small = false;             // ... not again: that launch left the step
+  int from = kFromText;              // where the launches of the step begin
   bool grams = false;                // the gram index and the rest buckets scan this step
   // An empty plan that keeps its vectors' storage.
   void clear() {
@@ -454,6 +473,9 @@ struct oasm_ctx {
   bool capturing = false;
 
   oasm_stats st{};
+  oasm_routes routes{};
+  Limits limits;
+  bool many_hits = false;    // the last step of a small step's size went over them
   uint64_t fingerprint = 0;  // patterns, thresholds and rules (stream checkpoints)
 };
 

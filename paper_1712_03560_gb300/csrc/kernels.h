@@ -178,6 +178,13 @@ cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramSca
 
 cudaError_t launch_verify(const StepParams& p, cudaStream_t s);
 
+// Bound of a wait at a grid barrier.  `extra` arrivals more than there are
+// blocks are waited for: 0, or 1 in a self-test that lets the wait run out.
+struct BarrierBound {
+  uint32_t polls = 1u << 22;  // a second or more
+  uint32_t extra = 0;
+};
+
 // Stable LSD radix sort (8-bit digits) of keys by bits [lo_bit, hi_bit),
 // with an optional 32-bit payload, in one cooperative launch.  The element
 // count is read on the device from *count (clamped to cap).  On return
@@ -195,6 +202,7 @@ struct SortArgs {
   int nblocks;                    // sort_grid(): blocks that are resident together
   unsigned int* bar;              // barrier arrivals, zero before the launch
   StepCounters* ctr;
+  BarrierBound bound;
 };
 int sort_grid(int num_sms);       // 0: the device cannot say
 size_t sort_hist_len(int nblocks);
@@ -222,8 +230,14 @@ cudaError_t launch_ordered_emit(const StepParams& p, const unsigned long long* s
                                 DevHit* dst, unsigned long long* run_start, cudaStream_t s);
 cudaError_t launch_tails(const StepParams& p, cudaStream_t s);
 // Everything after the candidates of a small step with ordered records, in one
-// cooperative launch (p.pair_pool and p.seg need no filling before it).
+// cooperative launch (p.pair_pool and p.seg need no filling before it).  With
+// more than max_cand candidates it ends at once, with more than max_hits hits
+// after the verification; *counters then carries kSmallLeft, and the launches
+// of other steps go on from there (a thread walks a pair's spanned hits one by
+// one while the others wait at a barrier, and that wait is bounded).
 struct SmallStep {
+  unsigned long long max_cand, max_hits;
+  BarrierBound bound;
   DevHit* dst;                    // records in canonical order
   DevHit* direct;                 // pinned host memory for up to direct_cap of them
   unsigned long long direct_cap;  // (more go to dst)

@@ -103,6 +103,8 @@ struct WinHdr {
   int32_t idx;
 };
 
+constexpr unsigned int kWaitOver = 1u << 16, kSmallLeft = 1u << 17;
+
 // Per-step device counters; copied back to the host after every step.
 struct StepCounters {
   unsigned long long n_cand;
@@ -113,7 +115,9 @@ struct StepCounters {
   unsigned int overflow;     // bit 0 candidates, 1 hits, 2 outputs, 3 pool,
                              // 5 the prefilter's candidate set (with bit 0),
                              // 6 an ordered record outside its segment (a bug),
-                             // 7 the gram index's suspects (with bit 0)
+                             // 7 the gram index's suspects (with bit 0),
+                             // 16 a bounded wait ran out, 17 a small step left its
+                             // launch (in the host's copy only)
   unsigned int bar[2];       // barrier arrivals of the hit sort, the record sort
   unsigned int pad;
   unsigned long long n_pref;  // distinct (pattern, end) pairs the prefilter proposed

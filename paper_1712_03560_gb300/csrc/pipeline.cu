@@ -420,7 +420,7 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kBins = 256;
 constexpr int kSortPer = 8;                         // keys per thread and tile
 constexpr int kSortTile = kSortThreads * kSortPer;  // 2,048
-constexpr uint32_t kBarrierSpins = 1u << 22;
+constexpr uint32_t kGaveUp = 1u << 30;              // over any count of arrivals
 // Blocks up to which each walks all blocks' digit counts itself, which saves a
 // barrier a pass (14,000 keys of four digits on 8 blocks: 58 -> 43 us).
 constexpr unsigned int kSortWalk = 64;
@@ -498,23 +498,31 @@ __device__ __forceinline__ unsigned int rank_tile(SortSmem& sm,
 }
 
 // All active blocks meet (*bar counts arrivals since the step began); false
-// when the bounded wait ran out.
+// when the bounded wait ran out.  The blocks agree on that: one whose wait runs
+// out takes kGaveUp from the count, unless the last block has arrived by then,
+// so a barrier that one block gives up is passed by none, and what follows the
+// last barrier of a launch runs in all blocks or in none.
 __device__ __forceinline__ bool sort_barrier(SortSmem& sm, unsigned int* bar, unsigned int target,
-                                             StepCounters* ctr) {
+                                             const BarrierBound& bound, StepCounters* ctr) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(bar, 1u);
-    unsigned int seen = 0;
-    uint32_t it = 0;
-    for (; it < kBarrierSpins; ++it) {
+    target += bound.extra;
+    bool met = false;
+    for (uint32_t it = 0;; ++it) {
+      unsigned int seen;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-      if (seen >= target) break;
-      __nanosleep(20);
+      met = int(seen) >= int(target);
+      if (met || int(seen) < 0) break;
+      if (it < bound.polls) __nanosleep(20);
+      // (an exchange fails where another block arrived or gave up meanwhile, as
+      // often as there are blocks at most)
+      else if (atomicCAS(bar, seen, seen - kGaveUp) == seen) break;
     }
-    sm.stop = it == kBarrierSpins;
+    sm.stop = !met;
     // (bit 0 keeps the filter off the unsorted keys)
-    if (sm.stop) atomicOr(&ctr->overflow, (1u << 16) | 1u);
+    if (!met) atomicOr(&ctr->overflow, kWaitOver | 1u);
     __threadfence();
   }
   __syncthreads();
@@ -524,7 +532,7 @@ __device__ __forceinline__ bool sort_barrier(SortSmem& sm, unsigned int* bar, un
 __device__ void sort_body(SortSmem& sm, unsigned long long* keys, unsigned long long* keys_alt,
                           uint32_t* vals, uint32_t* vals_alt, const unsigned long long* count,
                           unsigned long long cap, int lo_bit, int hi_bit, unsigned int* hist,
-                          unsigned int* bar, StepCounters* ctr) {
+                          unsigned int* bar, const BarrierBound& bound, StepCounters* ctr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned long long n = min(*count, cap);
   // keys per block: an even split, in whole tiles (two or more tiles to a block
@@ -599,7 +607,7 @@ __device__ void sort_body(SortSmem& sm, unsigned long long* keys, unsigned long 
       unsigned int* h = hist + size_t(parity) * kSortWalk * kBins;
       parity ^= 1u;  // (the other half may still be read)
       h[size_t(blockIdx.x) * kBins + threadIdx.x] = sm.base[threadIdx.x];
-      if (!sort_barrier(sm, bar, target += nb, ctr)) return;
+      if (!sort_barrier(sm, bar, target += nb, bound, ctr)) return;
 #pragma unroll 8
       for (unsigned int q = 0; q < nb; ++q) {
         const unsigned int v = __ldcg(h + size_t(q) * kBins + threadIdx.x);
@@ -608,7 +616,7 @@ __device__ void sort_body(SortSmem& sm, unsigned long long* keys, unsigned long 
       }
     } else {
       hist[size_t(threadIdx.x) * gridDim.x + blockIdx.x] = sm.base[threadIdx.x];
-      if (!sort_barrier(sm, bar, target += nb, ctr)) return;
+      if (!sort_barrier(sm, bar, target += nb, bound, ctr)) return;
       // each digit's counts scanned over the blocks: a digit per block and
       // turn, or, where few blocks would take many turns, per warp (3.7 M keys
       // on 608 blocks: 196 us per block, 226 per warp)
@@ -638,7 +646,7 @@ __device__ void sort_body(SortSmem& sm, unsigned long long* keys, unsigned long 
         }
         if (lane == 0) total[d] = run;
       }
-      if (!sort_barrier(sm, bar, target += nb, ctr)) return;
+      if (!sort_barrier(sm, bar, target += nb, bound, ctr)) return;
       tot = __ldcg(total + threadIdx.x);
       pre = __ldcg(hist + size_t(threadIdx.x) * gridDim.x + blockIdx.x);
     }
@@ -673,7 +681,7 @@ __device__ void sort_body(SortSmem& sm, unsigned long long* keys, unsigned long 
       __syncthreads();
       sm.base[threadIdx.x] += cnt;
     }
-    if (shift + 8 < hi_bit && !sort_barrier(sm, bar, target += nb, ctr)) return;
+    if (shift + 8 < hi_bit && !sort_barrier(sm, bar, target += nb, bound, ctr)) return;
     unsigned long long* tk = keys;
     keys = keys_alt;
     keys_alt = tk;
@@ -687,16 +695,16 @@ __global__ void __launch_bounds__(kSortThreads, 4)
     sort_kernel(unsigned long long* keys, unsigned long long* keys_alt, uint32_t* vals,
                 uint32_t* vals_alt, const unsigned long long* count, unsigned long long cap,
                 int lo_bit, int hi_bit, unsigned int* hist, unsigned int* bar,
-                StepCounters* ctr) {
+                const BarrierBound bound, StepCounters* ctr) {
   extern __shared__ __align__(16) unsigned char sort_smem[];
   sort_body(*reinterpret_cast<SortSmem*>(sort_smem), keys, keys_alt, vals, vals_alt, count, cap,
-            lo_bit, hi_bit, hist, bar, ctr);
+            lo_bit, hi_bit, hist, bar, bound, ctr);
 }
 
 __global__ void permute_kernel(const DevHit* __restrict__ src, const uint32_t* __restrict__ idx,
                                DevHit* __restrict__ dst, const StepCounters* ctr,
                                unsigned long long cap) {
-  if (ctr->overflow & (1u << 16)) return;  // the record sort gave up: idx is incomplete
+  if (ctr->overflow & kWaitOver) return;  // the record sort gave up: idx is incomplete
   const unsigned long long n = min(ctr->n_out, cap);
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (unsigned long long)gridDim.x * blockDim.x)
@@ -1271,16 +1279,25 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   unsigned int target = 0;
   const unsigned long long me = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x,
                            all = (unsigned long long)gridDim.x * blockDim.x;
-  // (the timeout bit is set by the barrier; the host gives up on the step)
-  auto meet = [&]() { return sort_barrier(sm, A.bar, target += gridDim.x, P.ctr); };
+  // (after a wait that ran out the host finds no counters, and runs the step
+  // again as separate launches: the state is as it was, see sort_barrier)
+  auto meet = [&]() { return sort_barrier(sm, A.bar, target += gridDim.x, A.bound, P.ctr); };
+  auto leave = [&]() {
+    if (me != 0) return;
+    StepCounters c = *P.ctr;
+    c.overflow |= kSmallLeft;
+    *A.counters = c;
+  };
   for (unsigned long long i = me; i < (unsigned long long)P.n_items * P.n_pat; i += all)
     P.pair_pool[i] = -1;
   for (unsigned long long i = me; i < A.seg_len / 4; i += all)
     reinterpret_cast<uint4*>(P.seg)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (P.ctr->n_cand > A.max_cand) return leave();
   verify_body<kWeighted>(P);
   if (!meet()) return;
+  if (__ldcg(&P.ctr->n_hits) > A.max_hits) return leave();
   sort_body(sm, P.keys, P.keys_alt, nullptr, nullptr, &P.ctr->n_hits, P.cap_hits, A.lo_bit,
-            A.hi_bit, A.hist, A.sort_bar, P.ctr);
+            A.hi_bit, A.hist, A.sort_bar, A.bound, P.ctr);
   if (!meet()) return;
   filter_body(P, A.sorted);
   if (!meet()) return;
@@ -1405,7 +1422,7 @@ cudaError_t launch_sort(const SortArgs& a, unsigned long long** keys_out, uint32
   cfg.numAttrs = 1;
   const cudaError_t e =
       cudaLaunchKernelEx(&cfg, sort_kernel, a.keys, a.keys_alt, a.vals, a.vals_alt, a.count, a.cap,
-                         a.lo_bit, a.hi_bit, a.hist, a.bar, a.ctr);
+                         a.lo_bit, a.hi_bit, a.hist, a.bar, a.bound, a.ctr);
   const bool odd = ((a.hi_bit - a.lo_bit + 7) / 8) & 1;
   *keys_out = odd ? a.keys_alt : a.keys;
   if (vals_out) *vals_out = odd ? a.vals_alt : a.vals;

@@ -8,7 +8,12 @@ namespace oasm {
 
 constexpr int64_t kPrefSeg = kPrefSegMax;  // start positions per piece-filter segment
 // Steps that run everything after the scan in one launch: at most this much new
-// text and this many head slots (pairs x (K_max + 1)).
+// text and this many head slots (pairs x (K_max + 1)).  Verification and filter
+// run there on one block per SM, elsewhere on more: a motif of 12 symbols with
+// few hits takes 83 us a step here and 119 in separate launches over 4 MiB, 100
+// and 133 over 8, 152 and 171 over 16, 240 and 222 over 32; one of 8 symbols
+// (110,000 hits in 8 MiB) 146 and 183, 213 and 213, 341 and 275, 587 and 380;
+// 1,024 motifs (37,000 hits) 149 and 200, 173 and 235, 230 and 278, 332 and 379.
 constexpr uint64_t kSmallBytes = 8 << 20;
 constexpr size_t kSmallSlots = 1 << 18;
 constexpr size_t kDirectRecords = 4096;  // records such a step writes to the host itself
@@ -169,6 +174,10 @@ cudaError_t record_event(oasm_ctx* ctx, cudaEvent_t e, cudaStream_t s) {
                         : cudaEventRecord(e, s);
 }
 
+// Text to candidates: the gather and the search for ends.
+static int enqueue_search(oasm_ctx* ctx, StepPlan& pl, const StepParams& P,
+                          const Region* d_regions, const CopyChunk* d_chunks, uint64_t& topo);
+
 // Enqueues the device work of one step (directly, or into a stream capture).
 int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Region* d_regions,
                  const CopyChunk* d_chunks) {
@@ -179,17 +188,110 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
   uint64_t topo = 1469598103934665603ull;
   auto topo_add = [&topo](uint64_t v) { topo = (topo ^ v) * 1099511628211ull; };
   topo_add(tm ? 1 : 0);
+  topo_add(uint64_t(pl.from));
+  const StepParams P = make_params(ctx, d_items, n_items, pl.sb, pl.kb, pl.ordered);
+  int rc;
+  if (pl.from == kFromText && (rc = enqueue_search(ctx, pl, P, d_regions, d_chunks, topo)))
+    return rc;
+  if (pl.small) {
+    SmallStep a{};
+    a.max_cand = ctx->limits.small_cand;
+    a.max_hits = ctx->limits.small_hits;
+    a.bound = ctx->limits.barrier;
+    a.dst = ctx->out_sorted[ctx->rec_buf].p;
+    a.direct = ctx->h_out[ctx->rec_buf];
+    a.direct_cap = kDirectRecords;
+    a.run_start = ctx->h_run_start;
+    a.counters = ctx->h_ctr;
+    a.part = ctx->seg_part.p;
+    a.hist = ctx->d_hist;
+    a.bar = &ctx->d_ctr->bar[1];
+    a.sort_bar = &ctx->d_ctr->bar[0];
+    CK(launch_small_step(P, a, ctx->small_blocks, s));
+    ctx->st.launches += 1;
+    topo_add(0x400);
+    ctx->step_topo = topo;
+    return OASM_OK;
+  }
+  CK(cudaMemsetAsync(ctx->pair_pool.p, 0xff, size_t(n_items) * ctx->n_pat * sizeof(int32_t), s));
+  if (tm) CK(record_event(ctx, ctx->ev[2], s));
+  if (pl.from != kFromHits) {
+    CK(launch_verify(P, s));
+    ctx->st.launches += 1;
+  }
+  if (tm) CK(record_event(ctx, ctx->ev[3], s));
+  unsigned long long* sorted = P.keys;
+  if (ctx->rules.output == OASM_OUT_FILTERED) {
+    SortArgs sa{P.keys, P.keys_alt, nullptr, nullptr, &ctx->d_ctr->n_hits, P.cap_hits,
+                kKBits, pl.kb, ctx->d_hist, ctx->sort_blocks, &ctx->d_ctr->bar[0], ctx->d_ctr,
+                ctx->limits.barrier};
+    CK(launch_sort(sa, &sorted, nullptr, s));
+    topo_add(0x100);
+    ctx->st.launches += 1;
+    if (tm) CK(record_event(ctx, ctx->ev[4], s));
+    if (pl.ordered) {
+      // records by segment; the window state is written only after the scan
+      // has checked that the records fit (a re-run starts from it unchanged)
+      CK(cudaMemsetAsync(ctx->seg.p, 0, ordered_seg_len(ctx->rtmp.cap) * sizeof(uint32_t), s));
+      CK(launch_filter(P, sorted, s));
+      CK(launch_finalize(P, sorted, kFinFlush, s));
+      CK(launch_ordered_scan(P, ctx->seg_part.p, s));
+      CK(launch_finalize(P, sorted, kFinCommit, s));
+      ctx->st.launches += 6;
+    } else {
+      CK(launch_filter(P, sorted, s));
+      CK(launch_finalize(P, sorted, kFinAll, s));
+      ctx->st.launches += 2;
+    }
+  } else if (tm) {
+    CK(record_event(ctx, ctx->ev[4], s));
+  }
+  CK(launch_tails(P, s));
+  ctx->st.launches += 1;
+  if (pl.ordered) {  // records from their segments to their offsets: canonical order
+    CK(launch_ordered_emit(P, sorted, ctx->out_sorted[ctx->rec_buf].p, ctx->run_start.p, s));
+    topo_add(0x300);
+    CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
+                       (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                       s));
+    ctx->st.launches += 2;
+  } else {  // emitted records -> canonical order (work item, pattern, decided_at, k, length)
+    unsigned long long* ks = nullptr;
+    uint32_t* vs = nullptr;
+    SortArgs sa{ctx->okeys.p, ctx->okeys_alt.p, ctx->ovals.p, ctx->ovals_alt.p,
+                &ctx->d_ctr->n_out, P.cap_out, 0, pl.kb, ctx->d_hist, ctx->sort_blocks,
+                &ctx->d_ctr->bar[1], ctx->d_ctr, ctx->limits.barrier};
+    CK(launch_sort(sa, &ks, &vs, s));
+    topo_add(0x200);
+    CK(launch_permute(ctx->out.p, vs, ctx->out_sorted[ctx->rec_buf].p, ctx->d_ctr, P.cap_out,
+                      ctx->num_sms, s));
+    // where each work item's (stream's) run of records starts
+    CK(launch_runs(ks, P, ctx->run_start.p, s));
+    CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
+                       (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                       s));
+    ctx->st.launches += 3;
+  }
+  if (tm) CK(record_event(ctx, ctx->ev[5], s));
+  CK(cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, sizeof(StepCounters), cudaMemcpyDeviceToHost, s));
+  topo_add(uint64_t(ctx->rules.output));
+  ctx->step_topo = topo;
+  return OASM_OK;
+}
+
+static int enqueue_search(oasm_ctx* ctx, StepPlan& pl, const StepParams& P,
+                          const Region* d_regions, const CopyChunk* d_chunks, uint64_t& topo) {
+  cudaStream_t s = ctx->stream;
+  const bool tm = ctx->cfg.timing != 0;
+  auto topo_add = [&topo](uint64_t v) { topo = (topo ^ v) * 1099511628211ull; };
   topo_add(pl.chunks.empty() ? 0 : 1);
   if (tm) CK(record_event(ctx, ctx->ev[0], s));
   CK(cudaMemsetAsync(ctx->d_ctr, 0, sizeof(StepCounters), s));
-  if (!pl.small)
-    CK(cudaMemsetAsync(ctx->pair_pool.p, 0xff, size_t(n_items) * ctx->n_pat * sizeof(int32_t), s));
   const bool short_chunks = pl.longest_chunk <= kShortChunk;
   topo_add(short_chunks ? 1 : 0);
   CK(launch_gather(d_chunks, int(pl.chunks.size()), short_chunks, ctx->arena.p, s));
   ctx->st.launches += pl.chunks.empty() ? 0 : 1;
   if (tm) CK(record_event(ctx, ctx->ev[1], s));
-  StepParams P = make_params(ctx, d_items, n_items, pl.sb, pl.kb, pl.ordered);
   const std::vector<Bucket>& buckets = step_buckets(ctx, pl);
   topo_add(pl.grams ? 0x61 : 0x60);
   if (pl.grams || ctx->n_pref_pat)
@@ -237,7 +339,7 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
     a.c_sub = int(ctx->costs.sub);
     a.c_ins = int(ctx->costs.ins);
     a.c_del = int(ctx->costs.del);
-    a.items = d_items;
+    a.items = P.items;
     a.arena = ctx->arena.p;
     a.cand = ctx->cand.p;
     a.cap_cand = ctx->cand.cap;
@@ -272,82 +374,6 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
       ctx->st.launches += 1;
     }
   }
-  if (pl.small) {
-    SmallStep a{};
-    a.dst = ctx->out_sorted[ctx->rec_buf].p;
-    a.direct = ctx->h_out[ctx->rec_buf];
-    a.direct_cap = kDirectRecords;
-    a.run_start = ctx->h_run_start;
-    a.counters = ctx->h_ctr;
-    a.part = ctx->seg_part.p;
-    a.hist = ctx->d_hist;
-    a.bar = &ctx->d_ctr->bar[1];
-    a.sort_bar = &ctx->d_ctr->bar[0];
-    CK(launch_small_step(P, a, ctx->small_blocks, s));
-    ctx->st.launches += 1;
-    topo_add(0x400);
-    ctx->step_topo = topo;
-    return OASM_OK;
-  }
-  if (tm) CK(record_event(ctx, ctx->ev[2], s));
-  CK(launch_verify(P, s));
-  ctx->st.launches += 1;
-  if (tm) CK(record_event(ctx, ctx->ev[3], s));
-  unsigned long long* sorted = P.keys;
-  if (ctx->rules.output == OASM_OUT_FILTERED) {
-    SortArgs sa{P.keys, P.keys_alt, nullptr, nullptr, &ctx->d_ctr->n_hits, P.cap_hits,
-                kKBits, pl.kb, ctx->d_hist, ctx->sort_blocks, &ctx->d_ctr->bar[0], ctx->d_ctr};
-    CK(launch_sort(sa, &sorted, nullptr, s));
-    topo_add(0x100);
-    ctx->st.launches += 1;
-    if (tm) CK(record_event(ctx, ctx->ev[4], s));
-    if (pl.ordered) {
-      // records by segment; the window state is written only after the scan
-      // has checked that the records fit (a re-run starts from it unchanged)
-      CK(cudaMemsetAsync(ctx->seg.p, 0, ordered_seg_len(ctx->rtmp.cap) * sizeof(uint32_t), s));
-      CK(launch_filter(P, sorted, s));
-      CK(launch_finalize(P, sorted, kFinFlush, s));
-      CK(launch_ordered_scan(P, ctx->seg_part.p, s));
-      CK(launch_finalize(P, sorted, kFinCommit, s));
-      ctx->st.launches += 6;
-    } else {
-      CK(launch_filter(P, sorted, s));
-      CK(launch_finalize(P, sorted, kFinAll, s));
-      ctx->st.launches += 2;
-    }
-  } else if (tm) {
-    CK(record_event(ctx, ctx->ev[4], s));
-  }
-  CK(launch_tails(P, s));
-  ctx->st.launches += 1;
-  if (pl.ordered) {  // records from their segments to their offsets: canonical order
-    CK(launch_ordered_emit(P, sorted, ctx->out_sorted[ctx->rec_buf].p, ctx->run_start.p, s));
-    topo_add(0x300);
-    CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
-                       (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                       s));
-    ctx->st.launches += 2;
-  } else {  // emitted records -> canonical order (work item, pattern, decided_at, k, length)
-    unsigned long long* ks = nullptr;
-    uint32_t* vs = nullptr;
-    SortArgs sa{ctx->okeys.p, ctx->okeys_alt.p, ctx->ovals.p, ctx->ovals_alt.p,
-                &ctx->d_ctr->n_out, P.cap_out, 0, pl.kb, ctx->d_hist, ctx->sort_blocks,
-                &ctx->d_ctr->bar[1], ctx->d_ctr};
-    CK(launch_sort(sa, &ks, &vs, s));
-    topo_add(0x200);
-    CK(launch_permute(ctx->out.p, vs, ctx->out_sorted[ctx->rec_buf].p, ctx->d_ctr, P.cap_out,
-                      ctx->num_sms, s));
-    // where each work item's (stream's) run of records starts
-    CK(launch_runs(ks, P, ctx->run_start.p, s));
-    CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
-                       (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                       s));
-    ctx->st.launches += 3;
-  }
-  if (tm) CK(record_event(ctx, ctx->ev[5], s));
-  CK(cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, sizeof(StepCounters), cudaMemcpyDeviceToHost, s));
-  topo_add(uint64_t(ctx->rules.output));
-  ctx->step_topo = topo;
   return OASM_OK;
 }
 
@@ -367,9 +393,10 @@ int prepare_records(oasm_ctx* ctx, StepPlan& pl) {
   const int ro = ctx->cfg.record_order;
   pl.ordered = ctx->rules.output == OASM_OUT_FILTERED &&
                (ro == 1 || (ro == 0 && npairs * head <= cap_hits));
-  // (with cfg.timing each kernel class is timed, so they are launched one by one)
-  pl.small = pl.ordered && !ctx->cfg.timing && pl.new_bytes <= kSmallBytes &&
-             npairs * head <= kSmallSlots;
+  // (with cfg.timing each kernel class is timed, so they are launched one by one;
+  // where the last such step had too many hits, so may this one)
+  pl.small = pl.ordered && !ctx->cfg.timing && !pl.no_small && !ctx->many_hits &&
+             pl.new_bytes <= kSmallBytes && npairs * head <= kSmallSlots;
   if (!pl.ordered) return OASM_OK;
   int rc;
   if ((rc = ensure(ctx, ctx->rtmp, cap_hits + npairs * head, "ordered records"))) return rc;
@@ -421,7 +448,7 @@ int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Regi
     reclaim_lent(ctx, ctx->rec_buf);
     if ((rc = ensure_h_out(ctx, ctx->rec_buf, kDirectRecords))) return rc;
     // the kernel writes the counters at its end: one that gave up leaves this
-    ctx->h_ctr->overflow = 1u << 16;
+    ctx->h_ctr->overflow = kWaitOver;
   }
   if (ctx->cfg.graphs) {
     // capture the step, then update the cached executable graph in place when
@@ -560,12 +587,31 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
             "windows %llu/%llu\n",
             pl.items.size(), c.overflow, c.n_cand, ctx->cand.cap, c.n_hits,
             (size_t)P.cap_hits, c.n_out, P.cap_out, c.n_pool, P.cap_pool);
-  if (c.overflow & (1u << 16))
+  const bool left = (c.overflow & kSmallLeft) != 0;
+  if (pl.small) {
+    ctx->routes.small_steps += 1;
+    ctx->routes.small_left += left || (c.overflow & kWaitOver);
+  }
+  if (pl.small && (c.overflow & kWaitOver)) {
+    // the launch has changed nothing that outlives the step: once more, with a
+    // launch for each phase
+    pl.no_small = *overflow = true;
+    ctx->st.reruns += 1;
+    return OASM_OK;
+  }
+  if (left && !(c.overflow & ~kSmallLeft)) {  // the launch's own work so far stands
+    pl.no_small = *overflow = true;
+    pl.from = c.n_cand > ctx->limits.small_cand ? kFromCandidates : kFromHits;
+    return OASM_OK;
+  }
+  if (c.overflow & kWaitOver)
     return fail(ctx, OASM_ETIMEOUT, "a bounded wait on the device (a TMA copy, a grid barrier) ran out");
   if (c.overflow & 64u)
     return fail(ctx, OASM_ECUDA, "internal error: an ordered record fell outside its segment");
   *overflow = c.overflow != 0;
   if (*overflow) {
+    pl.no_small = pl.no_small || left;
+    pl.from = kFromText;
     // grow what was too small; the step is re-run from unchanged state
     if ((c.overflow & 1u) || c.n_cand > ctx->cand.cap)
       if ((rc = ensure(ctx, ctx->cand, size_t(c.n_cand * 5 / 4 + 1024), "candidates"))) return rc;
@@ -618,6 +664,8 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]); ctx->st.filter_ms += ms;
     cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[5]); ctx->st.step_ms += ms;
   }
+  if (pl.new_bytes <= kSmallBytes)
+    ctx->many_hits = c.n_cand > ctx->limits.small_cand || c.n_hits > ctx->limits.small_hits;
   ctx->st.candidates += c.n_cand;
   ctx->st.word_steps += c.word_steps;  // cut-off classes: words run beyond word 0
   ctx->st.prefilter_candidates += c.n_pref;

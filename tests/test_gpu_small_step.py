@@ -67,3 +67,76 @@ def test_many_streams_and_rules_over_steps():
                 assert canon(rows) == oracle_rows(pats, ks, t, rules)
         finally:
             B.oasm_destroy(ctx)
+
+
+def one_symbol_runs(rng, n, at, length):
+    """A DNA text with one run of a symbol, and patterns that it matches
+    everywhere: all hits of a pattern in the run are one chain."""
+    text = W.DNA[rng.integers(0, 4, size=n)]
+    text[at:at + length] = ord("A")
+    pats = [np.full(12, ord("A"), np.uint8), W.DNA[rng.integers(0, 4, size=14)],
+            np.full(20, ord("A"), np.uint8)]
+    return pats, [3, 2, 8], text
+
+
+@pytest.mark.parametrize("graphs", [0, 1])
+def test_many_hits_leave_the_launch(graphs):
+    """A step of more hits than the bound goes on as separate launches from
+    the hits that it has, the next steps run so until one has few hits again."""
+    rng = np.random.default_rng(1200)
+    pats, ks, text = one_symbol_runs(rng, 24_000, 9_000, 3_000)
+    ctx = B.oasm_create(pats, ks, None, {"graphs": graphs})
+    try:
+        B.oasm_selftest_limits(ctx, small_hits=2_000)
+        sid = B.oasm_open_stream(ctx)
+        out, left = [], []
+        for part in np.split(text, [8_000, 10_000, 11_000, 16_000, 20_000]):
+            B.oasm_feed(ctx, sid, part)
+            out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 5))
+            left.append(tuple(B.oasm_get_routes(ctx).values()))
+        st = B.oasm_get_stats(ctx)
+    finally:
+        B.oasm_destroy(ctx)
+    # few hits; many; many twice, not tried; few, not tried; few again
+    assert left == [(1, 0), (2, 1), (2, 1), (2, 1), (2, 1), (3, 1)]
+    assert st["reruns"] == 0 and st["hits"] > 20_000
+    assert canon(gpu_rows(np.concatenate(out))) == oracle_rows(pats, ks, text)
+
+
+def test_a_long_chain_of_hits():
+    """With the library's own bounds: more hits in one chain than a launch with
+    barriers between its phases can wait for."""
+    text = np.zeros(1 << 20, np.uint8)
+    text[::99_991] = 1
+    pats, ks = [np.zeros(20, np.uint8)], [15]
+    got, st = run_gpu(pats, ks, text)
+    assert st["hits"] > 20_000_000
+    ref, _ = run_gpu(pats, ks, text, cfg={"timing": 1})  # a launch per phase
+    assert got == ref and len(got) > 50_000
+
+
+def test_a_wait_that_runs_out():
+    """The blocks of a small step wait for an arrival that never comes: the step
+    runs again as separate launches, with the same records.  With more hits than
+    a sort tile the separate sort's wait runs out as well: the call fails, and
+    the step is there to be run again, from the state it was to start from."""
+    rng = np.random.default_rng(1210)
+    pats, ks, text = one_symbol_runs(rng, 24_000, 9_000, 500)
+    ctx = B.oasm_create(pats, ks)
+    try:
+        sid = B.oasm_open_stream(ctx)
+        out = []
+        for i, part in enumerate(np.split(text, [5_000, 9_100, 15_000])):
+            B.oasm_feed(ctx, sid, part)
+            B.oasm_selftest_limits(ctx, barrier_polls=300)
+            if i == 2:
+                with pytest.raises(B.OasmError) as e:
+                    B.oasm_flush(ctx, sid)
+                assert e.value.code == B.OASM_ETIMEOUT
+                B.oasm_selftest_limits(ctx)
+            out.append(B.oasm_flush(ctx, sid, end_of_stream=i == 3))
+        st, routes = B.oasm_get_stats(ctx), B.oasm_get_routes(ctx)
+    finally:
+        B.oasm_destroy(ctx)
+    assert routes == {"small_steps": 5, "small_left": 4} and st["reruns"] == 4
+    assert canon(gpu_rows(np.concatenate(out))) == oracle_rows(pats, ks, text)
