@@ -214,8 +214,8 @@ cudaError_t launch_permute(const DevHit* src, const uint32_t* idx, DevHit* dst,
                            cudaStream_t s);
 cudaError_t launch_filter(const StepParams& p, const unsigned long long* sorted, cudaStream_t s);
 // Carried windows: kFinFlush emits the decidable ones of pairs without hits,
-// kFinCommit writes the new window state; kFinAll does both.
-constexpr int kFinFlush = 1, kFinCommit = 2, kFinAll = 3;
+// kFinCommit writes the new window state.
+constexpr int kFinFlush = 1, kFinCommit = 2;
 cudaError_t launch_finalize(const StepParams& p, const unsigned long long* sorted, int phase,
                             cudaStream_t s);
 // Ordered records (p.ordered).  The scan turns the segment counts into

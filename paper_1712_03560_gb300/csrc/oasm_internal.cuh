@@ -144,6 +144,9 @@ struct Rules {
   int32_t replace, order, acc, cmp, output;
 };
 
+// A pair without hits: nothing to write, or its carried window was decided.
+constexpr int32_t kPairNone = -1, kPairDecided = -2;
+
 // Everything a step's kernels need.
 struct StepParams {
   // context tables
@@ -179,7 +182,7 @@ struct StepParams {
   WinHdr* pool_hdr;              // pending windows left by multi-segment pairs
   MemRow* pool_mem;              // [cap_pool][kMaxK+1]
   unsigned long long cap_pool;
-  int32_t* pair_pool;            // [n_items * n_pat] pool index or -1
+  int32_t* pair_pool;            // [n_items * n_pat] pool index, or one of kPair*
   StepCounters* ctr;
   int32_t num_sms;               // the device's SM count (grid sizes of the step kernels)
   // Records in canonical order without a record sort (filtered output).  A

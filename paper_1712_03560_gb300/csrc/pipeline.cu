@@ -993,51 +993,45 @@ __device__ __forceinline__ unsigned long long pair_lower_bound(const unsigned lo
 
 // Phase kFinFlush emits the records of carried windows that pairs without
 // hits can now decide; kFinCommit installs the step's new windows (and
-// clears the decided ones) in the stream state.  The ordered record path
-// runs the two apart, so the state changes only once the record count is
-// known to fit (a step that overflows is re-run from unchanged state).
+// clears the decided ones) in the stream state.  The two run apart, so the
+// state changes only once the records are known to fit and, where they are
+// sorted, to be in order (a step that overflows is re-run from unchanged state).
+// The second phase reads a word per pair and no more of the pairs it passes by
+// (8 M pairs of 4,096 streams and 2,000 signatures).
 __device__ void finalize_body(const StepParams& P, const unsigned long long* S, int phase) {
   if (P.ctr->overflow) return;
   const unsigned long long npairs = (unsigned long long)P.n_items * P.n_pat;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long pr = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
        pr < npairs; pr += stride) {
+    const int32_t q = P.pair_pool[pr];
+    if (phase == kFinCommit ? q == kPairNone : q >= 0) continue;
     const int p = int(pr % P.n_pat);
     const WorkItem w = P.items[pr / P.n_pat];
     const int m = P.m[p], K = P.K[p];
     WinHdr* hd = P.hdr + size_t(w.slot) * P.n_pat + p;
     MemRow* rows = P.mem + size_t(w.slot) * P.mem_stride + P.mem_off[p];
-    const int32_t q = P.pair_pool[pr];
     if (q >= 0) {
-      if (!(phase & kFinCommit)) continue;
       *hd = P.pool_hdr[q];
       for (int lv = 0; lv <= K; ++lv) rows[lv] = P.pool_mem[size_t(q) * (kMaxK + 1) + lv];
+    } else if (phase == kFinCommit) {
+      WinHdr z;
+      z.pend = 0;
+      z.idx = K;
+      *hd = z;
+      for (int lv = 0; lv <= K; ++lv) rows[lv].valid = 0;
     } else if (hd->pend) {
       const MemRow& top = rows[hd->idx];
-      if (w.eos || top.start + top.len - 1 <= f_new(w, m, K)) {
-        if (!(phase & kFinFlush)) {
-          WinHdr z;
-          z.pend = 0;
-          z.idx = K;
-          *hd = z;
-          for (int lv = 0; lv <= K; ++lv) rows[lv].valid = 0;
-          continue;
-        }
-        Window Wn;
-        open_window(Wn, K);
-        load_window(Wn, *hd, rows, K);
-        if (P.ordered)  // a pair without hits: its segment is the pair's head
-          Wn.rpos = pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pr,
-                                     P.start_bits + kLowBits) + pr * unsigned(P.head);
-        flush(P, Wn, uint32_t(pr), p, K, w);
-        close_segment(P, Wn);
-        if (!(phase & kFinCommit)) continue;
-        WinHdr z;
-        z.pend = 0;
-        z.idx = K;
-        *hd = z;
-        for (int lv = 0; lv <= K; ++lv) rows[lv].valid = 0;
-      }
+      if (!w.eos && top.start + top.len - 1 > f_new(w, m, K)) continue;
+      Window Wn;
+      open_window(Wn, K);
+      load_window(Wn, *hd, rows, K);
+      if (P.ordered)  // a pair without hits: its segment is the pair's head
+        Wn.rpos = pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pr,
+                                   P.start_bits + kLowBits) + pr * unsigned(P.head);
+      flush(P, Wn, uint32_t(pr), p, K, w);
+      close_segment(P, Wn);
+      P.pair_pool[pr] = kPairDecided;
     }
   }
 }
@@ -1289,7 +1283,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
     *A.counters = c;
   };
   for (unsigned long long i = me; i < (unsigned long long)P.n_items * P.n_pat; i += all)
-    P.pair_pool[i] = -1;
+    P.pair_pool[i] = kPairNone;
   for (unsigned long long i = me; i < A.seg_len / 4; i += all)
     reinterpret_cast<uint4*>(P.seg)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (P.ctr->n_cand > A.max_cand) return leave();

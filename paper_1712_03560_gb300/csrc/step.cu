@@ -240,21 +240,21 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
       ctx->st.launches += 6;
     } else {
       CK(launch_filter(P, sorted, s));
-      CK(launch_finalize(P, sorted, kFinAll, s));
+      CK(launch_finalize(P, sorted, kFinFlush, s));
       ctx->st.launches += 2;
     }
   } else if (tm) {
     CK(record_event(ctx, ctx->ev[4], s));
   }
-  CK(launch_tails(P, s));
-  ctx->st.launches += 1;
-  if (pl.ordered) {  // records from their segments to their offsets: canonical order
+  if (pl.ordered) {
+    CK(launch_tails(P, s));
+    // records from their segments to their offsets: canonical order
     CK(launch_ordered_emit(P, sorted, ctx->out_sorted[ctx->rec_buf].p, ctx->run_start.p, s));
     topo_add(0x300);
     CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
                        (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                        s));
-    ctx->st.launches += 2;
+    ctx->st.launches += 3;
   } else {  // emitted records -> canonical order (work item, pattern, decided_at, k, length)
     unsigned long long* ks = nullptr;
     uint32_t* vs = nullptr;
@@ -270,7 +270,14 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
     CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
                        (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                        s));
-    ctx->st.launches += 3;
+    // the stream state last: a step whose records did not fit, or whose sort ran
+    // out of a wait, leaves it as it was
+    if (ctx->rules.output == OASM_OUT_FILTERED) {
+      CK(launch_finalize(P, sorted, kFinCommit, s));
+      ctx->st.launches += 1;
+    }
+    CK(launch_tails(P, s));
+    ctx->st.launches += 4;
   }
   if (tm) CK(record_event(ctx, ctx->ev[5], s));
   CK(cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, sizeof(StepCounters), cudaMemcpyDeviceToHost, s));

@@ -222,3 +222,53 @@ def test_split_steps_overlap_the_record_copy(ro):
     for i in range(4):
         for j in range(3):
             assert canon(got[(i, j)]) == oracle_rows(pats, ks, sets[i][j]), (i, j)
+
+
+PEND = np.frombuffer(b"ACGTACGTAC", np.uint8)
+PEND_TEXT = np.concatenate([np.full(30, ord("T"), np.uint8), PEND, np.full(46, ord("T"), np.uint8)])
+
+
+def decide_pending(streams, copies, polls=0):
+    """Every pair of `streams` x `copies` (equal patterns) carries a window over
+    a step without hits, which decides them all with records appended and then
+    sorted; with `polls`, the record sort's wait runs out at a first attempt."""
+    ctx = B.oasm_create([PEND] * copies, [1] * copies, None,
+                        {"max_streams": streams, "record_order": 2})
+    try:
+        sids = B.oasm_open_streams(ctx, streams)
+
+        def feed(part):
+            B.oasm_feed_many(ctx, sids, np.tile(part, streams),
+                             np.arange(streams, dtype=np.uint64) * part.size,
+                             np.full(streams, part.size, np.uint32))
+
+        feed(PEND_TEXT[:46])  # (the hits are met, and their window ends at 39 or later)
+        B.oasm_step(ctx)
+        assert B.oasm_drain(ctx).size == 0
+        hits = B.oasm_get_stats(ctx)["hits"]
+        feed(PEND_TEXT[46:])
+        if polls:
+            B.oasm_selftest_limits(ctx, barrier_polls=polls)
+            with pytest.raises(B.OasmError) as e:
+                B.oasm_step(ctx)
+            assert e.value.code == B.OASM_ETIMEOUT
+            B.oasm_selftest_limits(ctx)
+        B.oasm_step(ctx)
+        assert hits > 0 and B.oasm_get_stats(ctx)["hits"] == hits
+        return B.oasm_drain(ctx)
+    finally:
+        B.oasm_destroy(ctx)
+
+
+@pytest.mark.parametrize("streams,copies,polls", [(130, 20, 300), (4096, 20, 0)])
+def test_windows_are_cleared_only_with_their_records_in_order(streams, copies, polls):
+    """A step whose record sort runs out of its wait, or whose records overflow
+    their buffer while carried windows are decided, starts again from the
+    windows as they were."""
+    res = decide_pending(streams, copies, polls)
+    assert res.size == streams * copies
+    want = oracle_rows([PEND], [1], PEND_TEXT)
+    assert len(want) == 1
+    for f, v in zip(("decided_at", "k", "start", "len"), want[0][1:]):
+        assert (res[f] == v).all()
+    assert np.unique(res["stream_id"].astype(np.int64) * copies + res["pattern_id"]).size == res.size
