@@ -64,6 +64,13 @@ int ensure_out(oasm_ctx* ctx, size_t n, bool ordered) {
   return ensure(ctx, ctx->ovals_alt, n, "record order");
 }
 
+int ensure_pool(oasm_ctx* ctx, size_t n) {
+  int rc;
+  if ((rc = ensure(ctx, ctx->pool_hdr, n, "window pool"))) return rc;
+  if ((rc = ensure(ctx, ctx->pool_pair, n, "window pool"))) return rc;
+  return ensure(ctx, ctx->pool_mem, n * (kMaxK + 1), "window pool");
+}
+
 int bits_for(uint64_t v) {  // bits needed to hold 0..v
   int b = 0;
   while (b < 64 && (v >> b) != 0) ++b;
@@ -102,7 +109,7 @@ void free_ctx(oasm_ctx* c) {
   }
   f(c->d_tails); f(c->d_hdr); f(c->d_mem);
   f(c->arena.p); f(c->upload.p); f(c->stage[0].d.p); f(c->stage[1].d.p); f(c->cand.p); f(c->keys.p);
-  f(c->keys_alt.p); f(c->out.p); f(c->pool_hdr.p); f(c->pool_mem.p); f(c->pair_pool.p);
+  f(c->keys_alt.p); f(c->out.p); f(c->pool_hdr.p); f(c->pool_mem.p); f(c->pool_pair.p); f(c->pair_pool.p);
   if (c->copy_stream) cudaStreamSynchronize(c->copy_stream);
   f(c->out_sorted[0].p); f(c->out_sorted[1].p); f(c->okeys.p); f(c->okeys_alt.p); f(c->ovals.p); f(c->ovals_alt.p);
   f(c->d_ctr); f(c->d_hist); f(c->run_start.p); f(c->rtmp.p); f(c->seg.p); f(c->seg_part.p);

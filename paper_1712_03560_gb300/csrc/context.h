@@ -438,6 +438,7 @@ struct oasm_ctx {
   DevArray<uint32_t> ovals, ovals_alt;
   DevArray<WinHdr> pool_hdr;
   DevArray<MemRow> pool_mem;
+  DevArray<uint32_t> pool_pair;
   DevArray<int32_t> pair_pool;
   DevArray<DevHit> rtmp;             // ordered records by segment position
   DevArray<uint32_t> seg;             // segment counts, then output offsets
@@ -486,6 +487,7 @@ int ensure_host(oasm_ctx* ctx, uint8_t** p, size_t* cap, size_t n, size_t keep);
 // Output record buffers for n records; `ordered` steps need only the
 // canonically ordered one.
 int ensure_out(oasm_ctx* ctx, size_t n, bool ordered = false);
+int ensure_pool(oasm_ctx* ctx, size_t n);  // room for n windows that a step leaves
 int bits_for(uint64_t v);  // bits needed to hold 0..v
 
 int wait_event(oasm_ctx* ctx, cudaEvent_t ev);

@@ -213,10 +213,8 @@ cudaError_t launch_permute(const DevHit* src, const uint32_t* idx, DevHit* dst,
                            const StepCounters* ctr, unsigned long long cap, int num_sms,
                            cudaStream_t s);
 cudaError_t launch_filter(const StepParams& p, const unsigned long long* sorted, cudaStream_t s);
-// Carried windows: kFinFlush emits the decidable ones of pairs without hits,
-// kFinCommit writes the new window state.
-constexpr int kFinFlush = 1, kFinCommit = 2;
-cudaError_t launch_finalize(const StepParams& p, const unsigned long long* sorted, int phase,
+// Decides carried windows of pairs without hits.
+cudaError_t launch_finalize(const StepParams& p, const unsigned long long* sorted,
                             cudaStream_t s);
 // Ordered records (p.ordered).  The scan turns the segment counts into
 // offsets (the total into ctr->n_out, overflow bit 2 past cap_out); the emit
@@ -228,7 +226,8 @@ size_t ordered_seg_len(size_t cap_rtmp);
 cudaError_t launch_ordered_scan(const StepParams& p, unsigned long long* part, cudaStream_t s);
 cudaError_t launch_ordered_emit(const StepParams& p, const unsigned long long* sorted,
                                 DevHit* dst, unsigned long long* run_start, cudaStream_t s);
-cudaError_t launch_tails(const StepParams& p, cudaStream_t s);
+// The step's new windows and tails into the stream state.
+cudaError_t launch_state(const StepParams& p, cudaStream_t s);
 // Everything after the candidates of a small step with ordered records, in one
 // cooperative launch (p.pair_pool and p.seg need no filling before it).  With
 // more than max_cand candidates it ends at once, with more than max_hits hits

@@ -144,9 +144,6 @@ struct Rules {
   int32_t replace, order, acc, cmp, output;
 };
 
-// A pair without hits: nothing to write, or its carried window was decided.
-constexpr int32_t kPairNone = -1, kPairDecided = -2;
-
 // Everything a step's kernels need.
 struct StepParams {
   // context tables
@@ -179,10 +176,11 @@ struct StepParams {
   unsigned long long* okeys;     // canonical sort key of each record
   uint32_t* ovals;               // record index (the sort's payload)
   unsigned long long cap_out;
-  WinHdr* pool_hdr;              // pending windows left by multi-segment pairs
+  WinHdr* pool_hdr;              // windows (open, or empty) that the step leaves
   MemRow* pool_mem;              // [cap_pool][kMaxK+1]
+  uint32_t* pool_pair;           // their pairs
   unsigned long long cap_pool;
-  int32_t* pair_pool;            // [n_items * n_pat] pool index, or one of kPair*
+  int32_t* pair_pool;            // [n_items * n_pat] pool index or -1
   StepCounters* ctr;
   int32_t num_sms;               // the device's SM count (grid sizes of the step kernels)
   // Records in canonical order without a record sort (filtered output).  A

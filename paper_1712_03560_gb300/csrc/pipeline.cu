@@ -11,9 +11,9 @@
 //             where the filter state is provably empty, and each piece runs
 //             on its own thread; the first piece resumes the pair's pending
 //             window carried from the previous step
-//   finalize  installs the new pending windows, decides carried windows of
-//             pairs without hits, and the tails kernel keeps the last T
-//             symbols of every stream for the next step.
+//   finalize  decides carried windows of pairs without hits
+//   state     installs the new pending windows and keeps the last T symbols of
+//             every stream for the next step
 #include <algorithm>
 #include <utility>
 
@@ -813,6 +813,30 @@ __device__ void flush(const StepParams& P, Window& W, uint32_t pair, int p, int 
   W.valid = 0;
 }
 
+// A pair's window after this step, for commit_body.
+__device__ __forceinline__ void put_window(const StepParams& P, const Window& W, uint32_t pair,
+                                           int K) {
+  const unsigned long long q = atomicAdd(&P.ctr->n_pool, 1ull);
+  if (q >= P.cap_pool) {
+    atomicOr(&P.ctr->overflow, 8u);
+    return;
+  }
+  WinHdr hdr;
+  hdr.pend = W.pend;
+  hdr.idx = W.idx;
+  P.pool_hdr[q] = hdr;
+  for (int lv = 0; lv <= K; ++lv) {
+    const bool v = (W.valid >> lv) & 1u;
+    MemRow r;
+    r.start = v ? W.start[lv] : 0;
+    r.len = v ? W.len[lv] : 0;
+    r.valid = v;
+    P.pool_mem[q * (kMaxK + 1) + lv] = r;
+  }
+  P.pool_pair[q] = pair;
+  P.pair_pool[pair] = int32_t(q);
+}
+
 // R1-R3 applied to one hit met in (i, l) order (event form of Algorithm 1).
 __device__ __forceinline__ void apply(const StepParams& P, Window& W, uint32_t pair, int p, int K,
                                       const WorkItem& w, int64_t start, int len, int k) {
@@ -948,24 +972,7 @@ __device__ void filter_body(const StepParams& P, const unsigned long long* S) {
     } else {
       if (Wn.pend && (w.eos || Wn.top_start + Wn.top_len - 1 <= f_new(w, m, K)))
         flush(P, Wn, pair, p, K, w);
-      const unsigned long long q = atomicAdd(&P.ctr->n_pool, 1ull);
-      if (q >= P.cap_pool) {
-        atomicOr(&P.ctr->overflow, 8u);
-      } else {
-        WinHdr nhdr;
-        nhdr.pend = Wn.pend;
-        nhdr.idx = Wn.idx;
-        P.pool_hdr[q] = nhdr;
-        for (int lv = 0; lv <= K; ++lv) {
-          const bool v = (Wn.valid >> lv) & 1u;
-          MemRow r;
-          r.start = v ? Wn.start[lv] : 0;
-          r.len = v ? Wn.len[lv] : 0;
-          r.valid = v;
-          P.pool_mem[q * (kMaxK + 1) + lv] = r;
-        }
-        P.pair_pool[pair] = int32_t(q);
-      }
+      put_window(P, Wn, pair, K);
     }
     close_segment(P, Wn);
   }
@@ -991,54 +998,74 @@ __device__ __forceinline__ unsigned long long pair_lower_bound(const unsigned lo
   return lo;
 }
 
-// Phase kFinFlush emits the records of carried windows that pairs without
-// hits can now decide; kFinCommit installs the step's new windows (and
-// clears the decided ones) in the stream state.  The two run apart, so the
-// state changes only once the records are known to fit and, where they are
-// sorted, to be in order (a step that overflows is re-run from unchanged state).
-// The second phase reads a word per pair and no more of the pairs it passes by
-// (8 M pairs of 4,096 streams and 2,000 signatures).
-__device__ void finalize_body(const StepParams& P, const unsigned long long* S, int phase) {
+// A pair without hits whose window was carried in: its records, and its entry
+// for commit_body, if it can be decided now.
+__device__ __noinline__ void decide_window(const StepParams& P, const unsigned long long* S,
+                                           uint32_t pair) {
+  const int p = int(pair % P.n_pat);
+  const WorkItem w = P.items[pair / P.n_pat];
+  const int m = P.m[p], K = P.K[p];
+  const WinHdr hd = P.hdr[size_t(w.slot) * P.n_pat + p];
+  const MemRow* rows = P.mem + size_t(w.slot) * P.mem_stride + P.mem_off[p];
+  const MemRow& top = rows[hd.idx];
+  if (!w.eos && top.start + top.len - 1 > f_new(w, m, K)) return;
+  Window Wn;
+  open_window(Wn, K);
+  load_window(Wn, hd, rows, K);
+  if (P.ordered)  // its segment is the pair's head
+    Wn.rpos = pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pair,
+                               P.start_bits + kLowBits) +
+              (unsigned long long)pair * unsigned(P.head);
+  flush(P, Wn, pair, p, K, w);
+  close_segment(P, Wn);
+  put_window(P, Wn, pair, K);
+}
+
+// Emits the records of carried windows that pairs without hits can now decide.
+// The stream state changes later, in commit_body, once the records are known to
+// fit and, where they are sorted, to be in order (a step that overflows is
+// re-run from unchanged state); a decided window leaves an entry for it.
+// Nearly every pair of a served step is passed by, so a thread has the 12 bytes
+// of four pairs on their way at a time, and the rest of the work is a function
+// of its own, for the registers (8 M pairs: one at a time 56 us, this form 28; the pass that also cleared the windows 47).
+__device__ void finalize_body(const StepParams& P, const unsigned long long* S) {
   if (P.ctr->overflow) return;
+  constexpr int kAhead = 4;
   const unsigned long long npairs = (unsigned long long)P.n_items * P.n_pat;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long pr = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-       pr < npairs; pr += stride) {
-    const int32_t q = P.pair_pool[pr];
-    if (phase == kFinCommit ? q == kPairNone : q >= 0) continue;
-    const int p = int(pr % P.n_pat);
-    const WorkItem w = P.items[pr / P.n_pat];
-    const int m = P.m[p], K = P.K[p];
-    WinHdr* hd = P.hdr + size_t(w.slot) * P.n_pat + p;
-    MemRow* rows = P.mem + size_t(w.slot) * P.mem_stride + P.mem_off[p];
-    if (q >= 0) {
-      *hd = P.pool_hdr[q];
-      for (int lv = 0; lv <= K; ++lv) rows[lv] = P.pool_mem[size_t(q) * (kMaxK + 1) + lv];
-    } else if (phase == kFinCommit) {
-      WinHdr z;
-      z.pend = 0;
-      z.idx = K;
-      *hd = z;
-      for (int lv = 0; lv <= K; ++lv) rows[lv].valid = 0;
-    } else if (hd->pend) {
-      const MemRow& top = rows[hd->idx];
-      if (!w.eos && top.start + top.len - 1 > f_new(w, m, K)) continue;
-      Window Wn;
-      open_window(Wn, K);
-      load_window(Wn, *hd, rows, K);
-      if (P.ordered)  // a pair without hits: its segment is the pair's head
-        Wn.rpos = pair_lower_bound(S, min(P.ctr->n_hits, P.cap_hits), pr,
-                                   P.start_bits + kLowBits) + pr * unsigned(P.head);
-      flush(P, Wn, uint32_t(pr), p, K, w);
-      close_segment(P, Wn);
-      P.pair_pool[pr] = kPairDecided;
+       pr < npairs; pr += kAhead * stride) {
+    int32_t q[kAhead], pend[kAhead];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      const uint32_t i = uint32_t(min(pr + j * stride, npairs - 1)), it = i / P.n_pat;
+      q[j] = P.pair_pool[i];
+      pend[j] = P.hdr[size_t(P.items[it].slot) * P.n_pat + (i - it * P.n_pat)].pend;
     }
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j)
+      if (q[j] < 0 && pend[j] && pr + j * stride < npairs)
+        decide_window(P, S, uint32_t(pr + j * stride));
   }
 }
 
-__global__ void finalize_kernel(const StepParams P, const unsigned long long* __restrict__ S,
-                                int phase) {
-  finalize_body(P, S, phase);
+__global__ void finalize_kernel(const StepParams P, const unsigned long long* __restrict__ S) {
+  finalize_body(P, S);
+}
+
+// The step's new windows into the stream state.
+__device__ void commit_body(const StepParams& P) {
+  if (P.ctr->overflow) return;
+  const unsigned long long n = P.ctr->n_pool;
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
+       q += stride) {
+    const uint32_t pair = P.pool_pair[q];
+    const uint32_t p = pair % P.n_pat, slot = P.items[pair / P.n_pat].slot;
+    MemRow* rows = P.mem + size_t(slot) * P.mem_stride + P.mem_off[p];
+    P.hdr[size_t(slot) * P.n_pat + p] = P.pool_hdr[q];
+    for (int lv = 0; lv <= P.K[p]; ++lv) rows[lv] = P.pool_mem[q * (kMaxK + 1) + lv];
+  }
 }
 
 __device__ void tails_body(const StepParams& P) {
@@ -1053,7 +1080,10 @@ __device__ void tails_body(const StepParams& P) {
   }
 }
 
-__global__ void tails_kernel(const StepParams P) { tails_body(P); }
+__global__ void state_kernel(const StepParams P) {
+  commit_body(P);
+  tails_body(P);
+}
 
 // Run boundaries of the canonically sorted records: the records of work item
 // w are [start[w], start[w + 1]), the first index whose key belongs to a pair
@@ -1283,7 +1313,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
     *A.counters = c;
   };
   for (unsigned long long i = me; i < (unsigned long long)P.n_items * P.n_pat; i += all)
-    P.pair_pool[i] = kPairNone;
+    P.pair_pool[i] = -1;
   for (unsigned long long i = me; i < A.seg_len / 4; i += all)
     reinterpret_cast<uint4*>(P.seg)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (P.ctr->n_cand > A.max_cand) return leave();
@@ -1295,7 +1325,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   if (!meet()) return;
   filter_body(P, A.sorted);
   if (!meet()) return;
-  finalize_body(P, A.sorted, kFinFlush);
+  finalize_body(P, A.sorted);
   if (!meet()) return;
   seg_reduce_body(P, A.part);
   if (!meet()) return;
@@ -1322,7 +1352,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   }
   seg_down_body(P, uint32_t(before_s));
   if (!meet()) return;
-  finalize_body(P, A.sorted, kFinCommit);
+  commit_body(P);
   tails_body(P);
   compact_body(P, total_s <= A.direct_cap ? A.direct : A.dst);
   runs_ordered_body(P, A.sorted, A.run_start);
@@ -1436,12 +1466,13 @@ cudaError_t launch_filter(const StepParams& p, const unsigned long long* sorted,
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const StepParams& p, const unsigned long long* sorted, int phase,
+cudaError_t launch_finalize(const StepParams& p, const unsigned long long* sorted,
                             cudaStream_t s) {
   const unsigned long long npairs = (unsigned long long)p.n_items * p.n_pat;
-  finalize_kernel<<<grid_for(npairs, 256, p.num_sms * 16), 256, 0, s>>>(p, sorted, phase);
+  finalize_kernel<<<grid_for(npairs, 256, p.num_sms * 16), 256, 0, s>>>(p, sorted);
   return cudaGetLastError();
 }
+
 
 int ordered_scan_blocks(int num_sms) { return std::min(kScanMaxBlocks, num_sms * 4); }
 
@@ -1473,9 +1504,11 @@ cudaError_t launch_runs(const unsigned long long* sorted_keys, const StepParams&
   return cudaGetLastError();
 }
 
-cudaError_t launch_tails(const StepParams& p, cudaStream_t s) {
+cudaError_t launch_state(const StepParams& p, cudaStream_t s) {
   if (p.n_items == 0) return cudaSuccess;
-  tails_kernel<<<min(p.n_items, 65535u), 128, 0, s>>>(p);
+  const int windows = p.rules.output == OASM_OUT_FILTERED
+                          ? grid_for(p.cap_pool, 128, p.num_sms * 8) : 1;
+  state_kernel<<<std::max(int(min(p.n_items, 65535u)), windows), 128, 0, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -234,20 +234,19 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
       // has checked that the records fit (a re-run starts from it unchanged)
       CK(cudaMemsetAsync(ctx->seg.p, 0, ordered_seg_len(ctx->rtmp.cap) * sizeof(uint32_t), s));
       CK(launch_filter(P, sorted, s));
-      CK(launch_finalize(P, sorted, kFinFlush, s));
+      CK(launch_finalize(P, sorted, s));
       CK(launch_ordered_scan(P, ctx->seg_part.p, s));
-      CK(launch_finalize(P, sorted, kFinCommit, s));
-      ctx->st.launches += 6;
+      ctx->st.launches += 5;
     } else {
       CK(launch_filter(P, sorted, s));
-      CK(launch_finalize(P, sorted, kFinFlush, s));
+      CK(launch_finalize(P, sorted, s));
       ctx->st.launches += 2;
     }
   } else if (tm) {
     CK(record_event(ctx, ctx->ev[4], s));
   }
   if (pl.ordered) {
-    CK(launch_tails(P, s));
+    CK(launch_state(P, s));
     // records from their segments to their offsets: canonical order
     CK(launch_ordered_emit(P, sorted, ctx->out_sorted[ctx->rec_buf].p, ctx->run_start.p, s));
     topo_add(0x300);
@@ -272,11 +271,7 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
                        s));
     // the stream state last: a step whose records did not fit, or whose sort ran
     // out of a wait, leaves it as it was
-    if (ctx->rules.output == OASM_OUT_FILTERED) {
-      CK(launch_finalize(P, sorted, kFinCommit, s));
-      ctx->st.launches += 1;
-    }
-    CK(launch_tails(P, s));
+    CK(launch_state(P, s));
     ctx->st.launches += 4;
   }
   if (tm) CK(record_event(ctx, ctx->ev[5], s));
@@ -648,9 +643,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     }
     if (leave && ((rc = leave_grams(ctx, pl)) || (rc = upload_plan(ctx, pl)))) return rc;
     if ((c.overflow & 8u) || c.n_pool > P.cap_pool) {
-      const size_t want = size_t(c.n_pool * 5 / 4 + 1024);
-      if ((rc = ensure(ctx, ctx->pool_hdr, want, "window pool"))) return rc;
-      if ((rc = ensure(ctx, ctx->pool_mem, want * (kMaxK + 1), "window pool"))) return rc;
+      if ((rc = ensure_pool(ctx, size_t(c.n_pool * 5 / 4 + 1024)))) return rc;
     }
     ctx->st.reruns += 1;
     return OASM_OK;
@@ -821,10 +814,7 @@ int step_begin(oasm_ctx* ctx) {
     if (!rc) rc = ensure_grams(ctx, gram_capacity(ctx, pl, false));
     if (rc && (rc != OASM_ENOMEM || (rc = leave_grams(ctx, pl)))) return rc;
   }
-  if (!ctx->pool_hdr.p) {
-    if ((rc = ensure(ctx, ctx->pool_hdr, 1 << 14, "window pool"))) return rc;
-    if ((rc = ensure(ctx, ctx->pool_mem, size_t(1 << 14) * (kMaxK + 1), "window pool"))) return rc;
-  }
+  if (!ctx->pool_hdr.p && (rc = ensure_pool(ctx, 1 << 14))) return rc;
   if ((rc = upload_plan(ctx, pl))) return rc;
   // the host staging copies must be done before bytes fed while this step
   // runs may move a staging buffer (a growing buffer is reallocated)

@@ -489,7 +489,8 @@ StepParams make_params(oasm_ctx* ctx, const WorkItem* d_items, uint32_t n_items,
                                   size_t(0xffffffffu)});
   P.pool_hdr = ctx->pool_hdr.p;
   P.pool_mem = ctx->pool_mem.p;
-  P.cap_pool = std::min(ctx->pool_hdr.cap, ctx->pool_mem.cap / (kMaxK + 1));
+  P.pool_pair = ctx->pool_pair.p;
+  P.cap_pool = std::min({ctx->pool_hdr.cap, ctx->pool_pair.cap, ctx->pool_mem.cap / (kMaxK + 1)});
   P.pair_pool = ctx->pair_pool.p;
   P.ctr = ctx->d_ctr;
   P.num_sms = ctx->num_sms;
