@@ -465,6 +465,8 @@ typedef struct {
     uint64_t small_left;  /* steps that left that launch for separate ones: too many
                              hits for it, or a wait of its blocks for one another
                              ran out */
+    uint64_t set_slots;   /* slots cleared of the set of (pattern, end) pairs that the
+                             piece filter and the gram index fill */
 } oasm_routes;
 int oasm_get_routes(oasm_ctx *ctx, oasm_routes *out);
 

@@ -84,7 +84,7 @@ class oasm_stats(ctypes.Structure):
 
 
 class oasm_routes(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_uint64) for n in ("small_steps", "small_left")]
+    _fields_ = [(n, ctypes.c_uint64) for n in ("small_steps", "small_left", "set_slots")]
 
 
 class oasm_limits(ctypes.Structure):

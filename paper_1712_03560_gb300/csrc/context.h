@@ -316,6 +316,7 @@ struct StepPlan {
   bool small = false;                // everything after the candidates in one launch
   bool no_small = false;             // ... not again: that launch left the step
   int from = kFromText;              // where the launches of the step begin
+  size_t set_len = 0;                // slots of the (end, pattern) set it uses
   bool grams = false;                // the gram index and the rest buckets scan this step
   // An empty plan that keeps its vectors' storage.
   void clear() {
@@ -395,6 +396,7 @@ struct oasm_ctx {
   uint8_t* d_pbytes = nullptr;
   uint32_t* d_poff = nullptr;
   DevArray<unsigned long long> pset;  // (end, pattern) set, capacity a power of two
+  double set_rate = 1.0 / 16;         // slots per symbol of a step's text
   Grams grams;
 
   // streams

@@ -8,7 +8,7 @@ import pytest
 
 from paper_1712_03560_gb300 import binding as B
 from paper_1712_03560_gb300 import workloads as W
-from parity_util import canon, oracle_rows, run_gpu
+from parity_util import canon, gpu_rows, oracle_rows, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -191,3 +191,49 @@ def test_short_patterns_of_three_errors_beside_the_index(short):
     got, st = run_gpu(pats, ks, text)
     assert canon(got) == want
     assert st["word_steps"] == (short + 1) // 2 * n
+
+
+@pytest.mark.parametrize("piece", [0, 1])
+def test_the_set_of_ends_fits_each_step(piece):
+    """Steps after a large one clear the part of the (end, pattern) set that
+    their own text needs; a step that needs more runs again with more, and the
+    ones after it start there."""
+    import torch
+    rng = np.random.default_rng(890 + piece)
+    sigma = 256 if piece else 4
+    pats, ks, text = dictionary(rng, sigma, N_PAT, 24, 90, 140_000, lambda m: m // 10)
+    alphabet = np.unique(text)
+    one = alphabet[rng.integers(0, alphabet.size, size=80)]  # a pattern many times over
+    pats, ks = pats + [one] * 300, ks + [8] * 300
+    dense = text.copy()
+    for at in range(500, dense.size, 2_000):
+        dense[at:at + one.size] = one
+    big = torch.from_numpy(alphabet).cuda()[
+        torch.randint(0, alphabet.size, (1 << 25,), device="cuda")]
+    ctx = B.oasm_create(pats, ks, None, {"prefilter_piece": piece})
+
+    def step(t):
+        before = B.oasm_get_routes(ctx)["set_slots"], B.oasm_get_stats(ctx)["reruns"]
+        sid = B.oasm_open_stream(ctx)
+        (B.oasm_feed if isinstance(t, np.ndarray) else B.oasm_feed_device)(ctx, sid, t)
+        B.oasm_end_stream(ctx, sid)
+        B.oasm_step(ctx)
+        rows = gpu_rows(B.oasm_drain(ctx))
+        B.oasm_close_stream(ctx, sid)
+        return rows, B.oasm_get_routes(ctx)["set_slots"] - before[0], \
+            B.oasm_get_stats(ctx)["reruns"] - before[1]
+
+    try:
+        step(big)
+        step(big)
+        assert step(big)[1] >= 1 << 21
+        want, want_dense = oracle_rows(pats, ks, text), oracle_rows(pats, ks, dense)
+        rows, slots, _ = step(text)
+        assert canon(rows) == want and 0 < slots <= 1 << 19
+        for _ in range(2):
+            rows, slots, reruns = step(dense)
+            assert canon(rows) == want_dense
+        assert reruns == 0 and slots > 1 << 19
+        assert step(big)[1] >= 1 << 21
+    finally:
+        B.oasm_destroy(ctx)
