@@ -288,7 +288,13 @@ int oasm_end_stream(oasm_ctx *ctx, uint32_t sid);
 /* Runs one batched step over every stream with pending input or a pending
  * end: one pass of the whole device path (stage, bit-parallel scan, anchored
  * verification, ordering, filter, emit).  Returns when the step has finished
- * on the device and its decided hits are queued on their streams. */
+ * on the device and its decided hits are queued on their streams.
+ * The sort, and the launch that small steps run after the scan, are
+ * cooperative: their blocks (up to four per SM, one per SM) wait for one
+ * another at barriers, so such a launch starts when all of them find room
+ * beside whatever else runs on the device.  Next to kernels of other streams
+ * or contexts that hold SMs for long, a step starts those two later than
+ * ordinary launches would. */
 int oasm_step(oasm_ctx *ctx);
 
 /* oasm_step in two halves, so that host work can overlap the device.
@@ -553,7 +559,8 @@ typedef struct {
     uint64_t small_hits;     /* hits over which a small step leaves its launch */
     uint32_t barrier_polls;  /* polls at a grid barrier, which then also waits for an
                                 arrival that never comes: the wait runs out */
-    uint32_t reserved;
+    uint32_t no_small;       /* 1: as on a device that the launch of small steps does
+                                not fit: every step runs as separate launches */
 } oasm_limits;
 int oasm_selftest_limits(oasm_ctx *ctx, const oasm_limits *l);
 

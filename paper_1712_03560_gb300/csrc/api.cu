@@ -275,8 +275,8 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   }
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
   if (ctx->num_sms < 1) ctx->num_sms = 1;
-  if ((ctx->sort_blocks = sort_grid(ctx->num_sms)) < 1 ||
-      (ctx->small_blocks = small_step_grid(ctx->num_sms)) < 1) {
+  ctx->small_blocks = small_step_grid(ctx->num_sms);
+  if ((ctx->sort_blocks = sort_grid(ctx->num_sms)) < 1) {
     cudaGetLastError();
     fail(ctx, OASM_ECUDA, "the sort kernel does not fit the device");
     return bail(OASM_ECUDA);
@@ -904,6 +904,7 @@ int oasm_selftest_limits(oasm_ctx* ctx, const oasm_limits* l) {
   if (rc) return rc;
   ctx->limits = Limits();
   ctx->many_hits = false;
+  ctx->small_blocks = l && l->no_small ? 0 : small_step_grid(ctx->num_sms);
   if (!l) return OASM_OK;
   if (l->small_hits) ctx->limits.small_hits = l->small_hits;
   if (l->barrier_polls) ctx->limits.barrier = BarrierBound{l->barrier_polls, 1};

@@ -378,7 +378,8 @@ struct oasm_ctx {
   std::vector<GraphSlot> graphs;
   uint64_t graph_clock = 0;
   uint64_t step_topo = 0;    // topology of the step being enqueued
-  int small_blocks = 0;      // blocks of the small steps' launch (0: never used)
+  int small_blocks = 0;      // blocks of the small steps' launch (0: it does not fit
+                             // the device, and no step is launched so)
   int sort_blocks = 0;       // radix-sort blocks: as many as are resident together
   bool capturing = false;
 

@@ -1403,8 +1403,10 @@ int small_step_grid(int num_sms) {
                              int(sizeof(SortSmem))) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kSortThreads,
                                                       sizeof(SortSmem)) != cudaSuccess ||
-        per_sm < 1)
+        per_sm < 1) {
+      cudaGetLastError();  // (the next launch reads it otherwise)
       return 0;
+    }
   }
   return num_sms;
 }

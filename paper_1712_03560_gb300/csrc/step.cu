@@ -412,8 +412,8 @@ int prepare_records(oasm_ctx* ctx, StepPlan& pl) {
                (ro == 1 || (ro == 0 && npairs * head <= cap_hits));
   // (with cfg.timing each kernel class is timed, so they are launched one by one;
   // where the last such step had too many hits, so may this one)
-  pl.small = pl.ordered && !ctx->cfg.timing && !pl.no_small && !ctx->many_hits &&
-             pl.new_bytes <= kSmallBytes && npairs * head <= kSmallSlots;
+  pl.small = pl.ordered && ctx->small_blocks > 0 && !ctx->cfg.timing && !pl.no_small &&
+             !ctx->many_hits && pl.new_bytes <= kSmallBytes && npairs * head <= kSmallSlots;
   if (!pl.ordered) return OASM_OK;
   int rc;
   if ((rc = ensure(ctx, ctx->rtmp, cap_hits + npairs * head, "ordered records"))) return rc;

@@ -141,3 +141,21 @@ def test_a_wait_that_runs_out():
         B.oasm_destroy(ctx)
     assert (routes["small_steps"], routes["small_left"], st["reruns"]) == (5, 4, 4)
     assert canon(gpu_rows(np.concatenate(out))) == oracle_rows(pats, ks, text)
+
+
+def test_without_the_launch_of_small_steps():
+    """Where it does not fit the device, every step runs as separate launches."""
+    rng = np.random.default_rng(1220)
+    pats, ks, text = one_symbol_runs(rng, 9_000, 4_000, 60)
+    ctx = B.oasm_create(pats, ks)
+    try:
+        B.oasm_selftest_limits(ctx, no_small=1)
+        sid = B.oasm_open_stream(ctx)
+        out = []
+        for part in np.split(text, [3_000, 4_020]):
+            B.oasm_feed(ctx, sid, part)
+            out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 2))
+        assert B.oasm_get_routes(ctx)["small_steps"] == 0
+    finally:
+        B.oasm_destroy(ctx)
+    assert canon(gpu_rows(np.concatenate(out))) == oracle_rows(pats, ks, text)
