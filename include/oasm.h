@@ -564,6 +564,11 @@ typedef struct {
 } oasm_limits;
 int oasm_selftest_limits(oasm_ctx *ctx, const oasm_limits *l);
 
+/* Lets the fail_at-th device allocation that the calling thread makes in this
+ * library from now on fail as one that finds no memory (1: the next; 0: none).
+ * Returns how many it made since the last call. */
+uint64_t oasm_selftest_alloc(uint64_t fail_at);
+
 /* ---- search without device allocation (no counterpart in the paper) ----
  * For callers that cannot call cudaMalloc: code running inside a framework
  * whose caching allocator already holds the device's memory, code under a

@@ -151,7 +151,8 @@ EXPORTS = ["oasm_config_default", "oasm_rules_default", "oasm_create", "oasm_cre
            "oasm_save_stream", "oasm_restore_stream", "oasm_replay", "oasm_register_host",
            "oasm_unregister_host", "oasm_step_begin", "oasm_step_end", "oasm_replay_ops",
            "oasm_piece_filter_choice", "oasm_selftest_wait", "oasm_get_tuning",
-           "oasm_set_tuning", "oasm_get_routes", "oasm_selftest_limits"]
+           "oasm_set_tuning", "oasm_get_routes", "oasm_selftest_limits",
+           "oasm_selftest_alloc"]
 
 _lib = None
 _lock = threading.Lock()
@@ -201,6 +202,7 @@ def load(path: str | None = None):
             "oasm_strerror": ([i32], ctypes.c_char_p),
             "oasm_autotune": ([vp, vp, ctypes.c_size_t, ctypes.c_char_p, ctypes.c_size_t], i32),
             "oasm_selftest_wait": ([i32, u32, i32], i32),
+            "oasm_selftest_alloc": ([u64], u64),
             "oasm_get_routes": ([vp, ctypes.POINTER(oasm_routes)], i32),
             "oasm_selftest_limits": ([vp, ctypes.POINTER(oasm_limits)], i32),
             "oasm_get_tuning": ([vp, ctypes.POINTER(oasm_tuning), u32, ctypes.POINTER(u32)], i32),
@@ -495,6 +497,10 @@ def oasm_selftest_limits(ctx, **kw):
     library's own ones again."""
     lim = oasm_limits(**kw)
     return _check(load().oasm_selftest_limits(ctx, ctypes.byref(lim) if kw else None), ctx)
+
+
+def oasm_selftest_alloc(fail_at: int = 0) -> int:
+    return int(load().oasm_selftest_alloc(fail_at))
 
 
 def _check_device_buffer(d, need_bytes: int, what: str):

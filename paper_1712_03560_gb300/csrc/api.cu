@@ -71,6 +71,14 @@ int ensure_pool(oasm_ctx* ctx, size_t n) {
   return ensure(ctx, ctx->pool_mem, n * (kMaxK + 1), "window pool");
 }
 
+// Failure injection of oasm_selftest_alloc, per thread.
+thread_local uint64_t g_allocs = 0, g_alloc_fail = 0;
+
+cudaError_t dev_alloc(void** p, size_t bytes) {
+  if (++g_allocs == g_alloc_fail) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
 int bits_for(uint64_t v) {  // bits needed to hold 0..v
   int b = 0;
   while (b < 64 && (v >> b) != 0) ++b;
@@ -99,14 +107,8 @@ void free_ctx(oasm_ctx* c) {
   auto f = [](void* p) { if (p) cudaFree(p); };
   f(c->d_m); f(c->d_K); f(c->d_mem_off); f(c->d_peq_rev); f(c->d_bytes);
   f(c->d_pdir); f(c->d_pent); f(c->d_pbytes); f(c->d_poff); f(c->pset.p); f(c->d_pbloom);
-  for (auto* bs : {&c->buckets, &c->grams.rest})
-    for (auto& b : *bs) { f(b.d_groups); f(b.d_peq); f(b.d_peq_hi); f(b.d_wrow); }
-  {
-    Grams& gr = c->grams;
-    f(const_cast<uint32_t*>(gr.scan.bits)); f(const_cast<uint4*>(gr.scan.dir));
-    f(const_cast<GramEntry*>(gr.t.entries));
-    f(const_cast<uint32_t*>(gr.t.peq_fwd)); f(gr.susp.p); f(gr.longs.p); f(gr.ctr.p);
-  }
+  free_buckets(c->buckets);
+  drop_grams(c);
   f(c->d_tails); f(c->d_hdr); f(c->d_mem);
   f(c->arena.p); f(c->upload.p); f(c->stage[0].d.p); f(c->stage[1].d.p); f(c->cand.p); f(c->keys.p);
   f(c->keys_alt.p); f(c->out.p); f(c->pool_hdr.p); f(c->pool_mem.p); f(c->pool_pair.p); f(c->pair_pool.p);
@@ -335,9 +337,9 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
          ctx->stream_bytes);
     return bail(OASM_ENOMEM);
   }
-  if (cudaMalloc(&ctx->d_tails, size_t(S) * ctx->T) != cudaSuccess ||
-      cudaMalloc(&ctx->d_hdr, size_t(S) * n_pat * sizeof(WinHdr)) != cudaSuccess ||
-      cudaMalloc(&ctx->d_mem, size_t(S) * ctx->mem_stride * sizeof(MemRow)) != cudaSuccess) {
+  if (dev_alloc(&ctx->d_tails, size_t(S) * ctx->T) != cudaSuccess ||
+      dev_alloc(&ctx->d_hdr, size_t(S) * n_pat * sizeof(WinHdr)) != cudaSuccess ||
+      dev_alloc(&ctx->d_mem, size_t(S) * ctx->mem_stride * sizeof(MemRow)) != cudaSuccess) {
     cudaGetLastError();
     fail(ctx, OASM_ENOMEM, "stream state for %u streams does not fit", S);
     return bail(OASM_ENOMEM);
@@ -350,9 +352,9 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   }
   ctx->streams.resize(S);
   for (uint32_t i = 0; i < S; ++i) ctx->free_slots.push(i);
-  if (cudaMalloc(&ctx->d_ctr, sizeof(StepCounters)) != cudaSuccess ||
+  if (dev_alloc(&ctx->d_ctr, sizeof(StepCounters)) != cudaSuccess ||
       cudaHostAlloc(&ctx->h_ctr, sizeof(StepCounters), cudaHostAllocDefault) != cudaSuccess ||
-      cudaMalloc(&ctx->d_hist, sort_hist_len(ctx->sort_blocks) * sizeof(unsigned int)) != cudaSuccess) {
+      dev_alloc(&ctx->d_hist, sort_hist_len(ctx->sort_blocks) * sizeof(unsigned int)) != cudaSuccess) {
     cudaGetLastError();
     fail(ctx, OASM_ENOMEM, "step counters");
     return bail(OASM_ENOMEM);
@@ -367,6 +369,7 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   // the records' copies to the host run on their own stream, beside the next step
   if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
     return bail(fail(ctx, OASM_ECUDA, "cudaStreamCreate failed"));
+  if ((rc = build_index(ctx))) return bail(rc);
   // the tables' copies and the cleared state are complete before the first
   // step, which runs on a stream that does not wait for the default one
   if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
@@ -909,6 +912,13 @@ int oasm_selftest_limits(oasm_ctx* ctx, const oasm_limits* l) {
   if (l->small_hits) ctx->limits.small_hits = l->small_hits;
   if (l->barrier_polls) ctx->limits.barrier = BarrierBound{l->barrier_polls, 1};
   return OASM_OK;
+}
+
+uint64_t oasm_selftest_alloc(uint64_t fail_at) {
+  const uint64_t n = g_allocs;
+  g_allocs = 0;
+  g_alloc_fail = fail_at;
+  return n;
 }
 
 void* oasm_cuda_stream(oasm_ctx* ctx) { return ctx ? static_cast<void*>(ctx->stream) : nullptr; }

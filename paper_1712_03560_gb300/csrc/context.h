@@ -294,6 +294,7 @@ struct oasm_ctx {
   uint8_t* d_bytes = nullptr;  // [n_pat][OASM_MAX_PATTERN_LEN] pattern symbols
   std::vector<Bucket> buckets;
   // piece filter (cfg.prefilter_piece): tables of the patterns it serves
+  std::vector<char> on_filter;  // per pattern
   uint32_t n_pref_pat = 0;
   PrefSlot* d_pdir = nullptr;
   uint32_t pdir_bits = 0, pmax_probe = 0;
@@ -404,6 +405,17 @@ int wait_event(oasm_ctx* ctx, cudaEvent_t ev);
 void free_ctx(oasm_ctx* c);
 int build_prefilter(oasm_ctx* ctx, const std::vector<char>& pref);
 int build_tables(oasm_ctx* ctx);
+// The gram index, after everything that the context cannot do without: with no
+// device memory for all of it there is none.
+int build_index(oasm_ctx* ctx);
+void drop_grams(oasm_ctx* ctx);  // frees the index and its buffers
+void free_buckets(std::vector<Bucket>& bs);
+// cudaMalloc (that oasm_selftest_alloc can let fail).
+cudaError_t dev_alloc(void** p, size_t bytes);
+template <class T>
+cudaError_t dev_alloc(T** p, size_t bytes) {
+  return dev_alloc(reinterpret_cast<void**>(p), bytes);
+}
 // Tables of the gram index; served[p] = 1 for the patterns it takes (all 0
 // when it would not pay).
 int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>& served);
@@ -428,8 +440,7 @@ cudaError_t record_event(oasm_ctx* ctx, cudaEvent_t e, cudaStream_t s);
 int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Region* d_regions,
                  const CopyChunk* d_chunks);
 double ms_since(std::chrono::steady_clock::time_point t0);
-int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Region* d_regions,
-                const CopyChunk* d_chunks);
+int launch_step(oasm_ctx* ctx);
 int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* overflow);
 // Waits for the records of the last finished step to reach the host and
 // hands them to their streams' queues (no-op when none are on the way).
@@ -445,12 +456,17 @@ int check_sid(oasm_ctx* ctx, uint32_t sid);
 #define CK(call)                                                                        \
   do {                                                                                  \
     cudaError_t e_ = (call);                                                            \
+    if (e_ == cudaErrorMemoryAllocation) cudaGetLastError();                            \
     if (e_ != cudaSuccess)                                                              \
-      return fail(ctx, OASM_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_));     \
+      return fail(ctx, e_ == cudaErrorMemoryAllocation ? OASM_ENOMEM : OASM_ECUDA,      \
+                  "%s failed: %s", #call, cudaGetErrorString(e_));                      \
   } while (0)
 
+// Room for n elements (the old contents are not kept).  Without device memory
+// for it the gram index gives up its own, unless the room is for the index: a
+// step planned with it is planned again (launch_step).
 template <class T>
-int ensure(oasm_ctx* ctx, DevArray<T>& a, size_t n, const char* what) {
+int ensure(oasm_ctx* ctx, DevArray<T>& a, size_t n, const char* what, bool for_index = false) {
   if (a.cap >= n && a.p) return OASM_OK;
   size_t want = std::max<size_t>(n, a.cap + a.cap / 2);
   want = std::max<size_t>(want, 1024);
@@ -458,7 +474,12 @@ int ensure(oasm_ctx* ctx, DevArray<T>& a, size_t n, const char* what) {
   a.p = nullptr;
   a.cap = 0;
   ctx->st.buffer_grows += 1;
-  cudaError_t e = cudaMalloc(&a.p, want * sizeof(T));
+  cudaError_t e = dev_alloc(&a.p, want * sizeof(T));
+  if (e == cudaErrorMemoryAllocation && !for_index && ctx->grams.n_pat) {
+    cudaGetLastError();
+    drop_grams(ctx);
+    e = dev_alloc(&a.p, want * sizeof(T));
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     a.p = nullptr;
@@ -471,11 +492,12 @@ int ensure(oasm_ctx* ctx, DevArray<T>& a, size_t n, const char* what) {
 
 // A power-of-two capacity of at least n (the piece filter's open-addressing set).
 template <class T>
-int ensure_pow2(oasm_ctx* ctx, DevArray<T>& a, size_t n, const char* what) {
+int ensure_pow2(oasm_ctx* ctx, DevArray<T>& a, size_t n, const char* what,
+                bool for_index = false) {
   if (a.p && a.cap >= n) return OASM_OK;
   size_t want = 1024;
   while (want < n || want < 2 * a.cap) want <<= 1;
-  return ensure(ctx, a, want, what);
+  return ensure(ctx, a, want, what, for_index);
 }
 
 }  // namespace oasm

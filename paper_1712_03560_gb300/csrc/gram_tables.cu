@@ -387,7 +387,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   auto up = [&](auto** dst, const auto& v) -> cudaError_t {
     using T = typename std::decay<decltype(v[0])>::type;
     T* d = nullptr;
-    cudaError_t e = cudaMalloc(&d, v.size() * sizeof(T));
+    cudaError_t e = dev_alloc(&d, v.size() * sizeof(T));
     if (e != cudaSuccess) return e;
     *dst = d;
     return cudaMemcpy(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
@@ -396,11 +396,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   cudaError_t e = up(&a.bits, bits);
   if (e == cudaSuccess) e = up(&a.dir, dir);
   if (e == cudaSuccess) e = up(&gr.t.entries, entries);
-  if (e == cudaSuccess) e = cudaMalloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t));
-  if (e == cudaErrorMemoryAllocation) {  // no room for the index: the scan needs none
-    cudaGetLastError();
-    return none();  // (what was allocated goes with the context)
-  }
+  if (e == cudaSuccess) e = dev_alloc(&peq, size_t(n) * 256 * 4 * sizeof(uint32_t));
   CK(e);
   gr.t.peq_fwd = peq;
   a.entries = gr.t.entries;

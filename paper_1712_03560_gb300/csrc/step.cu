@@ -453,14 +453,72 @@ static int ensure_h_out(oasm_ctx* ctx, int b, size_t n) {
   return OASM_OK;
 }
 
+// Suspects a slice may hold: half as many again as expected, or, `most`, as
+// many as cost what the index saves (about 30 clocks each).
+static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) {
+  const Grams& gr = ctx->grams;
+  const double syms = double(std::min(pl.arena_bytes, gram_slice(pl)));
+  const double top = std::min(kGramMaxRate, gr.saved_clk / 30.0);
+  const double rate = most ? top : std::min(top, 1.5 * gr.rate + 0.03);
+  return size_t(syms * rate) + (size_t(1) << 14);
+}
+
+// Room for n suspects of a slice; those of long patterns that a second look
+// keeps are a small part.
+static int ensure_grams(oasm_ctx* ctx, size_t n) {
+  const int rc = ensure(ctx, ctx->grams.susp, n, "gram suspects", true);
+  if (rc || !ctx->grams.t.any_long) return rc;
+  return ensure(ctx, ctx->grams.longs, 3 * (n / 4 + (size_t(1) << 14)), "gram suspects", true);
+}
+
+// One upload: items | regions | chunks.
+static int upload_plan(oasm_ctx* ctx, StepPlan& pl) {
+  int rc;
+  const size_t bi = pl.items.size() * sizeof(WorkItem);
+  const size_t br = pl.regions.size() * sizeof(Region);
+  const size_t bc = pl.chunks.size() * sizeof(CopyChunk);
+  const size_t o_r = (bi + 255) & ~size_t(255), o_c = (o_r + br + 255) & ~size_t(255);
+  const size_t total = o_c + bc + 256;
+  if ((rc = ensure_host(ctx, &ctx->h_upload, &ctx->h_upload_cap, total, 0))) return rc;
+  if ((rc = ensure(ctx, ctx->upload, total, "step upload"))) return rc;
+  memcpy(ctx->h_upload, pl.items.data(), bi);
+  memcpy(ctx->h_upload + o_r, pl.regions.data(), br);
+  memcpy(ctx->h_upload + o_c, pl.chunks.data(), bc);
+  CK(cudaMemcpyAsync(ctx->upload.p, ctx->h_upload, total, cudaMemcpyHostToDevice, ctx->stream));
+  Flight& f = ctx->flight;
+  f.d_items = reinterpret_cast<const WorkItem*>(ctx->upload.p);
+  f.d_regions = reinterpret_cast<const Region*>(ctx->upload.p + o_r);
+  f.d_chunks = reinterpret_cast<const CopyChunk*>(ctx->upload.p + o_c);
+  return OASM_OK;
+}
+
+// The step, and the next ones, without the index: every pattern is scanned
+// (or filtered) with the buffers that this needs.  Used where the text is too
+// repetitive for the index, and where its buffers find no memory.
+static int leave_grams(oasm_ctx* ctx, StepPlan& pl) {
+  pl.grams = false;
+  ctx->grams.off_steps = 32;
+  ctx->err.clear();
+  plan_regions(ctx, pl);
+  if (!ctx->n_pref_pat) return OASM_OK;
+  const int rc = ctx->pset.p ? OASM_OK
+                             : ensure_pow2(ctx, ctx->pset, size_t(1) << 20, "piece filter set");
+  fit_set(ctx, pl);
+  return rc;
+}
+
 // Launches one step's device work (as a graph or directly) and records the
 // completion event; returns without waiting.
-int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Region* d_regions,
-                const CopyChunk* d_chunks) {
+int launch_step(oasm_ctx* ctx) {
   const auto t_launch = std::chrono::steady_clock::now();
   cudaStream_t s = ctx->stream;
+  Flight& f = ctx->flight;
+  StepPlan& pl = f.pl;
   int rc;
   if ((rc = prepare_records(ctx, pl))) return rc;
+  // a buffer of this step took the index's memory
+  if (pl.grams && !ctx->grams.n_pat && ((rc = leave_grams(ctx, pl)) || (rc = upload_plan(ctx, pl))))
+    return rc;
   if (pl.small) {  // the step may write its records straight into the pinned buffer
     reclaim_lent(ctx, ctx->rec_buf);
     if ((rc = ensure_h_out(ctx, ctx->rec_buf, kDirectRecords))) return rc;
@@ -472,7 +530,7 @@ int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Regi
     // the step has the same shape (kernel arguments and grids may differ)
     CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     ctx->capturing = true;
-    rc = enqueue_step(ctx, pl, d_items, d_regions, d_chunks);
+    rc = enqueue_step(ctx, pl, f.d_items, f.d_regions, f.d_chunks);
     ctx->capturing = false;
     cudaGraph_t g = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(s, &g);
@@ -521,65 +579,11 @@ int launch_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Regi
     cudaGraphDestroy(g);
     CK(cudaGraphLaunch(slot->exec, s));
   } else {
-    if ((rc = enqueue_step(ctx, pl, d_items, d_regions, d_chunks))) return rc;
+    if ((rc = enqueue_step(ctx, pl, f.d_items, f.d_regions, f.d_chunks))) return rc;
   }
   CK(cudaEventRecord(ctx->done, s));
   ctx->st.host_launch_ms += ms_since(t_launch);
   return OASM_OK;
-}
-
-// Suspects a slice may hold: half as many again as expected, or, `most`, as
-// many as cost what the index saves (about 30 clocks each).
-static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) {
-  const Grams& gr = ctx->grams;
-  const double syms = double(std::min(pl.arena_bytes, gram_slice(pl)));
-  const double top = std::min(kGramMaxRate, gr.saved_clk / 30.0);
-  const double rate = most ? top : std::min(top, 1.5 * gr.rate + 0.03);
-  return size_t(syms * rate) + (size_t(1) << 14);
-}
-
-// Room for n suspects of a slice; those of long patterns that a second look
-// keeps are a small part.
-static int ensure_grams(oasm_ctx* ctx, size_t n) {
-  const int rc = ensure(ctx, ctx->grams.susp, n, "gram suspects");
-  if (rc || !ctx->grams.t.any_long) return rc;
-  return ensure(ctx, ctx->grams.longs, 3 * (n / 4 + (size_t(1) << 14)), "gram suspects");
-}
-
-// One upload: items | regions | chunks.
-static int upload_plan(oasm_ctx* ctx, StepPlan& pl) {
-  int rc;
-  const size_t bi = pl.items.size() * sizeof(WorkItem);
-  const size_t br = pl.regions.size() * sizeof(Region);
-  const size_t bc = pl.chunks.size() * sizeof(CopyChunk);
-  const size_t o_r = (bi + 255) & ~size_t(255), o_c = (o_r + br + 255) & ~size_t(255);
-  const size_t total = o_c + bc + 256;
-  if ((rc = ensure_host(ctx, &ctx->h_upload, &ctx->h_upload_cap, total, 0))) return rc;
-  if ((rc = ensure(ctx, ctx->upload, total, "step upload"))) return rc;
-  memcpy(ctx->h_upload, pl.items.data(), bi);
-  memcpy(ctx->h_upload + o_r, pl.regions.data(), br);
-  memcpy(ctx->h_upload + o_c, pl.chunks.data(), bc);
-  CK(cudaMemcpyAsync(ctx->upload.p, ctx->h_upload, total, cudaMemcpyHostToDevice, ctx->stream));
-  Flight& f = ctx->flight;
-  f.d_items = reinterpret_cast<const WorkItem*>(ctx->upload.p);
-  f.d_regions = reinterpret_cast<const Region*>(ctx->upload.p + o_r);
-  f.d_chunks = reinterpret_cast<const CopyChunk*>(ctx->upload.p + o_c);
-  return OASM_OK;
-}
-
-// The step, and the next ones, without the index: every pattern is scanned
-// (or filtered) with the buffers that this needs.  Used where the text is too
-// repetitive for the index, and where its buffers find no memory.
-static int leave_grams(oasm_ctx* ctx, StepPlan& pl) {
-  pl.grams = false;
-  ctx->grams.off_steps = 32;
-  ctx->err.clear();
-  plan_regions(ctx, pl);
-  if (!ctx->n_pref_pat) return OASM_OK;
-  const int rc = ctx->pset.p ? OASM_OK
-                             : ensure_pow2(ctx, ctx->pset, size_t(1) << 20, "piece filter set");
-  fit_set(ctx, pl);
-  return rc;
 }
 
 // Waits for the launched step, then either grows the buffers that overflowed
@@ -645,7 +649,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     bool leave = false;
     if (c.overflow & 32u) {  // the (end, pattern) set filled up: room for 4x its inserts
       const size_t want = std::max(size_t(c.n_pref + c.n_gram) * 4, 2 * pl.set_len);
-      rc = ensure_pow2(ctx, ctx->pset, want, "piece filter set");
+      rc = ensure_pow2(ctx, ctx->pset, want, "piece filter set", pl.grams);
       leave = rc == OASM_ENOMEM && pl.grams;
       if (rc && !leave) return rc;
       ctx->set_rate = std::max(ctx->set_rate, double(want - 1) / double(pl.arena_bytes));
@@ -824,12 +828,14 @@ int step_begin(oasm_ctx* ctx) {
     ctx->h_run_start = reinterpret_cast<unsigned long long*>(p);
     ctx->h_run_start_cap = cap_bytes / sizeof(unsigned long long);
   }
+  if (pl.grams && !ctx->grams.n_pat && (rc = leave_grams(ctx, pl))) return rc;
   if (ctx->n_pref_pat && !pl.grams && !ctx->pset.p &&
       (rc = ensure_pow2(ctx, ctx->pset, size_t(1) << 20, "piece filter set")))
     return rc;
   if (pl.grams) {
-    rc = ctx->pset.p ? OASM_OK : ensure_pow2(ctx, ctx->pset, 4 * ctx->cand.cap, "piece filter set");
-    if (!rc) rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters");
+    rc = ctx->pset.p ? OASM_OK
+                     : ensure_pow2(ctx, ctx->pset, 4 * ctx->cand.cap, "piece filter set", true);
+    if (!rc) rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters", true);
     if (!rc) rc = ensure_grams(ctx, gram_capacity(ctx, pl, false));
     if (rc && (rc != OASM_ENOMEM || (rc = leave_grams(ctx, pl)))) return rc;
   }
@@ -842,7 +848,7 @@ int step_begin(oasm_ctx* ctx) {
     CK(cudaEventRecord(ctx->staged, ctx->stream));
   }
   ctx->st.host_plan_ms += ms_since(t_plan);
-  if ((rc = launch_step(ctx, pl, f.d_items, f.d_regions, f.d_chunks))) return rc;
+  if ((rc = launch_step(ctx))) return rc;
   if (copies && (rc = wait_event(ctx, ctx->staged))) return rc;
   f.on = true;
   // new host bytes go to the other buffer while this one is consumed
@@ -871,7 +877,7 @@ int step_end(oasm_ctx* ctx) {
                   std::min(ctx->keys.cap, ctx->keys_alt.cap), c.n_out, ctx->out.cap, c.n_pool,
                   ctx->pool_hdr.cap);
     }
-    if (attempt > 0 && (rc = launch_step(ctx, pl, f.d_items, f.d_regions, f.d_chunks))) {
+    if (attempt > 0 && (rc = launch_step(ctx))) {
       f.on = false;
       return rc;
     }

@@ -64,13 +64,13 @@ int build_prefilter(oasm_ctx* ctx, const std::vector<char>& pref) {
   }
   std::vector<PrefEntry> ev;
   for (const auto& e : ents) ev.push_back(e.second);
-  CK(cudaMalloc(&ctx->d_pdir, dir.size() * sizeof(PrefSlot)));
+  CK(dev_alloc(&ctx->d_pdir, dir.size() * sizeof(PrefSlot)));
   CK(cudaMemcpy(ctx->d_pdir, dir.data(), dir.size() * sizeof(PrefSlot), cudaMemcpyHostToDevice));
-  CK(cudaMalloc(&ctx->d_pent, ev.size() * sizeof(PrefEntry)));
+  CK(dev_alloc(&ctx->d_pent, ev.size() * sizeof(PrefEntry)));
   CK(cudaMemcpy(ctx->d_pent, ev.data(), ev.size() * sizeof(PrefEntry), cudaMemcpyHostToDevice));
-  CK(cudaMalloc(&ctx->d_pbytes, bytes.size()));
+  CK(dev_alloc(&ctx->d_pbytes, bytes.size()));
   CK(cudaMemcpy(ctx->d_pbytes, bytes.data(), bytes.size(), cudaMemcpyHostToDevice));
-  CK(cudaMalloc(&ctx->d_poff, size_t(n) * 4));
+  CK(dev_alloc(&ctx->d_poff, size_t(n) * 4));
   CK(cudaMemcpy(ctx->d_poff, poff.data(), size_t(n) * 4, cudaMemcpyHostToDevice));
   ctx->pdir_bits = bits;
   ctx->pmax_probe = max_probe;
@@ -88,7 +88,7 @@ int build_prefilter(oasm_ctx* ctx, const std::vector<char>& pref) {
     bloom[b1 >> 5] |= 1u << (b1 & 31);
     bloom[b2 >> 5] |= 1u << (b2 & 31);
   }
-  CK(cudaMalloc(&ctx->d_pbloom, bloom.size() * 4));
+  CK(dev_alloc(&ctx->d_pbloom, bloom.size() * 4));
   CK(cudaMemcpy(ctx->d_pbloom, bloom.data(), bloom.size() * 4, cudaMemcpyHostToDevice));
   ctx->pbloom_bits = bb;
   return OASM_OK;
@@ -156,7 +156,8 @@ static int build_weighted(oasm_ctx* ctx, std::vector<Bucket>& to, const std::vec
     warps[g].push_back(p);
     used[g] += L;
   }
-  Bucket bk;
+  to.emplace_back();
+  Bucket& bk = to.back();
   bk.W = kWRows;
   bk.algo = kAlgoWeighted;
   bk.gpw = 1;
@@ -197,12 +198,197 @@ static int build_weighted(oasm_ctx* ctx, std::vector<Bucket>& to, const std::vec
     bk.groups.push_back(G);
     rows.insert(rows.end(), wr.begin(), wr.end());
   }
-  CK(cudaMalloc(&bk.d_groups, bk.groups.size() * sizeof(LaneGroup)));
+  CK(dev_alloc(&bk.d_groups, bk.groups.size() * sizeof(LaneGroup)));
   CK(cudaMemcpy(bk.d_groups, bk.groups.data(), bk.groups.size() * sizeof(LaneGroup),
                 cudaMemcpyHostToDevice));
-  CK(cudaMalloc(&bk.d_wrow, rows.size() * sizeof(uint32_t)));
+  CK(dev_alloc(&bk.d_wrow, rows.size() * sizeof(uint32_t)));
   CK(cudaMemcpy(bk.d_wrow, rows.data(), rows.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
-  to.push_back(bk);
+  return OASM_OK;
+}
+
+// A scan class of the given patterns:
+// forward lane groups per word-count class, patterns sorted by length so a
+// group's lanes need similar warm-up.  One-word patterns with K <= 2 form
+// automaton classes (one per K) when there are at least 32 of them; their
+// lanes are packed with up to kMaxSlots patterns whose lengths sum to <= 32
+// (first-fit over lengths in decreasing order).
+static int add_bucket(oasm_ctx* ctx, std::vector<Bucket>& to, int W, int algo,
+                      std::vector<uint32_t> ids) {
+  to.emplace_back();  // (there from the start: what is allocated goes with the context)
+  Bucket& bk = to.back();
+  bk.W = W;
+  bk.algo = algo;
+  std::vector<std::vector<uint32_t>> lanes;  // patterns of each lane
+  if (algo > 0 && algo <= 3) {
+    std::stable_sort(ids.begin(), ids.end(),
+                     [&](uint32_t a0, uint32_t b0) { return ctx->m[a0] > ctx->m[b0]; });
+    std::vector<int> used;
+    for (uint32_t p : ids) {
+      size_t l = 0;
+      while (l < lanes.size() &&
+             !(used[l] + ctx->m[p] <= 32 && lanes[l].size() < size_t(kMaxSlots)))
+        ++l;
+      if (l == lanes.size()) {
+        lanes.emplace_back();
+        used.push_back(0);
+      }
+      lanes[l].push_back(p);
+      used[l] += ctx->m[p];
+    }
+  } else if (algo == 4) {  // two a lane, ended at bits 15 and 31
+    for (size_t i = 0; i < ids.size(); i += 2)
+      lanes.emplace_back(ids.begin() + i, ids.begin() + std::min(i + 2, ids.size()));
+  } else {
+    std::stable_sort(ids.begin(), ids.end(),
+                     [&](uint32_t a0, uint32_t b0) { return ctx->m[a0] < ctx->m[b0]; });
+    for (uint32_t p : ids) lanes.push_back({p});
+  }
+  const size_t RW = size_t(32) * W;  // words per symbol row: [w][lane]
+  std::vector<uint32_t> peq;
+  for (size_t g0 = 0; g0 < lanes.size(); g0 += kLaneGroup) {
+    const int np = int(std::min<size_t>(kLaneGroup, lanes.size() - g0));
+    // a class with 32 or more patterns runs one lane word per lane (idle
+    // lanes in its last group); a smaller one spreads each pattern over lanes
+    const int nseg = ids.size() >= size_t(kLaneGroup) ? 1 : std::max(1, kLaneGroup / np);
+    LaneGroup G;
+    memset(&G, 0, sizeof G);
+    G.nseg = nseg;
+    G.W = W;
+    G.ov = 1;
+    G.nslot = 1;
+    const size_t base = peq.size();
+    peq.resize(base + size_t(256) * RW, 0u);
+    for (int l = 0; l < kLaneGroup; ++l) {
+      const int pi = l / nseg, sg = l % nseg;
+      for (int q = 0; q < kMaxSlots; ++q) G.lastbit[q][l] = 31;
+      for (int q = 0; q + 1 < kMaxSlots; ++q) G.xpat[q][l] = -1;
+      if (pi >= np) {
+        G.pat[l] = -1;
+        G.m[l] = uint8_t(32 * W);
+        G.K[l] = 0;
+        G.seg[l] = 0;
+        continue;
+      }
+      const auto& lp = lanes[g0 + pi];
+      G.nslot = std::max<int>(G.nslot, int(lp.size()));
+      G.pat[l] = int32_t(lp[0]);
+      G.seg[l] = uint8_t(sg);
+      G.K[l] = ctx->K[lp[0]];
+      // Myers lanes are top-aligned (the last row at bit 31 of the top word);
+      // cut-off lanes and automaton lanes start at bit 0
+      int off = (algo != 0) ? 0 : 32 * W - ctx->m[lp[0]];
+      for (size_t q = 0; q < lp.size(); ++q) {
+        const uint32_t p = lp[q];
+        const auto& s = ctx->pats[p];
+        const int m = int(s.size());
+        if (algo == 4) off = 16 * int(q) + 16 - m;
+        if (q > 0) G.xpat[q - 1][l] = int32_t(p);
+        G.m[l] = std::max<uint8_t>(G.m[l], uint8_t(m));
+        G.ov = std::max(G.ov, m + ctx->K[p] - 1);
+        bk.kmax = std::max<int>(bk.kmax, ctx->K[p]);
+        for (int j = 0; j < m; ++j) {
+          const int bit = off + j;
+          peq[base + size_t(s[j]) * RW + size_t(bit >> 5) * 32 + l] |= 1u << (bit & 31);
+        }
+        if (algo > 0 && algo <= 4) {
+          G.first[l] |= 1u << off;
+          G.last[l] |= 1u << (off + m - 1);
+          G.lastbit[q][l] = uint8_t(off + m - 1);
+        }
+        off += m;
+      }
+    }
+    bk.ov_max = std::max(bk.ov_max, G.ov);
+    bk.max_nseg = std::max(bk.max_nseg, nseg);
+    bk.groups.push_back(G);
+  }
+  // untuned default: the Myers/Hyyro one-word scan runs two groups per warp
+  // (measured faster) unless an odd, small group count would leave much of
+  // the last warp idle; the automaton runs one
+  const size_t ng = bk.groups.size();
+  bk.gpw = (algo == 0 && W == 1 && bk.max_nseg == 1 && ng >= 2 && (ng % 2 == 0 || ng >= 7))
+               ? 2 : 1;
+  // (two K = 3 patterns a lane, 55 patterns over 64 MiB of DNA: 8 warps and
+  // 1,024-byte buffers 1.79 ms, 16 and 512 with regions twice as long 1.69)
+  if (algo == 4) bk.warps = 16, bk.chunk = 512, bk.region_scale = 2.0;
+  CK(dev_alloc(&bk.d_groups, bk.groups.size() * sizeof(LaneGroup)));
+  CK(cudaMemcpy(bk.d_groups, bk.groups.data(), bk.groups.size() * sizeof(LaneGroup),
+                cudaMemcpyHostToDevice));
+  if (algo == kAlgoCut) {
+    // the scan stages only word 0 of each lane (rows 1..32) in shared
+    // memory; the whole table stays in global memory for the full form
+    std::vector<uint32_t> w0(bk.groups.size() * size_t(256) * 32);
+    for (size_t g = 0; g < bk.groups.size(); ++g)
+      for (size_t c = 0; c < 256; ++c)
+        for (size_t l = 0; l < 32; ++l)
+          w0[(g * 256 + c) * 32 + l] = peq[g * 256 * RW + c * RW + l];
+    CK(dev_alloc(&bk.d_peq_hi, peq.size() * 4));
+    CK(cudaMemcpy(bk.d_peq_hi, peq.data(), peq.size() * 4, cudaMemcpyHostToDevice));
+    peq.swap(w0);
+  }
+  if (algo >= 3 && algo <= 4) {
+    // automaton classes of K = 2 and 3: each symbol row holds the match masks B
+    // and B >> 1
+    std::vector<uint32_t> two(bk.groups.size() * size_t(256) * 64);
+    for (size_t r = 0; r < bk.groups.size() * size_t(256); ++r)
+      for (size_t l = 0; l < 32; ++l) {
+        two[r * 64 + l] = peq[r * 32 + l];
+        two[r * 64 + 32 + l] = peq[r * 32 + l] >> 1;
+      }
+    peq.swap(two);
+  }
+  CK(dev_alloc(&bk.d_peq, peq.size() * 4));
+  CK(cudaMemcpy(bk.d_peq, peq.data(), peq.size() * 4, cudaMemcpyHostToDevice));
+  return OASM_OK;
+}
+
+// Cost of a one-word Myers/Hyyro class of x patterns.
+static double words_cost(size_t x) {
+  const size_t L = size_t(kLaneGroup);
+  return group_cost(1, 0) * (x >= L ? double((x + L - 1) / L) : x ? 1.0 / double(L / x) : 0.0);
+}
+
+// Scan classes of the patterns that `skip` leaves, for steps without the gram
+// index or beside it.
+static int add_classes(oasm_ctx* ctx, std::vector<Bucket>& to, const std::vector<char>& skip,
+                       bool beside_index) {
+  for (int W = 1; W <= kMaxW; ++W) {
+    std::vector<uint32_t> ids;
+    for (uint32_t p = 0; p < ctx->n_pat; ++p)
+      if ((ctx->m[p] + 31) / 32 == W && !skip[p]) ids.push_back(p);
+    if (W == 1 && !ctx->cfg.myers_only) {
+      for (int K = 0; K <= 2; ++K) {
+        std::vector<uint32_t> kid, others;
+        for (uint32_t p : ids) (ctx->K[p] == K ? kid : others).push_back(p);
+        if (kid.size() >= size_t(kLaneGroup)) {
+          int rc = add_bucket(ctx, to, 1, 1 + K, kid);
+          if (rc) return rc;
+          ids.swap(others);
+        }
+      }
+    }
+    // beside the gram index: patterns of up to 16 symbols with K = 3, two a
+    // lane, where that is cheaper than one a lane (55 of them over 64 MiB of
+    // DNA: 2.85 ms as two Myers/Hyyro groups, 1.69 as one of these)
+    if (beside_index && W == 1) {
+      std::vector<uint32_t> kid, others;
+      for (uint32_t p : ids) (ctx->K[p] == 3 && ctx->m[p] <= 16 ? kid : others).push_back(p);
+      if (kid.size() > size_t(kLaneGroup) &&
+          double((kid.size() + 63) / 64) * group_cost(1, 4) + words_cost(others.size()) <
+              words_cost(ids.size())) {
+        int rc = add_bucket(ctx, to, 1, 4, kid);
+        if (rc) return rc;
+        ids.swap(others);
+      }
+    }
+    if (ids.empty()) continue;
+    // multi-word classes of 32 or more patterns (dictionary mapping) run the
+    // cut-off form of the scan unless every word is asked for
+    const int algo = (W >= 2 && ids.size() >= size_t(kLaneGroup) && !ctx->cfg.full_words)
+                         ? kAlgoCut : 0;
+    int rc = add_bucket(ctx, to, W, algo, ids);
+    if (rc) return rc;
+  }
   return OASM_OK;
 }
 
@@ -212,9 +398,9 @@ int build_tables(oasm_ctx* ctx) {
   for (uint32_t p = 0; p < n; ++p)
     std::copy(ctx->pats[p].begin(), ctx->pats[p].end(),
               bytes.begin() + size_t(p) * OASM_MAX_PATTERN_LEN);
-  CK(cudaMalloc(&ctx->d_bytes, bytes.size()));
-  CK(cudaMalloc(&ctx->d_m, n));
-  CK(cudaMalloc(&ctx->d_K, n));
+  CK(dev_alloc(&ctx->d_bytes, bytes.size()));
+  CK(dev_alloc(&ctx->d_m, n));
+  CK(dev_alloc(&ctx->d_K, n));
   // (on the context's stream, which the kernel that reads them runs on)
   CK(cudaMemcpyAsync(ctx->d_bytes, bytes.data(), bytes.size(), cudaMemcpyHostToDevice,
                      ctx->stream));
@@ -222,7 +408,7 @@ int build_tables(oasm_ctx* ctx) {
   CK(cudaMemcpy(ctx->d_K, ctx->K.data(), n, cudaMemcpyHostToDevice));
   // reversed, bottom-aligned Peq (verification pass): [p][256][4], made on the
   // device (4 KiB per pattern would otherwise cross the link)
-  CK(cudaMalloc(&ctx->d_peq_rev, size_t(n) * 256 * 4 * sizeof(uint32_t)));
+  CK(dev_alloc(&ctx->d_peq_rev, size_t(n) * 256 * 4 * sizeof(uint32_t)));
   CK(launch_peq(ctx->d_bytes, ctx->d_m, n, ctx->d_peq_rev, true, ctx->stream));
   ctx->mem_off.resize(n);
   uint32_t off = 0;
@@ -231,154 +417,12 @@ int build_tables(oasm_ctx* ctx) {
     off += ctx->K[p] + 1u;
   }
   ctx->mem_stride = off;
-  CK(cudaMalloc(&ctx->d_mem_off, size_t(n) * 4));
+  CK(dev_alloc(&ctx->d_mem_off, size_t(n) * 4));
   CK(cudaMemcpy(ctx->d_mem_off, ctx->mem_off.data(), size_t(n) * 4, cudaMemcpyHostToDevice));
 
-  // forward lane groups per word-count class, patterns sorted by length so a
-  // group's lanes need similar warm-up.  One-word patterns with K <= 2 form
-  // automaton classes (one per K) when there are at least 32 of them; their
-  // lanes are packed with up to kMaxSlots patterns whose lengths sum to <= 32
-  // (first-fit over lengths in decreasing order).
-  auto add_bucket = [&](std::vector<Bucket>& to, int W, int algo,
-                        std::vector<uint32_t> ids) -> int {
-    Bucket bk;
-    bk.W = W;
-    bk.algo = algo;
-    std::vector<std::vector<uint32_t>> lanes;  // patterns of each lane
-    if (algo > 0 && algo <= 3) {
-      std::stable_sort(ids.begin(), ids.end(),
-                       [&](uint32_t a0, uint32_t b0) { return ctx->m[a0] > ctx->m[b0]; });
-      std::vector<int> used;
-      for (uint32_t p : ids) {
-        size_t l = 0;
-        while (l < lanes.size() &&
-               !(used[l] + ctx->m[p] <= 32 && lanes[l].size() < size_t(kMaxSlots)))
-          ++l;
-        if (l == lanes.size()) {
-          lanes.emplace_back();
-          used.push_back(0);
-        }
-        lanes[l].push_back(p);
-        used[l] += ctx->m[p];
-      }
-    } else if (algo == 4) {  // two a lane, ended at bits 15 and 31
-      for (size_t i = 0; i < ids.size(); i += 2)
-        lanes.emplace_back(ids.begin() + i, ids.begin() + std::min(i + 2, ids.size()));
-    } else {
-      std::stable_sort(ids.begin(), ids.end(),
-                       [&](uint32_t a0, uint32_t b0) { return ctx->m[a0] < ctx->m[b0]; });
-      for (uint32_t p : ids) lanes.push_back({p});
-    }
-    const size_t RW = size_t(32) * W;  // words per symbol row: [w][lane]
-    std::vector<uint32_t> peq;
-    for (size_t g0 = 0; g0 < lanes.size(); g0 += kLaneGroup) {
-      const int np = int(std::min<size_t>(kLaneGroup, lanes.size() - g0));
-      // a class with 32 or more patterns runs one lane word per lane (idle
-      // lanes in its last group); a smaller one spreads each pattern over lanes
-      const int nseg = ids.size() >= size_t(kLaneGroup) ? 1 : std::max(1, kLaneGroup / np);
-      LaneGroup G;
-      memset(&G, 0, sizeof G);
-      G.nseg = nseg;
-      G.W = W;
-      G.ov = 1;
-      G.nslot = 1;
-      const size_t base = peq.size();
-      peq.resize(base + size_t(256) * RW, 0u);
-      for (int l = 0; l < kLaneGroup; ++l) {
-        const int pi = l / nseg, sg = l % nseg;
-        for (int q = 0; q < kMaxSlots; ++q) G.lastbit[q][l] = 31;
-        for (int q = 0; q + 1 < kMaxSlots; ++q) G.xpat[q][l] = -1;
-        if (pi >= np) {
-          G.pat[l] = -1;
-          G.m[l] = uint8_t(32 * W);
-          G.K[l] = 0;
-          G.seg[l] = 0;
-          continue;
-        }
-        const auto& lp = lanes[g0 + pi];
-        G.nslot = std::max<int>(G.nslot, int(lp.size()));
-        G.pat[l] = int32_t(lp[0]);
-        G.seg[l] = uint8_t(sg);
-        G.K[l] = ctx->K[lp[0]];
-        // Myers lanes are top-aligned (the last row at bit 31 of the top word);
-        // cut-off lanes and automaton lanes start at bit 0
-        int off = (algo != 0) ? 0 : 32 * W - ctx->m[lp[0]];
-        for (size_t q = 0; q < lp.size(); ++q) {
-          const uint32_t p = lp[q];
-          const auto& s = ctx->pats[p];
-          const int m = int(s.size());
-          if (algo == 4) off = 16 * int(q) + 16 - m;
-          if (q > 0) G.xpat[q - 1][l] = int32_t(p);
-          G.m[l] = std::max<uint8_t>(G.m[l], uint8_t(m));
-          G.ov = std::max(G.ov, m + ctx->K[p] - 1);
-          bk.kmax = std::max<int>(bk.kmax, ctx->K[p]);
-          for (int j = 0; j < m; ++j) {
-            const int bit = off + j;
-            peq[base + size_t(s[j]) * RW + size_t(bit >> 5) * 32 + l] |= 1u << (bit & 31);
-          }
-          if (algo > 0 && algo <= 4) {
-            G.first[l] |= 1u << off;
-            G.last[l] |= 1u << (off + m - 1);
-            G.lastbit[q][l] = uint8_t(off + m - 1);
-          }
-          off += m;
-        }
-      }
-      bk.ov_max = std::max(bk.ov_max, G.ov);
-      bk.max_nseg = std::max(bk.max_nseg, nseg);
-      bk.groups.push_back(G);
-    }
-    // untuned default: the Myers/Hyyro one-word scan runs two groups per warp
-    // (measured faster) unless an odd, small group count would leave much of
-    // the last warp idle; the automaton runs one
-    const size_t ng = bk.groups.size();
-    bk.gpw = (algo == 0 && W == 1 && bk.max_nseg == 1 && ng >= 2 && (ng % 2 == 0 || ng >= 7))
-                 ? 2 : 1;
-    // (two K = 3 patterns a lane, 55 patterns over 64 MiB of DNA: 8 warps and
-    // 1,024-byte buffers 1.79 ms, 16 and 512 with regions twice as long 1.69)
-    if (algo == 4) bk.warps = 16, bk.chunk = 512, bk.region_scale = 2.0;
-    CK(cudaMalloc(&bk.d_groups, bk.groups.size() * sizeof(LaneGroup)));
-    CK(cudaMemcpy(bk.d_groups, bk.groups.data(), bk.groups.size() * sizeof(LaneGroup),
-                  cudaMemcpyHostToDevice));
-    if (algo == kAlgoCut) {
-      // the scan stages only word 0 of each lane (rows 1..32) in shared
-      // memory; the whole table stays in global memory for the full form
-      std::vector<uint32_t> w0(bk.groups.size() * size_t(256) * 32);
-      for (size_t g = 0; g < bk.groups.size(); ++g)
-        for (size_t c = 0; c < 256; ++c)
-          for (size_t l = 0; l < 32; ++l)
-            w0[(g * 256 + c) * 32 + l] = peq[g * 256 * RW + c * RW + l];
-      CK(cudaMalloc(&bk.d_peq_hi, peq.size() * 4));
-      CK(cudaMemcpy(bk.d_peq_hi, peq.data(), peq.size() * 4, cudaMemcpyHostToDevice));
-      peq.swap(w0);
-    }
-    if (algo >= 3 && algo <= 4) {
-      // automaton classes of K = 2 and 3: each symbol row holds the match masks B
-      // and B >> 1
-      std::vector<uint32_t> two(bk.groups.size() * size_t(256) * 64);
-      for (size_t r = 0; r < bk.groups.size() * size_t(256); ++r)
-        for (size_t l = 0; l < 32; ++l) {
-          two[r * 64 + l] = peq[r * 32 + l];
-          two[r * 64 + 32 + l] = peq[r * 32 + l] >> 1;
-        }
-      peq.swap(two);
-    }
-    CK(cudaMalloc(&bk.d_peq, peq.size() * 4));
-    CK(cudaMemcpy(bk.d_peq, peq.data(), peq.size() * 4, cudaMemcpyHostToDevice));
-    to.push_back(bk);
-    return OASM_OK;
-  };
-  if (ctx->weighted) {
-    std::vector<char> skip(n, 0), served;
-    int rc = build_weighted(ctx, ctx->buckets, skip);
-    if (rc) return rc;
-    if ((rc = build_grams(ctx, skip, served)) || !ctx->grams.n_pat) return rc;
-    if ((rc = build_weighted(ctx, ctx->grams.rest, served))) return rc;
-    finish_grams(ctx);
-    return OASM_OK;
-  }
-  // patterns for the piece filter instead of the forward scan
-  std::vector<char> pref(n, 0);
+  std::vector<char>& pref = ctx->on_filter;
+  pref.assign(n, 0);
+  if (ctx->weighted) return build_weighted(ctx, ctx->buckets, pref);
   if (ctx->cfg.prefilter_piece) {
     std::vector<const uint8_t*> ptr(n);
     std::vector<uint32_t> len(n), kk(n);
@@ -389,67 +433,50 @@ int build_tables(oasm_ctx* ctx) {
     }
     choose_piece_filter(ptr.data(), len.data(), kk.data(), n, ctx->cfg.prefilter_piece,
                         reinterpret_cast<uint8_t*>(pref.data()));
-  }
-  if (ctx->cfg.prefilter_piece) {
-    int rc = build_prefilter(ctx, pref);
+    const int rc = build_prefilter(ctx, pref);
     if (rc) return rc;
   }
-  // scan classes of the patterns that `skip` leaves
-  // cost of a one-word Myers/Hyyro class of x patterns
-  auto words_cost = [&](size_t x) {
-    const size_t L = size_t(kLaneGroup);
-    return group_cost(1, 0) * (x >= L ? double((x + L - 1) / L) : x ? 1.0 / double(L / x) : 0.0);
-  };
-  auto add_classes = [&](std::vector<Bucket>& to, const std::vector<char>& skip,
-                         bool rest) -> int {
-    for (int W = 1; W <= kMaxW; ++W) {
-      std::vector<uint32_t> ids;
-      for (uint32_t p = 0; p < n; ++p)
-        if ((ctx->m[p] + 31) / 32 == W && !skip[p]) ids.push_back(p);
-      if (W == 1 && !ctx->cfg.myers_only) {
-        for (int K = 0; K <= 2; ++K) {
-          std::vector<uint32_t> kid, rest;
-          for (uint32_t p : ids) (ctx->K[p] == K ? kid : rest).push_back(p);
-          if (kid.size() >= size_t(kLaneGroup)) {
-            int rc = add_bucket(to, 1, 1 + K, kid);
-            if (rc) return rc;
-            ids.swap(rest);
-          }
-        }
-      }
-      // beside the gram index: patterns of up to 16 symbols with K = 3, two a
-      // lane, where that is cheaper than one a lane (55 of them over 64 MiB of
-      // DNA: 2.85 ms as two Myers/Hyyro groups, 1.69 as one of these)
-      if (rest && W == 1) {
-        std::vector<uint32_t> kid, others;
-        for (uint32_t p : ids) (ctx->K[p] == 3 && ctx->m[p] <= 16 ? kid : others).push_back(p);
-        if (kid.size() > size_t(kLaneGroup) &&
-            double((kid.size() + 63) / 64) * group_cost(1, 4) + words_cost(others.size()) <
-                words_cost(ids.size())) {
-          int rc = add_bucket(to, 1, 4, kid);
-          if (rc) return rc;
-          ids.swap(others);
-        }
-      }
-      if (ids.empty()) continue;
-      // multi-word classes of 32 or more patterns (dictionary mapping) run the
-      // cut-off form of the scan unless every word is asked for
-      const int algo = (W >= 2 && ids.size() >= size_t(kLaneGroup) && !ctx->cfg.full_words)
-                           ? kAlgoCut : 0;
-      int rc = add_bucket(to, W, algo, ids);
-      if (rc) return rc;
-    }
-    return OASM_OK;
-  };
-  int rc = add_classes(ctx->buckets, pref, false);
-  if (rc) return rc;
+  return add_classes(ctx, ctx->buckets, pref, false);
+}
+
+static int index_tables(oasm_ctx* ctx) {
   std::vector<char> served;
-  if ((rc = build_grams(ctx, pref, served))) return rc;
-  if (!ctx->grams.n_pat) return OASM_OK;
-  for (uint32_t p = 0; p < n; ++p) served[p] |= pref[p];
-  if ((rc = add_classes(ctx->grams.rest, served, true))) return rc;
-  finish_grams(ctx);
+  int rc = build_grams(ctx, ctx->on_filter, served);
+  if (rc || !ctx->grams.n_pat) return rc;
+  for (uint32_t p = 0; p < ctx->n_pat; ++p) served[p] |= ctx->on_filter[p];
+  rc = ctx->weighted ? build_weighted(ctx, ctx->grams.rest, served)
+                     : add_classes(ctx, ctx->grams.rest, served, true);
+  if (!rc) finish_grams(ctx);
+  return rc;
+}
+
+int build_index(oasm_ctx* ctx) {
+  int rc = index_tables(ctx);
+  if (rc == OASM_ENOMEM) rc = OASM_OK, ctx->grams.n_pat = 0;
+  if (rc || ctx->grams.n_pat) return rc;
+  drop_grams(ctx);
+  ctx->err.clear();
   return OASM_OK;
+}
+
+void free_buckets(std::vector<Bucket>& bs) {
+  for (Bucket& b : bs)
+    for (void* p : {static_cast<void*>(b.d_groups), static_cast<void*>(b.d_peq),
+                    static_cast<void*>(b.d_peq_hi), static_cast<void*>(b.d_wrow)})
+      if (p) cudaFree(p);
+  bs.clear();
+}
+
+void drop_grams(oasm_ctx* ctx) {
+  Grams& gr = ctx->grams;
+  free_buckets(gr.rest);
+  for (const void* p : {static_cast<const void*>(gr.scan.bits), static_cast<const void*>(gr.scan.dir),
+                        static_cast<const void*>(gr.t.entries),
+                        static_cast<const void*>(gr.t.peq_fwd),
+                        static_cast<const void*>(gr.susp.p), static_cast<const void*>(gr.longs.p),
+                        static_cast<const void*>(gr.ctr.p)})
+    if (p) cudaFree(const_cast<void*>(p));
+  gr = Grams();
 }
 
 StepParams make_params(oasm_ctx* ctx, const WorkItem* d_items, uint32_t n_items, int sb, int kb,

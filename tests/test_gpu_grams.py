@@ -237,3 +237,54 @@ def test_the_set_of_ends_fits_each_step(piece):
         assert step(big)[1] >= 1 << 21
     finally:
         B.oasm_destroy(ctx)
+
+
+@pytest.mark.parametrize("piece,costs,scan", [(0, None, 0), (4, None, 0), (0, (1, 2, 2), 0),
+                                              (0, None, 1)])
+def test_memory_for_the_index_is_not_needed(piece, costs, scan):
+    """Each device allocation of a context and its first steps fails in turn,
+    once.  Those of the index only cost the index, and a step's own take its
+    memory; a context that finds no room for anything else is not created, and
+    a step of one without an index fails and is there to be run again."""
+    rng = np.random.default_rng(895 + piece)
+    pats, ks, text = dictionary(rng, 256 if piece else 4, N_PAT, 12, 70, 100_003,
+                                lambda m: m // 10)
+    want = oracle_rows(pats, ks, text, costs=costs)
+
+    def run(fail_at):
+        made = {"created": False, "failed_steps": 0}
+        B.oasm_selftest_alloc(fail_at)
+        try:
+            ctx = B.oasm_create(pats, ks, None, {"prefilter_piece": piece, "full_words": scan},
+                                costs=costs)
+        except B.OasmError as e:
+            assert e.code == B.OASM_ENOMEM
+            return made
+        try:
+            made["created"] = True
+            made["allocs"] = B.oasm_selftest_alloc(0)
+            B.oasm_selftest_alloc(max(fail_at - made["allocs"], 0))
+            sid, out = B.oasm_open_stream(ctx), []
+            for part in np.split(text, [text.size // 50]):
+                B.oasm_feed(ctx, sid, part)
+                try:
+                    out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 1))
+                except B.OasmError as e:
+                    assert e.code == B.OASM_ENOMEM
+                    made["failed_steps"] += 1
+                    out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 1))
+            made["step_allocs"] = B.oasm_selftest_alloc(0)
+            assert canon(gpu_rows(np.concatenate(out))) == want
+            return made
+        finally:
+            B.oasm_selftest_alloc(0)
+            B.oasm_destroy(ctx)
+
+    whole = run(0)
+    runs = [run(i) for i in range(1, whole["allocs"] + whole["step_allocs"] + 1)]
+    needed = [r["created"] for r in runs].index(True)  # allocations that a context needs
+    assert all(r["created"] for r in runs[needed:])
+    if scan:
+        assert needed == whole["allocs"] and any(r["failed_steps"] for r in runs)
+    else:
+        assert needed <= whole["allocs"] - 4 and not any(r["failed_steps"] for r in runs)
