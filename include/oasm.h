@@ -561,6 +561,8 @@ typedef struct {
                                 arrival that never comes: the wait runs out */
     uint32_t no_small;       /* 1: as on a device that the launch of small steps does
                                 not fit: every step runs as separate launches */
+    uint64_t gram_slice;     /* symbols of a step's text that share a buffer of the gram
+                                index (a multiple of 4,096; at most 256 slices a step) */
 } oasm_limits;
 int oasm_selftest_limits(oasm_ctx *ctx, const oasm_limits *l);
 

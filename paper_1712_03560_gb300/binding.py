@@ -89,7 +89,7 @@ class oasm_routes(ctypes.Structure):
 
 class oasm_limits(ctypes.Structure):
     _fields_ = [("small_hits", ctypes.c_uint64), ("barrier_polls", ctypes.c_uint32),
-                ("no_small", ctypes.c_uint32)]
+                ("no_small", ctypes.c_uint32), ("gram_slice", ctypes.c_uint64)]
 
 
 class oasm_costs(ctypes.Structure):

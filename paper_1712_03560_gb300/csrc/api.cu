@@ -907,6 +907,7 @@ int oasm_selftest_limits(oasm_ctx* ctx, const oasm_limits* l) {
   if (rc) return rc;
   ctx->limits = Limits();
   ctx->many_hits = false;
+  if (l && l->gram_slice) ctx->limits.gram_slice = (size_t(l->gram_slice) + 4095) & ~size_t(4095);
   ctx->small_blocks = l && l->no_small ? 0 : small_step_grid(ctx->num_sms);
   if (!l) return OASM_OK;
   if (l->small_hits) ctx->limits.small_hits = l->small_hits;

@@ -206,6 +206,7 @@ struct Limits {
   // 288).
   unsigned long long small_cand = 1ull << 22, small_hits = 1ull << 18;
   BarrierBound barrier;
+  size_t gram_slice = size_t(1) << 27;  // arena symbols per slice of suspects
 };
 
 struct StepPlan {

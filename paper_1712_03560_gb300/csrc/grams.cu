@@ -441,7 +441,7 @@ __device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, c
   for (uint32_t h = hit; h; h &= h - 1)
     if (!insert_key(S, ((s.arena0 + uint64_t(s.lo + __ffs(h) - 1)) << 24) | s.pat, &full))
       hit &= ~(h & (0u - h));
-  if (full) atomicOr(&P.ctr->overflow, 1u | 32u);
+  if (full) atomicOr(&P.ctr->overflow, kSetOverflow | 1u);
   __syncwarp();
   const int nf = __popc(hit);
   int incl = nf;
@@ -457,7 +457,7 @@ __device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, c
     o = atomicAdd(&P.ctr->n_cand, (unsigned long long)tot);
     const unsigned long long filled =
         atomicAdd(&P.ctr->n_gram, (unsigned long long)tot) + (unsigned long long)tot;
-    if (filled > (S.mask + 1) / 4) atomicOr(&P.ctr->overflow, 1u | 32u);
+    if (filled > (S.mask + 1) / 4) atomicOr(&P.ctr->overflow, kSetOverflow | 1u);
   }
   o = __shfl_sync(kFull, o, 0) + unsigned(incl - nf);
   bool over = false;
@@ -473,6 +473,12 @@ __device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, c
     }
   }
   if (over) atomicOr(&P.ctr->overflow, 1u);
+}
+
+// Ends found from here on would be too few, or not once each.  (Candidates over
+// their buffer are counted on, for the next run's.)  Called by whole warps.
+__device__ __forceinline__ bool incomplete(const StepParams& P) {
+  return __any_sync(kFull, P.ctr->overflow & (kSetOverflow | kGramOverflow));
 }
 
 constexpr int kEndThreads = 256;
@@ -502,7 +508,8 @@ __global__ void __launch_bounds__(kEndThreads)
   const unsigned long long n = min(C->n_susp, cap);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
-  if (__any_sync(kFull, P.ctr->overflow & 1u)) return;
+  if (incomplete(P)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&P.ctr->n_slices, 1ull);
   unsigned long long *pairs = list[0][warp], *passed = list[1][warp];
   int np = 0, nq = 0;  // listed suspects of this warp: whose pair, whose sides matched
   // the ends of the last 32 (or all) suspects that passed
@@ -601,7 +608,7 @@ __global__ void __launch_bounds__(kEndThreads)
     gram_long_kernel(const StepParams P, const GramTables G, const GramCounters* C,
                      const unsigned long long* __restrict__ longs, unsigned long long cap_long,
                      const EndSet S) {
-  if (__any_sync(kFull, P.ctr->overflow & 1u)) return;
+  if (incomplete(P)) return;
   unsigned long long n[3], warps = 0;
 #pragma unroll
   for (int l = 0; l < 3; ++l) {

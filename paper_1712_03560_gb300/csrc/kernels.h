@@ -114,7 +114,6 @@ cudaError_t prepare_prefilter_kernel(int max_smem_bytes);
 constexpr int kGramThreads = 1024;            // threads of an index scan block (one per SM)
 constexpr uint32_t kGramMaxWords = 45056;     // 176 KiB of table bits in shared memory
 constexpr int kGramLens = 6;                  // key lengths of an index
-constexpr unsigned kGramOverflow = 1u << 7;   // StepCounters::overflow: suspects over capacity
 // odd multipliers: table bits of hashed keys, directory
 constexpr uint32_t kGramBitMul = 0x9E3779B1u, kGramDirMul = 0x2C1B3C6Du;
 struct GramLen {             // one key length: the first symbols of a gram

@@ -105,6 +105,10 @@ struct WinHdr {
 
 constexpr unsigned int kWaitOver = 1u << 16, kSmallLeft = 1u << 17;
 
+// The (end, pattern) set over its fill, and the gram index's suspects over their
+// buffer, as bits of StepCounters::overflow.
+constexpr unsigned int kSetOverflow = 1u << 5, kGramOverflow = 1u << 7;
+
 // Per-step device counters; copied back to the host after every step.
 struct StepCounters {
   unsigned long long n_cand;
@@ -122,6 +126,7 @@ struct StepCounters {
   unsigned int pad;
   unsigned long long n_pref;  // distinct (pattern, end) pairs the prefilter proposed
   unsigned long long n_gram;  // distinct (pattern, end) pairs the gram index found
+  unsigned long long n_slices;  // slices of the text that they stand for
 };
 
 // Piece filter (exact pigeonhole prefilter).  A pattern with K errors split

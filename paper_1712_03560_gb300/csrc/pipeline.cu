@@ -1029,7 +1029,7 @@ __device__ __noinline__ void decide_window(const StepParams& P, const unsigned l
 // of four pairs on their way at a time, and the rest of the work is a function
 // of its own, for the registers (8 M pairs: one at a time 56 us, this form 28; the pass that also cleared the windows 47).
 __device__ void finalize_body(const StepParams& P, const unsigned long long* S) {
-  if (P.ctr->overflow) return;
+  if (P.ctr->overflow & ~4u) return;  // (records over their buffer are counted on)
   constexpr int kAhead = 4;
   const unsigned long long npairs = (unsigned long long)P.n_items * P.n_pat;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;

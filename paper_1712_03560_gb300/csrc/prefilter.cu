@@ -29,7 +29,6 @@ namespace oasm {
 namespace {
 
 constexpr unsigned kCandOverflow = 1u;
-constexpr unsigned kSetOverflow = 1u << 5;
 constexpr unsigned long long kEmpty = ~0ull;
 constexpr int kSetProbes = 64;
 

@@ -25,16 +25,15 @@ constexpr size_t kDirectRecords = 4096;  // records such a step writes to the ho
 // over 4,096 symbols 168 -> 76, 300 DNA patterns over 100,000 125 -> 98, over
 // 30,000 105 -> 92 (left to the scan).
 constexpr double kGramClk = 40e3, kScanLaunchClk = 6e3, kGramPlanClk = 30.0;
-constexpr size_t kGramSlice = size_t(1) << 27;  // arena symbols per slice of suspects
 constexpr double kGramMaxRate = 2.0;            // suspects per symbol that a slice may hold
 
 // Slices of the arena that share the suspect buffer: their symbols (a
 // multiple of a tile's, at most 256 slices) and count.
-static size_t gram_slice(const StepPlan& pl) {
-  return std::max(kGramSlice, (pl.arena_bytes / 256 + 4095) & ~size_t(4095));
+static size_t gram_slice(const oasm_ctx* ctx, const StepPlan& pl) {
+  return std::max(ctx->limits.gram_slice, (pl.arena_bytes / 256 + 4095) & ~size_t(4095));
 }
-static size_t gram_slices(const StepPlan& pl) {
-  return (pl.arena_bytes + gram_slice(pl) - 1) / gram_slice(pl);
+static size_t gram_slices(const oasm_ctx* ctx, const StepPlan& pl) {
+  return (pl.arena_bytes + gram_slice(ctx, pl) - 1) / gram_slice(ctx, pl);
 }
 
 // The part of the (end, pattern) set that a step uses and so clears: a power of
@@ -315,9 +314,9 @@ static int enqueue_search(oasm_ctx* ctx, StepPlan& pl, const StepParams& P,
   }
   if (pl.grams) {
     Grams& gr = ctx->grams;
-    const size_t slices = gram_slices(pl);
+    const size_t slices = gram_slices(ctx, pl);
     // whole tiles (the end padding is longer than a tile and holds no text)
-    const size_t n_tiles = (pl.arena_bytes - 16) / 512, slice = gram_slice(pl) / 512;
+    const size_t n_tiles = (pl.arena_bytes - 16) / 512, slice = gram_slice(ctx, pl) / 512;
     topo_add(slices);
     CK(cudaMemsetAsync(gr.ctr.p, 0, slices * sizeof(GramCounters), s));
     for (size_t q = 0; q < slices; ++q) {
@@ -457,7 +456,7 @@ static int ensure_h_out(oasm_ctx* ctx, int b, size_t n) {
 // many as cost what the index saves (about 30 clocks each).
 static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) {
   const Grams& gr = ctx->grams;
-  const double syms = double(std::min(pl.arena_bytes, gram_slice(pl)));
+  const double syms = double(std::min(pl.arena_bytes, gram_slice(ctx, pl)));
   const double top = std::min(kGramMaxRate, gr.saved_clk / 30.0);
   const double rate = most ? top : std::min(top, 1.5 * gr.rate + 0.03);
   return size_t(syms * rate) + (size_t(1) << 14);
@@ -633,12 +632,22 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
   if (c.overflow & 64u)
     return fail(ctx, OASM_ECUDA, "internal error: an ordered record fell outside its segment");
   *overflow = c.overflow != 0;
+  // n of the slices that the index got to, for all of them (at most 8 times
+  // what there was room for: the rest may hold fewer)
+  const size_t slices = pl.grams ? gram_slices(ctx, pl) : 1;
+  const auto of_all = [&](unsigned long long n, size_t room) {
+    if (c.n_slices == 0 || c.n_slices >= slices) return size_t(n);
+    return std::max(size_t(n), std::min(size_t(double(n) * double(slices) / double(c.n_slices)),
+                                        8 * room));
+  };
   if (*overflow) {
     pl.no_small = pl.no_small || left;
     pl.from = kFromText;
     // grow what was too small; the step is re-run from unchanged state
     if ((c.overflow & 1u) || c.n_cand > ctx->cand.cap)
-      if ((rc = ensure(ctx, ctx->cand, size_t(c.n_cand * 5 / 4 + 1024), "candidates"))) return rc;
+      if ((rc = ensure(ctx, ctx->cand, of_all(c.n_cand, ctx->cand.cap) * 5 / 4 + 1024,
+                       "candidates")))
+        return rc;
     if ((c.overflow & 2u) || c.n_hits > P.cap_hits) {
       const size_t want = size_t(c.n_hits * 5 / 4 + 1024);
       if ((rc = ensure(ctx, ctx->keys, want, "hit keys"))) return rc;
@@ -647,8 +656,8 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     if ((c.overflow & 4u) || c.n_out > P.cap_out)
       if ((rc = ensure_out(ctx, size_t(c.n_out * 5 / 4 + 1024), pl.ordered))) return rc;
     bool leave = false;
-    if (c.overflow & 32u) {  // the (end, pattern) set filled up: room for 4x its inserts
-      const size_t want = std::max(size_t(c.n_pref + c.n_gram) * 4, 2 * pl.set_len);
+    if (c.overflow & kSetOverflow) {  // the (end, pattern) set filled up: room for 4x its inserts
+      const size_t want = std::max(of_all(c.n_pref + c.n_gram, pl.set_len / 4) * 4, 2 * pl.set_len);
       rc = ensure_pow2(ctx, ctx->pset, want, "piece filter set", pl.grams);
       leave = rc == OASM_ENOMEM && pl.grams;
       if (rc && !leave) return rc;
@@ -835,7 +844,7 @@ int step_begin(oasm_ctx* ctx) {
   if (pl.grams) {
     rc = ctx->pset.p ? OASM_OK
                      : ensure_pow2(ctx, ctx->pset, 4 * ctx->cand.cap, "piece filter set", true);
-    if (!rc) rc = ensure(ctx, ctx->grams.ctr, gram_slices(pl), "gram counters", true);
+    if (!rc) rc = ensure(ctx, ctx->grams.ctr, gram_slices(ctx, pl), "gram counters", true);
     if (!rc) rc = ensure_grams(ctx, gram_capacity(ctx, pl, false));
     if (rc && (rc != OASM_ENOMEM || (rc = leave_grams(ctx, pl)))) return rc;
   }

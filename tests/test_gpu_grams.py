@@ -288,3 +288,28 @@ def test_memory_for_the_index_is_not_needed(piece, costs, scan):
         assert needed == whole["allocs"] and any(r["failed_steps"] for r in runs)
     else:
         assert needed <= whole["allocs"] - 4 and not any(r["failed_steps"] for r in runs)
+
+
+def test_a_first_step_sizes_its_buffers_in_few_runs():
+    """Many slices of a step's text, each with more ends than the buffers hold
+    at first: the counts of one run size them for the whole step."""
+    rng = np.random.default_rng(899)
+    pats, ks, text = dictionary(rng, 4, N_PAT, 24, 60, 1_500_000, lambda m: m // 10)
+    one = W.DNA[rng.integers(0, 4, size=40)]
+    pats, ks = pats + [one] * 300, ks + [4] * 300
+    for at in range(500, text.size - 100, 2_000):
+        text[at:at + one.size] = one
+    scan, _ = run_gpu(pats, ks, text, cfg={"full_words": 1, "myers_only": 1})
+    ctx = B.oasm_create(pats, ks)
+    try:
+        B.oasm_selftest_limits(ctx, gram_slice=1 << 15)
+        sid = B.oasm_open_stream(ctx)
+        B.oasm_feed(ctx, sid, text)
+        rows = gpu_rows(B.oasm_flush(ctx, sid, end_of_stream=True))
+        st = B.oasm_get_stats(ctx)
+    finally:
+        B.oasm_destroy(ctx)
+    assert canon(rows) == canon(scan)
+    # suspects; ends and their set, 31 times what there was room for, twice (8
+    # times at most); hits; records
+    assert st["candidates"] > 1_000_000 and st["reruns"] <= 5
