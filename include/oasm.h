@@ -473,6 +473,10 @@ typedef struct {
                              ran out */
     uint64_t set_slots;   /* slots cleared of the set of (pattern, end) pairs that the
                              piece filter and the gram index fill */
+    uint64_t index_steps; /* steps that the gram index served */
+    uint64_t index_left;  /* steps it was left for: a text too repetitive for it, or no
+                             device memory for its buffers (the 32 steps after such a
+                             one do not try it) */
 } oasm_routes;
 int oasm_get_routes(oasm_ctx *ctx, oasm_routes *out);
 

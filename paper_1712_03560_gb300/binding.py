@@ -84,7 +84,8 @@ class oasm_stats(ctypes.Structure):
 
 
 class oasm_routes(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_uint64) for n in ("small_steps", "small_left", "set_slots")]
+    _fields_ = [(n, ctypes.c_uint64) for n in ("small_steps", "small_left", "set_slots",
+                                                "index_steps", "index_left")]
 
 
 class oasm_limits(ctypes.Structure):

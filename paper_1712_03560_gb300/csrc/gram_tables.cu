@@ -152,7 +152,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   // The filter's patterns are taken all or none: one that is left keeps the
   // whole filter pass (4,096 patterns over 128 MiB with one filter pattern left
   // by a limit per pattern: 10.4 ms a step, against 3.6 ms with all taken).
-  double ends_clk = 0, pref_clk = 0, pref_rate = 0;
+  double ends_clk = 0, pref_clk = 0, pref_rate = 0, pref_looks = 0;
   bool pref_left = false;
   std::vector<double> ps, w, scratch;
   std::vector<uint8_t> sym;
@@ -189,7 +189,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
       }
       return at;
     };
-    double best = 1e30, best_q = 0;
+    double best = 1e30, best_q = 0, best_look = 0;
     int best_b = 0, best_h = 0;
     bool best_edit = false;
     // (a) E + 1 pieces of h symbols, two by two: a pair of them holds at most
@@ -207,6 +207,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
           double key = 1;
           for (int i = 0; i < kb; ++i) key *= ps[y + i];
           cost += key * kLookup + w[x] * (paired(t, E) ? kPair : kEnds);
+          best_look += key;
         }
         best = cost;
         best_h = h;
@@ -230,6 +231,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
           best_at = at;
           best_edit = true;
           best_q = q;
+          best_look = look;
         }
       }
     }
@@ -244,6 +246,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     gr.n_pat += 1;
     if (!pref[p]) ends_clk += best;
     (pref[p] ? pref_rate : gr.rate) += best_q;
+    (pref[p] ? pref_looks : gr.looks) += best_look;
     // a gram for pattern symbols [from, to)
     auto put = [&](uint64_t sym8, int len, int from, int to, int pair) {
       if (from > 32 || m - to > 32) gr.t.any_long = 1;
@@ -289,6 +292,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   } else {
     ends_clk += pref_clk;
     gr.rate += pref_rate;
+    gr.looks += pref_looks;
   }
   auto none = [&]() {
     served.assign(n, 0);

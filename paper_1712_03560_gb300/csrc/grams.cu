@@ -33,6 +33,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kQueue = 64;  // table hits, and suspects, buffered per warp
+constexpr uint32_t kLookReport = 1024;  // compared entries that a warp reports at a time
 
 // ------------------------------------------------------------------- scan
 // 2-bit symbols: (byte >> shift) & 3, 16 of them to a word.
@@ -90,7 +91,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
   }
   __syncthreads();
   int hn = 0, qn = 0;  // queued table hits and suspects of this warp
-  bool dead = false;   // the suspect buffer is full
+  uint32_t looked = 0;  // entries that it compared since it last said so
+  bool dead = false;   // the suspect buffer is full, or the text is not for the index
   auto flush = [&]() {
     __syncwarp();
     unsigned long long base = 0;
@@ -139,6 +141,19 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
       if (lane >= d) incl += x;
     }
     const uint32_t total = __shfl_sync(kFull, incl, 31);
+    looked += total;
+    if (looked >= kLookReport) {
+      // a key that many grams share, in a text full of it, would have every one
+      // of them compared at each of its places (16,384 grams of one key, 1 MiB
+      // of that key: 32 ms, and 2.5 for the scan): see gram_looks in step.cu
+      unsigned long long all = 0;
+      if (lane == 0) all = atomicAdd(&A.ctr_slice->n_look, (unsigned long long)looked) + looked;
+      looked = 0;
+      if (__shfl_sync(kFull, all, 0) > A.cap_look) {
+        dead = true;
+        if (lane == 0) atomicOr(&A.ctr->overflow, kGramDense | 1u);
+      }
+    }
     for (uint32_t base = 0; base < total && !dead; base += 32) {
       const uint32_t item = base + unsigned(lane);
       int own = 0;  // the lane whose look-up found the item: lanes with incl <= item
@@ -478,7 +493,7 @@ __device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, c
 // Ends found from here on would be too few, or not once each.  (Candidates over
 // their buffer are counted on, for the next run's.)  Called by whole warps.
 __device__ __forceinline__ bool incomplete(const StepParams& P) {
-  return __any_sync(kFull, P.ctr->overflow & (kSetOverflow | kGramOverflow));
+  return __any_sync(kFull, P.ctr->overflow & (kSetOverflow | kGramOverflow | kGramDense));
 }
 
 constexpr int kEndThreads = 256;

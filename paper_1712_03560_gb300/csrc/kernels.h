@@ -141,6 +141,7 @@ struct EndSet {              // (arena offset of an end << 24 | pattern) keys; a
 };
 struct GramCounters {        // one per slice of the arena
   unsigned long long n_susp;
+  unsigned long long n_look;     // entries compared with the text
   unsigned long long n_long[3];  // suspects left of patterns of two, three, four words
 };
 struct GramTables {
@@ -161,6 +162,7 @@ struct GramScan {
   unsigned long long t_begin, t_end;  // 512-symbol tiles of this slice
   unsigned long long* susp;  // arena offset of a gram << 24 | entry
   unsigned long long cap_susp;
+  unsigned long long cap_look;
   unsigned long long* longs; // [3][cap_long] suspects left, by word count
   unsigned long long cap_long;
   GramCounters* ctr_slice;

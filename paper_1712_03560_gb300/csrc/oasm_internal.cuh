@@ -105,9 +105,10 @@ struct WinHdr {
 
 constexpr unsigned int kWaitOver = 1u << 16, kSmallLeft = 1u << 17;
 
-// The (end, pattern) set over its fill, and the gram index's suspects over their
-// buffer, as bits of StepCounters::overflow.
-constexpr unsigned int kSetOverflow = 1u << 5, kGramOverflow = 1u << 7;
+// The (end, pattern) set over its fill, the gram index's suspects over their
+// buffer, and its look-ups over what it may save, as bits of
+// StepCounters::overflow.
+constexpr unsigned int kSetOverflow = 1u << 5, kGramOverflow = 1u << 7, kGramDense = 1u << 8;
 
 // Per-step device counters; copied back to the host after every step.
 struct StepCounters {
@@ -119,7 +120,7 @@ struct StepCounters {
   unsigned int overflow;     // bit 0 candidates, 1 hits, 2 outputs, 3 pool,
                              // 5 the prefilter's candidate set (with bit 0),
                              // 6 an ordered record outside its segment (a bug),
-                             // 7 the gram index's suspects (with bit 0),
+                             // 7 the gram index's suspects, 8 its look-ups (with bit 0),
                              // 16 a bounded wait ran out, 17 a small step left its
                              // launch (in the host's copy only)
   unsigned int bar[2];       // barrier arrivals of the hit sort, the record sort

@@ -32,6 +32,7 @@ constexpr double kGramMaxRate = 2.0;            // suspects per symbol that a sl
 static size_t gram_slice(const oasm_ctx* ctx, const StepPlan& pl) {
   return std::max(ctx->limits.gram_slice, (pl.arena_bytes / 256 + 4095) & ~size_t(4095));
 }
+static unsigned long long gram_looks(const oasm_ctx* ctx, const StepPlan& pl);
 static size_t gram_slices(const oasm_ctx* ctx, const StepPlan& pl) {
   return (pl.arena_bytes + gram_slice(ctx, pl) - 1) / gram_slice(ctx, pl);
 }
@@ -326,6 +327,7 @@ static int enqueue_search(oasm_ctx* ctx, StepPlan& pl, const StepParams& P,
       a.t_end = std::min(n_tiles, (q + 1) * slice);
       a.susp = gr.susp.p;
       a.cap_susp = gr.susp.cap;
+      a.cap_look = gram_looks(ctx, pl);
       a.longs = gr.longs.p;
       a.cap_long = gr.longs.cap / 3;
       a.ctr_slice = gr.ctr.p + q;
@@ -462,6 +464,15 @@ static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) 
   return size_t(syms * rate) + (size_t(1) << 14);
 }
 
+// Entries that the index may compare with a slice's text: three times what it
+// expects, or as many as cost half of what it saves (2.2 clocks each); a text of
+// more is left to the scan.
+static unsigned long long gram_looks(const oasm_ctx* ctx, const StepPlan& pl) {
+  const Grams& gr = ctx->grams;
+  const double syms = double(std::min(pl.arena_bytes, gram_slice(ctx, pl)));
+  return (unsigned long long)(syms * (3.0 * gr.looks + gr.saved_clk / 4.4)) + (1ull << 20);
+}
+
 // Room for n suspects of a slice; those of long patterns that a second look
 // keeps are a small part.
 static int ensure_grams(oasm_ctx* ctx, size_t n) {
@@ -497,6 +508,7 @@ static int upload_plan(oasm_ctx* ctx, StepPlan& pl) {
 static int leave_grams(oasm_ctx* ctx, StepPlan& pl) {
   pl.grams = false;
   ctx->grams.off_steps = 32;
+  ctx->routes.index_left += 1;
   ctx->err.clear();
   plan_regions(ctx, pl);
   if (!ctx->n_pref_pat) return OASM_OK;
@@ -655,11 +667,11 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     }
     if ((c.overflow & 4u) || c.n_out > P.cap_out)
       if ((rc = ensure_out(ctx, size_t(c.n_out * 5 / 4 + 1024), pl.ordered))) return rc;
-    bool leave = false;
+    bool leave = (c.overflow & kGramDense) != 0;
     if (c.overflow & kSetOverflow) {  // the (end, pattern) set filled up: room for 4x its inserts
       const size_t want = std::max(of_all(c.n_pref + c.n_gram, pl.set_len / 4) * 4, 2 * pl.set_len);
       rc = ensure_pow2(ctx, ctx->pset, want, "piece filter set", pl.grams);
-      leave = rc == OASM_ENOMEM && pl.grams;
+      leave = leave || (rc == OASM_ENOMEM && pl.grams);
       if (rc && !leave) return rc;
       ctx->set_rate = std::max(ctx->set_rate, double(want - 1) / double(pl.arena_bytes));
       fit_set(ctx, pl);
@@ -696,6 +708,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]); ctx->st.filter_ms += ms;
     cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[5]); ctx->st.step_ms += ms;
   }
+  ctx->routes.index_steps += pl.grams;
   if (pl.new_bytes <= kSmallBytes)
     ctx->many_hits = c.n_cand > ctx->limits.small_cand || c.n_hits > ctx->limits.small_hits;
   ctx->st.candidates += c.n_cand;

@@ -313,3 +313,31 @@ def test_a_first_step_sizes_its_buffers_in_few_runs():
     # suspects; ends and their set, 31 times what there was room for, twice (8
     # times at most); hits; records
     assert st["candidates"] > 1_000_000 and st["reruns"] <= 5
+
+
+def test_index_gives_way_to_a_text_of_one_shared_key():
+    """Every piece of every pattern starts with the same four symbols, and the
+    text repeats those: thousands of entries to compare at each of their
+    places, and no suspect."""
+    rng = np.random.default_rng(897)
+    a = np.frombuffer(b"ABCDEF", np.uint8)
+    pats = [np.concatenate([np.concatenate([a[:4], a[4 + rng.integers(0, 2, 4)]])
+                            for _ in range(4)]) for _ in range(2048)]
+    ks = [3] * len(pats)
+    text = np.tile(a[:4], 50_000)
+    text[1_000:1_032] = pats[7]
+    text[150_000:150_032] = pats[8]
+    ctx = B.oasm_create(pats, ks)
+    try:
+        sid = B.oasm_open_stream(ctx)
+        out, routes = [], []
+        for part in np.split(text, [140_000]):
+            B.oasm_feed(ctx, sid, part)
+            out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 1))
+            r = B.oasm_get_routes(ctx)
+            routes.append((r["index_steps"], r["index_left"]))
+    finally:
+        B.oasm_destroy(ctx)
+    want = oracle_rows(pats, ks, text)
+    assert canon(gpu_rows(np.concatenate(out))) == want and {r[0] for r in want} >= {7, 8}
+    assert routes == [(0, 1), (0, 1)]
