@@ -210,6 +210,13 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
         t[5] = nx.y;
       }
     }
+    // positions of the tile that hold text (behind the last item lies what an
+    // earlier, longer step or another buffer left there)
+    uint32_t own = 0xffffu;
+    if (tile >= A.text_end / 512) {
+      const long long at = (long long)(A.text_end - tile * 512) - lane * 16;
+      own = at >= 16 ? own : at > 0 ? (1u << at) - 1u : 0u;
+    }
 #pragma unroll 1
     for (int l = 0; l < A.n_len; ++l) {
       const GramLen& g = A.len[l];
@@ -229,7 +236,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
         const uint32_t w = bits_s[g.word0 + (h >> 5)];
         acc = __funnelshift_r(acc, __funnelshift_r(w, w, h), 1);
       }
-      uint32_t hits = acc >> 16;
+      uint32_t hits = (acc >> 16) & own;
       unsigned m;
       while ((m = __ballot_sync(kFull, hits != 0)) != 0) {
         if (hn > kQueue - 32) look_up();

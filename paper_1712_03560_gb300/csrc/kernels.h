@@ -160,6 +160,7 @@ struct GramScan {
   const GramEntry* entries;
   const uint8_t* arena;
   unsigned long long t_begin, t_end;  // 512-symbol tiles of this slice
+  unsigned long long text_end;        // arena offset after the last item's text
   unsigned long long* susp;  // arena offset of a gram << 24 | entry
   unsigned long long cap_susp;
   unsigned long long cap_look;

@@ -34,7 +34,7 @@ static size_t gram_slice(const oasm_ctx* ctx, const StepPlan& pl) {
 }
 static unsigned long long gram_looks(const oasm_ctx* ctx, const StepPlan& pl);
 static size_t gram_slices(const oasm_ctx* ctx, const StepPlan& pl) {
-  return (pl.arena_bytes + gram_slice(ctx, pl) - 1) / gram_slice(ctx, pl);
+  return (pl.arena_bytes - kEndPad + gram_slice(ctx, pl) - 1) / gram_slice(ctx, pl);
 }
 
 // The part of the (end, pattern) set that a step uses and so clears: a power of
@@ -316,15 +316,18 @@ static int enqueue_search(oasm_ctx* ctx, StepPlan& pl, const StepParams& P,
   if (pl.grams) {
     Grams& gr = ctx->grams;
     const size_t slices = gram_slices(ctx, pl);
-    // whole tiles (the end padding is longer than a tile and holds no text)
-    const size_t n_tiles = (pl.arena_bytes - 16) / 512, slice = gram_slice(ctx, pl) / 512;
+    // the tiles that hold text (the end padding is longer than a tile)
+    const WorkItem& last = pl.items.back();
+    const size_t text_end = last.arena_base + size_t(last.e_new - last.base_pos);
+    const size_t n_tiles = (text_end + 511) / 512, slice = gram_slice(ctx, pl) / 512;
     topo_add(slices);
     CK(cudaMemsetAsync(gr.ctr.p, 0, slices * sizeof(GramCounters), s));
     for (size_t q = 0; q < slices; ++q) {
       GramScan a = gr.scan;
       a.arena = ctx->arena.p;
-      a.t_begin = std::min(n_tiles, q * slice);
+      a.t_begin = std::min(n_tiles, std::max(q * slice, kFrontPad / 512));
       a.t_end = std::min(n_tiles, (q + 1) * slice);
+      a.text_end = text_end;
       a.susp = gr.susp.p;
       a.cap_susp = gr.susp.cap;
       a.cap_look = gram_looks(ctx, pl);

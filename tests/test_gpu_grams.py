@@ -96,7 +96,8 @@ def test_index_over_steps_and_streams():
 def test_index_gives_way_on_repetitive_text():
     """Every piece matches nearly everywhere: the suspects outgrow their
     buffer, the step is re-run on the forward scan, and so are the next
-    steps; symbols outside the patterns' alphabet match nothing."""
+    32, then the index is tried again; symbols outside the patterns' alphabet
+    match nothing."""
     rng = np.random.default_rng(840)
     unit = np.frombuffer(b"ACGGTCA", np.uint8)
     pats = [np.roll(np.tile(unit, 5), i % 7)[:25 + i % 9].copy() for i in range(N_PAT)]
@@ -104,20 +105,25 @@ def test_index_gives_way_on_repetitive_text():
     text = np.tile(unit, 24_000)[:90_000].copy()
     text[rng.integers(0, text.size, size=400)] = ord("T")
     text[40_000:40_100] = ord("N")
+    other = W.DNA[rng.integers(0, 4, size=100_000)]
     ctx = B.oasm_create(pats, ks)
     try:
-        out = []
+        out, routes = [], []
         sid = B.oasm_open_stream(ctx)
         for part in np.split(text, [85_000]):
             B.oasm_feed(ctx, sid, part)
             out.append(B.oasm_flush(ctx, sid, end_of_stream=len(out) == 1))
-        st = B.oasm_get_stats(ctx)
+        for part in 33 * [other] + [text[:85_000]]:
+            B.oasm_feed(ctx, sid, part)
+            B.oasm_flush(ctx, sid)
+            r = B.oasm_get_routes(ctx)
+            routes.append((r["index_steps"], r["index_left"]))
     finally:
         B.oasm_destroy(ctx)
     got = [(int(r["pattern_id"]), int(r["decided_at"]), int(r["k"]), int(r["start"]),
             int(r["len"])) for r in np.concatenate(out)]
     assert canon(got) == oracle_rows(pats, ks, text)
-    assert st["reruns"] >= 1
+    assert routes[30:] == [(0, 1), (0, 1), (1, 1), (1, 2)]
 
 
 @pytest.mark.parametrize("costs", [(1, 2, 2), (2, 3, 2), (1, 1, 1), (9, 5, 7)])
