@@ -51,7 +51,7 @@ def run_gpu(patterns, ks, text, rules=None, splits=None, device_feed=False, cfg=
                 out.append(B.oasm_flush(ctx, sid))  # decisions available so far
         out.append(B.oasm_flush(ctx, sid, end_of_stream=True))
         res = np.concatenate(out)
-        return gpu_rows(res), B.oasm_get_stats(ctx)
+        return gpu_rows(res), {**B.oasm_get_stats(ctx), **B.oasm_get_routes(ctx)}
     finally:
         B.oasm_destroy(ctx)
 

@@ -2,7 +2,8 @@
 the text that a piece of a pattern may appear as, and examine only the ends
 they allow.  The records must equal the oracle's element by element, and those
 of the forward scan alone (cfg.full_words = 1 and myers_only = 1 keep every
-pattern on it), at sizes just above those from which the index runs."""
+pattern on it), at sizes just above those from which the index runs; the
+counts of steps that it served or was left for say that it did."""
 import numpy as np
 import pytest
 
@@ -51,9 +52,9 @@ def test_index_equals_oracle_and_scan(case):
     got, st = run_gpu(pats, ks, text)
     scan, st_scan = run_gpu(pats, ks, text, cfg={"full_words": 1, "myers_only": 1})
     assert len(want) > 0 and canon(got) == canon(scan) == want
-    assert runs_index(st, st_scan)
-    dev, _ = run_gpu(pats, ks, text, device_feed=True, cfg={"graphs": 1})
-    assert canon(dev) == want
+    assert runs_index(st, st_scan) and st["index_steps"] == 1 and st_scan["index_steps"] == 0
+    dev, st = run_gpu(pats, ks, text, device_feed=True, cfg={"graphs": 1})
+    assert canon(dev) == want and st["index_steps"] == 1
 
 
 @pytest.mark.parametrize("mode,output", [("ends", "ends"), ("hits", "all_hits")])
@@ -61,8 +62,8 @@ def test_index_raw_outputs(mode, output):
     """Every end with D[e] <= K and every hit of Eq. 2: a missed end shows."""
     rng = np.random.default_rng(820)
     pats, ks, text = dictionary(rng, 4, N_PAT, 20, 60, 100_003, lambda m: m // 10)
-    got, _ = run_gpu(pats, ks, text, {"output": output})
-    assert canon(got) == oracle_rows(pats, ks, text, mode=mode)
+    got, st = run_gpu(pats, ks, text, {"output": output})
+    assert canon(got) == oracle_rows(pats, ks, text, mode=mode) and st["index_steps"] == 1
 
 
 def test_index_over_steps_and_streams():
@@ -73,8 +74,8 @@ def test_index_over_steps_and_streams():
     pats, ks, text = dictionary(rng, 4, N_PAT, 18, 70, 260_011, lambda m: m // 10, copies=6)
     want = oracle_rows(pats, ks, text)
     cuts = [88_001, 88_002, 88_040, 176_500]
-    rows, _ = run_gpu(pats, ks, text, splits=cuts)
-    assert canon(rows) == want
+    rows, st = run_gpu(pats, ks, text, splits=cuts)
+    assert canon(rows) == want and (st["steps"], st["index_steps"]) == (6, 3)
     lens = [1, 5, 63, 64, 65, 127, 1000, 4099, 20_001, 90_000]
     ctx = B.oasm_create(pats, ks, None, {"max_streams": 16})
     try:
@@ -89,6 +90,7 @@ def test_index_over_steps_and_streams():
             got = [(int(r["pattern_id"]), int(r["decided_at"]), int(r["k"]), int(r["start"]),
                     int(r["len"])) for r in res[res["stream_id"] == sid]]
             assert canon(got) == oracle_rows(pats, ks, t)
+        assert B.oasm_get_routes(ctx)["index_steps"] == 1
     finally:
         B.oasm_destroy(ctx)
 
@@ -132,9 +134,10 @@ def test_index_under_edit_costs(costs):
     rng = np.random.default_rng(850)
     pats, ks, text = dictionary(rng, 4, N_PAT, 10, 40, 100_003, lambda m: m // 7)
     got, st = run_gpu(pats, ks, text, costs=costs)
-    assert canon(got) == oracle_rows(pats, ks, text, costs=costs)
-    ends, _ = run_gpu(pats, ks, text, {"output": "ends"}, costs=costs)
+    assert canon(got) == oracle_rows(pats, ks, text, costs=costs) and st["index_steps"] == 1
+    ends, st = run_gpu(pats, ks, text, {"output": "ends"}, costs=costs)
     assert canon(ends) == oracle_rows(pats, ks, text, mode="ends", costs=costs)
+    assert st["index_steps"] == 1
 
 
 def test_index_runs_of_one_symbol():
@@ -143,32 +146,45 @@ def test_index_runs_of_one_symbol():
     rng = np.random.default_rng(860)
     pats, ks = [], []
     for i in range(N_PAT):
-        p = np.repeat(W.DNA[rng.integers(0, 4, size=20)], rng.integers(1, 4, size=20))
-        pats.append(p[:int(rng.integers(14, 32))].copy())
+        p = np.repeat(W.DNA[rng.integers(0, 4, size=60)], rng.integers(1, 4, size=60))
+        pats.append(p[:int(rng.integers(26, 60))].copy())
         ks.append(1 + i % 3)
-    text = np.repeat(W.DNA[rng.integers(0, 4, size=60_000)], rng.integers(1, 4, size=60_000))
+    n = 200_000
+    text = np.repeat(W.DNA[rng.integers(0, 4, size=n)], rng.integers(1, 4, size=n))
     for p, k in zip(pats, ks):
         for cp in W.edit_copies(rng, p, np.full(4, k), W.DNA):
             W.plant(rng, text, cp)
-    got, _ = run_gpu(pats, ks, text)
-    assert canon(got) == oracle_rows(pats, ks, text)
+    got, st = run_gpu(pats, ks, text)
+    assert canon(got) == oracle_rows(pats, ks, text) and st["index_steps"] == 1
 
 
 @pytest.mark.parametrize("piece", [1, 4])
 def test_index_takes_the_piece_filters_patterns(piece):
     """A large step looks the piece filter's patterns up in the index too, or,
-    with a pattern that the index leaves (one repeated symbol), runs the piece
-    filter beside it; small steps of the same stream run the filter."""
+    with patterns that it leaves (a symbol that most of the pattern text is
+    made of), runs the piece filter beside it; small steps of the same stream run the filter.  Half of
+    the patterns have pieces too short for the filter."""
     rng = np.random.default_rng(870 + piece)
-    pats, ks, text = dictionary(rng, 256, N_PAT, 12, 100, 400_003, lambda m: min(8, m // 6))
-    cuts = [390_000, 390_500, 399_990]
+    pats, ks, text = dictionary(rng, 256, N_PAT // 2, 12, 100, 300_003, lambda m: min(8, m // 6))
+    for _ in range(N_PAT // 2):
+        p = rng.permutation(256).astype(np.uint8)[:int(rng.integers(30, 46))]
+        pats, ks = pats + [p], ks + [p.size // 3 - 1]
+        for cp in W.edit_copies(rng, p, rng.integers(0, ks[-1] + 1, size=2),
+                                np.arange(256, dtype=np.uint8)):
+            W.plant(rng, text, cp)
+    assert B.oasm_piece_filter_choice(pats, ks, piece).sum() == N_PAT // 2
+    cuts = [290_000, 290_500, 299_990]
+    proposed = []
     for extra in (False, True):
         if extra:
-            pats = pats + [np.full(40, text[0], np.uint8)]
-            ks = ks + [1]
+            pats = pats + 400 * [np.full(128, text[0], np.uint8)]
+            ks = ks + 400 * [1]
             text[200_000:200_300] = text[0]
-        got, _ = run_gpu(pats, ks, text, splits=cuts, cfg={"prefilter_piece": piece})
+        got, st = run_gpu(pats, ks, text, splits=cuts, cfg={"prefilter_piece": piece})
         assert canon(got) == oracle_rows(pats, ks, text)
+        assert (st["steps"], st["index_steps"]) == (5, 1)
+        proposed.append(st["prefilter_candidates"])
+    assert 0 < 20 * proposed[0] < proposed[1]  # of the small steps; of the large one too
 
 
 def test_index_of_a_few_long_patterns():
@@ -177,7 +193,7 @@ def test_index_of_a_few_long_patterns():
     pats, ks, text = dictionary(rng, 256, 9, 60, 128, 1_000_003, lambda m: 3 + m // 11, copies=40)
     got, st = run_gpu(pats, ks, text)
     scan, st_scan = run_gpu(pats, ks, text, cfg={"full_words": 1})
-    assert runs_index(st, st_scan)
+    assert runs_index(st, st_scan) and st["index_steps"] == 1
     assert canon(got) == canon(scan) == oracle_rows(pats, ks, text)
 
 
@@ -196,7 +212,7 @@ def test_short_patterns_of_three_errors_beside_the_index(short):
     want = oracle_rows(pats, ks, text)
     got, st = run_gpu(pats, ks, text)
     assert canon(got) == want
-    assert st["word_steps"] == (short + 1) // 2 * n
+    assert st["word_steps"] == (short + 1) // 2 * n and st["index_steps"] == 1
 
 
 @pytest.mark.parametrize("piece", [0, 1])

@@ -33,8 +33,9 @@ def test_records_straight_to_the_host_or_copied(records):
     text = np.frombuffer(b"T" * (records * 12), np.uint8).copy()
     for i in range(records):
         text[12 * i:12 * i + 7] = np.frombuffer(b"GATTACA", np.uint8)
-    got, _ = run_gpu([b"GATTACA"], [0], text)
+    got, st = run_gpu([b"GATTACA"], [0], text)
     assert len(got) == records and canon(got) == oracle_rows([b"GATTACA"], [0], text)
+    assert st["small_steps"] == 1 and st["small_left"] == 0
 
 
 def test_many_streams_and_rules_over_steps():
@@ -65,6 +66,7 @@ def test_many_streams_and_rules_over_steps():
             for s, t in zip(sids, texts):
                 rows = gpu_rows(np.array(got[s], dtype=B.HIT_DTYPE))
                 assert canon(rows) == oracle_rows(pats, ks, t, rules)
+            assert B.oasm_get_routes(ctx)["small_steps"] == 7
         finally:
             B.oasm_destroy(ctx)
 
