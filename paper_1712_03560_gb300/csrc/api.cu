@@ -7,12 +7,13 @@
 // stream:
 //   gather -> [gram index ->] scan (one launch per class, of the patterns that
 //   the index leaves where it runs) [-> piece filter]
-//   -> verify -> radix sort -> filter -> finalize -> tails
-// (from verify on in one launch for small steps), then copies the per-step counters and the emitted records back.  If a
-// device buffer was too small, the kernels that change stream state skip
-// their work, the host grows the buffer and re-runs the step from the same
-// (unchanged) state.  This file holds context creation, streams and input,
-// queued output, checkpoints, statistics and the autotuner.
+//   -> verify -> radix sort -> filter -> finalize -> state
+// (from verify on in one launch for small steps), then copies the per-step
+// counters and the emitted records back.  If a device buffer was too small, the
+// kernels that change stream state skip their work, the host grows the buffer
+// and re-runs the step from the same (unchanged) state.  This file holds context
+// creation, streams and input, queued output, checkpoints, statistics and the
+// autotuner.
 #include "context.h"
 
 namespace oasm {

@@ -147,7 +147,8 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
   for (int c = 0; c < 256; ++c) fr[two ? (c >> shift2) & 3 : c] += cnt[c] / tot;
   if (two)
     for (int c = 0; c < 4; ++c) fr[c] = std::max(fr[c], 1e-3);
-  const int cmin = ctx->weighted ? int(std::min({ctx->costs.sub, ctx->costs.ins, ctx->costs.del})) : 1;
+  const oasm_costs& co = ctx->costs;
+  const int cmin = ctx->weighted ? int(std::min({co.sub, co.ins, co.del})) : 1;
   GramList by_len[kMaxKey2 + 1];
   // The filter's patterns are taken all or none: one that is left keeps the
   // whole filter pass (4,096 patterns over 128 MiB with one filter pattern left

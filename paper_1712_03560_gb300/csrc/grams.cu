@@ -26,6 +26,7 @@
 //
 // The cost per text position depends on the number of key lengths and on how
 // often grams appear, not on the number of patterns.
+#include "end_set.cuh"
 #include "kernels.h"
 
 namespace oasm {
@@ -259,31 +260,9 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
 }
 
 // ------------------------------------------------------------------- ends
-__device__ __forceinline__ unsigned long long mix_key(unsigned long long k) {
-  // a 64-bit finaliser (xor-shift-multiply), spreads keys over the table
-  k ^= k >> 33;
-  k *= 0xff51afd7ed558ccdull;
-  k ^= k >> 33;
-  k *= 0xc4ceb9fe1a85ec53ull;
-  k ^= k >> 33;
-  return k;
-}
-
-constexpr int kSetProbes = 64;
-__device__ bool insert_key(const EndSet& S, unsigned long long key, bool* full) {
-  unsigned long long h = mix_key(key) & S.mask;
-  for (int i = 0; i < kSetProbes; ++i) {
-    const unsigned long long prev = atomicCAS(&S.slots[h], ~0ull, key);
-    if (prev == ~0ull) return true;
-    if (prev == key) return false;
-    h = (h + 1) & S.mask;
-  }
-  *full = true;
-  return false;
-}
-
 // D[e] over the span + 1 ends from lo on, from the symbols before them (text
 // is the item's first symbol): bit j of the result is set when D[lo + j] <= E.
+// Two to four words.
 template <int W>
 __device__ uint32_t ends_run(const uint32_t* __restrict__ peq, const uint8_t* __restrict__ text,
                              int64_t lo, int span, int m, int E) {
@@ -302,15 +281,8 @@ __device__ uint32_t ends_run(const uint32_t* __restrict__ peq, const uint8_t* __
 #pragma unroll 4
   for (int i = 0; i < n; ++i) {
     const uint32_t* row = peq + size_t(t[i]) * 4;
-    uint32_t eq[W];
-    if (W == 1) {
-      eq[0] = __ldg(row);
-    } else {
-      const uint4 q = __ldg(reinterpret_cast<const uint4*>(row));
-      const uint32_t q4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int w = 0; w < W; ++w) eq[w] = q4[w];
-    }
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(row));
+    const uint32_t eq[4] = {q.x, q.y, q.z, q.w};
     uint32_t php = 0, mhp = 0, carry = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {

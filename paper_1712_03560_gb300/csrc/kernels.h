@@ -84,6 +84,12 @@ struct CopyChunk {
 cudaError_t launch_gather(const CopyChunk* chunks, int n, bool short_chunks, uint8_t* arena,
                           cudaStream_t s);
 
+// Set of (arena offset of an end << 24 | pattern) keys; all ones = empty.
+struct EndSet {
+  unsigned long long* slots;
+  unsigned long long mask;   // capacity - 1 (a power of two)
+};
+
 // Piece filter over segments of the step's text: exact matches of pattern
 // pieces propose candidate ends, deduplicated through an open-addressing set.
 struct PrefArgs {
@@ -96,8 +102,7 @@ struct PrefArgs {
   const Region* segs;            // text segments [a, b) of start positions
   int32_t n_segs;
   int32_t pad;
-  unsigned long long* set;       // (end, pattern) keys; all ones = empty
-  unsigned long long set_mask;   // capacity - 1 (a power of two)
+  EndSet set;
   const uint32_t* bloom;         // 2^bloom_bits bits: two hash bits per piece prefix
   uint32_t bloom_bits;
   int32_t grid;                  // resident blocks (each walks many segments)
@@ -134,10 +139,6 @@ struct GramEntry {           // one gram of a pattern
                              // bits 4-5: symbols of that part - len + 1
   uint8_t len;               // symbols of the gram
   uint32_t lo, hi;           // 16 2-bit symbols (lo), or eight bytes
-};
-struct EndSet {              // (arena offset of an end << 24 | pattern) keys; all ones = empty
-  unsigned long long* slots;
-  unsigned long long mask;   // capacity - 1 (a power of two)
 };
 struct GramCounters {        // one per slice of the arena
   unsigned long long n_susp;

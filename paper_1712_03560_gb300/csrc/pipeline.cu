@@ -1027,7 +1027,8 @@ __device__ __noinline__ void decide_window(const StepParams& P, const unsigned l
 // re-run from unchanged state); a decided window leaves an entry for it.
 // Nearly every pair of a served step is passed by, so a thread has the 12 bytes
 // of four pairs on their way at a time, and the rest of the work is a function
-// of its own, for the registers (8 M pairs: one at a time 56 us, this form 28; the pass that also cleared the windows 47).
+// of its own, for the registers (8 M pairs: one at a time 56 us, this form 28; a
+// pass that also cleared the windows 47).
 __device__ void finalize_body(const StepParams& P, const unsigned long long* S) {
   if (P.ctr->overflow & ~4u) return;  // (records over their buffer are counted on)
   constexpr int kAhead = 4;

@@ -23,41 +23,15 @@
 // of a pair writes a candidate, through a per-warp buffer in shared memory.
 // A set that fills up (or a candidate buffer that overflows) raises an
 // overflow bit: the step is re-run with more room.
+#include "end_set.cuh"
 #include "kernels.h"
 
 namespace oasm {
 namespace {
 
 constexpr unsigned kCandOverflow = 1u;
-constexpr unsigned long long kEmpty = ~0ull;
-constexpr int kSetProbes = 64;
-
-__device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
-  // a 64-bit finaliser (xor-shift-multiply), spreads keys over the table
-  k ^= k >> 33;
-  k *= 0xff51afd7ed558ccdull;
-  k ^= k >> 33;
-  k *= 0xc4ceb9fe1a85ec53ull;
-  k ^= k >> 33;
-  return k;
-}
-
 __device__ __forceinline__ uint32_t dir_hash(uint32_t key, uint32_t bits) {
   return (key * 0x9E3779B1u) >> (32u - bits);
-}
-
-// Inserts key; true if it was not in the set yet.  Sets the overflow bits
-// when no free slot turns up within the probe bound.
-__device__ bool set_insert(const PrefArgs& F, unsigned long long key, bool* full) {
-  unsigned long long h = mix64(key) & F.set_mask;
-  for (int i = 0; i < kSetProbes; ++i) {
-    const unsigned long long prev = atomicCAS(&F.set[h], kEmpty, key);
-    if (prev == kEmpty) return true;
-    if (prev == key) return false;
-    h = (h + 1) & F.set_mask;
-  }
-  *full = true;
-  return false;
 }
 
 __device__ __forceinline__ uint32_t bloom_h2(uint32_t key, uint32_t bits) {
@@ -91,7 +65,7 @@ __device__ void piece_entry(const StepParams& P, const PrefArgs& F, const WorkIt
   for (int64_t e = lo; e <= hi; ++e) {
     const unsigned long long arena_off = w.arena_base + uint64_t(e - w.base_pos);
     bool full = false;
-    const bool fresh = set_insert(F, (arena_off << 24) | pe.pat, &full);
+    const bool fresh = insert_key(F.set, (arena_off << 24) | pe.pat, &full);
     if (full) atomicOr(&P.ctr->overflow, kSetOverflow | kCandOverflow);
     if (!fresh) continue;
     Candidate c;
@@ -122,7 +96,7 @@ __device__ void flush_cands(const StepParams& P, const PrefArgs& F, WarpCands& w
     base = nb ? atomicAdd(&P.ctr->n_cand, (unsigned long long)nb) : 0ull;
     // every distinct proposal counts towards the set's fill
     const unsigned long long filled = atomicAdd(&P.ctr->n_pref, (unsigned long long)nf) + nf;
-    if (filled > (F.set_mask + 1) / 2) atomicOr(&P.ctr->overflow, kSetOverflow | kCandOverflow);
+    if (filled > (F.set.mask + 1) / 2) atomicOr(&P.ctr->overflow, kSetOverflow | kCandOverflow);
   }
   base = __shfl_sync(0xffffffffu, base, 0);
   for (unsigned i = lane; i < nb; i += 32) {

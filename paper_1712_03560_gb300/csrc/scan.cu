@@ -752,8 +752,9 @@ __device__ void scan_dict_nfa(const ScanArgs& A, const char* peq, uint8_t* tbuf,
 // replayed.  Bound by the logic pipe (ncu: 71% busy, 73% of the issue slots),
 // so the shifts go to the other one.  64 MiB of DNA, 55 patterns: two
 // Myers/Hyyro groups 2.85 ms; this form with shifts on the logic pipe 2.0, as
-// it stands 1.69 (the packed automaton above, with its replays, 4.5).  The bits between two patterns may hold anything: the first bit of
-// a pattern is set by E at every level above 0, and by E & B at level 0.
+// it stands 1.69 (the packed automaton above, with its replays, 4.5).  The bits
+// between two patterns may hold anything: the first bit of a pattern is set by E
+// at every level above 0, and by E & B at level 0.
 __device__ void scan_dict_pairs(const ScanArgs& A, const char* peq, uint8_t* tbuf, uint32_t bar0,
                                 const GroupSet<1>& GS, const Region& R, const WorkItem& wi,
                                 int lane) {

@@ -382,8 +382,7 @@ static int enqueue_search(oasm_ctx* ctx, StepPlan& pl, const StepParams& P,
     f.poff = ctx->d_poff;
     f.segs = d_regions + pl.region_off[nb];
     f.n_segs = int(pl.region_off[nb + 1] - pl.region_off[nb]);
-    f.set = ctx->pset.p;
-    f.set_mask = pl.set_len - 1;
+    f.set = EndSet{ctx->pset.p, pl.set_len - 1};
     f.bloom = ctx->d_pbloom;
     f.bloom_bits = ctx->pbloom_bits;
     f.dir_in_smem = (size_t(1) << f.dir_bits) * sizeof(PrefSlot) <= kPrefDirSmem ? 1u : 0u;
@@ -626,10 +625,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
             pl.items.size(), c.overflow, c.n_cand, ctx->cand.cap, c.n_hits,
             (size_t)P.cap_hits, c.n_out, P.cap_out, c.n_pool, P.cap_pool);
   const bool left = (c.overflow & kSmallLeft) != 0;
-  if (pl.small) {
-    ctx->routes.small_steps += 1;
-    ctx->routes.small_left += left || (c.overflow & kWaitOver);
-  }
+  if (pl.small && (left || (c.overflow & kWaitOver))) ctx->routes.small_left += 1;
   if (pl.small && (c.overflow & kWaitOver)) {
     // the launch has changed nothing that outlives the step: once more, with a
     // launch for each phase
@@ -643,7 +639,8 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     return OASM_OK;
   }
   if (c.overflow & kWaitOver)
-    return fail(ctx, OASM_ETIMEOUT, "a bounded wait on the device (a TMA copy, a grid barrier) ran out");
+    return fail(ctx, OASM_ETIMEOUT,
+                "a bounded wait on the device (a TMA copy, a grid barrier) ran out");
   if (c.overflow & 64u)
     return fail(ctx, OASM_ECUDA, "internal error: an ordered record fell outside its segment");
   *overflow = c.overflow != 0;
@@ -711,6 +708,7 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
     cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]); ctx->st.filter_ms += ms;
     cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[5]); ctx->st.step_ms += ms;
   }
+  ctx->routes.small_steps += pl.small;
   ctx->routes.index_steps += pl.grams;
   if (pl.new_bytes <= kSmallBytes)
     ctx->many_hits = c.n_cand > ctx->limits.small_cand || c.n_hits > ctx->limits.small_hits;
@@ -836,9 +834,9 @@ int step_begin(oasm_ctx* ctx) {
   if ((rc = ensure(ctx, ctx->arena, pl.arena_bytes, "text arena"))) return rc;
   if ((rc = ensure(ctx, ctx->pair_pool, pl.items.size() * size_t(ctx->n_pat), "pair table")))
     return rc;
-  if (!ctx->cand.p && (rc = ensure(ctx, ctx->cand, std::max<size_t>(1 << 16, pl.new_bytes / 64), "candidates"))) return rc;
+  const size_t h0 = std::max<size_t>(1 << 16, pl.new_bytes / 64);
+  if (!ctx->cand.p && (rc = ensure(ctx, ctx->cand, h0, "candidates"))) return rc;
   if (!ctx->keys.p) {
-    const size_t h0 = std::max<size_t>(1 << 16, pl.new_bytes / 64);
     if ((rc = ensure(ctx, ctx->keys, h0, "hit keys"))) return rc;
     if ((rc = ensure(ctx, ctx->keys_alt, h0, "hit keys"))) return rc;
   }

@@ -162,8 +162,8 @@ def test_index_runs_of_one_symbol():
 def test_index_takes_the_piece_filters_patterns(piece):
     """A large step looks the piece filter's patterns up in the index too, or,
     with patterns that it leaves (a symbol that most of the pattern text is
-    made of), runs the piece filter beside it; small steps of the same stream run the filter.  Half of
-    the patterns have pieces too short for the filter."""
+    made of), runs the piece filter beside it; small steps of the same stream
+    run the filter.  Half of the patterns have pieces too short for it."""
     rng = np.random.default_rng(870 + piece)
     pats, ks, text = dictionary(rng, 256, N_PAT // 2, 12, 100, 300_003, lambda m: min(8, m // 6))
     for _ in range(N_PAT // 2):

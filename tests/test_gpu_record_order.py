@@ -271,4 +271,5 @@ def test_windows_are_cleared_only_with_their_records_in_order(streams, copies, p
     assert len(want) == 1
     for f, v in zip(("decided_at", "k", "start", "len"), want[0][1:]):
         assert (res[f] == v).all()
-    assert np.unique(res["stream_id"].astype(np.int64) * copies + res["pattern_id"]).size == res.size
+    pairs = res["stream_id"].astype(np.int64) * copies + res["pattern_id"]
+    assert np.unique(pairs).size == res.size
