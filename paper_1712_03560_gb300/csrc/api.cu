@@ -316,6 +316,7 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
     ctx->kmax = std::max<int>(ctx->kmax, int(k[p]));
   }
   int rc = build_tables(ctx);
+  if (!rc) rc = build_index(ctx);
   if (rc) return bail(rc);
   {
     uint64_t h = 1469598103934665603ull;
@@ -338,9 +339,9 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
          ctx->stream_bytes);
     return bail(OASM_ENOMEM);
   }
-  if (dev_alloc(&ctx->d_tails, size_t(S) * ctx->T) != cudaSuccess ||
-      dev_alloc(&ctx->d_hdr, size_t(S) * n_pat * sizeof(WinHdr)) != cudaSuccess ||
-      dev_alloc(&ctx->d_mem, size_t(S) * ctx->mem_stride * sizeof(MemRow)) != cudaSuccess) {
+  if (must_alloc(ctx, &ctx->d_tails, size_t(S) * ctx->T) != cudaSuccess ||
+      must_alloc(ctx, &ctx->d_hdr, size_t(S) * n_pat * sizeof(WinHdr)) != cudaSuccess ||
+      must_alloc(ctx, &ctx->d_mem, size_t(S) * ctx->mem_stride * sizeof(MemRow)) != cudaSuccess) {
     cudaGetLastError();
     fail(ctx, OASM_ENOMEM, "stream state for %u streams does not fit", S);
     return bail(OASM_ENOMEM);
@@ -353,9 +354,10 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   }
   ctx->streams.resize(S);
   for (uint32_t i = 0; i < S; ++i) ctx->free_slots.push(i);
-  if (dev_alloc(&ctx->d_ctr, sizeof(StepCounters)) != cudaSuccess ||
+  if (must_alloc(ctx, &ctx->d_ctr, sizeof(StepCounters)) != cudaSuccess ||
       cudaHostAlloc(&ctx->h_ctr, sizeof(StepCounters), cudaHostAllocDefault) != cudaSuccess ||
-      dev_alloc(&ctx->d_hist, sort_hist_len(ctx->sort_blocks) * sizeof(unsigned int)) != cudaSuccess) {
+      must_alloc(ctx, &ctx->d_hist, sort_hist_len(ctx->sort_blocks) * sizeof(unsigned int)) !=
+          cudaSuccess) {
     cudaGetLastError();
     fail(ctx, OASM_ENOMEM, "step counters");
     return bail(OASM_ENOMEM);
@@ -370,7 +372,6 @@ int oasm_create_weighted(const uint8_t* const* pat, const uint32_t* len, const u
   // the records' copies to the host run on their own stream, beside the next step
   if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
     return bail(fail(ctx, OASM_ECUDA, "cudaStreamCreate failed"));
-  if ((rc = build_index(ctx))) return bail(rc);
   // the tables' copies and the cleared state are complete before the first
   // step, which runs on a stream that does not wait for the default one
   if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {

@@ -34,7 +34,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kQueue = 64;  // table hits, and suspects, buffered per warp
-constexpr uint32_t kLookReport = 1024;  // compared entries that a warp reports at a time
 
 // ------------------------------------------------------------------- scan
 // 2-bit symbols: (byte >> shift) & 3, 16 of them to a word.
@@ -78,6 +77,22 @@ struct GramWarp {
   uint32_t hit_lo[kQueue], hit_hi[kQueue];
 };
 
+// Counts a warp's look-ups that have many entries to compare; true once a slice
+// has more of them than pay.  A key that many grams share, in a text full of it,
+// would have every one of them compared at each of its places (16,384 grams of
+// one key, 1 MiB of that key: 32 ms, and 2.5 for the scan).  Called by whole
+// warps; a function of its own, for the registers of the scan.
+constexpr uint32_t kLookReport = 256;  // entries of 32 look-ups from which they are counted
+__device__ __noinline__ bool too_dense(GramCounters* c, StepCounters* ctr, unsigned long long cap,
+                                       uint32_t total) {
+  unsigned long long all = 0;
+  const bool first = (threadIdx.x & 31) == 0;
+  if (first) all = atomicAdd(&c->n_look, (unsigned long long)total) + total;
+  const bool over = __shfl_sync(kFull, all, 0) > cap;
+  if (first && over) atomicOr(&ctr->overflow, kGramDense | 1u);
+  return over;
+}
+
 template <bool kTwoBit>
 __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramScan A) {
   extern __shared__ __align__(16) uint32_t bits_s[];
@@ -92,7 +107,6 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
   }
   __syncthreads();
   int hn = 0, qn = 0;  // queued table hits and suspects of this warp
-  uint32_t looked = 0;  // entries that it compared since it last said so
   bool dead = false;   // the suspect buffer is full, or the text is not for the index
   auto flush = [&]() {
     __syncwarp();
@@ -115,10 +129,11 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
     const int i = max(hn - 32, 0) + lane;
     uint32_t first = 0, left = 0, lo = 0, hi = 0;
     unsigned long long pos = 0;
-    if (i < hn) {
+    // (behind the last item's text lies what an earlier, longer step or another
+    // buffer left there)
+    if (i < hn && (pos = Q.hit_pos[i]) < A.text_end << 4) {
       lo = Q.hit_lo[i];
       hi = Q.hit_hi[i];
-      pos = Q.hit_pos[i];
       const GramLen& g = A.len[pos & 15u];
       const uint32_t key = lo & g.mask;
       uint32_t s = (key * kGramDirMul) >> g.dir_shift;
@@ -142,19 +157,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
       if (lane >= d) incl += x;
     }
     const uint32_t total = __shfl_sync(kFull, incl, 31);
-    looked += total;
-    if (looked >= kLookReport) {
-      // a key that many grams share, in a text full of it, would have every one
-      // of them compared at each of its places (16,384 grams of one key, 1 MiB
-      // of that key: 32 ms, and 2.5 for the scan): see gram_looks in step.cu
-      unsigned long long all = 0;
-      if (lane == 0) all = atomicAdd(&A.ctr_slice->n_look, (unsigned long long)looked) + looked;
-      looked = 0;
-      if (__shfl_sync(kFull, all, 0) > A.cap_look) {
-        dead = true;
-        if (lane == 0) atomicOr(&A.ctr->overflow, kGramDense | 1u);
-      }
-    }
+    if (total >= kLookReport) dead = too_dense(A.ctr_slice, A.ctr, A.cap_look, total);
     for (uint32_t base = 0; base < total && !dead; base += 32) {
       const uint32_t item = base + unsigned(lane);
       int own = 0;  // the lane whose look-up found the item: lanes with incl <= item
@@ -211,13 +214,6 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
         t[5] = nx.y;
       }
     }
-    // positions of the tile that hold text (behind the last item lies what an
-    // earlier, longer step or another buffer left there)
-    uint32_t own = 0xffffu;
-    if (tile >= A.text_end / 512) {
-      const long long at = (long long)(A.text_end - tile * 512) - lane * 16;
-      own = at >= 16 ? own : at > 0 ? (1u << at) - 1u : 0u;
-    }
 #pragma unroll 1
     for (int l = 0; l < A.n_len; ++l) {
       const GramLen& g = A.len[l];
@@ -237,7 +233,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
         const uint32_t w = bits_s[g.word0 + (h >> 5)];
         acc = __funnelshift_r(acc, __funnelshift_r(w, w, h), 1);
       }
-      uint32_t hits = (acc >> 16) & own;
+      uint32_t hits = acc >> 16;
       unsigned m;
       while ((m = __ballot_sync(kFull, hits != 0)) != 0) {
         if (hn > kQueue - 32) look_up();

@@ -142,8 +142,8 @@ struct GramEntry {           // one gram of a pattern
 };
 struct GramCounters {        // one per slice of the arena
   unsigned long long n_susp;
-  unsigned long long n_look;     // entries compared with the text
   unsigned long long n_long[3];  // suspects left of patterns of two, three, four words
+  unsigned long long n_look;     // entries compared with the text, where they are many
 };
 struct GramTables {
   const GramEntry* entries;
@@ -161,14 +161,14 @@ struct GramScan {
   const GramEntry* entries;
   const uint8_t* arena;
   unsigned long long t_begin, t_end;  // 512-symbol tiles of this slice
-  unsigned long long text_end;        // arena offset after the last item's text
   unsigned long long* susp;  // arena offset of a gram << 24 | entry
   unsigned long long cap_susp;
-  unsigned long long cap_look;
   unsigned long long* longs; // [3][cap_long] suspects left, by word count
   unsigned long long cap_long;
   GramCounters* ctr_slice;
   StepCounters* ctr;
+  unsigned long long text_end;  // arena offset after the last item's text
+  unsigned long long cap_look;  // entries compared before the text is too dense
 };
 cudaError_t prepare_gram_kernels();
 // Match masks [n_pat][256][4] from the patterns' bytes ([n_pat][128]): bit j
