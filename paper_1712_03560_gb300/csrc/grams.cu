@@ -498,8 +498,10 @@ __global__ void __launch_bounds__(kEndThreads)
   const unsigned long long n = min(C->n_susp, cap);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
-  if (incomplete(P)) return;
-  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&P.ctr->n_slices, 1ull);
+  if (incomplete(P)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&P.ctr->n_skipped, 1ull);
+    return;
+  }
   unsigned long long *pairs = list[0][warp], *passed = list[1][warp];
   int np = 0, nq = 0;  // listed suspects of this warp: whose pair, whose sides matched
   // the ends of the last 32 (or all) suspects that passed

@@ -127,7 +127,7 @@ struct StepCounters {
   unsigned int pad;
   unsigned long long n_pref;  // distinct (pattern, end) pairs the prefilter proposed
   unsigned long long n_gram;  // distinct (pattern, end) pairs the gram index found
-  unsigned long long n_slices;  // slices of the text that they stand for
+  unsigned long long n_skipped;  // slices of the text that they do not stand for
 };
 
 // Piece filter (exact pigeonhole prefilter).  A pattern with K errors split

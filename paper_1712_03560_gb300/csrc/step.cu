@@ -648,9 +648,8 @@ int finish_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, bool* over
   // what there was room for: the rest may hold fewer)
   const size_t slices = pl.grams ? gram_slices(ctx, pl) : 1;
   const auto of_all = [&](unsigned long long n, size_t room) {
-    if (c.n_slices == 0 || c.n_slices >= slices) return size_t(n);
-    return std::max(size_t(n), std::min(size_t(double(n) * double(slices) / double(c.n_slices)),
-                                        8 * room));
+    const double part = 1.0 - double(c.n_skipped) / double(slices);
+    return std::max(size_t(n), std::min(size_t(double(n) / std::max(part, 1e-3)), 8 * room));
   };
   if (*overflow) {
     pl.no_small = pl.no_small || left;
