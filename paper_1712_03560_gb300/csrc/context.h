@@ -181,7 +181,8 @@ struct Grams {
   GramTables t{};
   GramScan scan{};            // tables; a step adds its text and buffers
   double rate = 0;            // expected suspects per text symbol
-  double looks = 0;           // expected entries compared per text symbol
+  double looks = 0;           // expected entries compared per text symbol,
+  double most_looks = 0;      // and the most that any text can cause
   double clk = 0;             // clocks of an SM per symbol it takes
   double saved_clk = 0;       // and saves, against the forward scan of every pattern
   bool all_pref = false;      // serves every pattern of the piece filter

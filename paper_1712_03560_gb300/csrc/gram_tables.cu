@@ -368,6 +368,7 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
     g.dir_mask = (1u << db) - 1u;
     g.max_probe = 0;
     dir.resize(dir.size() + (size_t(1) << db), make_uint4(0u, 0u, 0u, 0u));
+    uint32_t of_key = 0;  // entries of one key, at most
     for (size_t i = 0; i < list.size();) {
       const uint32_t key = list[i].lo & L.mask, h = (key * g.mul) >> g.shift;
       const uint32_t first = uint32_t(entries.size());
@@ -380,7 +381,9 @@ int build_grams(oasm_ctx* ctx, const std::vector<char>& pref, std::vector<char>&
       }
       dir[g.dir0 + s] = make_uint4(key, first, uint32_t(entries.size()) - first, 0u);
       g.max_probe = std::max(g.max_probe, pr);
+      of_key = std::max(of_key, uint32_t(entries.size()) - first);
     }
+    gr.most_looks += of_key;
     if (!two) false_bits += double(L.distinct) / double(size_t(1) << L.bits);
   }
   a.n_words = uint32_t((bits.size() + 3) & ~size_t(3));

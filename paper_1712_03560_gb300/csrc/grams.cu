@@ -77,11 +77,18 @@ struct GramWarp {
   uint32_t hit_lo[kQueue], hit_hi[kQueue];
 };
 
+// Ends found from here on would be too few, or not once each.  (Candidates over
+// their buffer are counted on, for the next run's.)  Called by whole warps.
+__device__ __forceinline__ bool incomplete(const StepCounters* ctr) {
+  return __any_sync(kFull, ctr->overflow & (kSetOverflow | kGramOverflow | kGramDense));
+}
+
 // Counts a warp's look-ups that have many entries to compare; true once a slice
 // has more of them than pay.  A key that many grams share, in a text full of it,
 // would have every one of them compared at each of its places (16,384 grams of
 // one key, 1 MiB of that key: 32 ms, and 2.5 for the scan).  Called by whole
-// warps; a function of its own, for the registers of the scan.
+// warps; a function of its own, for the registers of the scan.  (In the scan it
+// costs 1 to 2%, so kCounted is left out where the keys bound it well enough.)
 constexpr uint32_t kLookReport = 256;  // entries of 32 look-ups from which they are counted
 __device__ __noinline__ bool too_dense(GramCounters* c, StepCounters* ctr, unsigned long long cap,
                                        uint32_t total) {
@@ -93,7 +100,7 @@ __device__ __noinline__ bool too_dense(GramCounters* c, StepCounters* ctr, unsig
   return over;
 }
 
-template <bool kTwoBit>
+template <bool kTwoBit, bool kCounted>
 __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramScan A) {
   extern __shared__ __align__(16) uint32_t bits_s[];
   constexpr int kWarps = kGramThreads / 32;
@@ -106,6 +113,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
     for (uint32_t i = threadIdx.x; i < A.n_words / 4; i += kGramThreads) dst[i] = src[i];
   }
   __syncthreads();
+  if (blockIdx.x == 0 && warp == 0 && incomplete(A.ctr) && lane == 0)
+    atomicAdd(&A.ctr->n_skipped, 1ull);  // no ends of this slice will be looked for
   int hn = 0, qn = 0;  // queued table hits and suspects of this warp
   bool dead = false;   // the suspect buffer is full, or the text is not for the index
   auto flush = [&]() {
@@ -157,7 +166,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_scan_kernel(const GramSc
       if (lane >= d) incl += x;
     }
     const uint32_t total = __shfl_sync(kFull, incl, 31);
-    if (total >= kLookReport) dead = too_dense(A.ctr_slice, A.ctr, A.cap_look, total);
+    if (kCounted && total >= kLookReport)
+      dead = too_dense(A.ctr_slice, A.ctr, A.cap_look, total);
     for (uint32_t base = 0; base < total && !dead; base += 32) {
       const uint32_t item = base + unsigned(lane);
       int own = 0;  // the lane whose look-up found the item: lanes with incl <= item
@@ -465,12 +475,6 @@ __device__ __forceinline__ void put_ends(const StepParams& P, const EndSet& S, c
   if (over) atomicOr(&P.ctr->overflow, 1u);
 }
 
-// Ends found from here on would be too few, or not once each.  (Candidates over
-// their buffer are counted on, for the next run's.)  Called by whole warps.
-__device__ __forceinline__ bool incomplete(const StepParams& P) {
-  return __any_sync(kFull, P.ctr->overflow & (kSetOverflow | kGramOverflow | kGramDense));
-}
-
 constexpr int kEndThreads = 256;
 constexpr int kEndList = 64;
 
@@ -498,10 +502,7 @@ __global__ void __launch_bounds__(kEndThreads)
   const unsigned long long n = min(C->n_susp, cap);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
-  if (incomplete(P)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&P.ctr->n_skipped, 1ull);
-    return;
-  }
+  if (incomplete(P.ctr)) return;
   unsigned long long *pairs = list[0][warp], *passed = list[1][warp];
   int np = 0, nq = 0;  // listed suspects of this warp: whose pair, whose sides matched
   // the ends of the last 32 (or all) suspects that passed
@@ -600,7 +601,7 @@ __global__ void __launch_bounds__(kEndThreads)
     gram_long_kernel(const StepParams P, const GramTables G, const GramCounters* C,
                      const unsigned long long* __restrict__ longs, unsigned long long cap_long,
                      const EndSet S) {
-  if (incomplete(P)) return;
+  if (incomplete(P.ctr)) return;
   unsigned long long n[3], warps = 0;
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
@@ -657,12 +658,13 @@ size_t gram_smem(uint32_t n_words) {
 
 cudaError_t prepare_gram_kernels() {
   const int bytes = int(gram_smem(kGramMaxWords));
-  cudaError_t e = cudaFuncSetAttribute(gram_scan_kernel<true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gram_scan_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             bytes);
-  return e;
+  for (auto* kernel : {gram_scan_kernel<false, false>, gram_scan_kernel<false, true>,
+                       gram_scan_kernel<true, false>, gram_scan_kernel<true, true>}) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_peq(const uint8_t* bytes, const uint8_t* len, uint32_t n_pat, uint32_t* peq,
@@ -678,10 +680,9 @@ cudaError_t launch_grams(const StepParams& p, const GramTables& g, const GramSca
   const unsigned long long tiles = a.t_end - a.t_begin;
   const unsigned long long need = (tiles + kGramThreads / 32 - 1) / (kGramThreads / 32);
   const unsigned grid = unsigned(need < (unsigned long long)p.num_sms ? need : p.num_sms);
-  if (a.two_bit)
-    gram_scan_kernel<true><<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
-  else
-    gram_scan_kernel<false><<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
+  auto* scan = a.two_bit ? a.cap_look ? gram_scan_kernel<true, true> : gram_scan_kernel<true, false>
+               : a.cap_look ? gram_scan_kernel<false, true> : gram_scan_kernel<false, false>;
+  scan<<<grid, kGramThreads, gram_smem(a.n_words), s>>>(a);
   gram_ends_kernel<<<p.num_sms * 4, kEndThreads, 0, s>>>(p, g, a.susp, a.ctr_slice, a.cap_susp,
                                                          a.longs, a.cap_long, set);
   if (g.any_long)

@@ -168,7 +168,7 @@ struct GramScan {
   GramCounters* ctr_slice;
   StepCounters* ctr;
   unsigned long long text_end;  // arena offset after the last item's text
-  unsigned long long cap_look;  // entries compared before the text is too dense
+  unsigned long long cap_look;  // entries compared before the text is too dense; 0: any
 };
 cudaError_t prepare_gram_kernels();
 // Match masks [n_pat][256][4] from the patterns' bytes ([n_pat][128]): bit j

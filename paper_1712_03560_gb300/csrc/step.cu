@@ -468,9 +468,11 @@ static size_t gram_capacity(const oasm_ctx* ctx, const StepPlan& pl, bool most) 
 
 // Entries that the index may compare with a slice's text: three times what it
 // expects, or as many as cost half of what it saves (2.2 clocks each); a text of
-// more is left to the scan.
+// more is left to the scan.  0 where no text can cost more than the scan: with
+// few grams to a key, or many patterns.
 static unsigned long long gram_looks(const oasm_ctx* ctx, const StepPlan& pl) {
   const Grams& gr = ctx->grams;
+  if (gr.most_looks * 2.2 <= gr.saved_clk) return 0;
   const double syms = double(std::min(pl.arena_bytes, gram_slice(ctx, pl)));
   return (unsigned long long)(syms * (3.0 * gr.looks + gr.saved_clk / 4.4)) + (1ull << 20);
 }

@@ -368,8 +368,12 @@ static int add_classes(oasm_ctx* ctx, std::vector<Bucket>& to, const std::vector
       }
     }
     // beside the gram index: patterns of up to 16 symbols with K = 3, two a
-    // lane, where that is cheaper than one a lane (55 of them over 64 MiB of
-    // DNA: 2.85 ms as two Myers/Hyyro groups, 1.69 as one of these)
+    // lane, where that is cheaper than one a lane (search for ends over 64 MiB of
+    // DNA with so many of them beside 500 indexed patterns, Myers/Hyyro groups and
+    // this form: 33 2.88 and 1.73 ms, 64 3.10 and 1.81, 65 4.26 and 3.54, 96 4.38
+    // and 3.53, 128 6.50 and 3.54, 192 9.26 and 5.18; up to 32 are one group
+    // either way).  Short patterns with more errors have no such form: 33 with
+    // K = 4 take 3.39 ms, 128 8.1.
     if (beside_index && W == 1) {
       std::vector<uint32_t> kid, others;
       for (uint32_t p : ids) (ctx->K[p] == 3 && ctx->m[p] <= 16 ? kid : others).push_back(p);
