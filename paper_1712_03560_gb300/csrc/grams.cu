@@ -65,8 +65,10 @@ __device__ __forceinline__ void window(const uint32_t (&t)[6], int j, uint32_t& 
 // and compared with the text in full where its table bit and directory slot
 // are found.  Table hits go through a per-warp queue, so that the directory
 // (L2) is read 32 look-ups at a time, and the entries of those look-ups are
-// dealt out one per lane.  Bound by instruction issue and the shared-memory
-// conflicts of the random table reads.
+// dealt out one per lane.  Bound by the look-ups' latency and issue (ncu, 32 MiB
+// of bytes: 61% of the issue slots busy, 31% of the cycles without a warp to
+// issue, 21 of 32 lanes active, shared-memory pipe 53%) and, on 2-bit text, by
+// the shared-memory pipe (65%, L1 74%; 54% of the issue slots); DRAM 4%.
 // (First forms: hashed tables for every gram length, up to 13 symbols, let
 // four positions in ten through to the directory, one look-up per lane and
 // length at a time: 535 us per 64 MiB of DNA against 1,024 patterns; with the
@@ -489,6 +491,9 @@ constexpr int kEndList = 64;
 // or one gram with its edit; that one's suspect finds its end.)  With more than
 // 32 symbols on a side, the 32 next to the gram are matched, and the few
 // suspects that pass are left to gram_long_kernel.
+// Bound by the latency of the suspects' text and masks (ncu, 3 M suspects: 46% of
+// the issue slots busy, half of a warp's cycles wait for a load, 11 of 32 lanes
+// active; gram_long_kernel 27%, 25 lanes; DRAM 4%).
 // (4,096 byte patterns over 32 MiB, 3 M suspects: the whole pattern for every
 // suspect 892 us; its first 32 rows first 576; both sides at once, 9 lanes of a
 // warp busy, 965; two rounds, long patterns apart, 375; this form 331; and 85
