@@ -279,12 +279,13 @@ int enqueue_step(oasm_ctx* ctx, StepPlan& pl, const WorkItem* d_items, const Reg
                       ctx->num_sms, s));
     // where each work item's (stream's) run of records starts
     CK(launch_runs(ks, P, ctx->run_start.p, s));
+    // the stream state last: a step whose records did not fit, or whose sort ran
+    // out of a wait, leaves it as it was (before the copies, which run on another
+    // engine: a kernel between two of them starts 5 us later)
+    CK(launch_state(P, s));
     CK(cudaMemcpyAsync(ctx->h_run_start, ctx->run_start.p,
                        (size_t(n_items) + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                        s));
-    // the stream state last: a step whose records did not fit, or whose sort ran
-    // out of a wait, leaves it as it was
-    CK(launch_state(P, s));
     ctx->st.launches += 4;
   }
   if (tm) CK(record_event(ctx, ctx->ev[5], s));
