@@ -136,3 +136,11 @@ def test_tuning_and_selftest_reject_bad_arguments_on_the_host():
     assert lib.oasm_get_tuning(None, None, 0, ctypes.byref(n)) == B.OASM_EINVAL
     assert lib.oasm_set_tuning(None, None, 0) == B.OASM_EINVAL
     assert lib.oasm_selftest_wait(0, 0, 0) == B.OASM_EINVAL
+
+
+def test_routes_and_limits_reject_a_missing_context():
+    lib = B.load()
+    assert lib.oasm_get_routes(None, ctypes.byref(B.oasm_routes())) == B.OASM_EINVAL
+    assert lib.oasm_selftest_limits(None, None) == B.OASM_EINVAL
+    B.oasm_selftest_alloc(0)
+    assert B.oasm_selftest_alloc(0) == 0  # nothing allocated since the call before
