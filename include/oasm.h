@@ -292,9 +292,9 @@ int oasm_end_stream(oasm_ctx *ctx, uint32_t sid);
  * The sort, and the launch that small steps run after the scan, are
  * cooperative: their blocks (up to four per SM, one per SM) wait for one
  * another at barriers, so such a launch starts when all of them find room
- * beside whatever else runs on the device.  Next to kernels of other streams
- * or contexts that hold SMs for long, a step starts those two later than
- * ordinary launches would. */
+ * beside whatever else runs on the device.  A kernel of another stream or
+ * context that holds every SM delays ordinary launches as long; one that holds
+ * a few SMs delays only these two. */
 int oasm_step(oasm_ctx *ctx);
 
 /* oasm_step in two halves, so that host work can overlap the device.
